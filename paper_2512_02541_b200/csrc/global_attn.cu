@@ -8,11 +8,10 @@
 // loads and first product run under the current item's epilogue.
 // Roles (20 warps):
 //   warps 0-15  softmax.  Warp 8 t + 4 h + q works on query tile t, rows
-//               [32 q + 16 h, 32 q + 16 h + 16), all 128 columns of a key step.
+//               [32 q + 16 h, 32 q + 16 h + 16), all 112 columns of a key step.
 //               It reads tensor memory in the 16-lane shapes, which spread a row
 //               over the four threads of a quad (two rows per thread): a row's
-//               maximum and sums are two shuffles away and every row lives in one
-//               warp.  Four softmax warps per scheduler keep the exponential unit
+//               maximum is two shuffles away and every row lives in one warp.  Four softmax warps per scheduler keep the exponential unit
 //               busy while others wait on tensor memory or barriers.
 //   warp  16    TMA producer: Q tiles once per work item, then the compacted K/V
 //               of the head through a ring of shared-memory stages (128-byte
@@ -23,11 +22,10 @@
 //               accumulators in tensor memory
 //   warp  19    idle (it completes the fifth warpgroup so that registers can
 //               be moved to the softmax warpgroups)
-// Tensor memory per tile: S 128 columns (fp32), P 64 columns (bf16 pairs),
-// O 64 columns (fp32); 512 columns in all.  A softmax thread pulls its 64 scores
-// of S into registers and the warp frees its rows at once, so the next Q K^T runs
-// under the exponentials; P V of step j runs under the softmax of step j+1.  One
-// block of 8 key columns in eight takes its exponentials from a polynomial on
+// Tensor memory per tile (256 columns): two places for S and P that alternate (see kColSOdd), O (64) and the row
+// sums of P (16).  A softmax thread pulls its 56 scores of S into registers and the warp frees its rows at once,
+// so the next Q K^T runs under the exponentials; P V of step j runs under the softmax of step j+1.  Three
+// blocks of 8 key columns in fourteen take their exponentials from a polynomial on
 // the FMA pipe.  The accumulator is rescaled lazily: only when the running
 // maximum grew by more than 2^8 since the last rescale.  The epilogue folds the
 // diagonal and the mean-fill column into the same normalisation:
@@ -47,9 +45,12 @@ namespace {
 
 constexpr int kTileQ = 128;      // query rows per tile
 constexpr int kQTiles = 2;       // tiles per CTA
-constexpr int kTileKV = 128;     // keys per step
+constexpr int kTileKV = 112;     // keys per step
+constexpr int kBlocks = kTileKV / 8;   // blocks of 8 key columns in a step
 constexpr int kHeadDim = 64;
-constexpr uint32_t kTileBytes = kTileKV * kHeadDim * 2;   // 16 KiB: one 128 x 64 bf16 tile
+constexpr uint32_t kTileBytes = kTileQ * kHeadDim * 2;      // 16 KiB: one tile of 128 query rows (or of the queries' own K/V rows); also a ring stage
+constexpr uint32_t kKeyTileBytes = kTileKV * kHeadDim * 2;  // 14 KiB: one tile of keys or values
+constexpr uint32_t kOnesBytes = 2 * 1024;                   // the block of value columns 64..79 (ones_block)
 // K ring and V ring depth.  The subsampled layer runs the same at 2 to 5; frame attention, whose strided key
 // tiles take longer to arrive, gained 6 % from the fourth stage and nothing from a fifth.
 #ifndef AVGGT_STAGES
@@ -61,19 +62,32 @@ constexpr int kSoftmaxWarps = 16;
 constexpr int kTmaWarp = 16;
 constexpr int kMmaWarp = 17;
 constexpr uint32_t kTmemCols = 512;
-constexpr uint32_t kTmemTileStride = 256;   // columns per query tile: S [0,128) P [128,192) O [192,256)
-constexpr uint32_t kColP = 128, kColO = 192;
+// Tensor memory of a query tile (256 columns): scores and probabilities of the even steps of the tile, S at 0 and P at 0
+// (over the scores it was computed from); of the odd steps, S at 64 and P at 112; O at 176, the row sums of P at 240.
+// P of a step and S of the next one never share a column, so a step's Q K^T needs only that the previous step's scores
+// have been read.
+constexpr uint32_t kTmemTileStride = 256;
+constexpr uint32_t kColSOdd = 64, kColPOdd = 112, kColO = 176, kColL = kColO + kHeadDim;
+constexpr int kPvCols = kHeadDim + 16;   // N of P V: the value columns and the block whose first column is all ones
+static_assert(kTileKV <= kColPOdd && kTileKV / 2 <= kColSOdd && kColSOdd + kTileKV <= kColO && kColPOdd + kTileKV / 2 <= kColO &&
+              kColO + kPvCols <= kTmemTileStride, "tensor memory of a tile");
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kRescaleThreshold = 8.0f;   // log2 units
+// The tensor core truncates when it accumulates: a sum of many positive terms comes out short by up to 2^-24 for each of the
+// seven products of a step (measured 1.8e-3 after 4,086 steps, as large as a bf16 rounding step).  Every so many steps the
+// row sums are therefore moved to the next column, to which P V adds exact zeros; what is left of the error is 2.7e-5.
+constexpr int kFlushSteps = 64;
 
-// Of every 8 blocks of 8 key columns, this many take their exponentials from a polynomial on the FMA pipe instead of
-// the special-function unit (which, at 16 results per clock per SM, is the scarcest arithmetic unit of the softmax at
-// head dimension 64).  One in eight measured best: 723 ms on the 800-frame layer against 768 ms with none and 767 ms
-// with two in eight.
-#ifndef AVGGT_POLY_EIGHTHS
-#define AVGGT_POLY_EIGHTHS 1
+// Blocks of 8 key columns (bit b: columns [8 b, 8 b + 8) of a step) whose exponentials come from a polynomial on the
+// FMA pipe instead of the special-function unit, which at 16 results per clock per SM would otherwise set the pace.
+// The polynomial costs more instructions and more energy, and the long launches run at the card's power limit, so the
+// choice that takes the fewest clocks gains least.  137,400 queries x 36,600 keys, 27 launches in a row (clocks per
+// step of 2 x 128 rows x 112 keys; SM clock): no block 23.45 ms (1984; 1.62 GHz), two 22.60 (1809; 1.53), three 22.55
+// (1771; 1.50), five 22.71 (1755; 1.47); a single launch 21.5, 20.1, 19.9, 20.2 ms.
+#ifndef AVGGT_POLY_BLOCKS
+#define AVGGT_POLY_BLOCKS 0x0888
 #endif
-constexpr int kPolyEighths = AVGGT_POLY_EIGHTHS;
+constexpr uint32_t kPolyBlocks = AVGGT_POLY_BLOCKS;
 
 struct AttnArgs {
   Plan pl;
@@ -86,13 +100,14 @@ struct AttnArgs {
   int32_t frame_mode;   // 0: subsampled global attention over the compact keys.  1: frame attention (Sec. 4.2):
                         //    every frame is a problem of its own, keys and values are the frame's own rows of K and V
   int64_t n_keys;       // keys of one problem: M, or the tokens of a frame
-  int32_t n_kv_tiles;   // ceil(n_keys / 128)
+  int32_t n_kv_tiles;   // ceil(n_keys / kTileKV)
   int32_t n_work;       // work items (pairs of query tiles x heads x problems) of the launch; a CTA takes the items
                         // blockIdx.x, blockIdx.x + gridDim.x, ...  (more than one per CTA only in frame attention)
   int32_t pairs;        // pairs of query tiles of one problem
   int32_t use_diag;     // diag on and |D| > 0
   int32_t use_mean;     // mean_fill on and |D| > 0
   float scale_log2;     // softmax scale * log2(e)
+  float inv_scale_log2;
 };
 
 struct __align__(8) Barriers {
@@ -103,8 +118,10 @@ struct __align__(8) Barriers {
   uint64_t v_full[kStages], v_empty[kStages];
   uint64_t s_full[kQTiles];    // MMA -> softmax: S_t(j) is in tensor memory
   uint64_t s_free[kQTiles];    // softmax -> MMA: S_t(j) has been read into registers
-  uint64_t p_full[kQTiles];    // softmax -> MMA: P_t(j) stored (and O_t rescaled)
-  uint64_t o_done[kQTiles];    // MMA -> softmax: P_t(j) V_j has completed
+  uint64_t p_full[kQTiles][2]; // softmax -> MMA: P_t(j) stored (and O_t rescaled); even and odd steps apart, since a warp may
+                               // have finished a step before another warp of its tile has finished the step before
+  uint64_t o_done[kQTiles][2]; // MMA -> softmax: P_t(j) V_j has completed; even and odd steps apart, since the softmax learns of
+                               // P V of step j-2 from the scores of step j only, and of later ones here
   uint64_t mma_idle[kQTiles];  // MMA issuer t -> itself: every tcgen05.mma it issued has completed
   uint32_t tmem_base;
   uint32_t abort_flag;
@@ -142,6 +159,12 @@ __device__ __forceinline__ bool wait_bar(uint64_t* bar, uint32_t parity, Barrier
 __device__ __forceinline__ float max3(float a, float b, float c) {
   float d;
   asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+  return d;
+}
+
+__device__ __forceinline__ float min3(float a, float b, float c) {
+  float d;
+  asm("min.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
   return d;
 }
 
@@ -186,6 +209,7 @@ struct SmemLayout {
   uint8_t* q[kQTiles];
   uint8_t* k;   // kStages tiles
   uint8_t* v;   // kStages tiles
+  uint8_t* ones;   // 16 rows of 64 values: 1 in column 0, else 0 (ones_block)
 };
 
 // The producer and the MMA issuers run with all 32 lanes of their warp in step (every branch
@@ -244,7 +268,7 @@ __device__ __forceinline__ void producer_role(const CUtensorMap* tm_q, const CUt
 #endif
       if (elect_one() && !skip_load) {
         const uint32_t kb = smem_u32(&bars->k_full[stage]);
-        mbar_arrive_expect_tx(kb, kTileBytes);
+        mbar_arrive_expect_tx(kb, it < n_kv ? kKeyTileBytes : kTileBytes);
         if (a.frame_mode) tma_load_2d(smem_u32(sm.k + stage * kTileBytes), tm_k, head * kHeadDim, cta.key_row0 + it * kTileKV, kb);
         else if (it < n_kv) tma_load_3d(smem_u32(sm.k + stage * kTileBytes), tm_kc, 0, it * kTileKV, head, kb);
         else tma_load_2d(smem_u32(sm.k + stage * kTileBytes), tm_k, head * kHeadDim, q0 + (it - n_kv) * kTileQ, kb);
@@ -255,7 +279,7 @@ __device__ __forceinline__ void producer_role(const CUtensorMap* tm_q, const CUt
       if (!ok) break;
       if (elect_one()) {
         const uint32_t vb = smem_u32(&bars->v_full[stage]);
-        mbar_arrive_expect_tx(vb, kTileBytes);
+        mbar_arrive_expect_tx(vb, it < n_kv ? kKeyTileBytes : kTileBytes);
         if (a.frame_mode) tma_load_2d(smem_u32(sm.v + stage * kTileBytes), tm_v, head * kHeadDim, cta.key_row0 + it * kTileKV, vb);
         else if (it < n_kv) tma_load_3d(smem_u32(sm.v + stage * kTileBytes), tm_vc, 0, it * kTileKV, head, vb);
         else tma_load_2d(smem_u32(sm.v + stage * kTileBytes), tm_v, head * kHeadDim, q0 + (it - n_kv) * kTileQ, vb);
@@ -280,34 +304,40 @@ __device__ __forceinline__ void producer_role(const CUtensorMap* tm_q, const CUt
 // ------------------------------------------------------------------ MMA issuer (one warp per query tile)
 // Per tile the order of events is fixed: S_t(j) is read by the softmax (s_free) before P_t(j) is
 // stored (p_full), which precedes the read of S_t(j+1).  The issuer of tile t therefore waits, in
-// turn, for "S_t free and K_{j+1} loaded" -> Q K^T of step j+1, then "P_t(j) stored and V_j
-// loaded" -> P V of step j.  A K or V stage is released when both tiles' issuers have committed
+// turn, for "S_t(j) read and K_{j+1} loaded" -> Q K^T of step j+1, then "P_t(j) stored and V_j
+// loaded" -> P V of step j.  S_t(j+1) overwrites P_t(j-1) and part of S_t(j): the tensor core takes
+// a thread's products in the order they were issued, and P V of step j-1 was issued before.
+// A K or V stage is released when both tiles' issuers have committed
 // their product on it (the empty barriers count two arrivals).
 template <int t>
 __device__ __forceinline__ void issue_qk(const AttnArgs& a, Barriers* bars, uint32_t tmem, uint64_t desc_q, uint32_t k_base,
-                                         int stage, int j) {
+                                         int stage, bool odd) {
   if (elect_one()) {
     constexpr uint32_t idesc = umma_idesc_bf16(kTileQ, kTileKV, false);
     const uint64_t desc_k = umma_desc_sw128(k_base + stage * kTileBytes);
+    const uint32_t d = tmem + t * kTmemTileStride + (odd ? kColSOdd : 0);
 #pragma unroll
-    for (int k = 0; k < kHeadDim / 16; ++k)
-      umma_ss(tmem + t * kTmemTileStride, desc_q + (k * 32 >> 4), desc_k + (k * 32 >> 4), idesc, k > 0);
+    for (int k = 0; k < kHeadDim / 16; ++k) umma_ss(d, desc_q + (k * 32 >> 4), desc_k + (k * 32 >> 4), idesc, k > 0);
     umma_commit(smem_u32(&bars->s_full[t]));
     umma_commit(smem_u32(&bars->k_empty[stage]));
   }
   __syncwarp();
 }
 
+// O_t += P_t V and, as columns 64..79 of the same product, the row sums of P: the descriptor's leading byte offset leads
+// from a slice of 16 keys of the V tile to the ones block, which serves as value columns 64..79 of every slice.
 template <int t>
-__device__ __forceinline__ void issue_pv(const AttnArgs& a, Barriers* bars, uint32_t tmem, uint32_t v_base, int stage, int j) {
+__device__ __forceinline__ void issue_pv(const AttnArgs& a, Barriers* bars, uint32_t tmem, uint32_t v_base, uint32_t ones,
+                                         int stage, bool odd, bool first) {
   if (elect_one()) {
-    constexpr uint32_t idesc = umma_idesc_bf16(kTileQ, kHeadDim, true);
-    const uint64_t desc_v = umma_desc_sw128(v_base + stage * kTileBytes);
+    constexpr uint32_t idesc = umma_idesc_bf16(kTileQ, kPvCols, true);
+    const uint32_t v = v_base + stage * kTileBytes;
+    const uint32_t p = tmem + t * kTmemTileStride + (odd ? kColPOdd : 0);
 #pragma unroll
     for (int k = 0; k < kTileKV / 16; ++k)
-      umma_ts(tmem + t * kTmemTileStride + kColO, tmem + t * kTmemTileStride + kColP + k * 8, desc_v + (k * 2048 >> 4),
-              idesc, (j > 0 || k > 0) ? 1u : 0u);
-    umma_commit(smem_u32(&bars->o_done[t]));
+      umma_ts(tmem + t * kTmemTileStride + kColO, p + k * 8, umma_desc_sw128(v + k * 2048, ones - (v + k * 2048)), idesc,
+              (!first || k > 0) ? 1u : 0u);
+    umma_commit(smem_u32(&bars->o_done[t][odd]));
     umma_commit(smem_u32(&bars->v_empty[stage]));
   }
   __syncwarp();
@@ -318,7 +348,7 @@ __device__ __forceinline__ void mma_issue_loop(const AttnArgs& a, Barriers* bars
   static_assert(kStages >= 2, "the K ring must hold the tile in use and the next one");
   const int n_kv = a.n_kv_tiles;
   const uint64_t desc_q = umma_desc_sw128(smem_u32(sm.q[t]));
-  const uint32_t k_base = smem_u32(sm.k), v_base = smem_u32(sm.v);
+  const uint32_t k_base = smem_u32(sm.k), v_base = smem_u32(sm.v), ones = smem_u32(sm.ones);
   if (n_kv == 0) return;   // no retained keys: the epilogue's two extra columns are the whole layer
 
   // Running over all work items of the CTA: the ring positions of the next K and V tile, and g, the number of key
@@ -334,26 +364,26 @@ __device__ __forceinline__ void mma_issue_loop(const AttnArgs& a, Barriers* bars
     if (n_done > 0 && !wait_bar_warp(&bars->s_free[t], (g - 1) & 1, bars, a, 22 + t, g - 1)) return;
     if (!wait_bar_warp(&bars->k_full[k_stage], k_parity, bars, a, 21, g)) return;
     tc_fence_after();
-    issue_qk<t>(a, bars, tmem, desc_q, k_base, k_stage, 0);
+    issue_qk<t>(a, bars, tmem, desc_q, k_base, k_stage, (g & 1) != 0);
     if (++k_stage == kStages) { k_stage = 0; k_parity ^= 1; }
     for (int j = 0; j < n_kv; ++j) {
       if (j + 1 < n_kv) {
         if (!wait_bar_warp(&bars->s_free[t], (g + j) & 1, bars, a, 22 + t, g + j)) return;
         if (!wait_bar_warp(&bars->k_full[k_stage], k_parity, bars, a, 24 + t, g + j)) return;
         tc_fence_after();
-        issue_qk<t>(a, bars, tmem, desc_q, k_base, k_stage, j + 1);
+        issue_qk<t>(a, bars, tmem, desc_q, k_base, k_stage, ((g + j + 1) & 1) != 0);
         if (++k_stage == kStages) { k_stage = 0; k_parity ^= 1; }
       } else {
         // every Q K^T of this work item has been issued: when they have completed, Q may be overwritten
         if (elect_one()) umma_commit(smem_u32(&bars->q_empty));
         __syncwarp();
       }
-      if (!wait_bar_warp(&bars->p_full[t], (g + j) & 1, bars, a, 26 + t, g + j)) return;
+      if (!wait_bar_warp(&bars->p_full[t][(g + j) & 1], ((g + j) >> 1) & 1, bars, a, 26 + t, g + j)) return;
       if (!wait_bar_warp(&bars->v_full[v_stage], v_parity, bars, a, 28 + t, g + j)) return;
       // the first P V of a work item overwrites O_t: the previous item's epilogue must have read it out
       if (j == 0 && n_done > 0 && !wait_bar_warp(&bars->o_free[t], (n_done - 1) & 1, bars, a, 29, n_done)) return;
       tc_fence_after();
-      issue_pv<t>(a, bars, tmem, v_base, v_stage, j);
+      issue_pv<t>(a, bars, tmem, v_base, ones, v_stage, ((g + j) & 1) != 0, j == 0);
       if (++v_stage == kStages) { v_stage = 0; v_parity ^= 1; }
     }
     // ring positions of the work item's own K/V rows (read by the softmax epilogue, not by any product)
@@ -382,11 +412,8 @@ __device__ __forceinline__ void mma_role(const AttnArgs& a, Barriers* bars, cons
 // 2^x for a pair of values on the FMA pipe.  x = n + r with n = round(x), |r| <= 1/2: adding
 // 1.5 * 2^23 leaves n in the low mantissa bits of the sum; 2^r is a degree-3 minimax polynomial
 // (relative error 7.5e-5, a twenty-sixth of the bf16 rounding step the result goes through);
-// 2^n is applied by adding n to the exponent field.  Valid for x <= 100; x is clamped at -125.
+// 2^n is applied by adding n to the exponent field.  Valid for -126 <= x <= 100; the caller sees to that.
 __device__ __forceinline__ void exp2_poly_pair(uint64_t x2, float& p0, float& p1) {
-  float x0, x1;
-  unpack_f32x2(x2, x0, x1);
-  x2 = pack_f32x2(fmaxf(x0, -125.0f), fmaxf(x1, -125.0f));
   const uint64_t magic = pack_f32x2(12582912.0f, 12582912.0f);
   const uint64_t t = add_f32x2(x2, magic);
   const uint64_t r = sub_f32x2(x2, sub_f32x2(t, magic));
@@ -399,17 +426,13 @@ __device__ __forceinline__ void exp2_poly_pair(uint64_t x2, float& p0, float& p1
   p0 = __uint_as_float(__float_as_uint(q0) + (__float_as_uint(t0) << 23));
   p1 = __uint_as_float(__float_as_uint(q1) + (__float_as_uint(t1) << 23));
 }
+constexpr float kPolyLowest = -125.0f;   // scores are raised to this many log2 units below the reference before the polynomial sees them
 
-// Block b of 8 key columns (0..15 within a step) goes to the polynomial when kPoly of eight blocks do.  The choice
-// depends on the column alone, so a query row's result does not depend on where in a tile the row sits.
-template <int kPoly>
-__device__ __forceinline__ constexpr bool block_uses_poly(int b) { return (((b & 7) + 1) * kPoly) / 8 != ((b & 7) * kPoly) / 8; }
-
-// What a softmax thread knows about itself.  A softmax warp works on 16 query rows of its tile, all 128 columns
+// What a softmax thread knows about itself.  A softmax warp works on 16 query rows of its tile, all columns
 // of a key step: the tensor-memory lanes [32 q + 16 h, 32 q + 16 h + 16) of the tile.  Its tensor-memory
 // accesses use the 16-lane shapes, which spread a row over the four threads of a quad: thread `lane` holds,
 // of every block of 8 columns, columns 2 i and 2 i + 1 (i = lane % 4) of the rows lane / 4 and lane / 4 + 8.
-// A row's maximum and sums therefore take two shuffles within the quad and no shared memory, and every row
+// A row's maximum therefore takes two shuffles within the quad and no shared memory, and every row
 // is handled inside one warp.
 struct SoftmaxThread {
   int t;        // query tile of the CTA
@@ -418,28 +441,46 @@ struct SoftmaxThread {
   int lane;
   int i;        // position in the quad: columns 2 i, 2 i + 1 of every 8
   int r[2];     // the thread's two rows within the tile
-  uint32_t tS, tP, tO;   // tensor-memory addresses (first lane of the warp's 16) of S, P and O of the tile
+  uint32_t base;   // tensor-memory address of the tile's columns, first lane of the warp's 16
 };
 
-// tensor memory <-> registers in the 16-lane shapes (layout above): S (128 columns) and O (64 columns) as 32-bit
-// columns, P as 64 columns of bf16 pairs
-__device__ __forceinline__ void tmem_ld_rows16_c128(uint32_t taddr, uint32_t (&r)[64]) {
+// tensor memory <-> registers in the 16-lane shapes (layout above): S, O and the row sums as 32-bit columns, P as
+// columns of bf16 pairs
+__device__ __forceinline__ void tmem_ld_rows16_c8(uint32_t taddr, uint32_t (&r)[4]) {
+  asm volatile("tcgen05.ld.sync.aligned.16x256b.x1.b32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(taddr)
+               : "memory");
+}
+__device__ __forceinline__ void tmem_st_rows16_c8(uint32_t taddr, const uint32_t (&r)[4]) {
+  asm volatile("tcgen05.st.sync.aligned.16x256b.x1.b32 [%0], {%1, %2, %3, %4};"
+               ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3])
+               : "memory");
+}
+// the 112 score columns of a step in three pieces: 64, 32 and 16
+__device__ __forceinline__ void tmem_ld_rows16_scores(uint32_t taddr, uint32_t (&r)[4 * kBlocks]) {
+  static_assert(kTileKV == 112, "three pieces");
   asm volatile(
-      "tcgen05.ld.sync.aligned.16x256b.x16.b32 "
+      "tcgen05.ld.sync.aligned.16x256b.x8.b32 "
       "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, "
-      "%32, %33, %34, %35, %36, %37, %38, %39, %40, %41, %42, %43, %44, %45, %46, %47, "
-      "%48, %49, %50, %51, %52, %53, %54, %55, %56, %57, %58, %59, %60, %61, %62, %63}, [%64];"
+      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
       : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
         "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
         "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-        "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31]),
-        "=r"(r[32]), "=r"(r[33]), "=r"(r[34]), "=r"(r[35]), "=r"(r[36]), "=r"(r[37]), "=r"(r[38]), "=r"(r[39]),
-        "=r"(r[40]), "=r"(r[41]), "=r"(r[42]), "=r"(r[43]), "=r"(r[44]), "=r"(r[45]), "=r"(r[46]), "=r"(r[47]),
-        "=r"(r[48]), "=r"(r[49]), "=r"(r[50]), "=r"(r[51]), "=r"(r[52]), "=r"(r[53]), "=r"(r[54]), "=r"(r[55]),
-        "=r"(r[56]), "=r"(r[57]), "=r"(r[58]), "=r"(r[59]), "=r"(r[60]), "=r"(r[61]), "=r"(r[62]), "=r"(r[63])
+        "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
       : "r"(taddr)
       : "memory");
+  asm volatile(
+      "tcgen05.ld.sync.aligned.16x256b.x4.b32 "
+      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+      : "=r"(r[32]), "=r"(r[33]), "=r"(r[34]), "=r"(r[35]), "=r"(r[36]), "=r"(r[37]), "=r"(r[38]), "=r"(r[39]),
+        "=r"(r[40]), "=r"(r[41]), "=r"(r[42]), "=r"(r[43]), "=r"(r[44]), "=r"(r[45]), "=r"(r[46]), "=r"(r[47])
+      : "r"(taddr + 64)
+      : "memory");
+  asm volatile("tcgen05.ld.sync.aligned.16x256b.x2.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=r"(r[48]), "=r"(r[49]), "=r"(r[50]), "=r"(r[51]), "=r"(r[52]), "=r"(r[53]), "=r"(r[54]), "=r"(r[55])
+               : "r"(taddr + 96)
+               : "memory");
 }
 __device__ __forceinline__ void tmem_ld_rows16_c64(uint32_t taddr, uint32_t (&r)[32]) {
   asm volatile(
@@ -471,6 +512,12 @@ __device__ __forceinline__ void tmem_st_rows16_p16(uint32_t taddr, const uint32_
                : "memory");
 }
 
+__device__ __forceinline__ void tmem_st_rows16_p8(uint32_t taddr, const uint32_t (&r)[8]) {   // of 2 blocks
+  asm volatile("tcgen05.st.sync.aligned.16x128b.x2.b32 [%0], {%1, %2, %3, %4};"
+               ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3])
+               : "memory");
+}
+
 // value over the four threads of a quad
 __device__ __forceinline__ float quad_max(float v) {
   v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, 1));
@@ -498,125 +545,163 @@ __device__ __forceinline__ void quad_transpose(uint32_t& w0, uint32_t& w1, uint3
 
 // Running state of the thread's two rows (the same in all four threads of a quad, except the partial sums).
 struct RowState {
-  float m_used[2];    // reference maximum of the stored exponentials (log2 units)
-  float l_run[2];     // this thread's part of the sum of the bf16-rounded 2^(scale_log2 * s - m_used): normaliser of O
-  float l_exact[2];   // the same sum without the rounding: log-sum-exp output only
+  float m[2];             // reference maximum of the stored exponentials (log2 units)
+  float neg_m[2];         // -m (0 before the first tile)
+  float jump_above[2];    // raw score above which the reference has to move (-inf before the first tile)
+  float clamp_below[2];   // raw score below which the polynomial is not valid
+  float l_exact[2];       // this thread's part of the sum of the unrounded 2^(scale_log2 * s - m): log-sum-exp output only
 };
 
-// The thread's 64 scores of a key step (register 4 b + 2 hi + e: row hi, column 8 b + 2 i + e) -> bf16
-// probabilities, stored to tensor memory at tP, relative to the rows' reference maxima folded into neg_m2; adds
-// to the sums for the normaliser (of the rounded values) and for the log-sum-exp (unrounded).  Written pair by
-// pair in dependency order; the instruction scheduler interleaves the pairs.
-template <bool kMasked, bool kLse, int kPoly>
-__device__ __forceinline__ void softmax_rows(const uint32_t (&s)[64], uint64_t scale2, const uint64_t (&neg_m2)[2],
-                                             float (&sum_lo)[2], float (&sum_hi)[2], uint64_t (&sum_exact2)[2], uint32_t tP,
-                                             int n_blocks) {
+// Blocks 4 kGroup .. of the thread's scores of a key step (register 4 b + 2 hi + e: row hi, column 8 b + 2 i + e) -> bf16
+// probabilities relative to the rows' reference maxima; kLse: adds the unrounded ones to sum_exact2.  Written pair by pair in
+// dependency order; the instruction scheduler interleaves the pairs.
+template <int kGroup, bool kMasked, bool kLse, uint32_t kPoly>
+__device__ __forceinline__ void exp_group(const uint32_t (&s)[4 * kBlocks], const RowState& st, uint64_t scale2,
+                                          uint64_t (&sum_exact2)[2], uint32_t (&pk)[8], int n_blocks) {
 #pragma unroll
-  for (int g = 0; g < 4; ++g) {
-    uint32_t pk[8];   // P of 32 keys x 2 rows as bf16 pairs
-#pragma unroll
-    for (int n = 0; n < 4; ++n) {
-      // ragged last step: a block of 8 columns with no key in it gives zeros without any arithmetic
-      if (kMasked && 4 * g + n >= n_blocks) {
-        pk[2 * n] = 0u;
-        pk[2 * n + 1] = 0u;
-        continue;
-      }
-#pragma unroll
-      for (int hi = 0; hi < 2; ++hi) {
-        const int c = 4 * (4 * g + n) + 2 * hi;
-        const uint64_t x2 = fma_f32x2(pack_f32x2(__uint_as_float(s[c]), __uint_as_float(s[c + 1])), scale2, neg_m2[hi]);
-        float p0, p1;
-        if (block_uses_poly<kPoly>(4 * g + n)) {
-          exp2_poly_pair(x2, p0, p1);
-        } else {
-          float x0, x1;
-          unpack_f32x2(x2, x0, x1);
-          p0 = ex2_approx(x0);
-          p1 = ex2_approx(x1);
-        }
-        const uint32_t w = pack_bf16x2(p0, p1);
-        pk[2 * n + hi] = w;
-        if (kLse) sum_exact2[hi] = add_f32x2(sum_exact2[hi], pack_f32x2(p0, p1));
-        add_bf16x2_to_f32(w, sum_lo[hi], sum_hi[hi]);
-      }
+  for (int n = 0; n < 4; ++n) {
+    const int b = 4 * kGroup + n;
+    if (b >= kBlocks) break;
+    // ragged last step: a block of 8 columns with no key in it gives zeros without any arithmetic
+    if (kMasked && b >= n_blocks) {
+      pk[2 * n] = 0u;
+      pk[2 * n + 1] = 0u;
+      continue;
     }
-    tmem_st_rows16_p16(tP + g * 16, pk);
+#pragma unroll
+    for (int hi = 0; hi < 2; ++hi) {
+      const int c = 4 * b + 2 * hi;
+      const uint64_t x2 = fma_f32x2(pack_f32x2(__uint_as_float(s[c]), __uint_as_float(s[c + 1])), scale2,
+                                    pack_f32x2(st.neg_m[hi], st.neg_m[hi]));
+      float p0, p1;
+      if ((kPoly >> b) & 1) {
+        exp2_poly_pair(x2, p0, p1);
+      } else {
+        float x0, x1;
+        unpack_f32x2(x2, x0, x1);
+        p0 = ex2_approx(x0);
+        p1 = ex2_approx(x1);
+      }
+      pk[2 * n + hi] = pack_bf16x2(p0, p1);
+      if (kLse) sum_exact2[hi] = add_f32x2(sum_exact2[hi], pack_f32x2(p0, p1));
+    }
   }
 }
 
 // One step of the online softmax of the thread's two rows: S_t(j) in tensor memory -> P_t(j) in tensor
-// memory, running reference maxima and partial sums updated.
+// memory, running reference maxima updated.
 //
-// The 64 scores are pulled into registers at once and the warp's share of S_t is released, so that the next
-// Q K^T runs under this step's exponentials.  The row maxima (two shuffles within the quad) decide whether a
-// reference maximum moves (lazy rescale).
-// j: step within the work item; g: the tile's steps in the CTA's earlier work items.  kPoly: blocks of 8 columns per eight
+// The 56 scores are pulled into registers at once and the warp's share of S_t is released, so that the next
+// Q K^T runs under this step's exponentials.  What the step does next depends on the row maxima only when one of them is
+// far above its reference (lazy rescale: more than 2^8), so the first group of exponentials is computed against the old
+// references while the maxima are being taken, and the common case ends in one vote: no shuffles, no wait for the previous
+// P V (P has a place of its own in alternate steps).  The other case moves the references (a row decides by its own maximum,
+// so its bits do not depend on its neighbours), rescales O and the row sums, raises the scores that lie below the range of
+// the polynomial, and computes the first group again.
+// Measured with the tensor core in the loop but without memory traffic, for 2 tiles x 128 keys on one SM: 2270 clocks
+// with the maxima shuffled, the sums taken by the softmax warps and a wait for P V in every step, 1990 without those
+// waits and sums, 1860 with the vote instead of the shuffles, 1740 with the first group ahead of it, 1695 with the range check
+// of the polynomial in the same vote instead of a clamp per score.
+//
+// j: step within the work item; g: the tile's steps in the CTA's earlier work items.  kPoly: blocks of 8 columns
 // whose exponentials are polynomials.  kLse: also keep the sum of the unrounded exponentials, for the
 // log-sum-exp output.  kMasked: columns >= valid are excluded (valid may be <= 0).
-template <bool kMasked, bool kLse, int kPoly>
-__device__ __forceinline__ bool softmax_step(const SoftmaxThread& me, int j, int g, int valid, float scale_log2,
-                                             RowState& st, Barriers* bars, const AttnArgs& a) {
+template <bool kMasked, bool kLse, uint32_t kPoly>
+__device__ __forceinline__ bool softmax_step(const SoftmaxThread& me, int j, int g, int valid, RowState& st, Barriers* bars,
+                                             const AttnArgs& a) {
   const int gj = g + j;   // this tile's key steps so far, over all work items of the CTA: the phase of the per-step barriers
-  uint32_t s[64];
-  tmem_ld_rows16_c128(me.tS, s);
-  tmem_wait_ld();
+  const bool odd = (gj & 1) != 0;
+  const uint32_t tP = me.base + (odd ? kColPOdd : 0);
+  uint32_t s[4 * kBlocks];
+  tmem_ld_rows16_scores(me.base + (odd ? kColSOdd : 0), s);
+  tmem_wait_ld();     // for the whole warp: lane 0 may speak for it
   tc_fence_before();
-  __syncwarp();
   if (me.lane == 0) mbar_arrive(smem_u32(&bars->s_free[me.t]));
 
   if (kMasked) {
 #pragma unroll
-    for (int c = 0; c < 64; ++c)
+    for (int c = 0; c < 4 * kBlocks; ++c)
       if (8 * (c >> 2) + 2 * me.i + (c & 1) >= valid) s[c] = __float_as_uint(-INFINITY);
   }
-  float alpha[2];
-  bool jump_any = false;
-#pragma unroll
-  for (int hi = 0; hi < 2; ++hi) {
-    float mx = fmaxf(__uint_as_float(s[2 * hi]), __uint_as_float(s[2 * hi + 1]));
-#pragma unroll
-    for (int b = 1; b < 16; ++b) mx = max3(mx, __uint_as_float(s[4 * b + 2 * hi]), __uint_as_float(s[4 * b + 2 * hi + 1]));
-    const float tile_max = quad_max(mx) * scale_log2;
-    // lazy rescale: keep the old reference maximum unless the new one is far above it
-    const bool jump = tile_max > st.m_used[hi] + kRescaleThreshold;
-    alpha[hi] = 1.0f;
-    if (jump) {
-      alpha[hi] = ex2_approx(st.m_used[hi] - tile_max);   // 0 on the first tile (m_used = -inf)
-      st.m_used[hi] = tile_max;
-      st.l_run[hi] *= alpha[hi];
-      if (kLse) st.l_exact[hi] *= alpha[hi];
-    }
-    jump_any = jump_any || jump;
-  }
-  const bool rescale = (j > 0) && __any_sync(0xffffffffu, jump_any);
-
-  // P_t(j-1) must have been consumed, and O_t be at rest, before either is written
-  if (j > 0) {
-    if (!wait_bar(&bars->o_done[me.t], (gj - 1) & 1, bars, a, 30 + me.t, gj)) return false;
-    tc_fence_after();
-  }
-  if (rescale) {   // the warp's 16 rows of the accumulator: register 4 b + 2 hi + e is row hi
-    uint32_t o[32];
-    tmem_ld_rows16_c64(me.tO, o);
-    tmem_wait_ld();
-#pragma unroll
-    for (int c = 0; c < 32; ++c) o[c] = __float_as_uint(__uint_as_float(o[c]) * alpha[(c >> 1) & 1]);
-    tmem_st_rows16_c64(me.tO, o);
-  }
-
-  // exponentials, rounded to bf16 for the value product; the normaliser sums the
-  // rounded values so that numerator and denominator carry the same weights
-  const uint64_t scale2 = pack_f32x2(scale_log2, scale_log2);
-  const uint64_t neg_m2[2] = {pack_f32x2(-st.m_used[0], -st.m_used[0]), pack_f32x2(-st.m_used[1], -st.m_used[1])};
-  float sum_lo[2] = {0.f, 0.f}, sum_hi[2] = {0.f, 0.f};   // even and odd columns
+  const int n_blocks = kMasked ? (valid + 7) >> 3 : kBlocks;   // blocks of 8 columns that hold a key
+  const uint64_t scale2 = pack_f32x2(a.scale_log2, a.scale_log2);
   uint64_t sum_exact2[2] = {pack_f32x2(0.f, 0.f), pack_f32x2(0.f, 0.f)};
-  const int n_blocks = kMasked ? (valid + 7) >> 3 : 16;   // blocks of 8 columns that hold a key
-  softmax_rows<kMasked, kLse, kPoly>(s, scale2, neg_m2, sum_lo, sum_hi, sum_exact2, me.tP, n_blocks);
+  uint32_t pk[8];   // P of 32 keys x 2 rows as bf16 pairs
+  constexpr bool kAhead = !kLse && !kMasked;   // first group before the vote
+  if (kAhead) exp_group<0, kMasked, kLse, kPoly>(s, st, scale2, sum_exact2, pk, n_blocks);
+
+  float mx[2], mn[2];
+  bool look = false;
 #pragma unroll
   for (int hi = 0; hi < 2; ++hi) {
-    st.l_run[hi] += sum_lo[hi] + sum_hi[hi];
-    if (kLse) {
+    float x = fmaxf(__uint_as_float(s[2 * hi]), __uint_as_float(s[2 * hi + 1]));
+    float y = fmaxf(__uint_as_float(s[2 * kBlocks + 2 * hi]), __uint_as_float(s[2 * kBlocks + 2 * hi + 1]));
+#pragma unroll
+    for (int b = 1; b < kBlocks / 2; ++b) {
+      x = max3(x, __uint_as_float(s[4 * b + 2 * hi]), __uint_as_float(s[4 * b + 2 * hi + 1]));
+      y = max3(y, __uint_as_float(s[2 * kBlocks + 4 * b + 2 * hi]), __uint_as_float(s[2 * kBlocks + 4 * b + 2 * hi + 1]));
+    }
+    mx[hi] = fmaxf(x, y);
+    mn[hi] = INFINITY;
+#pragma unroll
+    for (int b = 0; b < kBlocks; ++b)
+      if ((kPoly >> b) & 1) mn[hi] = min3(mn[hi], __uint_as_float(s[4 * b + 2 * hi]), __uint_as_float(s[4 * b + 2 * hi + 1]));
+    look = look || mx[hi] > st.jump_above[hi] || (kPoly != 0 && mn[hi] < st.clamp_below[hi]);
+  }
+  if (__any_sync(0xffffffffu, look)) {
+    float alpha[2];
+    bool jump_any = false;
+#pragma unroll
+    for (int hi = 0; hi < 2; ++hi) {
+      const float row_max = quad_max(mx[hi]);
+      alpha[hi] = 1.0f;
+      if (row_max > st.jump_above[hi]) {
+        const float m = row_max * a.scale_log2;
+        alpha[hi] = ex2_approx(st.m[hi] - m);   // 0 on the first tile (m = -inf)
+        st.m[hi] = m;
+        st.neg_m[hi] = -m;
+        st.jump_above[hi] = (m + kRescaleThreshold) * a.inv_scale_log2;
+        st.clamp_below[hi] = (m + kPolyLowest) * a.inv_scale_log2;
+        if (kLse) st.l_exact[hi] *= alpha[hi];
+        jump_any = true;
+      }
+    }
+    if (j > 0 && __any_sync(0xffffffffu, jump_any)) {
+      // O_t must be at rest
+      if (!wait_bar(&bars->o_done[me.t][!odd], ((gj - 1) >> 1) & 1, bars, a, 30 + me.t, gj)) return false;
+      tc_fence_after();
+      uint32_t o[32], l[4];   // the warp's 16 rows of the accumulator: register 4 b + 2 hi + e is row hi
+      tmem_ld_rows16_c64(me.base + kColO, o);
+      tmem_ld_rows16_c8(me.base + kColL, l);
+      tmem_wait_ld();
+#pragma unroll
+      for (int c = 0; c < 32; ++c) o[c] = __float_as_uint(__uint_as_float(o[c]) * alpha[(c >> 1) & 1]);
+#pragma unroll
+      for (int c = 0; c < 4; ++c) l[c] = __float_as_uint(__uint_as_float(l[c]) * alpha[c >> 1]);
+      tmem_st_rows16_c64(me.base + kColO, o);
+      tmem_st_rows16_c8(me.base + kColL, l);
+    }
+    if (kPoly != 0) {
+#pragma unroll
+      for (int c = 0; c < 4 * kBlocks; ++c)
+        if ((kPoly >> (c >> 2)) & 1) s[c] = __float_as_uint(fmaxf(__uint_as_float(s[c]), st.clamp_below[(c >> 1) & 1]));
+    }
+    if (kAhead) exp_group<0, kMasked, kLse, kPoly>(s, st, scale2, sum_exact2, pk, n_blocks);
+  }
+
+  // exponentials, rounded to bf16 for the value product (whose column of ones sums the rounded values, so that numerator
+  // and denominator carry the same weights)
+  if (!kAhead) exp_group<0, kMasked, kLse, kPoly>(s, st, scale2, sum_exact2, pk, n_blocks);
+  tmem_st_rows16_p16(tP, pk);
+  exp_group<1, kMasked, kLse, kPoly>(s, st, scale2, sum_exact2, pk, n_blocks);
+  tmem_st_rows16_p16(tP + 16, pk);
+  exp_group<2, kMasked, kLse, kPoly>(s, st, scale2, sum_exact2, pk, n_blocks);
+  tmem_st_rows16_p16(tP + 32, pk);
+  exp_group<3, kMasked, kLse, kPoly>(s, st, scale2, sum_exact2, pk, n_blocks);
+  tmem_st_rows16_p8(tP + 48, pk);
+  if (kLse) {
+#pragma unroll
+    for (int hi = 0; hi < 2; ++hi) {
       float sum_a, sum_b;
       unpack_f32x2(sum_exact2[hi], sum_a, sum_b);
       st.l_exact[hi] += sum_a + sum_b;
@@ -624,8 +709,24 @@ __device__ __forceinline__ bool softmax_step(const SoftmaxThread& me, int j, int
   }
   tmem_wait_st();
   tc_fence_before();
-  __syncwarp();
-  if (me.lane == 0) mbar_arrive(smem_u32(&bars->p_full[me.t]));
+  if (me.lane == 0) mbar_arrive(smem_u32(&bars->p_full[me.t][odd]));
+  return true;
+}
+
+// The row sums move to the column after theirs (see kFlushSteps).  Thread 0 of a quad has both columns, the others zeros.
+// last: the tile's latest step; its P V has to be done, and the next one waits for this warp's next P.
+__device__ __forceinline__ bool flush_row_sums(const SoftmaxThread& me, int last, Barriers* bars, const AttnArgs& a) {
+  if (!wait_bar(&bars->o_done[me.t][last & 1], (last >> 1) & 1, bars, a, 32 + me.t, last)) return false;
+  tc_fence_after();
+  uint32_t l[4];
+  tmem_ld_rows16_c8(me.base + kColL, l);
+  tmem_wait_ld();
+#pragma unroll
+  for (int hi = 0; hi < 2; ++hi) {
+    l[2 * hi + 1] = __float_as_uint(__uint_as_float(l[2 * hi]) + __uint_as_float(l[2 * hi + 1]));
+    l[2 * hi] = 0u;
+  }
+  tmem_st_rows16_c8(me.base + kColL, l);
   return true;
 }
 
@@ -643,27 +744,40 @@ __device__ __forceinline__ bool softmax_item(const AttnArgs& a, Barriers* bars, 
   const int t = me.t, lane = me.lane;
   RowState st;
 #pragma unroll
-  for (int hi = 0; hi < 2; ++hi) { st.m_used[hi] = -INFINITY; st.l_run[hi] = 0.f; st.l_exact[hi] = 0.f; }
+  for (int hi = 0; hi < 2; ++hi) {
+    st.m[hi] = -INFINITY;
+    st.neg_m[hi] = 0.f;
+    st.jump_above[hi] = -INFINITY;
+    st.clamp_below[hi] = -INFINITY;
+    st.l_exact[hi] = 0.f;
+  }
   const bool want_lse = a.lse != nullptr;
 
+  int j = 0;
 #pragma unroll 1
-  for (int j = 0; j < n_kv; ++j) {
-    if (!wait_bar(&bars->s_full[t], (g + j) & 1, bars, a, 40 + t, g + j)) return false;
-    tc_fence_after();
-    const int valid = static_cast<int>(a.n_keys - static_cast<int64_t>(j) * kTileKV);
-    bool ok;
-    // the masked (last, ragged) tile keeps every exponential on the special-function unit, where -inf gives an exact 0
-    if (valid < kTileKV) ok = want_lse ? softmax_step<true, true, 0>(me, j, g, valid, a.scale_log2, st, bars, a)
-                                       : softmax_step<true, false, 0>(me, j, g, valid, a.scale_log2, st, bars, a);
-    else if (want_lse) ok = softmax_step<false, true, kPolyEighths>(me, j, g, valid, a.scale_log2, st, bars, a);
-    else ok = softmax_step<false, false, kPolyEighths>(me, j, g, valid, a.scale_log2, st, bars, a);
-    if (!ok) return false;
+  while (j < n_kv) {
+    const int stop = n_kv - j > kFlushSteps ? j + kFlushSteps : n_kv;
+#pragma unroll 1
+    for (; j < stop; ++j) {
+      if (!wait_bar(&bars->s_full[t], (g + j) & 1, bars, a, 40 + t, g + j)) return false;
+      tc_fence_after();
+      const int valid = static_cast<int>(a.n_keys - static_cast<int64_t>(j) * kTileKV);
+      bool ok;
+      // the masked (last, ragged) tile keeps every exponential on the special-function unit, where -inf gives an exact 0
+      if (valid < kTileKV) ok = want_lse ? softmax_step<true, true, 0>(me, j, g, valid, st, bars, a)
+                                         : softmax_step<true, false, 0>(me, j, g, valid, st, bars, a);
+      else if (want_lse) ok = softmax_step<false, true, kPolyBlocks>(me, j, g, valid, st, bars, a);
+      else ok = softmax_step<false, false, kPolyBlocks>(me, j, g, valid, st, bars, a);
+      if (!ok) return false;
+    }
+    if (j < n_kv && !flush_row_sums(me, g + j - 1, bars, a)) return false;
   }
 
   // ---- epilogue: diagonal and mean-fill terms, normalisation, store of this thread's 16 output dimensions of two rows
   const int head = cta.head;
   if (n_kv > 0) {
-    if (!wait_bar(&bars->o_done[t], (g + n_kv - 1) & 1, bars, a, 50 + t, g + n_kv)) return false;
+    const int last = g + n_kv - 1;
+    if (!wait_bar(&bars->o_done[t][last & 1], (last >> 1) & 1, bars, a, 50 + t, last)) return false;
     tc_fence_after();
   }
   // completed long ago: makes the Q tile visible to this thread.  Only the two extra columns read Q here, and a CTA
@@ -680,8 +794,10 @@ __device__ __forceinline__ bool softmax_item(const AttnArgs& a, Barriers* bars, 
   const uint8_t* sQ = sm.q[t];
 
   uint32_t o[32];   // register 4 b + 2 hi + e: row hi, output dimension 8 b + 2 i + e
+  uint32_t l[4];    // thread 0 of a quad: the row sums, in two parts, in registers 0 + 1 (row 0) and 2 + 3 (row 1)
   if (n_kv > 0) {
-    tmem_ld_rows16_c64(me.tO, o);
+    tmem_ld_rows16_c64(me.base + kColO, o);
+    tmem_ld_rows16_c8(me.base + kColL, l);
     tmem_wait_ld();
     // O_t is in registers: the next work item's first P V may overwrite it
     tc_fence_before();
@@ -690,6 +806,8 @@ __device__ __forceinline__ bool softmax_item(const AttnArgs& a, Barriers* bars, 
   } else {   // no retained keys at all: the accumulator was never written
 #pragma unroll
     for (int c = 0; c < 32; ++c) o[c] = 0u;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) l[c] = 0u;
   }
 
 #pragma unroll
@@ -702,10 +820,10 @@ __device__ __forceinline__ bool softmax_item(const AttnArgs& a, Barriers* bars, 
       const int32_t f = row / pl.L;
       is_dropped = (a.slot_of_token != nullptr ? a.slot_of_token[row] : compact_slot(pl, f, row - f * pl.L)) < 0;
     }
-    // the row's sums over its four threads
-    const float l_run = quad_sum(st.l_run[hi]);
+    // the row's sums: of the rounded probabilities (the normaliser), of the unrounded ones (log-sum-exp)
+    const float l_run = __shfl_sync(0xffffffffu, __uint_as_float(l[2 * hi]) + __uint_as_float(l[2 * hi + 1]), lane & ~3);
     const float l_exact = want_lse ? quad_sum(st.l_exact[hi]) : 0.f;
-    const float m_used = st.m_used[hi];
+    const float m_used = st.m[hi];
     // base-2 logits of the two extra columns: each thread of the quad takes its 16 dimensions, then the quad adds up
     // (every thread runs the shuffles; rows without the term carry zeros)
     const bool has_diag = a.use_diag && is_dropped;
@@ -792,10 +910,7 @@ __device__ __forceinline__ void softmax_role(const AttnArgs& a, Barriers* bars, 
   me.i = lane & 3;
   me.r[0] = 32 * me.q + 16 * me.h + (lane >> 2);
   me.r[1] = me.r[0] + 8;
-  const uint32_t tile_base = tmem + me.t * kTmemTileStride + (static_cast<uint32_t>(32 * me.q + 16 * me.h) << 16);   // TMEM lane = row
-  me.tS = tile_base;
-  me.tP = tile_base + kColP;
-  me.tO = tile_base + kColO;
+  me.base = tmem + me.t * kTmemTileStride + (static_cast<uint32_t>(32 * me.q + 16 * me.h) << 16);   // TMEM lane = row
   const int n_kv = a.n_kv_tiles;
   int g = 0, n_done = 0;
 #pragma unroll 1
@@ -804,6 +919,19 @@ __device__ __forceinline__ void softmax_role(const AttnArgs& a, Barriers* bars, 
     g += n_kv;
     ++n_done;
   }
+}
+
+// Value columns 64..79 of a slice of 16 keys, in the 128-byte-swizzled layout of the V tiles: column 64 all ones, the others
+// zero, so that P V sums the rows of P on the tensor core.  It is the sum of the bf16-rounded probabilities that the value
+// product uses, in fp32, and it costs the softmax warps nothing (adding the rounded values up took one instruction per score
+// of the 6.5 that a score took).  128-byte rows: only 32 bytes of each are read.
+__device__ __forceinline__ void ones_block(uint8_t* ones, int tid) {
+  if (tid < static_cast<int>(kOnesBytes / 16)) {
+    const int row = tid >> 3, chunk = tid & 7;
+    const uint32_t first = chunk == (row & 7) ? 0x3f80u : 0u;   // bf16 1 in the row's first value
+    *reinterpret_cast<uint4*>(ones + tid * 16) = make_uint4(first, 0u, 0u, 0u);
+  }
+  fence_proxy_async_smem();
 }
 
 __global__ void __launch_bounds__(kThreads, 1)
@@ -817,6 +945,7 @@ global_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
   sm.q[1] = smem + kTileBytes;
   sm.k = smem + kQTiles * kTileBytes;
   sm.v = sm.k + kStages * kTileBytes;
+  sm.ones = sm.v + kStages * kTileBytes;
   __shared__ Barriers bars;
 
   const int tid = threadIdx.x;
@@ -836,8 +965,10 @@ global_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
     for (int t = 0; t < kQTiles; ++t) {
       mbar_init(smem_u32(&bars.s_full[t]), 1);
       mbar_init(smem_u32(&bars.s_free[t]), kSoftmaxWarps / kQTiles);
-      mbar_init(smem_u32(&bars.p_full[t]), kSoftmaxWarps / kQTiles);
-      mbar_init(smem_u32(&bars.o_done[t]), 1);
+      for (int e = 0; e < 2; ++e) {
+        mbar_init(smem_u32(&bars.p_full[t][e]), kSoftmaxWarps / kQTiles);
+        mbar_init(smem_u32(&bars.o_done[t][e]), 1);
+      }
       mbar_init(smem_u32(&bars.mma_idle[t]), 1);
       mbar_init(smem_u32(&bars.o_free[t]), kSoftmaxWarps / kQTiles);
     }
@@ -848,6 +979,7 @@ global_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
     tmem_alloc(smem_u32(&bars.tmem_base), kTmemCols);
     tmem_relinquish();
   }
+  ones_block(sm.ones, tid);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -871,7 +1003,7 @@ global_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
   if (warp == kTmaWarp) tmem_dealloc(tmem, kTmemCols);
 }
 
-constexpr size_t kAttnSmemBytes = static_cast<size_t>(kTileBytes) * (kQTiles + 2 * kStages) + 1024;
+constexpr size_t kAttnSmemBytes = static_cast<size_t>(kTileBytes) * (kQTiles + 2 * kStages) + kOnesBytes + 1024;
 
 }  // namespace
 
@@ -922,6 +1054,7 @@ cudaError_t launch_attn(const Plan& pl, int sm_count, bool frame_mode, const voi
   a.use_diag = (!frame_mode && pl.diag != 0 && pl.n_dropped > 0) ? 1 : 0;
   a.use_mean = (!frame_mode && pl.mean_fill != 0 && pl.n_dropped > 0) ? 1 : 0;
   a.scale_log2 = pl.scale * kLog2e;
+  a.inv_scale_log2 = 1.0f / a.scale_log2;
   const int64_t rows = frame_mode ? pl.L : pl.n_tok;
   a.pairs = static_cast<int32_t>((rows + kQTiles * kTileQ - 1) / (kQTiles * kTileQ));
   a.n_work = a.pairs * pl.H * (frame_mode ? pl.n_frames : 1);
@@ -932,10 +1065,12 @@ cudaError_t launch_attn(const Plan& pl, int sm_count, bool frame_mode, const voi
   const uint64_t tok_dims[2] = {static_cast<uint64_t>(pl.H) * pl.d, static_cast<uint64_t>(pl.n_tok)};
   const uint64_t tok_str[1] = {static_cast<uint64_t>(pl.H) * pl.d * 2};
   const uint32_t tok_box[2] = {kHeadDim, kTileQ};
+  // tiles of a frame's keys, or the queries' own rows
+  const uint32_t kv_box[2] = {kHeadDim, static_cast<uint32_t>(frame_mode ? kTileKV : kTileQ)};
   const bool reads_kv = frame_mode || a.use_diag;
   bool good = make_tmap_bf16(&tm_q, Q, 2, tok_dims, tok_str, tok_box);
-  good = good && make_tmap_bf16(&tm_k, reads_kv ? K : Q, 2, tok_dims, tok_str, tok_box);
-  good = good && make_tmap_bf16(&tm_v, reads_kv ? V : Q, 2, tok_dims, tok_str, tok_box);
+  good = good && make_tmap_bf16(&tm_k, reads_kv ? K : Q, 2, tok_dims, tok_str, kv_box);
+  good = good && make_tmap_bf16(&tm_v, reads_kv ? V : Q, 2, tok_dims, tok_str, kv_box);
   if (frame_mode || pl.M == 0) {
     tm_kc = tm_k;   // not read
     tm_vc = tm_v;

@@ -118,13 +118,14 @@ __device__ __forceinline__ void umma_commit(uint32_t bar) {
 // descriptor serves a K-major operand (rows = M or N index, 64 contiguous K
 // elements per row) and an MN-major operand (rows = K index, 64 contiguous
 // M/N elements per row): in both the 8-row groups are 1024 bytes apart.
+// An MN-major operand wider than 64 elements continues, at every row, `leading` bytes further on.
 //   bits  0-13 start address >> 4      bits 16-29 leading byte offset >> 4
 //   bits 32-45 stride byte offset >> 4 bits 46-47 descriptor version (1)
 //   bits 61-63 swizzle mode (2 = 128 bytes)
-__device__ __forceinline__ uint64_t umma_desc_sw128(uint32_t saddr) {
+__device__ __forceinline__ uint64_t umma_desc_sw128(uint32_t saddr, uint32_t leading = 16) {
   uint64_t d = 0;
   d |= static_cast<uint64_t>((saddr & 0x3ffffu) >> 4);
-  d |= static_cast<uint64_t>(1) << 16;            // leading byte offset: unused for one 128-byte span
+  d |= static_cast<uint64_t>((leading & 0x3ffffu) >> 4) << 16;   // unused for one 128-byte span
   d |= static_cast<uint64_t>(1024 >> 4) << 32;    // stride between 8-row groups
   d |= static_cast<uint64_t>(1) << 46;
   d |= static_cast<uint64_t>(2) << 61;
@@ -220,16 +221,6 @@ __device__ __forceinline__ uint64_t sub_f32x2(uint64_t a, uint64_t b) {
   uint64_t d;
   asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
   return d;
-}
-// lo += low bf16 half of w, hi += high bf16 half of w: the mixed-precision add of sm_100 takes the bf16
-// operand as it is (exact widening), so the sum of rounded values costs no unpacking.
-__device__ __forceinline__ void add_bf16x2_to_f32(uint32_t w, float& lo, float& hi) {
-  asm("{\n\t.reg .b16 l, h;\n\t"
-      "mov.b32 {l, h}, %2;\n\t"
-      "add.rn.f32.bf16 %0, l, %0;\n\t"
-      "add.rn.f32.bf16 %1, h, %1;\n\t}"
-      : "+f"(lo), "+f"(hi)
-      : "r"(w));
 }
 // two floats -> packed bf16x2 (lo in the low half), round to nearest even
 __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
