@@ -2,10 +2,10 @@
 // warp-specialised flash-style kernel for sm_100a; the same kernel runs frame
 // attention (Sec. 4.2) as many small dense problems.
 //
-// A work item is two tiles of 128 query rows of one head.  In the subsampled
-// layer a CTA has one work item (hundreds of key steps); in frame attention one
-// CTA per SM walks over many (a dozen key steps each), so that the next item's
-// loads and first product run under the current item's epilogue.
+// A work item is two tiles of 128 query rows of one head.  One CTA per SM walks
+// over the work items; the next item's loads and first product run under the
+// current item's last step, and the epilogue of an item comes after the first
+// step of the next one, when its last product has long completed.
 // Roles (20 warps):
 //   warps 0-15  softmax.  Warp 8 t + 4 h + q works on query tile t, rows
 //               [32 q + 16 h, 32 q + 16 h + 16), all 112 columns of a key step.
@@ -13,10 +13,8 @@
 //               over the four threads of a quad (two rows per thread): a row's
 //               maximum is two shuffles away and every row lives in one warp.  Four softmax warps per scheduler keep the exponential unit
 //               busy while others wait on tensor memory or barriers.
-//   warp  16    TMA producer: Q tiles once per work item, then the compacted K/V
-//               of the head through a ring of shared-memory stages (128-byte
-//               swizzle); in the subsampled layer the last two ring items are the
-//               K/V rows of the CTA's own queries (the preserved diagonal)
+//   warp  16    TMA producer: Q tiles once per work item (two places), then the compacted
+//               K/V of the head through a ring of shared-memory stages (128-byte swizzle)
 //   warps 17-18 MMA issuers, one per query tile: S_t = Q_t Kc_j^T and
 //               O_t += P_t Vc_j with tcgen05.mma, bf16 operands, fp32
 //               accumulators in tensor memory
@@ -30,6 +28,7 @@
 // maximum grew by more than 2^8 since the last rescale.  The epilogue folds the
 // diagonal and the mean-fill column into the same normalisation:
 //   O = (a_S O_S + p_d v_i + p_m vmean) / (a_S l_S + p_d + p_m).
+#include <cmath>
 #include <mutex>
 
 #include <cuda_bf16.h>
@@ -48,8 +47,9 @@ constexpr int kQTiles = 2;       // tiles per CTA
 constexpr int kTileKV = 112;     // keys per step
 constexpr int kBlocks = kTileKV / 8;   // blocks of 8 key columns in a step
 constexpr int kHeadDim = 64;
-constexpr uint32_t kTileBytes = kTileQ * kHeadDim * 2;      // 16 KiB: one tile of 128 query rows (or of the queries' own K/V rows); also a ring stage
-constexpr uint32_t kKeyTileBytes = kTileKV * kHeadDim * 2;  // 14 KiB: one tile of keys or values
+constexpr uint32_t kTileBytes = kTileQ * kHeadDim * 2;      // 16 KiB: one tile of 128 query rows
+constexpr uint32_t kKeyTileBytes = kTileKV * kHeadDim * 2;  // 14 KiB: one tile of keys or values, one ring stage
+static_assert(kKeyTileBytes % 1024 == 0, "swizzle atoms");
 constexpr uint32_t kOnesBytes = 2 * 1024;                   // the block of value columns 64..79 (ones_block)
 // K ring and V ring depth.  The subsampled layer runs the same at 2 to 5; frame attention, whose strided key
 // tiles take longer to arrive, gained 6 % from the fourth stage and nothing from a fifth.
@@ -91,6 +91,9 @@ constexpr uint32_t kPolyBlocks = AVGGT_POLY_BLOCKS;
 
 struct AttnArgs {
   Plan pl;
+  const uint4* Q;       // [n_tok, H, d], read by the diagonal and mean terms; K and V by the diagonal term only
+  const uint4* K;
+  const uint4* V;
   const float* kmean;   // [H, d] or null
   const float* vmean;
   __nv_bfloat16* O;     // [n_tok, H, d]
@@ -101,18 +104,21 @@ struct AttnArgs {
                         //    every frame is a problem of its own, keys and values are the frame's own rows of K and V
   int64_t n_keys;       // keys of one problem: M, or the tokens of a frame
   int32_t n_kv_tiles;   // ceil(n_keys / kTileKV)
+  int32_t last_tile_keys;   // keys of a ragged last tile, else 0
   int32_t n_work;       // work items (pairs of query tiles x heads x problems) of the launch; a CTA takes the items
-                        // blockIdx.x, blockIdx.x + gridDim.x, ...  (more than one per CTA only in frame attention)
+                        // blockIdx.x, blockIdx.x + gridDim.x, ...
   int32_t pairs;        // pairs of query tiles of one problem
   int32_t use_diag;     // diag on and |D| > 0
   int32_t use_mean;     // mean_fill on and |D| > 0
   float scale_log2;     // softmax scale * log2(e)
   float inv_scale_log2;
+  float poly_range;     // raw score units from the polynomial's lowest score (kPolyLowest) to the threshold of a rescale
+  float log2_count[2];  // log2 weight of the mean column for a retained and for a dropped query (0: unit weight; -inf: absent)
 };
 
 struct __align__(8) Barriers {
-  uint64_t q_full;             // producer -> all: the work item's Q tiles are in shared memory
-  uint64_t q_empty;            // MMA issuers -> producer: every Q K^T of the work item has completed, Q may be overwritten
+  uint64_t q_full[2];          // producer -> MMA: the work item's Q tiles are in shared memory (items take the two places in turn)
+  uint64_t q_empty[2];         // MMA issuers -> producer: every Q K^T of the work item has completed, Q may be overwritten
   uint64_t o_free[kQTiles];    // softmax -> MMA: O_t of the finished work item has been read out
   uint64_t k_full[kStages], k_empty[kStages];
   uint64_t v_full[kStages], v_empty[kStages];
@@ -178,35 +184,50 @@ static_assert(kRegsSoftmax * kSoftmaxWarps + kRegsOther * (kThreads / 32 - kSoft
 template <int N> __device__ __forceinline__ void reg_inc() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N)); }
 template <int N> __device__ __forceinline__ void reg_dec() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N)); }
 
-// What one CTA works on.
-struct CtaProblem {
+// A work item.
+struct WorkItem {
   int head;
-  int q0;             // first query row (token index) of the CTA's two tiles
-  int64_t row_end;    // query rows at or beyond this token index are not stored
-  int key_row0;       // frame attention: token index of the frame's first key
+  int key_row0;   // frame attention: token index of the frame's first key
+  int row0;       // first query row (token index)
+  int64_t end;    // one past the problem's last query row
+};
+// One of its query tiles.
+struct QueryTile {
+  int q0;         // token index of lane 0 (negative where the lanes before `first` reach back that far)
+  int first;      // query rows [first, last) are wanted
+  int64_t last;
 };
 
-// Work item -> problem.  Items are numbered with the pair of query tiles fastest, then the head, then (frame
+// Items are numbered with the pair of query tiles fastest, then the head, then (frame
 // attention) the frame, so that the CTAs running side by side share one head's keys in L2.
-__device__ __forceinline__ CtaProblem work_item(const AttnArgs& a, int item) {
-  CtaProblem c;
-  const int qp = item % a.pairs;
-  const int rest = item / a.pairs;
-  c.head = rest % a.pl.H;
-  if (a.frame_mode) {
-    c.key_row0 = (rest / a.pl.H) * a.pl.L;
-    c.q0 = c.key_row0 + qp * (kQTiles * kTileQ);
-    c.row_end = static_cast<int64_t>(c.key_row0) + a.pl.L;
-  } else {
-    c.key_row0 = 0;
-    c.q0 = qp * (kQTiles * kTileQ);
-    c.row_end = a.pl.n_tok;
-  }
-  return c;
+__device__ __forceinline__ WorkItem work_item(const AttnArgs& a, uint32_t item) {
+  WorkItem w;
+  const uint32_t rest = item / static_cast<uint32_t>(a.pairs);
+  const uint32_t qp = item - rest * static_cast<uint32_t>(a.pairs);
+  const uint32_t frame = rest / static_cast<uint32_t>(a.pl.H);
+  w.head = static_cast<int>(rest - frame * static_cast<uint32_t>(a.pl.H));
+  w.key_row0 = static_cast<int>(frame) * a.pl.L;   // the subsampled layer has one problem
+  w.row0 = w.key_row0 + static_cast<int>(qp) * (kQTiles * kTileQ);
+  w.end = a.frame_mode ? static_cast<int64_t>(w.key_row0) + a.pl.L : a.pl.n_tok;
+  return w;
+}
+
+// A last pair with rows for one tile only is cut in two halves by groups of 16 rows (one softmax warp), the second
+// half in the upper lanes of its tile: every scheduler then has two warps with work at most, and both tiles' products
+// overlap.  Warps without rows compute nothing.
+__device__ __forceinline__ QueryTile query_tile(const WorkItem& w, int t) {
+  QueryTile q;
+  const bool two = w.end - w.row0 > kTileQ;
+  const int groups = two ? 16 : static_cast<int>(w.end - w.row0 + 15) >> 4;
+  const int cut = w.row0 + 16 * ((groups + 1) >> 1);   // first row of tile 1
+  q.first = t == 0 ? w.row0 : cut;
+  q.q0 = t == 0 ? w.row0 : (two ? cut : cut - kTileQ / 2);
+  q.last = t == 0 && cut < w.end ? cut : w.end;
+  return q;
 }
 
 struct SmemLayout {
-  uint8_t* q[kQTiles];
+  uint8_t* q;   // 2 places of kQTiles tiles
   uint8_t* k;   // kStages tiles
   uint8_t* v;   // kStages tiles
   uint8_t* ones;   // 16 rows of 64 values: 1 in column 0, else 0 (ones_block)
@@ -225,14 +246,13 @@ __device__ __forceinline__ bool wait_bar_warp(uint64_t* bar, uint32_t parity, Ba
 
 // ------------------------------------------------------------------ TMA producer (one warp)
 __device__ __forceinline__ void producer_role(const CUtensorMap* tm_q, const CUtensorMap* tm_k, const CUtensorMap* tm_v,
-                                              const CUtensorMap* tm_kc, const CUtensorMap* tm_vc, const AttnArgs& a,
-                                              Barriers* bars, const SmemLayout& sm) {
+                                              const AttnArgs& a, Barriers* bars, const SmemLayout& sm) {
   const int n_kv = a.n_kv_tiles;
-  const int n_ring = n_kv + (a.use_diag ? kQTiles : 0);   // ring items of one work item
+  if (n_kv == 0) return;   // no retained keys: nothing goes through shared memory
   if (elect_one()) {
     prefetch_tensormap(tm_q);
-    prefetch_tensormap(tm_kc);
-    prefetch_tensormap(tm_vc);
+    prefetch_tensormap(tm_k);
+    prefetch_tensormap(tm_v);
   }
   int k_issued = 0, v_issued = 0;   // K / V copies issued so far, over all work items
   int stage = 0;
@@ -240,23 +260,29 @@ __device__ __forceinline__ void producer_role(const CUtensorMap* tm_q, const CUt
   bool ok = true;
   int n_done = 0;              // work items completed by this role
   int q_issued = 0;            // work items whose Q copies have been issued
-  for (int item = blockIdx.x; item < a.n_work && ok; item += gridDim.x, ++n_done) {
-    const CtaProblem cta = work_item(a, item);
-    const int head = cta.head, q0 = cta.q0;
-    // the Q tiles of the previous work item are no longer read by any Q K^T
-    if (n_done > 0) {
-      ok = wait_bar_warp(&bars->q_empty, (n_done - 1) & 1, bars, a, 14, n_done);
-      if (!ok) break;
+  for (uint32_t item = blockIdx.x; item < static_cast<uint32_t>(a.n_work) && ok; item += gridDim.x, ++n_done) {
+    const WorkItem wi = work_item(a, item);
+    const int head = wi.head;
+    const int place = n_done & 1;
+    // a wait has run out in another thread block: the launch is abandoned
+    if (n_done > 0 && __any_sync(kFullMask, *reinterpret_cast<volatile uint32_t*>(a.status) != 0u)) {
+      *reinterpret_cast<volatile uint32_t*>(&bars->abort_flag) = 1u;
+      ok = false;
+      break;
     }
+    // the Q tiles of the work item before the last one are no longer read by any Q K^T
+    ok = wait_bar_warp(&bars->q_empty[place], ((n_done >> 1) & 1) ^ 1, bars, a, 14, n_done);
+    if (!ok) break;
     if (elect_one()) {
-      mbar_arrive_expect_tx(smem_u32(&bars->q_full), kQTiles * kTileBytes);
+      const uint32_t qb = smem_u32(&bars->q_full[place]);
+      mbar_arrive_expect_tx(qb, kQTiles * kTileBytes);
 #pragma unroll
       for (int t = 0; t < kQTiles; ++t)
-        tma_load_2d(smem_u32(sm.q[t]), tm_q, head * kHeadDim, q0 + t * kTileQ, smem_u32(&bars->q_full));
+        tma_load_2d(smem_u32(sm.q + (place * kQTiles + t) * kTileBytes), tm_q, head * kHeadDim, query_tile(wi, t).q0, qb);
     }
     __syncwarp();
     ++q_issued;
-    for (int it = 0; it < n_ring; ++it) {
+    for (int it = 0; it < n_kv; ++it) {
       ok = wait_bar_warp(&bars->k_empty[stage], empty_parity, bars, a, 10, it);
       if (!ok) break;
 #ifdef AVGGT_TEST_SKIP_K_LOAD
@@ -268,10 +294,9 @@ __device__ __forceinline__ void producer_role(const CUtensorMap* tm_q, const CUt
 #endif
       if (elect_one() && !skip_load) {
         const uint32_t kb = smem_u32(&bars->k_full[stage]);
-        mbar_arrive_expect_tx(kb, it < n_kv ? kKeyTileBytes : kTileBytes);
-        if (a.frame_mode) tma_load_2d(smem_u32(sm.k + stage * kTileBytes), tm_k, head * kHeadDim, cta.key_row0 + it * kTileKV, kb);
-        else if (it < n_kv) tma_load_3d(smem_u32(sm.k + stage * kTileBytes), tm_kc, 0, it * kTileKV, head, kb);
-        else tma_load_2d(smem_u32(sm.k + stage * kTileBytes), tm_k, head * kHeadDim, q0 + (it - n_kv) * kTileQ, kb);
+        mbar_arrive_expect_tx(kb, kKeyTileBytes);
+        if (a.frame_mode) tma_load_2d(smem_u32(sm.k + stage * kKeyTileBytes), tm_k, head * kHeadDim, wi.key_row0 + it * kTileKV, kb);
+        else tma_load_3d(smem_u32(sm.k + stage * kKeyTileBytes), tm_k, 0, it * kTileKV, head, kb);
       }
       __syncwarp();
       ++k_issued;
@@ -279,10 +304,9 @@ __device__ __forceinline__ void producer_role(const CUtensorMap* tm_q, const CUt
       if (!ok) break;
       if (elect_one()) {
         const uint32_t vb = smem_u32(&bars->v_full[stage]);
-        mbar_arrive_expect_tx(vb, it < n_kv ? kKeyTileBytes : kTileBytes);
-        if (a.frame_mode) tma_load_2d(smem_u32(sm.v + stage * kTileBytes), tm_v, head * kHeadDim, cta.key_row0 + it * kTileKV, vb);
-        else if (it < n_kv) tma_load_3d(smem_u32(sm.v + stage * kTileBytes), tm_vc, 0, it * kTileKV, head, vb);
-        else tma_load_2d(smem_u32(sm.v + stage * kTileBytes), tm_v, head * kHeadDim, q0 + (it - n_kv) * kTileQ, vb);
+        mbar_arrive_expect_tx(vb, kKeyTileBytes);
+        if (a.frame_mode) tma_load_2d(smem_u32(sm.v + stage * kKeyTileBytes), tm_v, head * kHeadDim, wi.key_row0 + it * kTileKV, vb);
+        else tma_load_3d(smem_u32(sm.v + stage * kKeyTileBytes), tm_v, 0, it * kTileKV, head, vb);
       }
       __syncwarp();
       ++v_issued;
@@ -290,9 +314,12 @@ __device__ __forceinline__ void producer_role(const CUtensorMap* tm_q, const CUt
     }
   }
   if (!ok) {
-    // let the copies still in flight land before the CTA gives up its shared memory: the Q tiles of the last work
-    // item begun, and the last kStages issued into either ring (earlier ones completed before their stage was reused)
-    if (q_issued > 0) (void)wait_bar_warp(&bars->q_full, (q_issued - 1) & 1, bars, a, 12, 0, false);
+    // let the copies still in flight land before the CTA gives up its shared memory: the Q tiles of the last two work
+    // items begun, and the last kStages issued into either ring (earlier ones completed before their stage was reused)
+    for (int back = 1; back <= 2; ++back) {
+      const int jq = q_issued - back;
+      if (jq >= 0) (void)wait_bar_warp(&bars->q_full[jq & 1], (jq >> 1) & 1, bars, a, 12, jq, false);
+    }
     for (int back = 1; back <= kStages; ++back) {
       const int jk = k_issued - back, jv = v_issued - back;
       if (jk >= 0) (void)wait_bar_warp(&bars->k_full[jk % kStages], (jk / kStages) & 1, bars, a, 12, jk, false);
@@ -304,20 +331,22 @@ __device__ __forceinline__ void producer_role(const CUtensorMap* tm_q, const CUt
 // ------------------------------------------------------------------ MMA issuer (one warp per query tile)
 // Per tile the order of events is fixed: S_t(j) is read by the softmax (s_free) before P_t(j) is
 // stored (p_full), which precedes the read of S_t(j+1).  The issuer of tile t therefore waits, in
-// turn, for "S_t(j) read and K_{j+1} loaded" -> Q K^T of step j+1, then "P_t(j) stored and V_j
-// loaded" -> P V of step j.  S_t(j+1) overwrites P_t(j-1) and part of S_t(j): the tensor core takes
+// turn, for "S_t(j) read and K_{j+1} loaded" -> Q K^T of step j+1 (or of step 0 of the next work
+// item), then "P_t(j) stored and V_j loaded" -> P V of step j.  S_t(j+1) overwrites P_t(j-1) and part of S_t(j): the tensor core takes
 // a thread's products in the order they were issued, and P V of step j-1 was issued before.
 // A K or V stage is released when both tiles' issuers have committed
 // their product on it (the empty barriers count two arrivals).
+//
+// The issuing is on the chain from the slowest warp of a step to the next scores, and it shares its scheduler with four softmax
+// warps, so each instruction of it counts: the lower halves of the operand descriptors advance by additions of a constant, the
+// upper halves are constants, and of several waits the one that is satisfied last comes last.
 template <int t>
-__device__ __forceinline__ void issue_qk(const AttnArgs& a, Barriers* bars, uint32_t tmem, uint64_t desc_q, uint32_t k_base,
-                                         int stage, bool odd) {
+__device__ __forceinline__ void issue_qk(Barriers* bars, uint32_t tmem, uint32_t desc_q, uint32_t desc_k, int stage, bool odd) {
   if (elect_one()) {
     constexpr uint32_t idesc = umma_idesc_bf16(kTileQ, kTileKV, false);
-    const uint64_t desc_k = umma_desc_sw128(k_base + stage * kTileBytes);
     const uint32_t d = tmem + t * kTmemTileStride + (odd ? kColSOdd : 0);
 #pragma unroll
-    for (int k = 0; k < kHeadDim / 16; ++k) umma_ss(d, desc_q + (k * 32 >> 4), desc_k + (k * 32 >> 4), idesc, k > 0);
+    for (int k = 0; k < kHeadDim / 16; ++k) umma_ss_lo(d, desc_q + (k * 32 >> 4), desc_k + (k * 32 >> 4), idesc, k > 0);
     umma_commit(smem_u32(&bars->s_full[t]));
     umma_commit(smem_u32(&bars->k_empty[stage]));
   }
@@ -327,16 +356,16 @@ __device__ __forceinline__ void issue_qk(const AttnArgs& a, Barriers* bars, uint
 // O_t += P_t V and, as columns 64..79 of the same product, the row sums of P: the descriptor's leading byte offset leads
 // from a slice of 16 keys of the V tile to the ones block, which serves as value columns 64..79 of every slice.
 template <int t>
-__device__ __forceinline__ void issue_pv(const AttnArgs& a, Barriers* bars, uint32_t tmem, uint32_t v_base, uint32_t ones,
-                                         int stage, bool odd, bool first) {
+__device__ __forceinline__ void issue_pv(Barriers* bars, uint32_t tmem, uint32_t desc_v, int stage, bool odd, bool first) {
   if (elect_one()) {
     constexpr uint32_t idesc = umma_idesc_bf16(kTileQ, kPvCols, true);
-    const uint32_t v = v_base + stage * kTileBytes;
+    constexpr uint32_t kSlice = 16 * kHeadDim * 2;   // bytes of 16 keys: the start moves on, the offset to the ones shrinks
+    constexpr uint32_t kAdvance = (kSlice >> 4) - ((kSlice >> 4) << 16);
     const uint32_t p = tmem + t * kTmemTileStride + (odd ? kColPOdd : 0);
+    umma_ts_lo(tmem + t * kTmemTileStride + kColO, p, desc_v, idesc, !first);
 #pragma unroll
-    for (int k = 0; k < kTileKV / 16; ++k)
-      umma_ts(tmem + t * kTmemTileStride + kColO, p + k * 8, umma_desc_sw128(v + k * 2048, ones - (v + k * 2048)), idesc,
-              (!first || k > 0) ? 1u : 0u);
+    for (int k = 1; k < kTileKV / 16; ++k)
+      umma_ts_lo(tmem + t * kTmemTileStride + kColO, p + k * 8, desc_v + k * kAdvance, idesc, true);
     umma_commit(smem_u32(&bars->o_done[t][odd]));
     umma_commit(smem_u32(&bars->v_empty[stage]));
   }
@@ -347,51 +376,47 @@ template <int t>
 __device__ __forceinline__ void mma_issue_loop(const AttnArgs& a, Barriers* bars, const SmemLayout& sm, uint32_t tmem) {
   static_assert(kStages >= 2, "the K ring must hold the tile in use and the next one");
   const int n_kv = a.n_kv_tiles;
-  const uint64_t desc_q = umma_desc_sw128(smem_u32(sm.q[t]));
-  const uint32_t k_base = smem_u32(sm.k), v_base = smem_u32(sm.v), ones = smem_u32(sm.ones);
+  // lower halves of the descriptors (umma_desc_lo)
+  const uint32_t q_desc = umma_desc_lo(smem_u32(sm.q) + t * kTileBytes, 16), k_desc = umma_desc_lo(smem_u32(sm.k), 16);
+  const uint32_t v_desc = umma_desc_lo(smem_u32(sm.v), smem_u32(sm.ones) - smem_u32(sm.v));
+  constexpr uint32_t kStage = kKeyTileBytes >> 4;         // a stage further on the start advances ...
+  constexpr uint32_t kStageV = kStage - (kStage << 16);   // ... and the offset to the ones shrinks
   if (n_kv == 0) return;   // no retained keys: the epilogue's two extra columns are the whole layer
 
   // Running over all work items of the CTA: the ring positions of the next K and V tile, and g, the number of key
-  // steps of this tile so far (the phase of the per-step barriers).  The rings carry the work item's own rows
-  // (the diagonal) only in the subsampled layer, where a CTA has one work item.
+  // steps of this tile so far (the phase of the per-step barriers).
   int k_stage = 0, v_stage = 0;
   uint32_t k_parity = 0, v_parity = 0;   // parity of their "full" phase
   int g = 0;
   int n_done = 0;
-  for (int item = blockIdx.x; item < a.n_work; item += gridDim.x, ++n_done, g += n_kv) {
-    if (!wait_bar_warp(&bars->q_full, n_done & 1, bars, a, 20, n_done)) return;
-    // first product of the work item: S_t must have been read by the softmax of the previous item's last step
-    if (n_done > 0 && !wait_bar_warp(&bars->s_free[t], (g - 1) & 1, bars, a, 22 + t, g - 1)) return;
-    if (!wait_bar_warp(&bars->k_full[k_stage], k_parity, bars, a, 21, g)) return;
-    tc_fence_after();
-    issue_qk<t>(a, bars, tmem, desc_q, k_base, k_stage, (g & 1) != 0);
-    if (++k_stage == kStages) { k_stage = 0; k_parity ^= 1; }
-    for (int j = 0; j < n_kv; ++j) {
-      if (j + 1 < n_kv) {
-        if (!wait_bar_warp(&bars->s_free[t], (g + j) & 1, bars, a, 22 + t, g + j)) return;
+  for (uint32_t item = blockIdx.x; item < static_cast<uint32_t>(a.n_work); item += gridDim.x, ++n_done, g += n_kv) {
+    const bool more = item + gridDim.x < static_cast<uint32_t>(a.n_work);
+    // j = -1: Q K^T of the CTA's first step, which no P V precedes
+    for (int j = n_done == 0 ? -1 : 0; j < n_kv; ++j) {
+      const bool last = j + 1 == n_kv;
+      if (!last || more) {
+        const int next = last ? 0 : j + 1;                  // step within its work item
+        const int next_item = last ? n_done + 1 : n_done;
+        const int place = next_item & 1;
+        if (next == 0 && !wait_bar_warp(&bars->q_full[place], (next_item >> 1) & 1, bars, a, 20, n_done)) return;
         if (!wait_bar_warp(&bars->k_full[k_stage], k_parity, bars, a, 24 + t, g + j)) return;
+        if (j >= 0 && !wait_bar_warp(&bars->s_free[t], (g + j) & 1, bars, a, 22 + t, g + j)) return;
         tc_fence_after();
-        issue_qk<t>(a, bars, tmem, desc_q, k_base, k_stage, ((g + j + 1) & 1) != 0);
+        issue_qk<t>(bars, tmem, q_desc + place * (kQTiles * kTileBytes >> 4), k_desc + k_stage * kStage, k_stage, ((g + j + 1) & 1) != 0);
         if (++k_stage == kStages) { k_stage = 0; k_parity ^= 1; }
-      } else {
-        // every Q K^T of this work item has been issued: when they have completed, Q may be overwritten
-        if (elect_one()) umma_commit(smem_u32(&bars->q_empty));
-        __syncwarp();
+        if (next + 1 == n_kv) {   // every Q K^T of the work item has been issued: when they have completed, Q may be overwritten
+          if (elect_one()) umma_commit(smem_u32(&bars->q_empty[place]));
+          __syncwarp();
+        }
       }
-      if (!wait_bar_warp(&bars->p_full[t][(g + j) & 1], ((g + j) >> 1) & 1, bars, a, 26 + t, g + j)) return;
+      if (j < 0) continue;
       if (!wait_bar_warp(&bars->v_full[v_stage], v_parity, bars, a, 28 + t, g + j)) return;
       // the first P V of a work item overwrites O_t: the previous item's epilogue must have read it out
       if (j == 0 && n_done > 0 && !wait_bar_warp(&bars->o_free[t], (n_done - 1) & 1, bars, a, 29, n_done)) return;
+      if (!wait_bar_warp(&bars->p_full[t][(g + j) & 1], ((g + j) >> 1) & 1, bars, a, 26 + t, g + j)) return;
       tc_fence_after();
-      issue_pv<t>(a, bars, tmem, v_base, ones, v_stage, ((g + j) & 1) != 0, j == 0);
+      issue_pv<t>(bars, tmem, v_desc + v_stage * kStageV, v_stage, ((g + j) & 1) != 0, j == 0);
       if (++v_stage == kStages) { v_stage = 0; v_parity ^= 1; }
-    }
-    // ring positions of the work item's own K/V rows (read by the softmax epilogue, not by any product)
-    if (a.use_diag) {
-      for (int i = 0; i < kQTiles; ++i) {
-        if (++k_stage == kStages) { k_stage = 0; k_parity ^= 1; }
-        if (++v_stage == kStages) { v_stage = 0; v_parity ^= 1; }
-      }
     }
   }
 }
@@ -439,8 +464,6 @@ struct SoftmaxThread {
   int h;        // which 16 of the 32 lanes of the warp's tensor-memory quarter
   int q;        // tensor-memory quarter (and scheduler): lanes [32 q, 32 q + 32)
   int lane;
-  int i;        // position in the quad: columns 2 i, 2 i + 1 of every 8
-  int r[2];     // the thread's two rows within the tile
   uint32_t base;   // tensor-memory address of the tile's columns, first lane of the warp's 16
 };
 
@@ -482,27 +505,21 @@ __device__ __forceinline__ void tmem_ld_rows16_scores(uint32_t taddr, uint32_t (
                : "r"(taddr + 96)
                : "memory");
 }
-__device__ __forceinline__ void tmem_ld_rows16_c64(uint32_t taddr, uint32_t (&r)[32]) {
+__device__ __forceinline__ void tmem_ld_rows16_c32(uint32_t taddr, uint32_t (&r)[16]) {
   asm volatile(
-      "tcgen05.ld.sync.aligned.16x256b.x8.b32 "
-      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+      "tcgen05.ld.sync.aligned.16x256b.x4.b32 "
+      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
       : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-        "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-        "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
       : "r"(taddr)
       : "memory");
 }
-__device__ __forceinline__ void tmem_st_rows16_c64(uint32_t taddr, const uint32_t (&r)[32]) {
+__device__ __forceinline__ void tmem_st_rows16_c32(uint32_t taddr, const uint32_t (&r)[16]) {
   asm volatile(
-      "tcgen05.st.sync.aligned.16x256b.x8.b32 [%0], "
-      "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, "
-      "%17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32};"
+      "tcgen05.st.sync.aligned.16x256b.x4.b32 [%0], "
+      "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};"
       ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]),
-        "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]),
-        "r"(r[16]), "r"(r[17]), "r"(r[18]), "r"(r[19]), "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]),
-        "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]), "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31])
+        "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
       : "memory");
 }
 // bf16 pairs of 4 blocks of 8 keys: register 2 n + hi -> row hi of the thread, pair column 4 n + i
@@ -545,10 +562,8 @@ __device__ __forceinline__ void quad_transpose(uint32_t& w0, uint32_t& w1, uint3
 
 // Running state of the thread's two rows (the same in all four threads of a quad, except the partial sums).
 struct RowState {
-  float m[2];             // reference maximum of the stored exponentials (log2 units)
-  float neg_m[2];         // -m (0 before the first tile)
-  float jump_above[2];    // raw score above which the reference has to move (-inf before the first tile)
-  float clamp_below[2];   // raw score below which the polynomial is not valid
+  float neg_m[2];         // minus the reference maximum of the stored exponentials (log2 units); +inf before the first tile
+  float jump_above[2];    // raw score above which the reference has to move; -inf before the first tile
   float l_exact[2];       // this thread's part of the sum of the unrounded 2^(scale_log2 * s - m): log-sum-exp output only
 };
 
@@ -603,15 +618,16 @@ __device__ __forceinline__ void exp_group(const uint32_t (&s)[4 * kBlocks], cons
 // waits and sums, 1860 with the vote instead of the shuffles, 1740 with the first group ahead of it, 1695 with the range check
 // of the polynomial in the same vote instead of a clamp per score.
 //
-// j: step within the work item; g: the tile's steps in the CTA's earlier work items.  kPoly: blocks of 8 columns
+// gj: this tile's key steps so far, over all work items of the CTA.  kPoly: blocks of 8 columns
 // whose exponentials are polynomials.  kLse: also keep the sum of the unrounded exponentials, for the
-// log-sum-exp output.  kMasked: columns >= valid are excluded (valid may be <= 0).
+// log-sum-exp output.  kMasked: columns >= valid are excluded.
 template <bool kMasked, bool kLse, uint32_t kPoly>
-__device__ __forceinline__ bool softmax_step(const SoftmaxThread& me, int j, int g, int valid, RowState& st, Barriers* bars,
+__device__ __forceinline__ bool softmax_step(const SoftmaxThread& me, int gj, int valid, RowState& st, Barriers* bars,
                                              const AttnArgs& a) {
-  const int gj = g + j;   // this tile's key steps so far, over all work items of the CTA: the phase of the per-step barriers
   const bool odd = (gj & 1) != 0;
   const uint32_t tP = me.base + (odd ? kColPOdd : 0);
+  if (!wait_bar(&bars->s_full[me.t], gj & 1, bars, a, 40 + me.t, gj)) return false;
+  tc_fence_after();
   uint32_t s[4 * kBlocks];
   tmem_ld_rows16_scores(me.base + (odd ? kColSOdd : 0), s);
   tmem_wait_ld();     // for the whole warp: lane 0 may speak for it
@@ -621,7 +637,7 @@ __device__ __forceinline__ bool softmax_step(const SoftmaxThread& me, int j, int
   if (kMasked) {
 #pragma unroll
     for (int c = 0; c < 4 * kBlocks; ++c)
-      if (8 * (c >> 2) + 2 * me.i + (c & 1) >= valid) s[c] = __float_as_uint(-INFINITY);
+      if (8 * (c >> 2) + 2 * (me.lane & 3) + (c & 1) >= valid) s[c] = __float_as_uint(-INFINITY);
   }
   const int n_blocks = kMasked ? (valid + 7) >> 3 : kBlocks;   // blocks of 8 columns that hold a key
   const uint64_t scale2 = pack_f32x2(a.scale_log2, a.scale_log2);
@@ -646,7 +662,7 @@ __device__ __forceinline__ bool softmax_step(const SoftmaxThread& me, int j, int
 #pragma unroll
     for (int b = 0; b < kBlocks; ++b)
       if ((kPoly >> b) & 1) mn[hi] = min3(mn[hi], __uint_as_float(s[4 * b + 2 * hi]), __uint_as_float(s[4 * b + 2 * hi + 1]));
-    look = look || mx[hi] > st.jump_above[hi] || (kPoly != 0 && mn[hi] < st.clamp_below[hi]);
+    look = look || mx[hi] > st.jump_above[hi] || (kPoly != 0 && mn[hi] < st.jump_above[hi] - a.poly_range);
   }
   if (__any_sync(0xffffffffu, look)) {
     float alpha[2];
@@ -657,34 +673,39 @@ __device__ __forceinline__ bool softmax_step(const SoftmaxThread& me, int j, int
       alpha[hi] = 1.0f;
       if (row_max > st.jump_above[hi]) {
         const float m = row_max * a.scale_log2;
-        alpha[hi] = ex2_approx(st.m[hi] - m);   // 0 on the first tile (m = -inf)
-        st.m[hi] = m;
+        jump_any = jump_any || st.neg_m[hi] != INFINITY;   // nothing to rescale on the first tile
+        alpha[hi] = ex2_approx(-m - st.neg_m[hi]);
         st.neg_m[hi] = -m;
         st.jump_above[hi] = (m + kRescaleThreshold) * a.inv_scale_log2;
-        st.clamp_below[hi] = (m + kPolyLowest) * a.inv_scale_log2;
         if (kLse) st.l_exact[hi] *= alpha[hi];
-        jump_any = true;
       }
     }
-    if (j > 0 && __any_sync(0xffffffffu, jump_any)) {
+    if (__any_sync(0xffffffffu, jump_any)) {
       // O_t must be at rest
       if (!wait_bar(&bars->o_done[me.t][!odd], ((gj - 1) >> 1) & 1, bars, a, 30 + me.t, gj)) return false;
       tc_fence_after();
-      uint32_t o[32], l[4];   // the warp's 16 rows of the accumulator: register 4 b + 2 hi + e is row hi
-      tmem_ld_rows16_c64(me.base + kColO, o);
+      // the warp's 16 rows of the accumulator, 32 columns at a time (register 4 b + 2 hi + e is row hi): with the scores in
+      // registers there is no room for more
+#pragma unroll 1
+      for (int half = 0; half < 2; ++half) {
+        uint32_t o[16];
+        tmem_ld_rows16_c32(me.base + kColO + 32 * half, o);
+        tmem_wait_ld();
+#pragma unroll
+        for (int c = 0; c < 16; ++c) o[c] = __float_as_uint(__uint_as_float(o[c]) * alpha[(c >> 1) & 1]);
+        tmem_st_rows16_c32(me.base + kColO + 32 * half, o);
+      }
+      uint32_t l[4];
       tmem_ld_rows16_c8(me.base + kColL, l);
       tmem_wait_ld();
 #pragma unroll
-      for (int c = 0; c < 32; ++c) o[c] = __float_as_uint(__uint_as_float(o[c]) * alpha[(c >> 1) & 1]);
-#pragma unroll
       for (int c = 0; c < 4; ++c) l[c] = __float_as_uint(__uint_as_float(l[c]) * alpha[c >> 1]);
-      tmem_st_rows16_c64(me.base + kColO, o);
       tmem_st_rows16_c8(me.base + kColL, l);
     }
     if (kPoly != 0) {
 #pragma unroll
       for (int c = 0; c < 4 * kBlocks; ++c)
-        if ((kPoly >> (c >> 2)) & 1) s[c] = __float_as_uint(fmaxf(__uint_as_float(s[c]), st.clamp_below[(c >> 1) & 1]));
+        if ((kPoly >> (c >> 2)) & 1) s[c] = __float_as_uint(fmaxf(__uint_as_float(s[c]), st.jump_above[(c >> 1) & 1] - a.poly_range));
     }
     if (kAhead) exp_group<0, kMasked, kLse, kPoly>(s, st, scale2, sum_exact2, pk, n_blocks);
   }
@@ -730,195 +751,292 @@ __device__ __forceinline__ bool flush_row_sums(const SoftmaxThread& me, int last
   return true;
 }
 
-// 4-byte word (two bf16) number w (0..31) of row r of a 128-byte-swizzled tile
-__device__ __forceinline__ uint32_t ld_swizzled_word(const uint8_t* tile, int r, int w) {
-  return *reinterpret_cast<const uint32_t*>(tile + r * 128 + (((w >> 2) ^ (r & 7)) << 4) + ((w & 3) << 2));
+// acc + the sum over the 8 products of two 16-byte pieces of bf16, or of one with 8 floats
+__device__ __forceinline__ float dot_bf16x8(const uint4& x, const uint4& y, float acc) {
+  acc = fma_bf16x2_to_f32(x.x, y.x, acc);
+  acc = fma_bf16x2_to_f32(x.y, y.y, acc);
+  acc = fma_bf16x2_to_f32(x.z, y.z, acc);
+  return fma_bf16x2_to_f32(x.w, y.w, acc);
+}
+__device__ __forceinline__ float dot_bf16x8_f32(const uint4& x, const float4& a, const float4& b, float acc) {
+  acc = fmaf(__uint_as_float(x.x << 16), a.x, acc);
+  acc = fmaf(__uint_as_float(x.x & 0xffff0000u), a.y, acc);
+  acc = fmaf(__uint_as_float(x.y << 16), a.z, acc);
+  acc = fmaf(__uint_as_float(x.y & 0xffff0000u), a.w, acc);
+  acc = fmaf(__uint_as_float(x.z << 16), b.x, acc);
+  acc = fmaf(__uint_as_float(x.z & 0xffff0000u), b.y, acc);
+  acc = fmaf(__uint_as_float(x.w << 16), b.z, acc);
+  return fmaf(__uint_as_float(x.w & 0xffff0000u), b.w, acc);
 }
 
-// One work item of a softmax thread: the key steps, then the epilogue.  g: this tile's key steps in the CTA's earlier
-// work items; n_done: work items before this one.
-__device__ __forceinline__ bool softmax_item(const AttnArgs& a, Barriers* bars, const SmemLayout& sm, const SoftmaxThread& me,
-                                             const CtaProblem& cta, int g, int n_done) {
+// What the epilogue of a work item needs of its rows' running state (shared memory; a row's warp writes and reads it).
+struct RowResults {
+  float neg_m[kQTiles * kTileQ];     // minus the reference maximum
+  float l_exact[kQTiles * kTileQ];   // sum of the unrounded exponentials: log-sum-exp output only
+};
+
+// Epilogue of a work item: diagonal and mean-fill terms, normalisation, store of this thread's 16 output dimensions of two
+// rows.  last: the tile's latest key step, the item's last.
+//
+// The queries' own Q, K and V rows are read straight from global memory (at the item's start the warp asked for them to be
+// brought to L2), 16 bytes per thread and half row, and asked for before the first use.
+template <bool kLse, bool kExtra>
+__device__ __forceinline__ bool softmax_epilogue(const AttnArgs& a, Barriers* bars, const SoftmaxThread& me, const RowResults* res,
+                                                 uint32_t item, int last) {
   const Plan& pl = a.pl;
-  const int n_kv = a.n_kv_tiles;
-  const int t = me.t, lane = me.lane;
-  RowState st;
+  const WorkItem wi = work_item(a, item);
+  const QueryTile tile = query_tile(wi, me.t);
+  const int t = me.t, head = wi.head;
+  const int i = me.lane & 3;                             // position in the quad
+  const int r0 = 32 * me.q + 16 * me.h + (me.lane >> 2);   // the thread's two rows within the tile: r0, r0 + 8
+
+  // base-2 logits of the two extra columns: each thread of the quad takes 16 dimensions (8 i .. and 32 + 8 i ..), then the quad
+  // adds up (every thread runs the shuffles; rows without the term carry zeros)
+  float l_d[2] = {-INFINITY, -INFINITY}, l_m[2] = {-INFINITY, -INFINITY};
+  uint32_t vw[2][8];   // the row's own V: chunks i and 4 + i of 16 bytes, then the words 4 b + i
+  if (kExtra) {
+    uint4 q[2][2], k[2][2];
+    float4 km[4];
+    bool dropped[2] = {false, false};
 #pragma unroll
-  for (int hi = 0; hi < 2; ++hi) {
-    st.m[hi] = -INFINITY;
-    st.neg_m[hi] = 0.f;
-    st.jump_above[hi] = -INFINITY;
-    st.clamp_below[hi] = -INFINITY;
-    st.l_exact[hi] = 0.f;
-  }
-  const bool want_lse = a.lse != nullptr;
-
-  int j = 0;
-#pragma unroll 1
-  while (j < n_kv) {
-    const int stop = n_kv - j > kFlushSteps ? j + kFlushSteps : n_kv;
-#pragma unroll 1
-    for (; j < stop; ++j) {
-      if (!wait_bar(&bars->s_full[t], (g + j) & 1, bars, a, 40 + t, g + j)) return false;
-      tc_fence_after();
-      const int valid = static_cast<int>(a.n_keys - static_cast<int64_t>(j) * kTileKV);
-      bool ok;
-      // the masked (last, ragged) tile keeps every exponential on the special-function unit, where -inf gives an exact 0
-      if (valid < kTileKV) ok = want_lse ? softmax_step<true, true, 0>(me, j, g, valid, st, bars, a)
-                                         : softmax_step<true, false, 0>(me, j, g, valid, st, bars, a);
-      else if (want_lse) ok = softmax_step<false, true, kPolyBlocks>(me, j, g, valid, st, bars, a);
-      else ok = softmax_step<false, false, kPolyBlocks>(me, j, g, valid, st, bars, a);
-      if (!ok) return false;
+    for (int hi = 0; hi < 2; ++hi) {
+      const int row = tile.q0 + r0 + 8 * hi;   // query token
+      uint4 v0 = make_uint4(0u, 0u, 0u, 0u), v1 = v0;
+      q[hi][0] = q[hi][1] = k[hi][0] = k[hi][1] = v0;
+      if (row >= tile.first && row < tile.last) {
+        const size_t at = (static_cast<size_t>(row) * pl.H + head) * (kHeadDim / 8) + i;
+        q[hi][0] = __ldg(a.Q + at);
+        q[hi][1] = __ldg(a.Q + at + 4);
+        if (a.use_diag) {
+          k[hi][0] = __ldg(a.K + at);
+          k[hi][1] = __ldg(a.K + at + 4);
+          v0 = __ldg(a.V + at);
+          v1 = __ldg(a.V + at + 4);
+        }
+      }
+      vw[hi][0] = v0.x; vw[hi][1] = v0.y; vw[hi][2] = v0.z; vw[hi][3] = v0.w;
+      vw[hi][4] = v1.x; vw[hi][5] = v1.y; vw[hi][6] = v1.z; vw[hi][7] = v1.w;
     }
-    if (j < n_kv && !flush_row_sums(me, g + j - 1, bars, a)) return false;
+    if (a.use_mean) {
+      const float4* src = reinterpret_cast<const float4*>(a.kmean + head * kHeadDim + 8 * i);
+      km[0] = __ldg(src);
+      km[1] = __ldg(src + 1);
+      km[2] = __ldg(src + 8);
+      km[3] = __ldg(src + 9);
+    }
+    if (a.use_diag) {
+#pragma unroll
+      for (int hi = 0; hi < 2; ++hi) {
+        const int row = tile.q0 + r0 + 8 * hi;
+        if (row >= tile.first && row < tile.last) {
+          const int32_t f = row / pl.L;
+          dropped[hi] = (a.slot_of_token != nullptr ? a.slot_of_token[row] : compact_slot(pl, f, row - f * pl.L)) < 0;
+        }
+      }
+#pragma unroll
+      for (int hi = 0; hi < 2; ++hi) {
+        const float acc = quad_sum(dot_bf16x8(q[hi][1], k[hi][1], dot_bf16x8(q[hi][0], k[hi][0], 0.f)));
+        if (dropped[hi]) l_d[hi] = acc * a.scale_log2;
+      }
+    }
+    if (a.use_mean) {
+#pragma unroll
+      for (int hi = 0; hi < 2; ++hi) {
+        const float acc = quad_sum(dot_bf16x8_f32(q[hi][1], km[2], km[3], dot_bf16x8_f32(q[hi][0], km[0], km[1], 0.f)));
+        l_m[hi] = fmaf(acc, a.scale_log2, a.log2_count[dropped[hi] ? 1 : 0]);
+      }
+    }
+    if (a.use_diag) {
+#pragma unroll
+      for (int hi = 0; hi < 2; ++hi) {
+        quad_transpose(vw[hi][0], vw[hi][1], vw[hi][2], vw[hi][3], i);
+        quad_transpose(vw[hi][4], vw[hi][5], vw[hi][6], vw[hi][7], i);
+      }
+    }
   }
 
-  // ---- epilogue: diagonal and mean-fill terms, normalisation, store of this thread's 16 output dimensions of two rows
-  const int head = cta.head;
-  if (n_kv > 0) {
-    const int last = g + n_kv - 1;
+  uint32_t l[4] = {0u, 0u, 0u, 0u};   // thread 0 of a quad: the row sums, in two parts, in registers 0 + 1 (row 0) and 2 + 3 (row 1)
+  if (a.n_kv_tiles > 0) {
     if (!wait_bar(&bars->o_done[t][last & 1], (last >> 1) & 1, bars, a, 50 + t, last)) return false;
     tc_fence_after();
-  }
-  // completed long ago: makes the Q tile visible to this thread.  Only the two extra columns read Q here, and a CTA
-  // that has them has one work item (a later item's Q may already be on its way otherwise).
-  if ((a.use_diag || a.use_mean) && !wait_bar(&bars->q_full, n_done & 1, bars, a, 52, 0)) return false;
-  const int item = n_kv + t;                         // ring item holding this tile's own K/V rows
-  const uint8_t* sKd = sm.k + (item % kStages) * kTileBytes;
-  const uint8_t* sVd = sm.v + (item % kStages) * kTileBytes;
-  if (a.use_diag) {
-    const uint32_t par = (item / kStages) & 1;
-    if (!wait_bar(&bars->k_full[item % kStages], par, bars, a, 53, item)) return false;
-    if (!wait_bar(&bars->v_full[item % kStages], par, bars, a, 54, item)) return false;
-  }
-  const uint8_t* sQ = sm.q[t];
-
-  uint32_t o[32];   // register 4 b + 2 hi + e: row hi, output dimension 8 b + 2 i + e
-  uint32_t l[4];    // thread 0 of a quad: the row sums, in two parts, in registers 0 + 1 (row 0) and 2 + 3 (row 1)
-  if (n_kv > 0) {
-    tmem_ld_rows16_c64(me.base + kColO, o);
     tmem_ld_rows16_c8(me.base + kColL, l);
     tmem_wait_ld();
-    // O_t is in registers: the next work item's first P V may overwrite it
-    tc_fence_before();
-    __syncwarp();
-    if (lane == 0) mbar_arrive(smem_u32(&bars->o_free[t]));
-  } else {   // no retained keys at all: the accumulator was never written
-#pragma unroll
-    for (int c = 0; c < 32; ++c) o[c] = 0u;
-#pragma unroll
-    for (int c = 0; c < 4; ++c) l[c] = 0u;
   }
-
+  float w_s[2], w_d[2], w_m[2];   // weights of the accumulator, of the row's own V and of the mean Value
 #pragma unroll
   for (int hi = 0; hi < 2; ++hi) {
-    const int r = me.r[hi];
-    const int row = cta.q0 + t * kTileQ + r;           // query token
-    const bool row_valid = row < cta.row_end;
-    bool is_dropped = false;   // only the diagonal term asks
-    if (a.use_diag && row_valid) {
-      const int32_t f = row / pl.L;
-      is_dropped = (a.slot_of_token != nullptr ? a.slot_of_token[row] : compact_slot(pl, f, row - f * pl.L)) < 0;
-    }
+    const int r = r0 + 8 * hi;
     // the row's sums: of the rounded probabilities (the normaliser), of the unrounded ones (log-sum-exp)
-    const float l_run = __shfl_sync(0xffffffffu, __uint_as_float(l[2 * hi]) + __uint_as_float(l[2 * hi + 1]), lane & ~3);
-    const float l_exact = want_lse ? quad_sum(st.l_exact[hi]) : 0.f;
-    const float m_used = st.m[hi];
-    // base-2 logits of the two extra columns: each thread of the quad takes its 16 dimensions, then the quad adds up
-    // (every thread runs the shuffles; rows without the term carry zeros)
-    const bool has_diag = a.use_diag && is_dropped;
-    const int64_t count = pl.n_dropped - (has_diag ? 1 : 0);
-    const bool has_mean = a.use_mean && count > 0;
-    float acc_d = 0.f, acc_m = 0.f;
-    if (a.use_diag || a.use_mean) {
-#pragma unroll
-      for (int b = 0; b < 8; ++b) {
-        const uint32_t qw = ld_swizzled_word(sQ, r, 4 * b + me.i);
-        const float q0 = __uint_as_float(qw << 16), q1 = __uint_as_float(qw & 0xffff0000u);
-        if (has_diag) {
-          const uint32_t kw = ld_swizzled_word(sKd, r, 4 * b + me.i);
-          acc_d = fmaf(q0, __uint_as_float(kw << 16), acc_d);
-          acc_d = fmaf(q1, __uint_as_float(kw & 0xffff0000u), acc_d);
-        }
-        if (has_mean) {
-          const float2 km = __ldg(reinterpret_cast<const float2*>(a.kmean + head * kHeadDim + 8 * b + 2 * me.i));
-          acc_m = fmaf(q0, km.x, acc_m);
-          acc_m = fmaf(q1, km.y, acc_m);
-        }
+    const float l_run = __shfl_sync(0xffffffffu, __uint_as_float(l[2 * hi]) + __uint_as_float(l[2 * hi + 1]), me.lane & ~3);
+    float p_d = 0.f, p_m = 0.f, a_s = 1.0f, m_fin = 0.f;
+    if (kExtra || kLse) {
+      const float m = -res->neg_m[t * kTileQ + r];
+      m_fin = m;
+      if (kExtra) {
+        m_fin = fmaxf(m, fmaxf(l_d[hi], l_m[hi]));
+        a_s = exp2f(m - m_fin);
+        p_d = exp2f(l_d[hi] - m_fin);              // 0 when the term is absent
+        p_m = exp2f(l_m[hi] - m_fin);
       }
-      acc_d = quad_sum(acc_d);
-      acc_m = quad_sum(acc_m);
-    }
-    float m_fin = m_used, a_s = 1.0f, p_d = 0.f, p_m = 0.f;
-    if (a.use_diag || a.use_mean) {   // the same for every row of the launch; frame attention has neither
-      float l_d = -INFINITY, l_m = -INFINITY;
-      if (has_diag) l_d = acc_d * a.scale_log2;
-      if (has_mean) {
-        l_m = acc_m * a.scale_log2;
-        if (pl.mean_fill == AVGGT_MEAN_FILL) l_m += log2f(static_cast<float>(count));
-      }
-      m_fin = fmaxf(m_used, fmaxf(l_d, l_m));
-      a_s = exp2f(m_used - m_fin);
-      p_d = exp2f(l_d - m_fin);              // 0 when the term is absent
-      p_m = exp2f(l_m - m_fin);
     }
     const float z = fmaf(l_run, a_s, p_d + p_m);
     const float inv_z = __fdividef(1.0f, z);   // z is at least one exponential of a row maximum, far from the ends of the range
-    const float w_s = a_s * inv_z, w_d = p_d * inv_z, w_m = p_m * inv_z;
-    // the thread's 8 words of the output row: word 4 b + i (dimensions 8 b + 2 i, 8 b + 2 i + 1)
-    uint32_t w[8];
-#pragma unroll
-    for (int b = 0; b < 8; ++b) {
-      float v0 = __uint_as_float(o[4 * b + 2 * hi]) * w_s, v1 = __uint_as_float(o[4 * b + 2 * hi + 1]) * w_s;
-      if (w_d != 0.f) {
-        const uint32_t vw = ld_swizzled_word(sVd, r, 4 * b + me.i);
-        v0 = fmaf(w_d, __uint_as_float(vw << 16), v0);
-        v1 = fmaf(w_d, __uint_as_float(vw & 0xffff0000u), v1);
-      }
-      if (has_mean) {
-        const float2 vm = __ldg(reinterpret_cast<const float2*>(a.vmean + head * kHeadDim + 8 * b + 2 * me.i));
-        v0 = fmaf(w_m, vm.x, v0);
-        v1 = fmaf(w_m, vm.y, v1);
-      }
-      w[b] = pack_bf16x2(v0, v1);
-    }
-    // Transposed within the quad, a thread holds 16 contiguous bytes of each half of the row: 4 stores of 16 bytes
-    // per thread instead of 16 of 4 bytes (whose 8 rows x 16 bytes per warp instruction kept the store path of the
-    // SM busy for thousands of clocks per work item).
-    quad_transpose(w[0], w[1], w[2], w[3], me.i);
-    quad_transpose(w[4], w[5], w[6], w[7], me.i);
-    if (row_valid) {
-      uint4* dst = reinterpret_cast<uint4*>(a.O + (static_cast<size_t>(row) * pl.H + head) * kHeadDim);
-      dst[me.i] = make_uint4(w[0], w[1], w[2], w[3]);
-      dst[4 + me.i] = make_uint4(w[4], w[5], w[6], w[7]);
-      if (want_lse && me.i == 0) {
-        const float z_exact = fmaf(l_exact, a_s, p_d + p_m);
+    w_s[hi] = a_s * inv_z;
+    w_d[hi] = p_d * inv_z;
+    w_m[hi] = p_m * inv_z;
+    if (kLse && i == 0) {
+      const int row = tile.q0 + r;
+      const float z_exact = fmaf(res->l_exact[t * kTileQ + r], a_s, p_d + p_m);
+      if (row >= tile.first && row < tile.last)
         a.lse[static_cast<size_t>(row) * pl.H + head] = (m_fin + log2f(z_exact)) * 0.6931471805599453f;
+    }
+  }
+#pragma unroll
+  for (int half = 0; half < 2; ++half) {   // 32 output dimensions at a time: with more the registers run over
+    float2 vm[4];     // the mean Value at the thread's output dimensions 8 b + 2 i, 8 b + 2 i + 1
+    if (kExtra && a.use_mean) {
+      const float2* src = reinterpret_cast<const float2*>(a.vmean + head * kHeadDim + 32 * half) + i;
+#pragma unroll
+      for (int b = 0; b < 4; ++b) vm[b] = __ldg(src + 4 * b);
+    }
+    uint32_t o[16];   // register 4 b + 2 hi + e: row hi, output dimension 8 b + 2 i + e; zero with no retained keys at all
+#pragma unroll
+    for (int c = 0; c < 16; ++c) o[c] = 0u;
+    if (a.n_kv_tiles > 0) {
+      tmem_ld_rows16_c32(me.base + kColO + 32 * half, o);
+      tmem_wait_ld();
+      if (half == 1) {   // O_t has been read: the next work item's first P V may overwrite it
+        tc_fence_before();
+        if (me.lane == 0) mbar_arrive(smem_u32(&bars->o_free[t]));
+      }
+    }
+#pragma unroll
+    for (int hi = 0; hi < 2; ++hi) {
+      const int row = tile.q0 + r0 + 8 * hi;
+      uint32_t w[4];   // the thread's words of the output row: word 4 b + i (dimensions 8 b + 2 i, 8 b + 2 i + 1)
+#pragma unroll
+      for (int b = 0; b < 4; ++b) {
+        float v0 = __uint_as_float(o[4 * b + 2 * hi]) * w_s[hi], v1 = __uint_as_float(o[4 * b + 2 * hi + 1]) * w_s[hi];
+        if (kExtra && a.use_diag) {
+          v0 = fmaf(w_d[hi], __uint_as_float(vw[hi][4 * half + b] << 16), v0);
+          v1 = fmaf(w_d[hi], __uint_as_float(vw[hi][4 * half + b] & 0xffff0000u), v1);
+        }
+        if (kExtra && a.use_mean) {
+          v0 = fmaf(w_m[hi], vm[b].x, v0);
+          v1 = fmaf(w_m[hi], vm[b].y, v1);
+        }
+        w[b] = pack_bf16x2(v0, v1);
+      }
+      // Transposed within the quad, a thread holds 16 contiguous bytes of the row: 4 stores of 16 bytes
+      // per thread instead of 16 of 4 bytes (whose 8 rows x 16 bytes per warp instruction kept the store path of the
+      // SM busy for thousands of clocks per work item).
+      quad_transpose(w[0], w[1], w[2], w[3], i);
+      if (row >= tile.first && row < tile.last) {
+        uint4* dst = reinterpret_cast<uint4*>(a.O + (static_cast<size_t>(row) * pl.H + head) * kHeadDim);
+        dst[4 * half + i] = make_uint4(w[0], w[1], w[2], w[3]);
       }
     }
   }
   return true;
 }
 
-__device__ __forceinline__ void softmax_role(const AttnArgs& a, Barriers* bars, const SmemLayout& sm, uint32_t tmem, int warp,
-                                             int lane) {
+// The work items of a softmax thread.  The epilogue of an item runs after the first step of the next item: by then its last
+// P V has completed, the next item's P V waits for O to be read out (o_free) but its scores do not, and the tensor core and the
+// copies are a step ahead.
+template <bool kLse, bool kExtra>
+__device__ __forceinline__ void softmax_items(const AttnArgs& a, Barriers* bars, const SoftmaxThread& me, RowResults* res) {
+  const int n_kv = a.n_kv_tiles;
+  const int t = me.t;
+  const bool ragged = a.last_tile_keys != 0;
+  bool res_rows = false;   // the warp had rows in the item before
+  int gj = 0;              // this tile's key steps so far, over all work items of the CTA: the phase of the per-step barriers
+#pragma unroll 1
+  for (uint32_t item = blockIdx.x;; item += gridDim.x) {
+    const bool have = item < static_cast<uint32_t>(a.n_work);
+    bool pending = item != blockIdx.x;   // the epilogue of the item before
+    if (!have && !pending) return;
+    RowState st;
+#pragma unroll
+    for (int hi = 0; hi < 2; ++hi) {
+      st.neg_m[hi] = INFINITY;
+      st.jump_above[hi] = -INFINITY;
+      st.l_exact[hi] = 0.f;
+    }
+    bool rows = false;
+    if (have) {
+      const WorkItem wi = work_item(a, item);
+      const QueryTile tile = query_tile(wi, t);
+      const int row0 = tile.q0 + 32 * me.q + 16 * me.h;   // the warp's first row
+      rows = row0 + 16 > tile.first && row0 < tile.last;
+      if (kExtra && a.use_diag) {   // each thread asks for one line: K of row lane / 2, or V
+        const int row = row0 + (me.lane >> 1);
+        if (row >= tile.first && row < tile.last)
+          prefetch_l2(((me.lane & 1) ? a.V : a.K) + (static_cast<size_t>(row) * a.pl.H + wi.head) * (kHeadDim / 8));
+      }
+    }
+    int left = have ? n_kv : 0;
+#pragma unroll 1
+    do {
+      const int most = pending ? 1 : kFlushSteps;
+      const int chunk = left < most ? left : most;
+      left -= chunk;
+      const int stop = gj + chunk;
+      if (rows) {
+        // the ragged last tile apart, with every exponential on the special-function unit, where -inf gives an exact 0
+        const int full = left == 0 && ragged ? stop - 1 : stop;
+#pragma unroll 1
+        for (; gj < full; ++gj)
+          if (!softmax_step<false, kLse, kPolyBlocks>(me, gj, kTileKV, st, bars, a)) return;
+        if (gj < stop) {
+          if (!softmax_step<true, kLse, 0>(me, gj, a.last_tile_keys, st, bars, a)) return;
+          ++gj;
+        }
+      } else {   // nothing to compute: the warp's share of S and P is released at once
+#pragma unroll 1
+        for (; gj < stop; ++gj) {
+          if (!wait_bar(&bars->s_full[t], gj & 1, bars, a, 40 + t, gj)) return;
+          if (me.lane == 0) {
+            mbar_arrive(smem_u32(&bars->s_free[t]));
+            mbar_arrive(smem_u32(&bars->p_full[t][gj & 1]));
+          }
+        }
+      }
+      if (pending) {
+        if (res_rows) {
+          if (!softmax_epilogue<kLse, kExtra>(a, bars, me, res, item - gridDim.x, stop - chunk - 1)) return;
+        } else if (me.lane == 0 && n_kv > 0) {
+          mbar_arrive(smem_u32(&bars->o_free[t]));
+        }
+        pending = false;
+      } else if (left > 0 && rows && !flush_row_sums(me, gj - 1, bars, a)) {
+        return;
+      }
+    } while (left > 0);
+    if (!have) return;
+    __syncwarp();   // every lane has read the results of the item before
+#pragma unroll
+    for (int hi = 0; hi < 2; ++hi) {
+      const int at = t * kTileQ + 32 * me.q + 16 * me.h + (me.lane >> 2) + 8 * hi;
+      const float l_exact = kLse ? quad_sum(st.l_exact[hi]) : 0.f;
+      if ((me.lane & 3) == 0) {
+        res->neg_m[at] = st.neg_m[hi];
+        if (kLse) res->l_exact[at] = l_exact;
+      }
+    }
+    __syncwarp();
+    res_rows = rows;
+  }
+}
+
+template <bool kLse, bool kExtra>
+__device__ __forceinline__ void softmax_role(const AttnArgs& a, Barriers* bars, RowResults* res, uint32_t tmem, int warp, int lane) {
   SoftmaxThread me;
   me.t = warp >> 3;
   me.h = (warp >> 2) & 1;
   me.q = warp & 3;
   me.lane = lane;
-  me.i = lane & 3;
-  me.r[0] = 32 * me.q + 16 * me.h + (lane >> 2);
-  me.r[1] = me.r[0] + 8;
   me.base = tmem + me.t * kTmemTileStride + (static_cast<uint32_t>(32 * me.q + 16 * me.h) << 16);   // TMEM lane = row
-  const int n_kv = a.n_kv_tiles;
-  int g = 0, n_done = 0;
-#pragma unroll 1
-  for (int item = blockIdx.x; item < a.n_work; item += gridDim.x) {
-    if (!softmax_item(a, bars, sm, me, work_item(a, item), g, n_done)) return;
-    g += n_kv;
-    ++n_done;
-  }
+  softmax_items<kLse, kExtra>(a, bars, me, res);
 }
 
 // Value columns 64..79 of a slice of 16 keys, in the 128-byte-swizzled layout of the V tiles: column 64 all ones, the others
@@ -934,18 +1052,19 @@ __device__ __forceinline__ void ones_block(uint8_t* ones, int tid) {
   fence_proxy_async_smem();
 }
 
+// kLse: write the log-sum-exp.  kExtra: there is a diagonal or a mean column (frame attention and the dense layer have neither).
+template <bool kLse, bool kExtra>
 __global__ void __launch_bounds__(kThreads, 1)
 global_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
-                   const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_kc,
-                   const __grid_constant__ CUtensorMap tm_vc, const AttnArgs a) {
+                   const __grid_constant__ CUtensorMap tm_v, const AttnArgs a) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   SmemLayout sm;
-  sm.q[0] = smem;
-  sm.q[1] = smem + kTileBytes;
-  sm.k = smem + kQTiles * kTileBytes;
-  sm.v = sm.k + kStages * kTileBytes;
-  sm.ones = sm.v + kStages * kTileBytes;
+  sm.q = smem;
+  sm.k = smem + 2 * kQTiles * kTileBytes;
+  sm.v = sm.k + kStages * kKeyTileBytes;
+  sm.ones = sm.v + kStages * kKeyTileBytes;
+  __shared__ RowResults row_results;
   __shared__ Barriers bars;
 
   const int tid = threadIdx.x;
@@ -954,8 +1073,10 @@ global_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
   if (__syncthreads_or(*reinterpret_cast<volatile uint32_t*>(a.status) != 0u)) return;
 
   if (tid == 0) {
-    mbar_init(smem_u32(&bars.q_full), 1);
-    mbar_init(smem_u32(&bars.q_empty), kQTiles);
+    for (int e = 0; e < 2; ++e) {
+      mbar_init(smem_u32(&bars.q_full[e]), 1);
+      mbar_init(smem_u32(&bars.q_empty[e]), kQTiles);
+    }
     for (int s = 0; s < kStages; ++s) {
       mbar_init(smem_u32(&bars.k_full[s]), 1);
       mbar_init(smem_u32(&bars.k_empty[s]), kQTiles);
@@ -987,10 +1108,10 @@ global_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
 
   if (warp < kSoftmaxWarps) {
     reg_inc<kRegsSoftmax>();
-    softmax_role(a, &bars, sm, tmem, warp, tid & 31);
+    softmax_role<kLse, kExtra>(a, &bars, &row_results, tmem, warp, tid & 31);
   } else {
     reg_dec<kRegsOther>();
-    if (warp == kTmaWarp) producer_role(&tm_q, &tm_k, &tm_v, &tm_kc, &tm_vc, a, &bars, sm);
+    if (warp == kTmaWarp) producer_role(&tm_q, &tm_k, &tm_v, a, &bars, sm);
     else if (warp == kMmaWarp) mma_role<0>(a, &bars, sm, tmem);
     else if (warp == kMmaWarp + 1) mma_role<1>(a, &bars, sm, tmem);
   }
@@ -1003,7 +1124,7 @@ global_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
   if (warp == kTmaWarp) tmem_dealloc(tmem, kTmemCols);
 }
 
-constexpr size_t kAttnSmemBytes = static_cast<size_t>(kTileBytes) * (kQTiles + 2 * kStages) + kOnesBytes + 1024;
+constexpr size_t kAttnSmemBytes = static_cast<size_t>(kTileBytes) * (2 * kQTiles) + static_cast<size_t>(kKeyTileBytes) * (2 * kStages) + kOnesBytes + 1024;
 
 }  // namespace
 
@@ -1015,7 +1136,11 @@ namespace {
 // registers the role split hands out.  setmaxnreg.inc waits, without a time limit, for registers that other
 // warps release; if the compiler gave the kernel fewer than kRegsLaunch registers per thread the pool could
 // never cover the softmax warps' share and the kernel would hang, so such a build refuses to launch.
-cudaError_t prepare_kernel() {
+typedef void (*AttnKernel)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const AttnArgs);
+constexpr AttnKernel kAttnKernels[4] = {global_attn_kernel<false, false>, global_attn_kernel<false, true>,
+                                        global_attn_kernel<true, false>, global_attn_kernel<true, true>};
+
+cudaError_t prepare_kernels() {
   static std::mutex mu;
   static bool ready[64] = {};
   int dev = 0;
@@ -1024,13 +1149,15 @@ cudaError_t prepare_kernel() {
   if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
   std::lock_guard<std::mutex> lock(mu);
   if (ready[dev]) return cudaSuccess;
-  cudaFuncAttributes fa;
-  e = cudaFuncGetAttributes(&fa, global_attn_kernel);
-  if (e != cudaSuccess) return e;
-  if (fa.numRegs * (kThreads / 32) < kRegsSoftmax * kSoftmaxWarps + kRegsOther * (kThreads / 32 - kSoftmaxWarps))
-    return cudaErrorLaunchOutOfResources;
-  e = cudaFuncSetAttribute(global_attn_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kAttnSmemBytes));
-  if (e != cudaSuccess) return e;
+  for (AttnKernel k : kAttnKernels) {
+    cudaFuncAttributes fa;
+    e = cudaFuncGetAttributes(&fa, k);
+    if (e != cudaSuccess) return e;
+    if (fa.numRegs * (kThreads / 32) < kRegsSoftmax * kSoftmaxWarps + kRegsOther * (kThreads / 32 - kSoftmaxWarps))
+      return cudaErrorLaunchOutOfResources;
+    e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kAttnSmemBytes));
+    if (e != cudaSuccess) return e;
+  }
   ready[dev] = true;
   return cudaSuccess;
 }
@@ -1043,6 +1170,9 @@ cudaError_t launch_attn(const Plan& pl, int sm_count, bool frame_mode, const voi
   AttnArgs a;
   a.pl = pl;
   a.slot_of_token = slot_of_token;
+  a.Q = static_cast<const uint4*>(Q);
+  a.K = static_cast<const uint4*>(K);
+  a.V = static_cast<const uint4*>(V);
   a.kmean = kmean;
   a.vmean = vmean;
   a.O = static_cast<__nv_bfloat16*>(O);
@@ -1051,48 +1181,48 @@ cudaError_t launch_attn(const Plan& pl, int sm_count, bool frame_mode, const voi
   a.frame_mode = frame_mode ? 1 : 0;
   a.n_keys = frame_mode ? pl.L : pl.M;
   a.n_kv_tiles = static_cast<int32_t>((a.n_keys + kTileKV - 1) / kTileKV);
+  a.last_tile_keys = static_cast<int32_t>(a.n_keys % kTileKV);
+  for (int dropped = 0; dropped < 2; ++dropped) {   // the mean column stands for every dropped column but the query's own
+    const int64_t count = pl.n_dropped - dropped;
+    a.log2_count[dropped] = count <= 0 ? -INFINITY : pl.mean_fill == AVGGT_MEAN_FILL ? log2f(static_cast<float>(count)) : 0.0f;
+  }
   a.use_diag = (!frame_mode && pl.diag != 0 && pl.n_dropped > 0) ? 1 : 0;
   a.use_mean = (!frame_mode && pl.mean_fill != 0 && pl.n_dropped > 0) ? 1 : 0;
   a.scale_log2 = pl.scale * kLog2e;
   a.inv_scale_log2 = 1.0f / a.scale_log2;
+  a.poly_range = (kRescaleThreshold - kPolyLowest) * a.inv_scale_log2;
   const int64_t rows = frame_mode ? pl.L : pl.n_tok;
   a.pairs = static_cast<int32_t>((rows + kQTiles * kTileQ - 1) / (kQTiles * kTileQ));
   a.n_work = a.pairs * pl.H * (frame_mode ? pl.n_frames : 1);
 
-  // token-major [n_tok, H*d] maps for Q and for K, V (the diagonal tiles; all tiles of frame attention);
-  // head-major [H, M, d] maps for Kc, Vc
-  CUtensorMap tm_q, tm_k, tm_v, tm_kc, tm_vc;
+  // token-major [n_tok, H*d] maps for Q and, in frame attention, K and V; head-major [H, M, d] maps for Kc, Vc otherwise
+  CUtensorMap tm_q, tm_k, tm_v;
   const uint64_t tok_dims[2] = {static_cast<uint64_t>(pl.H) * pl.d, static_cast<uint64_t>(pl.n_tok)};
   const uint64_t tok_str[1] = {static_cast<uint64_t>(pl.H) * pl.d * 2};
-  const uint32_t tok_box[2] = {kHeadDim, kTileQ};
-  // tiles of a frame's keys, or the queries' own rows
-  const uint32_t kv_box[2] = {kHeadDim, static_cast<uint32_t>(frame_mode ? kTileKV : kTileQ)};
-  const bool reads_kv = frame_mode || a.use_diag;
-  bool good = make_tmap_bf16(&tm_q, Q, 2, tok_dims, tok_str, tok_box);
-  good = good && make_tmap_bf16(&tm_k, reads_kv ? K : Q, 2, tok_dims, tok_str, kv_box);
-  good = good && make_tmap_bf16(&tm_v, reads_kv ? V : Q, 2, tok_dims, tok_str, kv_box);
-  if (frame_mode || pl.M == 0) {
-    tm_kc = tm_k;   // not read
-    tm_vc = tm_v;
-  } else {
+  const uint32_t q_box[2] = {kHeadDim, kTileQ};
+  bool good = make_tmap_bf16(&tm_q, Q, 2, tok_dims, tok_str, q_box);
+  if (frame_mode) {
+    const uint32_t kv_box[2] = {kHeadDim, kTileKV};
+    good = good && make_tmap_bf16(&tm_k, K, 2, tok_dims, tok_str, kv_box);
+    good = good && make_tmap_bf16(&tm_v, V, 2, tok_dims, tok_str, kv_box);
+  } else if (pl.M > 0) {
     const uint64_t c_dims[3] = {static_cast<uint64_t>(pl.d), static_cast<uint64_t>(pl.M), static_cast<uint64_t>(pl.H)};
     const uint64_t c_str[2] = {static_cast<uint64_t>(pl.d) * 2, static_cast<uint64_t>(pl.M) * pl.d * 2};
     const uint32_t c_box[3] = {kHeadDim, kTileKV, 1};
-    good = good && make_tmap_bf16(&tm_kc, Kc, 3, c_dims, c_str, c_box);
-    good = good && make_tmap_bf16(&tm_vc, Vc, 3, c_dims, c_str, c_box);
+    good = good && make_tmap_bf16(&tm_k, Kc, 3, c_dims, c_str, c_box);
+    good = good && make_tmap_bf16(&tm_v, Vc, 3, c_dims, c_str, c_box);
+  } else {
+    tm_k = tm_v = tm_q;   // not read
   }
   if (!good) { *tmap_failed = true; return cudaSuccess; }
 
-  cudaError_t e = prepare_kernel();
+  cudaError_t e = prepare_kernels();
   if (e != cudaSuccess) return e;
   e = cudaMemsetAsync(ws, 0, kAttnStatusBytes, st);
   if (e != cudaSuccess) return e;
-  // The subsampled layer: one work item per CTA (hundreds of key steps each).  Frame attention: a dozen key steps
-  // per work item, so one CTA per SM walks over many of them and the next item's loads and first product run
-  // under the current item's epilogue.
-  const unsigned grid = frame_mode ? static_cast<unsigned>(a.n_work < sm_count ? a.n_work : sm_count)
-                                   : static_cast<unsigned>(a.n_work);
-  global_attn_kernel<<<grid, kThreads, kAttnSmemBytes, st>>>(tm_q, tm_k, tm_v, tm_kc, tm_vc, a);
+  const unsigned grid = static_cast<unsigned>(a.n_work < sm_count ? a.n_work : sm_count);
+  const int which = (lse != nullptr ? 2 : 0) + (a.use_diag || a.use_mean ? 1 : 0);
+  kAttnKernels[which]<<<grid, kThreads, kAttnSmemBytes, st>>>(tm_q, tm_k, tm_v, a);
   return cudaGetLastError();
 }
 

@@ -61,6 +61,8 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
 #define AVGGT_WAIT_LIMIT_NS 200000000ull
 #endif
 
+__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+
 // ---------------------------------------------------------------- TMA
 __device__ __forceinline__ void prefetch_tensormap(const CUtensorMap* m) {
   asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(m)) : "memory");
@@ -122,15 +124,21 @@ __device__ __forceinline__ void umma_commit(uint32_t bar) {
 //   bits  0-13 start address >> 4      bits 16-29 leading byte offset >> 4
 //   bits 32-45 stride byte offset >> 4 bits 46-47 descriptor version (1)
 //   bits 61-63 swizzle mode (2 = 128 bytes)
-__device__ __forceinline__ uint64_t umma_desc_sw128(uint32_t saddr, uint32_t leading = 16) {
+__device__ __forceinline__ uint64_t umma_desc_sw128(uint32_t saddr) {
   uint64_t d = 0;
   d |= static_cast<uint64_t>((saddr & 0x3ffffu) >> 4);
-  d |= static_cast<uint64_t>((leading & 0x3ffffu) >> 4) << 16;   // unused for one 128-byte span
+  d |= static_cast<uint64_t>(1) << 16;            // leading byte offset: unused for one 128-byte span
   d |= static_cast<uint64_t>(1024 >> 4) << 32;    // stride between 8-row groups
   d |= static_cast<uint64_t>(1) << 46;
   d |= static_cast<uint64_t>(2) << 61;
   return d;
 }
+
+// The same descriptor as two halves: the upper one is a constant, and an operand advances by additions to the lower one.
+__device__ __forceinline__ uint32_t umma_desc_lo(uint32_t saddr, uint32_t leading) {
+  return ((saddr & 0x3ffffu) >> 4) | (((leading & 0x3ffffu) >> 4) << 16);
+}
+constexpr uint32_t kUmmaDescHi = (1024u >> 4) | (1u << 14) | (2u << 29);
 
 // Instruction descriptor for kind::f16 with bf16 operands and fp32 accumulate.
 //   bits 4-5 D format (1 = f32), 7-9 A format (1 = bf16), 10-12 B format (1 = bf16),
@@ -149,13 +157,24 @@ __device__ __forceinline__ void umma_ss(uint32_t d_tmem, uint64_t a_desc, uint64
       ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
       : "memory");
 }
-// D[tmem] (+)= A[tmem] * B[smem]; issued by a single thread.
-__device__ __forceinline__ void umma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
+// The same with the descriptors given by their lower halves, and D[tmem] (+)= A[tmem] * B[smem].
+__device__ __forceinline__ void umma_ss_lo(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t idesc, bool accumulate) {
   asm volatile(
-      "{\n\t.reg .pred p;\n\t"
+      "{\n\t.reg .pred p;\n\t.reg .b64 a, b;\n\t"
       "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
-      ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
+      "mov.b64 a, {%1, %5};\n\t"
+      "mov.b64 b, {%2, %5};\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, p;\n\t}"
+      ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(idesc), "r"(accumulate ? 1u : 0u), "n"(kUmmaDescHi)
+      : "memory");
+}
+__device__ __forceinline__ void umma_ts_lo(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t idesc, bool accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t.reg .b64 b;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "mov.b64 b, {%2, %5};\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], b, %3, p;\n\t}"
+      ::"r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(idesc), "r"(accumulate ? 1u : 0u), "n"(kUmmaDescHi)
       : "memory");
 }
 
@@ -221,6 +240,17 @@ __device__ __forceinline__ uint64_t sub_f32x2(uint64_t a, uint64_t b) {
   uint64_t d;
   asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
   return d;
+}
+// acc + the dot product of two pairs of bf16: the mixed-precision fma of sm_100 takes bf16 operands as they are (exact products)
+__device__ __forceinline__ float fma_bf16x2_to_f32(uint32_t x, uint32_t y, float acc) {
+  asm("{\n\t.reg .b16 xl, xh, yl, yh;\n\t"
+      "mov.b32 {xl, xh}, %1;\n\t"
+      "mov.b32 {yl, yh}, %2;\n\t"
+      "fma.rn.f32.bf16 %0, xl, yl, %0;\n\t"
+      "fma.rn.f32.bf16 %0, xh, yh, %0;\n\t}"
+      : "+f"(acc)
+      : "r"(x), "r"(y));
+  return acc;
 }
 // two floats -> packed bf16x2 (lo in the low half), round to nearest even
 __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
