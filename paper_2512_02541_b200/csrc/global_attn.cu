@@ -22,7 +22,7 @@
 //               be moved to the softmax warpgroups)
 // Tensor memory per tile (256 columns): two places for S and P that alternate (see kColSOdd), O (64) and the row
 // sums of P (16).  A softmax thread pulls its 56 scores of S into registers and the warp frees its rows at once,
-// so the next Q K^T runs under the exponentials; P V of step j runs under the softmax of step j+1.  Three
+// so the next Q K^T runs under the exponentials; P V of step j runs under the softmax of step j+1.  Two
 // blocks of 8 key columns in fourteen take their exponentials from a polynomial on
 // the FMA pipe.  The accumulator is rescaled lazily: only when the running
 // maximum grew by more than 2^8 since the last rescale.  The epilogue folds the
@@ -81,16 +81,36 @@ constexpr int kFlushSteps = 64;
 // Blocks of 8 key columns (bit b: columns [8 b, 8 b + 8) of a step) whose exponentials come from a polynomial on the
 // FMA pipe instead of the special-function unit, which at 16 results per clock per SM would otherwise set the pace.
 // The polynomial costs more instructions and more energy, and the long launches run at the card's power limit, so the
-// choice that takes the fewest clocks gains least.  137,400 queries x 36,600 keys, 27 launches in a row (clocks per
-// step of 2 x 128 rows x 112 keys; SM clock): no block 23.45 ms (1984; 1.62 GHz), two 22.60 (1809; 1.53), three 22.55
-// (1771; 1.50), five 22.71 (1755; 1.47); a single launch 21.5, 20.1, 19.9, 20.2 ms.
+// choice that takes the fewest clocks gains least.  137,400 queries x 36,600 keys, launches in a row, when the kernel
+// still had one work item per CTA (clocks per step of 2 x 128 rows x 112 keys; SM clock): no block 23.45 ms (1984; 1.62 GHz),
+// two 22.60 (1809; 1.53), three 22.55 (1771; 1.50), five 22.71 (1755; 1.47).  Now two and three do the same there (22.76
+// and 22.61 ms) and two is ahead where steps are few (frame attention, 10 frames: 130.7 us against 133.2).
 #ifndef AVGGT_POLY_BLOCKS
-#define AVGGT_POLY_BLOCKS 0x0888
+#define AVGGT_POLY_BLOCKS 0x2040
 #endif
 constexpr uint32_t kPolyBlocks = AVGGT_POLY_BLOCKS;
 
+// Division of n < 2^31 by a number known at launch as a multiplication: n / d = n m >> s with m = ceil(2^s / d),
+// s = 31 + ceil(log2 d), exact because m d - 2^s < d <= 2^(s - 31).  (The epilogue asks six such questions per row; as
+// divisions they were a quarter of its time.)
+struct Divisor {
+  uint32_t d, m, s;
+};
+Divisor make_divisor(uint32_t d) {
+  Divisor v{d, 0, 31};
+  while ((uint64_t(1) << (v.s - 31)) < d) ++v.s;
+  v.m = static_cast<uint32_t>(((uint64_t(1) << v.s) + d - 1) / d);
+  return v;
+}
+__device__ __forceinline__ uint32_t divide(uint32_t n, const Divisor& v, uint32_t& rest) {
+  const uint32_t q = static_cast<uint32_t>((static_cast<uint64_t>(n) * v.m) >> v.s);
+  rest = n - q * v.d;
+  return q;
+}
+
 struct AttnArgs {
   Plan pl;
+  Divisor by_pairs, by_heads, by_L, by_grid_w, by_s_h, by_s_w;
   const uint4* Q;       // [n_tok, H, d], read by the diagonal and mean terms; K and V by the diagonal term only
   const uint4* K;
   const uint4* V;
@@ -202,10 +222,9 @@ struct QueryTile {
 // attention) the frame, so that the CTAs running side by side share one head's keys in L2.
 __device__ __forceinline__ WorkItem work_item(const AttnArgs& a, uint32_t item) {
   WorkItem w;
-  const uint32_t rest = item / static_cast<uint32_t>(a.pairs);
-  const uint32_t qp = item - rest * static_cast<uint32_t>(a.pairs);
-  const uint32_t frame = rest / static_cast<uint32_t>(a.pl.H);
-  w.head = static_cast<int>(rest - frame * static_cast<uint32_t>(a.pl.H));
+  uint32_t qp, head;
+  const uint32_t frame = divide(divide(item, a.by_pairs, qp), a.by_heads, head);
+  w.head = static_cast<int>(head);
   w.key_row0 = static_cast<int>(frame) * a.pl.L;   // the subsampled layer has one problem
   w.row0 = w.key_row0 + static_cast<int>(qp) * (kQTiles * kTileQ);
   w.end = a.frame_mode ? static_cast<int64_t>(w.key_row0) + a.pl.L : a.pl.n_tok;
@@ -630,9 +649,10 @@ __device__ __forceinline__ bool softmax_step(const SoftmaxThread& me, int gj, in
   tc_fence_after();
   uint32_t s[4 * kBlocks];
   tmem_ld_rows16_scores(me.base + (odd ? kColSOdd : 0), s);
-  tmem_wait_ld();     // for the whole warp: lane 0 may speak for it
+  tmem_wait_ld();     // for the whole warp: one lane may speak for it
   tc_fence_before();
-  if (me.lane == 0) mbar_arrive(smem_u32(&bars->s_free[me.t]));
+  // (elected rather than lane 0: a branch on the lane number costs a reconvergence, 4 % of a ten-frame layer)
+  if (elect_one()) mbar_arrive(smem_u32(&bars->s_free[me.t]));
 
   if (kMasked) {
 #pragma unroll
@@ -730,7 +750,7 @@ __device__ __forceinline__ bool softmax_step(const SoftmaxThread& me, int gj, in
   }
   tmem_wait_st();
   tc_fence_before();
-  if (me.lane == 0) mbar_arrive(smem_u32(&bars->p_full[me.t][odd]));
+  if (elect_one()) mbar_arrive(smem_u32(&bars->p_full[me.t][odd]));
   return true;
 }
 
@@ -767,6 +787,17 @@ __device__ __forceinline__ float dot_bf16x8_f32(const uint4& x, const float4& a,
   acc = fmaf(__uint_as_float(x.z & 0xffff0000u), b.y, acc);
   acc = fmaf(__uint_as_float(x.w << 16), b.z, acc);
   return fmaf(__uint_as_float(x.w & 0xffff0000u), b.w, acc);
+}
+
+// The window rule: compact_slot(frame, slot) < 0
+__device__ __forceinline__ bool is_dropped(const AttnArgs& a, int row) {
+  uint32_t slot, c, rest_h, rest_w;
+  const uint32_t frame = divide(row, a.by_L, slot);
+  const uint32_t n_special = a.pl.n_special;
+  const uint32_t r = divide(slot >= n_special ? slot - n_special : 0u, a.by_grid_w, c);
+  divide(r, a.by_s_h, rest_h);
+  divide(c, a.by_s_w, rest_w);
+  return slot >= n_special && !(a.pl.keep_first && frame == 0) && (rest_h | rest_w) != 0;
 }
 
 // What the epilogue of a work item needs of its rows' running state (shared memory; a row's warp writes and reads it).
@@ -829,8 +860,7 @@ __device__ __forceinline__ bool softmax_epilogue(const AttnArgs& a, Barriers* ba
       for (int hi = 0; hi < 2; ++hi) {
         const int row = tile.q0 + r0 + 8 * hi;
         if (row >= tile.first && row < tile.last) {
-          const int32_t f = row / pl.L;
-          dropped[hi] = (a.slot_of_token != nullptr ? a.slot_of_token[row] : compact_slot(pl, f, row - f * pl.L)) < 0;
+          dropped[hi] = a.slot_of_token != nullptr ? a.slot_of_token[row] < 0 : is_dropped(a, row);
         }
       }
 #pragma unroll
@@ -907,7 +937,7 @@ __device__ __forceinline__ bool softmax_epilogue(const AttnArgs& a, Barriers* ba
       tmem_wait_ld();
       if (half == 1) {   // O_t has been read: the next work item's first P V may overwrite it
         tc_fence_before();
-        if (me.lane == 0) mbar_arrive(smem_u32(&bars->o_free[t]));
+        if (elect_one()) mbar_arrive(smem_u32(&bars->o_free[t]));
       }
     }
 #pragma unroll
@@ -916,15 +946,15 @@ __device__ __forceinline__ bool softmax_epilogue(const AttnArgs& a, Barriers* ba
       uint32_t w[4];   // the thread's words of the output row: word 4 b + i (dimensions 8 b + 2 i, 8 b + 2 i + 1)
 #pragma unroll
       for (int b = 0; b < 4; ++b) {
-        float v0 = __uint_as_float(o[4 * b + 2 * hi]) * w_s[hi], v1 = __uint_as_float(o[4 * b + 2 * hi + 1]) * w_s[hi];
+        uint64_t v = mul_f32x2(pack_f32x2(__uint_as_float(o[4 * b + 2 * hi]), __uint_as_float(o[4 * b + 2 * hi + 1])),
+                               pack_f32x2(w_s[hi], w_s[hi]));
         if (kExtra && a.use_diag) {
-          v0 = fmaf(w_d[hi], __uint_as_float(vw[hi][4 * half + b] << 16), v0);
-          v1 = fmaf(w_d[hi], __uint_as_float(vw[hi][4 * half + b] & 0xffff0000u), v1);
+          const uint32_t own = vw[hi][4 * half + b];
+          v = fma_f32x2(pack_f32x2(w_d[hi], w_d[hi]), pack_f32x2(__uint_as_float(own << 16), __uint_as_float(own & 0xffff0000u)), v);
         }
-        if (kExtra && a.use_mean) {
-          v0 = fmaf(w_m[hi], vm[b].x, v0);
-          v1 = fmaf(w_m[hi], vm[b].y, v1);
-        }
+        if (kExtra && a.use_mean) v = fma_f32x2(pack_f32x2(w_m[hi], w_m[hi]), pack_f32x2(vm[b].x, vm[b].y), v);
+        float v0, v1;
+        unpack_f32x2(v, v0, v1);
         w[b] = pack_bf16x2(v0, v1);
       }
       // Transposed within the quad, a thread holds 16 contiguous bytes of the row: 4 stores of 16 bytes
@@ -1193,6 +1223,12 @@ cudaError_t launch_attn(const Plan& pl, int sm_count, bool frame_mode, const voi
   a.poly_range = (kRescaleThreshold - kPolyLowest) * a.inv_scale_log2;
   const int64_t rows = frame_mode ? pl.L : pl.n_tok;
   a.pairs = static_cast<int32_t>((rows + kQTiles * kTileQ - 1) / (kQTiles * kTileQ));
+  a.by_pairs = make_divisor(a.pairs);
+  a.by_heads = make_divisor(pl.H);
+  a.by_L = make_divisor(pl.L);
+  a.by_grid_w = make_divisor(pl.grid_w);
+  a.by_s_h = make_divisor(pl.s_h);
+  a.by_s_w = make_divisor(pl.s_w);
   a.n_work = a.pairs * pl.H * (frame_mode ? pl.n_frames : 1);
 
   // token-major [n_tok, H*d] maps for Q and, in frame attention, K and V; head-major [H, M, d] maps for Kc, Vc otherwise
