@@ -181,6 +181,16 @@ int avggt_global_attn(const avggt_params* p, const void* Q, const void* K, const
                       void* O, float* lse, void* ws, size_t ws_bytes, void* cuda_stream);
 
 /*
+ * The whole layer in one call: avggt_build_kv and then avggt_global_attn with the same arguments and results.  The status
+ * block is cleared by the compaction kernel, so the layer is two or three kernels and nothing else, each of which
+ * prepares itself while the one before it ends.
+ */
+int avggt_layer(const avggt_params* p, const void* Q, const void* K, const void* V,
+                void* Kc, void* Vc, int32_t* idx, float* kmean, float* vmean, void* O, float* lse,
+                void* build_ws, size_t build_ws_bytes, void* attn_ws, size_t attn_ws_bytes,
+                void* cuda_stream);
+
+/*
  * The same layer with a retained set chosen by the caller instead of the window rule (the
  * alternative selectors of the supplement, "Comparison with other subsampling strategies":
  * random, norm-ranked or feature-based picks).  `idx` lists the n_kept retained tokens; every

@@ -24,7 +24,7 @@ AVGGT_MEAN_OFF, AVGGT_MEAN_UNIT, AVGGT_MEAN_FILL = 0, 1, 2
 
 # every symbol include/avggt.h declares
 EXPORTS = (
-    "avggt_kv_count", "avggt_workspace_bytes", "avggt_build_kv", "avggt_build_kv_noalloc", "avggt_global_attn",
+    "avggt_kv_count", "avggt_workspace_bytes", "avggt_build_kv", "avggt_build_kv_noalloc", "avggt_global_attn", "avggt_layer",
     "avggt_frame_attn", "avggt_build_kv_indexed", "avggt_global_attn_indexed", "avggt_global_attn_shard",
     "avggt_build_kv_shard", "avggt_shard_assemble", "avggt_project_workspace_bytes", "avggt_project_build_kv",
     "avggt_check_status", "avggt_strerror", "avggt_last_cuda_error", "avggt_version",
@@ -75,6 +75,7 @@ def load_library(path):
         "avggt_build_kv": [pp, vp, vp, vp, vp, vp, vp, vp, vp, sz, vp],
         "avggt_build_kv_noalloc": [pp, vp, vp, vp, vp, vp, vp, vp, vp],
         "avggt_global_attn": [pp, vp, vp, vp, vp, vp, vp, vp, vp, vp, vp, sz, vp],
+        "avggt_layer": [pp, vp, vp, vp, vp, vp, vp, vp, vp, vp, vp, vp, sz, vp, sz, vp],
         "avggt_frame_attn": [pp, vp, vp, vp, vp, vp, vp, sz, vp],
         "avggt_build_kv_indexed": [pp, vp, i64, vp, vp, vp, vp, vp, vp, vp, vp, sz, vp],
         "avggt_global_attn_indexed": [pp, i64, vp, vp, vp, vp, vp, vp, vp, vp, vp, vp, vp, sz, vp],
@@ -167,6 +168,13 @@ def avggt_global_attn(params, Q, K, V, Kc, Vc, kmean, vmean, O, lse, ws, ws_byte
     """Enqueue the subsampled global attention."""
     _check(lib().avggt_global_attn(ctypes.byref(params), _ptr(Q), _ptr(K), _ptr(V), _ptr(Kc), _ptr(Vc), _ptr(kmean),
                                    _ptr(vmean), _ptr(O), _ptr(lse), _ptr(ws), ws_bytes, stream), "avggt_global_attn")
+
+
+def avggt_layer(params, Q, K, V, Kc, Vc, idx, kmean, vmean, O, lse, build_ws, build_ws_bytes, attn_ws, attn_ws_bytes, stream=None):
+    """Enqueue the whole layer: compaction + mean reduction, then the attention."""
+    _check(lib().avggt_layer(ctypes.byref(params), _ptr(Q), _ptr(K), _ptr(V), _ptr(Kc), _ptr(Vc), _ptr(idx), _ptr(kmean),
+                             _ptr(vmean), _ptr(O), _ptr(lse), _ptr(build_ws), build_ws_bytes, _ptr(attn_ws), attn_ws_bytes,
+                             stream), "avggt_layer")
 
 
 def avggt_build_kv_indexed(params, idx, n_kept, K, V, Kc, Vc, slot_of_token, kmean, vmean, ws, ws_bytes, stream=None):

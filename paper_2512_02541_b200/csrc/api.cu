@@ -126,20 +126,27 @@ int avggt_workspace_bytes(const avggt_params* p, size_t* build_ws_bytes, size_t*
   return AVGGT_OK;
 }
 
-int avggt_build_kv(const avggt_params* p, const void* K, const void* V, void* Kc, void* Vc, int32_t* idx,
-                   float* kmean, float* vmean, void* ws, size_t ws_bytes, void* cuda_stream) {
-  Plan pl;
-  int rc = make_plan(p, &pl);
-  if (rc != AVGGT_OK) return rc;
+// Validation of the compaction's arguments.
+static int check_build(const Plan& pl, const void* K, const void* V, const void* Kc, const void* Vc, const int32_t* idx,
+                       const float* kmean, const float* vmean, const void* ws, size_t ws_bytes, DeviceInfo* di) {
   if (!K || !V || !Kc || !Vc || !ws) return AVGGT_ERR_INVALID_ARG;
   if (pl.mean_fill != 0 && (!kmean || !vmean)) return AVGGT_ERR_INVALID_ARG;
   if (!aligned16(K) || !aligned16(V) || !aligned16(Kc) || !aligned16(Vc) || !aligned16(ws) ||
       (reinterpret_cast<uintptr_t>(idx) & 3u) || !aligned16(kmean) || !aligned16(vmean))
     return AVGGT_ERR_ALIGNMENT;
-  DeviceInfo di;
-  rc = device_info(&di);
+  const int rc = device_info(di);
   if (rc != AVGGT_OK) return rc;
-  if (ws_bytes < build_kv_ws_bytes(pl, di.sm_count)) return AVGGT_ERR_WORKSPACE_TOO_SMALL;
+  return ws_bytes < build_kv_ws_bytes(pl, di->sm_count) ? AVGGT_ERR_WORKSPACE_TOO_SMALL : AVGGT_OK;
+}
+
+int avggt_build_kv(const avggt_params* p, const void* K, const void* V, void* Kc, void* Vc, int32_t* idx,
+                   float* kmean, float* vmean, void* ws, size_t ws_bytes, void* cuda_stream) {
+  Plan pl;
+  int rc = make_plan(p, &pl);
+  if (rc != AVGGT_OK) return rc;
+  DeviceInfo di;
+  rc = check_build(pl, K, V, Kc, Vc, idx, kmean, vmean, ws, ws_bytes, &di);
+  if (rc != AVGGT_OK) return rc;
   return record_cuda(launch_build_kv(pl, di.sm_count, K, V, Kc, Vc, idx, kmean, vmean, ws, static_cast<cudaStream_t>(cuda_stream)));
 }
 
@@ -154,11 +161,12 @@ struct AttnCall {
   void* stream;
   const int32_t* slot_of_token;   // caller-chosen retained set, else null
   bool frame_mode;                // frame attention (Sec. 4.2): Kc, Vc, kmean, vmean play no part
+  bool status_cleared = false;    // the compaction before it in the stream clears the status block
 };
 
-// Validation and launch shared by every attention entry point.  Everything that can be rejected on the
-// host is rejected before anything is enqueued.
-static int run_attn(const Plan& pl, const AttnCall& c) {
+// Validation shared by every attention entry point: everything that can be rejected on the host is rejected before
+// anything is enqueued.
+static int check_attn(const Plan& pl, const AttnCall& c, DeviceInfo* di) {
   const bool need_diag = !c.frame_mode && pl.diag != 0 && pl.n_dropped > 0;
   const bool need_mean = !c.frame_mode && pl.mean_fill != 0 && pl.n_dropped > 0;
   if (!c.Q || !c.O || !c.ws) return AVGGT_ERR_INVALID_ARG;
@@ -169,18 +177,26 @@ static int run_attn(const Plan& pl, const AttnCall& c) {
       !aligned16(c.ws) || !aligned16(c.kmean) || !aligned16(c.vmean) || (reinterpret_cast<uintptr_t>(c.lse) & 3u) ||
       (reinterpret_cast<uintptr_t>(c.slot_of_token) & 3u))
     return AVGGT_ERR_ALIGNMENT;
-  DeviceInfo di;
-  int rc = device_info(&di);
+  int rc = device_info(di);
   if (rc != AVGGT_OK) return rc;
-  if (c.ws_bytes < global_attn_ws_bytes(pl, di.sm_count)) return AVGGT_ERR_WORKSPACE_TOO_SMALL;
+  return c.ws_bytes < global_attn_ws_bytes(pl, di->sm_count) ? AVGGT_ERR_WORKSPACE_TOO_SMALL : AVGGT_OK;
+}
+
+static int enqueue_attn(const Plan& pl, const DeviceInfo& di, const AttnCall& c) {
   bool tmap_failed = false;
   const cudaStream_t st = static_cast<cudaStream_t>(c.stream);
   const cudaError_t e = c.frame_mode
       ? launch_frame_attn(pl, di.sm_count, c.Q, c.K, c.V, c.O, c.lse, c.ws, st, &tmap_failed)
       : launch_global_attn(pl, di.sm_count, c.Q, c.K, c.V, c.Kc, c.Vc, c.kmean, c.vmean, c.O, c.lse, c.ws, st,
-                           &tmap_failed, c.slot_of_token);
+                           &tmap_failed, c.slot_of_token, c.status_cleared);
   if (tmap_failed) return record_message("cuTensorMapEncodeTiled failed");
   return record_cuda(e);
+}
+
+static int run_attn(const Plan& pl, const AttnCall& c) {
+  DeviceInfo di;
+  const int rc = check_attn(pl, c, &di);
+  return rc != AVGGT_OK ? rc : enqueue_attn(pl, di, c);
 }
 
 int avggt_global_attn(const avggt_params* p, const void* Q, const void* K, const void* V, const void* Kc,
@@ -190,6 +206,25 @@ int avggt_global_attn(const avggt_params* p, const void* Q, const void* K, const
   int rc = make_plan(p, &pl);
   if (rc != AVGGT_OK) return rc;
   return run_attn(pl, AttnCall{Q, K, V, Kc, Vc, kmean, vmean, O, lse, ws, ws_bytes, cuda_stream, nullptr, false});
+}
+
+int avggt_layer(const avggt_params* p, const void* Q, const void* K, const void* V, void* Kc, void* Vc, int32_t* idx,
+                float* kmean, float* vmean, void* O, float* lse, void* build_ws, size_t build_ws_bytes, void* attn_ws,
+                size_t attn_ws_bytes, void* cuda_stream) {
+  Plan pl;
+  int rc = make_plan(p, &pl);
+  if (rc != AVGGT_OK) return rc;
+  DeviceInfo di;
+  rc = check_build(pl, K, V, Kc, Vc, idx, kmean, vmean, build_ws, build_ws_bytes, &di);
+  if (rc != AVGGT_OK) return rc;
+  AttnCall c{Q, K, V, Kc, Vc, kmean, vmean, O, lse, attn_ws, attn_ws_bytes, cuda_stream, nullptr, false};
+  rc = check_attn(pl, c, &di);
+  if (rc != AVGGT_OK) return rc;
+  rc = record_cuda(launch_build_kv(pl, di.sm_count, K, V, Kc, Vc, idx, kmean, vmean, build_ws, static_cast<cudaStream_t>(cuda_stream),
+                                   nullptr, nullptr, 0, false, attn_ws));
+  if (rc != AVGGT_OK) return rc;
+  c.status_cleared = true;
+  return enqueue_attn(pl, di, c);
 }
 
 // Plan of a problem whose retained set is a caller-supplied list of n_kept tokens.

@@ -13,6 +13,7 @@
 #include <cuda_runtime.h>
 
 #include "internal.h"
+#include "ptx.cuh"
 
 namespace avggt {
 
@@ -45,13 +46,23 @@ template <int PASSES>
 __global__ void __launch_bounds__(kBuildThreads)
 build_kv_kernel(const Plan pl, const uint4* __restrict__ K, const uint4* __restrict__ V, uint4* __restrict__ Kc,
                 uint4* __restrict__ Vc, const int64_t kc_rows, int32_t* __restrict__ idx, float* __restrict__ partials,
-                const int do_mean, const int32_t* __restrict__ slot_of_token) {
+                const int do_mean, const int32_t* __restrict__ slot_of_token, uint32_t* __restrict__ status,
+                float* __restrict__ zero_kmean, float* __restrict__ zero_vmean) {
   extern __shared__ float red[];   // [kBuildWarps][PASSES * 256]
   const int lane = threadIdx.x & 31;
   const int warp = threadIdx.x >> 5;
   const uint32_t chunks_per_row = static_cast<uint32_t>(pl.H) * 8u;   // 16-byte chunks (d = 64 bf16 = 8 chunks per head)
   const uint32_t n_tok = static_cast<uint32_t>(pl.n_tok);
   const uint32_t warps_total = gridDim.x * kBuildWarps;
+
+  grid_dependency_wait();
+  if (blockIdx.x == 0) {
+    // what would otherwise be launches of their own: the status block of the attention that follows, and the mean pair of
+    // a problem that drops nothing
+    if (status != nullptr && threadIdx.x < kAttnStatusBytes / 4) status[threadIdx.x] = 0u;
+    if (zero_kmean != nullptr)
+      for (int i = threadIdx.x; i < pl.H * pl.d; i += kBuildThreads) { zero_kmean[i] = 0.f; zero_vmean[i] = 0.f; }
+  }
 
   float acc_k[PASSES][8], acc_v[PASSES][8];
 #pragma unroll
@@ -93,6 +104,8 @@ build_kv_kernel(const Plan pl, const uint4* __restrict__ K, const uint4* __restr
     }
   }
 
+  // the next kernel may take its place on the chip while the blocks reduce and end (earlier it would only be in the way)
+  grid_launch_dependents();
   if (!do_mean) return;
   // block reduction, K then V, fixed order over warps
   const int cols = pl.H * pl.d;   // = chunks_per_row * 8
@@ -120,11 +133,13 @@ __global__ void __launch_bounds__(1024)
 mean_finalize_kernel(const float* __restrict__ partials, int n_blocks, int cols2, float inv_count,
                      float* __restrict__ kmean, float* __restrict__ vmean) {
   __shared__ float tile[32][33];
+  grid_launch_dependents();
+  grid_dependency_wait();
   const int c = threadIdx.x & 31, g = threadIdx.x >> 5;
   const int col = blockIdx.x * 32 + c;
   float s = 0.f;
   if (col < cols2)
-    for (int b = g; b < n_blocks; b += 32) s += partials[static_cast<size_t>(b) * cols2 + col];
+    for (int b = g; b < n_blocks; b += 32) s += __ldcg(partials + static_cast<size_t>(b) * cols2 + col);
   tile[c][g] = s;
   __syncthreads();
   // warp g now owns column blockIdx.x*32 + g; lane c holds the partial of group c
@@ -156,16 +171,16 @@ __global__ void scatter_slots_kernel(const int32_t* __restrict__ idx, int64_t M,
 
 template <int PASSES>
 cudaError_t launch_build(const Plan& pl, int grid, const void* K, const void* V, void* Kc, void* Vc, int64_t kc_rows,
-                         int32_t* idx, float* partials, int do_mean, const int32_t* slot_of_token, cudaStream_t st) {
+                         int32_t* idx, float* partials, int do_mean, const int32_t* slot_of_token, uint32_t* status,
+                         float* zero_kmean, float* zero_vmean, cudaStream_t st) {
   const size_t smem = do_mean ? static_cast<size_t>(kBuildWarps) * PASSES * 256 * sizeof(float) : 0;
   if (smem > 48 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(build_kv_kernel<PASSES>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
     if (e != cudaSuccess) return e;
   }
-  build_kv_kernel<PASSES><<<grid, kBuildThreads, smem, st>>>(pl, static_cast<const uint4*>(K), static_cast<const uint4*>(V),
-                                                           static_cast<uint4*>(Kc), static_cast<uint4*>(Vc), kc_rows, idx, partials,
-                                                           do_mean, slot_of_token);
-  return cudaGetLastError();
+  return launch_dependent(build_kv_kernel<PASSES>, grid, kBuildThreads, smem, st, pl, static_cast<const uint4*>(K),
+                          static_cast<const uint4*>(V), static_cast<uint4*>(Kc), static_cast<uint4*>(Vc), kc_rows, idx, partials,
+                          do_mean, slot_of_token, status, zero_kmean, zero_vmean);
 }
 
 // Exchange buffer [n_ranks][2][H][slot_rows][d] (every rank's compact K then V, padded to slot_rows rows per
@@ -235,7 +250,8 @@ size_t build_kv_ws_bytes(const Plan& pl, int sm_count) {
 
 cudaError_t launch_build_kv(const Plan& pl, int sm_count, const void* K, const void* V, void* Kc, void* Vc,
                             int32_t* idx, float* kmean, float* vmean, void* ws, cudaStream_t st,
-                            const int32_t* caller_idx, int32_t* slot_of_token, int64_t kc_rows, bool sums_only) {
+                            const int32_t* caller_idx, int32_t* slot_of_token, int64_t kc_rows, bool sums_only,
+                            void* clear_status) {
   if (kc_rows <= 0) kc_rows = pl.M;
   if (slot_of_token != nullptr) {
     // caller-chosen retained set: build the token -> compact position map first
@@ -249,32 +265,27 @@ cudaError_t launch_build_kv(const Plan& pl, int sm_count, const void* K, const v
   const int grid = build_kv_grid(pl, sm_count);
   const int do_mean = (pl.mean_fill != 0 && pl.n_dropped > 0) ? 1 : 0;
   float* partials = static_cast<float*>(ws);
+  uint32_t* status = static_cast<uint32_t*>(clear_status);
+  const bool zero_mean = pl.mean_fill != 0 && !do_mean;
+  float* zk = zero_mean ? kmean : nullptr;
+  float* zv = zero_mean ? vmean : nullptr;
   const int passes = (pl.H * 8 + 31) / 32;
   cudaError_t e;
   switch (passes) {
-    case 1: e = launch_build<1>(pl, grid, K, V, Kc, Vc, kc_rows, idx, partials, do_mean, slot_of_token, st); break;
-    case 2: e = launch_build<2>(pl, grid, K, V, Kc, Vc, kc_rows, idx, partials, do_mean, slot_of_token, st); break;
-    case 3: e = launch_build<3>(pl, grid, K, V, Kc, Vc, kc_rows, idx, partials, do_mean, slot_of_token, st); break;
-    case 4: e = launch_build<4>(pl, grid, K, V, Kc, Vc, kc_rows, idx, partials, do_mean, slot_of_token, st); break;
-    case 5: e = launch_build<5>(pl, grid, K, V, Kc, Vc, kc_rows, idx, partials, do_mean, slot_of_token, st); break;
-    case 6: e = launch_build<6>(pl, grid, K, V, Kc, Vc, kc_rows, idx, partials, do_mean, slot_of_token, st); break;
-    case 7: e = launch_build<7>(pl, grid, K, V, Kc, Vc, kc_rows, idx, partials, do_mean, slot_of_token, st); break;
-    case 8: e = launch_build<8>(pl, grid, K, V, Kc, Vc, kc_rows, idx, partials, do_mean, slot_of_token, st); break;
+    case 1: e = launch_build<1>(pl, grid, K, V, Kc, Vc, kc_rows, idx, partials, do_mean, slot_of_token, status, zk, zv, st); break;
+    case 2: e = launch_build<2>(pl, grid, K, V, Kc, Vc, kc_rows, idx, partials, do_mean, slot_of_token, status, zk, zv, st); break;
+    case 3: e = launch_build<3>(pl, grid, K, V, Kc, Vc, kc_rows, idx, partials, do_mean, slot_of_token, status, zk, zv, st); break;
+    case 4: e = launch_build<4>(pl, grid, K, V, Kc, Vc, kc_rows, idx, partials, do_mean, slot_of_token, status, zk, zv, st); break;
+    case 5: e = launch_build<5>(pl, grid, K, V, Kc, Vc, kc_rows, idx, partials, do_mean, slot_of_token, status, zk, zv, st); break;
+    case 6: e = launch_build<6>(pl, grid, K, V, Kc, Vc, kc_rows, idx, partials, do_mean, slot_of_token, status, zk, zv, st); break;
+    case 7: e = launch_build<7>(pl, grid, K, V, Kc, Vc, kc_rows, idx, partials, do_mean, slot_of_token, status, zk, zv, st); break;
+    case 8: e = launch_build<8>(pl, grid, K, V, Kc, Vc, kc_rows, idx, partials, do_mean, slot_of_token, status, zk, zv, st); break;
     default: return cudaErrorInvalidValue;
   }
-  if (e != cudaSuccess) return e;
-  if (pl.mean_fill != 0) {
-    const int cols2 = 2 * pl.H * pl.d;
-    if (do_mean) {
-      const float inv_count = sums_only ? 1.0f : 1.0f / static_cast<float>(pl.n_dropped);
-      mean_finalize_kernel<<<(cols2 + 31) / 32, 1024, 0, st>>>(partials, grid, cols2, inv_count, kmean, vmean);
-      e = cudaGetLastError();
-    } else {
-      e = cudaMemsetAsync(kmean, 0, static_cast<size_t>(pl.H) * pl.d * sizeof(float), st);
-      if (e == cudaSuccess) e = cudaMemsetAsync(vmean, 0, static_cast<size_t>(pl.H) * pl.d * sizeof(float), st);
-    }
-  }
-  return e;
+  if (e != cudaSuccess || !do_mean) return e;
+  const int cols2 = 2 * pl.H * pl.d;
+  const float inv_count = sums_only ? 1.0f : 1.0f / static_cast<float>(pl.n_dropped);
+  return launch_dependent(mean_finalize_kernel, (cols2 + 31) / 32, 1024, 0, st, partials, grid, cols2, inv_count, kmean, vmean);
 }
 
 }  // namespace avggt

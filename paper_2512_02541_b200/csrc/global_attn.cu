@@ -127,7 +127,8 @@ struct AttnArgs {
   int32_t last_tile_keys;   // keys of a ragged last tile, else 0
   int32_t n_work;       // work items (pairs of query tiles x heads x problems) of the launch; a CTA takes the items
                         // blockIdx.x, blockIdx.x + gridDim.x, ...
-  int32_t pairs;        // pairs of query tiles of one problem
+  int32_t item_rows;    // query rows of a work item: 256 (two full tiles), or 128 or 64 spread over both tiles
+  int32_t pairs;        // work items of one problem and head
   int32_t use_diag;     // diag on and |D| > 0
   int32_t use_mean;     // mean_fill on and |D| > 0
   float scale_log2;     // softmax scale * log2(e)
@@ -209,7 +210,7 @@ struct WorkItem {
   int head;
   int key_row0;   // frame attention: token index of the frame's first key
   int row0;       // first query row (token index)
-  int64_t end;    // one past the problem's last query row
+  int64_t end;    // one past the item's last query row
 };
 // One of its query tiles.
 struct QueryTile {
@@ -226,12 +227,13 @@ __device__ __forceinline__ WorkItem work_item(const AttnArgs& a, uint32_t item) 
   const uint32_t frame = divide(divide(item, a.by_pairs, qp), a.by_heads, head);
   w.head = static_cast<int>(head);
   w.key_row0 = static_cast<int>(frame) * a.pl.L;   // the subsampled layer has one problem
-  w.row0 = w.key_row0 + static_cast<int>(qp) * (kQTiles * kTileQ);
-  w.end = a.frame_mode ? static_cast<int64_t>(w.key_row0) + a.pl.L : a.pl.n_tok;
+  w.row0 = w.key_row0 + static_cast<int>(qp) * a.item_rows;
+  const int64_t end = a.frame_mode ? static_cast<int64_t>(w.key_row0) + a.pl.L : a.pl.n_tok;
+  w.end = end - w.row0 > a.item_rows ? static_cast<int64_t>(w.row0) + a.item_rows : end;
   return w;
 }
 
-// A last pair with rows for one tile only is cut in two halves by groups of 16 rows (one softmax warp), the second
+// An item with rows for one tile only is cut in two halves by groups of 16 rows (one softmax warp), the second
 // half in the upper lanes of its tile: every scheduler then has two warps with work at most, and both tiles' products
 // overlap.  Warps without rows compute nothing.
 __device__ __forceinline__ QueryTile query_tile(const WorkItem& w, int t) {
@@ -848,12 +850,12 @@ __device__ __forceinline__ bool softmax_epilogue(const AttnArgs& a, Barriers* ba
       vw[hi][0] = v0.x; vw[hi][1] = v0.y; vw[hi][2] = v0.z; vw[hi][3] = v0.w;
       vw[hi][4] = v1.x; vw[hi][5] = v1.y; vw[hi][6] = v1.z; vw[hi][7] = v1.w;
     }
-    if (a.use_mean) {
+    if (a.use_mean) {   // (past L1: written by the kernel before this one, which may have ended after this one began)
       const float4* src = reinterpret_cast<const float4*>(a.kmean + head * kHeadDim + 8 * i);
-      km[0] = __ldg(src);
-      km[1] = __ldg(src + 1);
-      km[2] = __ldg(src + 8);
-      km[3] = __ldg(src + 9);
+      km[0] = __ldcg(src);
+      km[1] = __ldcg(src + 1);
+      km[2] = __ldcg(src + 8);
+      km[3] = __ldcg(src + 9);
     }
     if (a.use_diag) {
 #pragma unroll
@@ -927,7 +929,7 @@ __device__ __forceinline__ bool softmax_epilogue(const AttnArgs& a, Barriers* ba
     if (kExtra && a.use_mean) {
       const float2* src = reinterpret_cast<const float2*>(a.vmean + head * kHeadDim + 32 * half) + i;
 #pragma unroll
-      for (int b = 0; b < 4; ++b) vm[b] = __ldg(src + 4 * b);
+      for (int b = 0; b < 4; ++b) vm[b] = __ldcg(src + 4 * b);
     }
     uint32_t o[16];   // register 4 b + 2 hi + e: row hi, output dimension 8 b + 2 i + e; zero with no retained keys at all
 #pragma unroll
@@ -1099,9 +1101,6 @@ global_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
 
   const int tid = threadIdx.x;
   const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // warp-uniform by construction
-  // a launch in which a wait has already run out is abandoned: the remaining CTAs leave at once
-  if (__syncthreads_or(*reinterpret_cast<volatile uint32_t*>(a.status) != 0u)) return;
-
   if (tid == 0) {
     for (int e = 0; e < 2; ++e) {
       mbar_init(smem_u32(&bars.q_full[e]), 1);
@@ -1131,12 +1130,16 @@ global_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
     tmem_relinquish();
   }
   ones_block(sm.ones, tid);
+  // everything above may run while the kernel before this one ends
+  grid_dependency_wait();
   tc_fence_before();
-  __syncthreads();
+  // a launch in which a wait has already run out is abandoned: the remaining CTAs leave at once
+  const bool abandoned = __syncthreads_or(*reinterpret_cast<volatile uint32_t*>(a.status) != 0u) != 0;
   tc_fence_after();
   const uint32_t tmem = bars.tmem_base;
 
-  if (warp < kSoftmaxWarps) {
+  if (abandoned) {
+  } else if (warp < kSoftmaxWarps) {
     reg_inc<kRegsSoftmax>();
     softmax_role<kLse, kExtra>(a, &bars, &row_results, tmem, warp, tid & 31);
   } else {
@@ -1152,6 +1155,13 @@ global_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
   tc_fence_before();
   __syncthreads();
   if (warp == kTmaWarp) tmem_dealloc(tmem, kTmemCols);
+}
+
+// The status block of a launch that no compaction precedes.
+__global__ void clear_status_kernel(uint32_t* status) {
+  grid_dependency_wait();
+  grid_launch_dependents();
+  if (threadIdx.x < kAttnStatusBytes / 4) status[threadIdx.x] = 0u;
 }
 
 constexpr size_t kAttnSmemBytes = static_cast<size_t>(kTileBytes) * (2 * kQTiles) + static_cast<size_t>(kKeyTileBytes) * (2 * kStages) + kOnesBytes + 1024;
@@ -1192,10 +1202,17 @@ cudaError_t prepare_kernels() {
   return cudaSuccess;
 }
 
+// Query rows of a work item.  Half items leave half of a tile's products idle and cost 0.6 of a full one at best (a lone wave
+// of 13 key steps: 32.8 us in two rounds against 23.7 us in one), so they pay only where the chip has room for all of them at
+// once (1,044 queries x 532 keys x 16 heads, 80 items or 144: 18.3 against 16.2 us).
+int choose_item_rows(int64_t rows, int64_t problems, int sm_count) {
+  return (rows + kTileQ - 1) / kTileQ * problems <= sm_count ? kTileQ : kQTiles * kTileQ;
+}
+
 // Tensor maps and launch shared by the two entry points.  frame_mode: see AttnArgs.
 cudaError_t launch_attn(const Plan& pl, int sm_count, bool frame_mode, const void* Q, const void* K, const void* V, const void* Kc,
                         const void* Vc, const float* kmean, const float* vmean, void* O, float* lse, void* ws,
-                        cudaStream_t st, bool* tmap_failed, const int32_t* slot_of_token) {
+                        cudaStream_t st, bool* tmap_failed, const int32_t* slot_of_token, bool status_cleared) {
   *tmap_failed = false;
   AttnArgs a;
   a.pl = pl;
@@ -1222,14 +1239,16 @@ cudaError_t launch_attn(const Plan& pl, int sm_count, bool frame_mode, const voi
   a.inv_scale_log2 = 1.0f / a.scale_log2;
   a.poly_range = (kRescaleThreshold - kPolyLowest) * a.inv_scale_log2;
   const int64_t rows = frame_mode ? pl.L : pl.n_tok;
-  a.pairs = static_cast<int32_t>((rows + kQTiles * kTileQ - 1) / (kQTiles * kTileQ));
+  const int64_t problems = static_cast<int64_t>(pl.H) * (frame_mode ? pl.n_frames : 1);
+  a.item_rows = choose_item_rows(rows, problems, sm_count);
+  a.pairs = static_cast<int32_t>((rows + a.item_rows - 1) / a.item_rows);
   a.by_pairs = make_divisor(a.pairs);
   a.by_heads = make_divisor(pl.H);
   a.by_L = make_divisor(pl.L);
   a.by_grid_w = make_divisor(pl.grid_w);
   a.by_s_h = make_divisor(pl.s_h);
   a.by_s_w = make_divisor(pl.s_w);
-  a.n_work = a.pairs * pl.H * (frame_mode ? pl.n_frames : 1);
+  a.n_work = static_cast<int32_t>(a.pairs * problems);
 
   // token-major [n_tok, H*d] maps for Q and, in frame attention, K and V; head-major [H, M, d] maps for Kc, Vc otherwise
   CUtensorMap tm_q, tm_k, tm_v;
@@ -1254,25 +1273,28 @@ cudaError_t launch_attn(const Plan& pl, int sm_count, bool frame_mode, const voi
 
   cudaError_t e = prepare_kernels();
   if (e != cudaSuccess) return e;
-  e = cudaMemsetAsync(ws, 0, kAttnStatusBytes, st);
-  if (e != cudaSuccess) return e;
+  if (!status_cleared) {
+    e = launch_dependent(clear_status_kernel, 1, 64, 0, st, static_cast<uint32_t*>(ws));
+    if (e != cudaSuccess) return e;
+  }
   const unsigned grid = static_cast<unsigned>(a.n_work < sm_count ? a.n_work : sm_count);
   const int which = (lse != nullptr ? 2 : 0) + (a.use_diag || a.use_mean ? 1 : 0);
-  kAttnKernels[which]<<<grid, kThreads, kAttnSmemBytes, st>>>(tm_q, tm_k, tm_v, a);
-  return cudaGetLastError();
+  return launch_dependent(kAttnKernels[which], grid, kThreads, kAttnSmemBytes, st, tm_q, tm_k, tm_v, a);
 }
 
 }  // namespace
 
 cudaError_t launch_global_attn(const Plan& pl, int sm_count, const void* Q, const void* K, const void* V,
                                const void* Kc, const void* Vc, const float* kmean, const float* vmean, void* O,
-                               float* lse, void* ws, cudaStream_t st, bool* tmap_failed, const int32_t* slot_of_token) {
-  return launch_attn(pl, sm_count, false, Q, K, V, Kc, Vc, kmean, vmean, O, lse, ws, st, tmap_failed, slot_of_token);
+                               float* lse, void* ws, cudaStream_t st, bool* tmap_failed, const int32_t* slot_of_token,
+                               bool status_cleared) {
+  return launch_attn(pl, sm_count, false, Q, K, V, Kc, Vc, kmean, vmean, O, lse, ws, st, tmap_failed, slot_of_token,
+                     status_cleared);
 }
 
 cudaError_t launch_frame_attn(const Plan& pl, int sm_count, const void* Q, const void* K, const void* V, void* O, float* lse,
                               void* ws, cudaStream_t st, bool* tmap_failed) {
-  return launch_attn(pl, sm_count, true, Q, K, V, nullptr, nullptr, nullptr, nullptr, O, lse, ws, st, tmap_failed, nullptr);
+  return launch_attn(pl, sm_count, true, Q, K, V, nullptr, nullptr, nullptr, nullptr, O, lse, ws, st, tmap_failed, nullptr, false);
 }
 
 }  // namespace avggt

@@ -18,6 +18,25 @@ int record_cuda(cudaError_t e);
 // Keep `text` for avggt_last_cuda_error; returns AVGGT_ERR_CUDA.
 int record_message(const char* text);
 
+// Launch of a kernel that may be scheduled, up to its grid_dependency_wait, while the kernel before it in the stream ends:
+// the launch and the preparation of the layer's kernels (tensor memory, barriers) hide behind one another.
+template <typename... P, typename... A>
+cudaError_t launch_dependent(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t st, const A&... args) {
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
+constexpr size_t kAttnStatusBytes = 256;   // status block at the start of the attention workspace
+
 // ---- K/V compaction (build_kv.cu)
 int build_kv_grid(const Plan& pl, int sm_count);
 size_t build_kv_ws_bytes(const Plan& pl, int sm_count);
@@ -25,10 +44,11 @@ size_t build_kv_ws_bytes(const Plan& pl, int sm_count);
 // the M retained token indices (device) and the [n_tok] map the call fills (device).
 // kc_rows: rows per head of Kc / Vc (0 = M; larger when they are one rank's slot of an exchange buffer).
 // sums_only: kmean / vmean receive the un-normalised sums over the dropped rows instead of the means.
+// clear_status: the status block (kAttnStatusBytes) of the attention launch that follows in the stream, or null.
 cudaError_t launch_build_kv(const Plan& pl, int sm_count, const void* K, const void* V, void* Kc, void* Vc,
                             int32_t* idx, float* kmean, float* vmean, void* ws, cudaStream_t st,
                             const int32_t* caller_idx = nullptr, int32_t* slot_of_token = nullptr,
-                            int64_t kc_rows = 0, bool sums_only = false);
+                            int64_t kc_rows = 0, bool sums_only = false, void* clear_status = nullptr);
 
 // Frame-sharded layer: the ranks' slots of the exchange buffer -> one compact K/V pair, and the mean
 // pair from the all-reduced sums.
@@ -38,14 +58,14 @@ cudaError_t launch_assemble_shards(const void* gathered, int n_ranks, const int6
                                    float* vmean, cudaStream_t st);
 
 // ---- attention (global_attn.cu)
-constexpr size_t kAttnStatusBytes = 256;   // status block at the start of the attention workspace
 size_t global_attn_ws_bytes(const Plan& pl, int sm_count);
 // Returns cudaSuccess, or an error; *tmap_failed is set when a tensor map could not be encoded.
 // slot_of_token: null for the window rule; else the map written by the indexed compaction.
+// status_cleared: the compaction before it in the stream has cleared the status block.
 cudaError_t launch_global_attn(const Plan& pl, int sm_count, const void* Q, const void* K, const void* V,
                                const void* Kc, const void* Vc, const float* kmean, const float* vmean, void* O,
                                float* lse, void* ws, cudaStream_t st, bool* tmap_failed,
-                               const int32_t* slot_of_token = nullptr);
+                               const int32_t* slot_of_token = nullptr, bool status_cleared = false);
 
 // Frame attention (Sec. 4.2): the same kernel, one independent dense problem per frame.
 cudaError_t launch_frame_attn(const Plan& pl, int sm_count, const void* Q, const void* K, const void* V, void* O, float* lse,

@@ -17,11 +17,13 @@ class SubsampledGlobalAttention:
             raise RuntimeError("libavggt needs a CUDA device (sm_100); there is no CPU fallback")
         self.params = params
         self.device = torch.device(device)
+        self._index = torch.cuda.current_device() if self.device.index is None else self.device.index
         with torch.cuda.device(self.device):
             self.M, self.n_dropped = B.avggt_kv_count(params)
             self.build_ws_bytes, self.attn_ws_bytes = B.avggt_workspace_bytes(params)
         H, d = params.n_heads, params.head_dim
         self.n_tok = params.n_frames * params.tokens_per_frame
+        self._shape = torch.Size((self.n_tok, H, d))
         dev = self.device
         self.Kc = torch.empty((H, self.M, d), dtype=torch.bfloat16, device=dev)
         self.Vc = torch.empty((H, self.M, d), dtype=torch.bfloat16, device=dev)
@@ -33,7 +35,8 @@ class SubsampledGlobalAttention:
         self.lse = torch.empty((self.n_tok, H), dtype=torch.float32, device=dev) if want_lse else None
 
     def _stream(self):
-        return torch.cuda.current_stream(self.device).cuda_stream
+        # what torch.cuda.current_stream(device).cuda_stream gives, without building the Stream object (4 us of a 30 us layer)
+        return torch._C._cuda_getCurrentRawStream(self._index)
 
     def build_kv(self, K, V):
         B.avggt_build_kv(self.params, K, V, self.Kc, self.Vc, self.idx, self.kmean, self.vmean,
@@ -51,17 +54,25 @@ class SubsampledGlobalAttention:
         self._check_inputs(Q, K, V)
         if out is None:
             out = torch.empty_like(Q)
-        with torch.cuda.device(self.device):
+        with torch.cuda.device(self._index):
             B.avggt_frame_attn(self.params, Q, K, V, out, self.lse, self.attn_ws, self.attn_ws.numel(), self._stream())
         return out
 
     def forward(self, Q, K, V, out=None):
         self._check_inputs(Q, K, V)
-        with torch.cuda.device(self.device):
-            self.build_kv(K, V)
-            return self.attend(Q, K, V, out)
+        if torch.cuda.current_device() != self._index:
+            with torch.cuda.device(self._index):
+                return self._layer(Q, K, V, out)
+        return self._layer(Q, K, V, out)
 
     __call__ = forward
+
+    def _layer(self, Q, K, V, out):
+        if out is None:
+            out = torch.empty_like(Q)
+        B.avggt_layer(self.params, Q, K, V, self.Kc, self.Vc, self.idx, self.kmean, self.vmean, out, self.lse, self.build_ws,
+                      self.build_ws.numel(), self.attn_ws, self.attn_ws.numel(), self._stream())
+        return out
 
     def forward_host(self, hQ, hK, hV, hO, n_chunks=8):
         """The layer on host buffers (pinned memory), with the copies hidden behind the kernels.
@@ -156,7 +167,6 @@ class SubsampledGlobalAttention:
                 B.avggt_check_status(ws)
 
     def _check_inputs(self, *tensors):
-        shape = (self.n_tok, self.params.n_heads, self.params.head_dim)
         for t in tensors:
-            if t.dtype != torch.bfloat16 or tuple(t.shape) != shape or not t.is_contiguous() or t.device.type != "cuda":
-                raise ValueError(f"expected contiguous bf16 CUDA tensors of shape {shape}")
+            if t.dtype is not torch.bfloat16 or t.shape != self._shape or not t.is_contiguous() or not t.is_cuda:
+                raise ValueError(f"expected contiguous bf16 CUDA tensors of shape {tuple(self._shape)}")

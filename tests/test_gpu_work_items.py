@@ -1,0 +1,51 @@
+"""How the attention kernel cuts a launch: full items (256 rows), half items where the chip has room for all of them, a last
+item whose rows are spread over both tiles, several items per thread block, key counts around the 112-key step; and the
+one-call layer against its two calls."""
+
+import pytest
+import torch
+
+import paper_2512_02541_b200 as P
+from paper_2512_02541_b200 import binding as B
+from paper_2512_02541_b200 import inputs
+
+from test_gpu_parity import _check_attn, _host, _run_gpu
+
+pytestmark = pytest.mark.gpu
+
+
+# 32 heads: 7 or more half items per head do not fit the chip at once, so the items are full ones and some thread blocks have
+# two; the last item has 1, 16, 17, 128, 129 or 255 rows.  4 heads: half items.
+@pytest.mark.parametrize("heads,n_tok", [(32, 768 + r) for r in (1, 16, 17, 128, 129, 255)] + [(4, r) for r in (6, 64, 65, 129, 300)])
+@pytest.mark.parametrize("sigma,lse", [(1, False), (2, True)])
+def test_rows_of_the_last_item(heads, n_tok, sigma, lse):
+    wl = inputs.Workload("items", 1, 1, n_tok - 5, 5, heads, 64, sigma, 1, 2, "iid")
+    params, ocfg, layer, Q, K, V, O = _run_gpu(wl, seed=3, want_lse=lse)
+    _check_attn(ocfg, Q, _host(K), _host(V), O, lse=layer.lse)
+
+
+# keys 111, 112, 113, 224 and, past the 64 steps after which the row sums move on, 64 x 112 - 1, 64 x 112, 65 x 112 + 1
+@pytest.mark.parametrize("n_keys", (111, 112, 113, 224, 7167, 7168, 7281))
+def test_key_counts_around_a_step(n_keys):
+    wl = inputs.Workload("keys", 1, 1, n_keys, 0, 1, 64, 1, 0, 0, "iid")
+    _, ocfg, layer, Q, K, V, O = _run_gpu(wl, seed=4, want_lse=True)
+    rows = inputs.sample_rows(wl, 300).numpy()
+    _check_attn(ocfg, Q, _host(K), _host(V), O, rows=rows, lse=layer.lse)
+
+
+@pytest.mark.parametrize("sigma,mean_fill", [(4, 2), (4, 0), (1, 2)])   # (1, 2): nothing dropped, the mean pair is zero-filled
+def test_layer_call_gives_the_bits_of_its_two_calls(sigma, mean_fill):
+    wl = inputs.Workload("layer", 3, 9, 11, 5, 6, 64, sigma, 1, mean_fill, "proj")
+    params, _, layer, Q, K, V, O = _run_gpu(wl, seed=5)
+    two = P.SubsampledGlobalAttention(params)
+    for t in (two.kmean, two.vmean):
+        t.fill_(float("nan"))
+    two.build_kv(K, V)
+    assert torch.equal(two.attend(Q, K, V), O)
+    for a, b in ((two.Kc, layer.Kc), (two.Vc, layer.Vc), (two.idx, layer.idx)):
+        assert torch.equal(a, b)
+    if mean_fill:
+        assert torch.equal(two.kmean, layer.kmean) and torch.equal(two.vmean, layer.vmean)
+    with pytest.raises(B.AvggtError):   # everything is rejected before anything is enqueued
+        B.avggt_layer(params, Q, K, V, layer.Kc, layer.Vc, layer.idx, layer.kmean, layer.vmean, O, None, layer.build_ws, 0,
+                      layer.attn_ws, layer.attn_ws.numel(), None)
