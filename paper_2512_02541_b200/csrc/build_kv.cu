@@ -157,11 +157,15 @@ mean_finalize_kernel(const float* __restrict__ partials, int n_blocks, int cols2
 // slot_of_token[t] = -1 for every token, then m for the m-th retained token.  Entries of idx outside
 // [0, n_tok) are skipped.
 __global__ void fill_slots_kernel(int32_t* __restrict__ slot_of_token, int64_t n_tok) {
+  grid_launch_dependents();
+  grid_dependency_wait();
   const int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
   if (i < n_tok) slot_of_token[i] = -1;
 }
 __global__ void scatter_slots_kernel(const int32_t* __restrict__ idx, int64_t M, int32_t* __restrict__ slot_of_token,
                                      int64_t n_tok) {
+  grid_launch_dependents();
+  grid_dependency_wait();
   const int64_t m = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
   if (m < M) {
     const int32_t t = idx[m];
@@ -255,10 +259,10 @@ cudaError_t launch_build_kv(const Plan& pl, int sm_count, const void* K, const v
   if (kc_rows <= 0) kc_rows = pl.M;
   if (slot_of_token != nullptr) {
     // caller-chosen retained set: build the token -> compact position map first
-    fill_slots_kernel<<<static_cast<unsigned>((pl.n_tok + 255) / 256), 256, 0, st>>>(slot_of_token, pl.n_tok);
-    if (pl.M > 0 && caller_idx != nullptr)
-      scatter_slots_kernel<<<static_cast<unsigned>((pl.M + 255) / 256), 256, 0, st>>>(caller_idx, pl.M, slot_of_token, pl.n_tok);
-    cudaError_t e0 = cudaGetLastError();
+    cudaError_t e0 = launch_dependent(fill_slots_kernel, static_cast<unsigned>((pl.n_tok + 255) / 256), 256, 0, st, slot_of_token, pl.n_tok);
+    if (e0 == cudaSuccess && pl.M > 0 && caller_idx != nullptr)
+      e0 = launch_dependent(scatter_slots_kernel, static_cast<unsigned>((pl.M + 255) / 256), 256, 0, st, caller_idx, pl.M, slot_of_token,
+                            pl.n_tok);
     if (e0 != cudaSuccess) return e0;
     idx = nullptr;
   }

@@ -1168,6 +1168,10 @@ constexpr size_t kAttnSmemBytes = static_cast<size_t>(kTileBytes) * (2 * kQTiles
 
 }  // namespace
 
+cudaError_t launch_clear_status(void* status, cudaStream_t st) {
+  return launch_dependent(clear_status_kernel, 1, 64, 0, st, static_cast<uint32_t*>(status));
+}
+
 size_t global_attn_ws_bytes(const Plan&, int) { return kAttnStatusBytes; }
 
 namespace {
@@ -1274,7 +1278,7 @@ cudaError_t launch_attn(const Plan& pl, int sm_count, bool frame_mode, const voi
   cudaError_t e = prepare_kernels();
   if (e != cudaSuccess) return e;
   if (!status_cleared) {
-    e = launch_dependent(clear_status_kernel, 1, 64, 0, st, static_cast<uint32_t*>(ws));
+    e = launch_clear_status(ws, st);
     if (e != cudaSuccess) return e;
   }
   const unsigned grid = static_cast<unsigned>(a.n_work < sm_count ? a.n_work : sm_count);

@@ -37,6 +37,9 @@ cudaError_t launch_dependent(void (*kernel)(P...), unsigned grid, unsigned block
 
 constexpr size_t kAttnStatusBytes = 256;   // status block at the start of the attention workspace
 
+// Clears the status block of a launch that no kernel of this library has cleared it for (global_attn.cu).
+cudaError_t launch_clear_status(void* status, cudaStream_t st);
+
 // ---- K/V compaction (build_kv.cu)
 int build_kv_grid(const Plan& pl, int sm_count);
 size_t build_kv_ws_bytes(const Plan& pl, int sm_count);

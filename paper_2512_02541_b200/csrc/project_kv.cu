@@ -26,6 +26,8 @@
 // fetched from HBM once and from L2 by the others.  Per-CTA partial sums go to the workspace and
 // a small second kernel adds them in a fixed order: no floating-point atomics, results identical
 // from run to run.
+#include <mutex>
+
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -65,6 +67,9 @@ struct ProjArgs {
   float* partials;        // [gridDim.x][4 warps][256]: sums over the dropped rows this warp has seen
   uint32_t* status;       // 4 words, as in the attention kernel
   int32_t do_mean;
+  int32_t zero_means;     // zero-fill kmean and vmean
+  float* kmean;
+  float* vmean;
 };
 
 struct __align__(8) ProjBarriers {
@@ -143,8 +148,6 @@ project_kv_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
   const int tok0 = blockIdx.x / (2 * a.n_col_tiles);              // first token tile
   const int n_kb = a.C / kBlockK;
 
-  if (__syncthreads_or(*reinterpret_cast<volatile uint32_t*>(a.status) != 0u)) return;
-
   if (threadIdx.x == 0) {
     for (int s = 0; s < kProjStages; ++s) {
       mbar_init(smem_u32(&bars.full[s]), 1);
@@ -162,12 +165,18 @@ project_kv_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
     tmem_alloc(smem_u32(&bars.tmem_base), kProjTmemCols);
     tmem_relinquish();
   }
+  // everything above may run while the kernel before this one ends
+  grid_dependency_wait();
+  if (blockIdx.x == 0 && a.zero_means && threadIdx.x < 256) {   // a problem that drops nothing
+    for (int i = threadIdx.x; i < a.pl.H * a.pl.d; i += 256) { a.kmean[i] = 0.f; a.vmean[i] = 0.f; }
+  }
   tc_fence_before();
-  __syncthreads();
+  const bool abandoned = __syncthreads_or(*reinterpret_cast<volatile uint32_t*>(a.status) != 0u) != 0;
   tc_fence_after();
   const uint32_t tmem = bars.tmem_base;
 
-  if (warp == 0) {
+  if (abandoned) {
+  } else if (warp == 0) {
     // ------------------------------------------------------------ TMA producer
     const CUtensorMap* tm_w = which == 0 ? &tm_wk : &tm_wv;
     if (elect_one()) {
@@ -338,6 +347,7 @@ project_kv_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
     }
   }
 
+  grid_launch_dependents();
   tmem_wait_ld();
   tc_fence_before();
   __syncthreads();
@@ -348,17 +358,36 @@ project_kv_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
 __global__ void __launch_bounds__(256)
 project_mean_kernel(const float* __restrict__ partials, int grid, int n_col_tiles, int cols_total, float inv_count,
                     float* __restrict__ kmean, float* __restrict__ vmean) {
+  grid_launch_dependents();
+  grid_dependency_wait();
   const int g = blockIdx.x * blockDim.x + threadIdx.x;     // column of [K | V]
   if (g >= 2 * cols_total) return;
   const int which = g / cols_total, col = g - which * cols_total;
   const int col_tile_all = which * n_col_tiles + col / kTileCol, in_tile = col % kTileCol;
   float s = 0.f;
   for (int cta = col_tile_all; cta < grid; cta += 2 * n_col_tiles)
-    for (int w = 0; w < 4; ++w) s += partials[(static_cast<size_t>(cta) * 4 + w) * kTileCol + in_tile];
+    for (int w = 0; w < 4; ++w) s += __ldcg(partials + (static_cast<size_t>(cta) * 4 + w) * kTileCol + in_tile);
   (which == 0 ? kmean : vmean)[col] = s * inv_count;
 }
 
 constexpr size_t kProjSmemBytes = static_cast<size_t>(kProjStages) * (kBytesA + kBytesB) + 8 * kStageBytes + 1024;
+
+// Once per device: the dynamic shared-memory limit of the kernel.
+cudaError_t prepare_kernel() {
+  static std::mutex mu;
+  static bool ready[64] = {};
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+  std::lock_guard<std::mutex> lock(mu);
+  if (!ready[dev]) {
+    e = cudaFuncSetAttribute(project_kv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kProjSmemBytes));
+    if (e != cudaSuccess) return e;
+    ready[dev] = true;
+  }
+  return cudaSuccess;
+}
 
 int project_grid(const Plan& pl, int sm_count) {
   const int per_tok = 2 * ((pl.H * pl.d + kTileCol - 1) / kTileCol);
@@ -397,6 +426,9 @@ cudaError_t launch_project_kv(const Plan& pl, int sm_count, int model_dim, const
   a.status = static_cast<uint32_t*>(ws);
   a.partials = reinterpret_cast<float*>(static_cast<char*>(ws) + kAttnStatusBytes);
   a.do_mean = (pl.mean_fill != 0 && pl.n_dropped > 0) ? 1 : 0;
+  a.zero_means = pl.mean_fill != 0 && !a.do_mean;
+  a.kmean = kmean;
+  a.vmean = vmean;
 
   CUtensorMap tm_x, tm_wk, tm_wv, tm_kfull, tm_vfull;
   const uint64_t x_dims[2] = {static_cast<uint64_t>(model_dim), static_cast<uint64_t>(pl.n_tok)};
@@ -418,23 +450,13 @@ cudaError_t launch_project_kv(const Plan& pl, int sm_count, int model_dim, const
   else tm_vfull = tm_x;
   if (!good) { *tmap_failed = true; return cudaSuccess; }
 
-  cudaError_t e = cudaFuncSetAttribute(project_kv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kProjSmemBytes));
-  if (e != cudaSuccess) return e;
-  e = cudaMemsetAsync(ws, 0, kAttnStatusBytes, st);
-  if (e != cudaSuccess) return e;
-  project_kv_kernel<<<grid, kProjThreads, kProjSmemBytes, st>>>(tm_x, tm_wk, tm_wv, tm_kfull, tm_vfull, a);
-  e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  if (pl.mean_fill != 0) {
-    if (a.do_mean) {
-      project_mean_kernel<<<(2 * cols_total + 255) / 256, 256, 0, st>>>(a.partials, grid, a.n_col_tiles, cols_total,
-                                                                      1.0f / static_cast<float>(pl.n_dropped), kmean, vmean);
-      e = cudaGetLastError();
-    } else {
-      e = cudaMemsetAsync(kmean, 0, static_cast<size_t>(cols_total) * sizeof(float), st);
-      if (e == cudaSuccess) e = cudaMemsetAsync(vmean, 0, static_cast<size_t>(cols_total) * sizeof(float), st);
-    }
-  }
+  cudaError_t e = prepare_kernel();
+  if (e == cudaSuccess) e = launch_clear_status(ws, st);
+  if (e == cudaSuccess)
+    e = launch_dependent(project_kv_kernel, grid, kProjThreads, kProjSmemBytes, st, tm_x, tm_wk, tm_wv, tm_kfull, tm_vfull, a);
+  if (e == cudaSuccess && a.do_mean)
+    e = launch_dependent(project_mean_kernel, (2 * cols_total + 255) / 256, 256, 0, st, a.partials, grid, a.n_col_tiles, cols_total,
+                         1.0f / static_cast<float>(pl.n_dropped), kmean, vmean);
   return e;
 }
 
