@@ -90,27 +90,10 @@ constexpr int kFlushSteps = 64;
 #endif
 constexpr uint32_t kPolyBlocks = AVGGT_POLY_BLOCKS;
 
-// Division of n < 2^31 by a number known at launch as a multiplication: n / d = n m >> s with m = ceil(2^s / d),
-// s = 31 + ceil(log2 d), exact because m d - 2^s < d <= 2^(s - 31).  (The epilogue asks six such questions per row; as
-// divisions they were a quarter of its time.)
-struct Divisor {
-  uint32_t d, m, s;
-};
-Divisor make_divisor(uint32_t d) {
-  Divisor v{d, 0, 31};
-  while ((uint64_t(1) << (v.s - 31)) < d) ++v.s;
-  v.m = static_cast<uint32_t>(((uint64_t(1) << v.s) + d - 1) / d);
-  return v;
-}
-__device__ __forceinline__ uint32_t divide(uint32_t n, const Divisor& v, uint32_t& rest) {
-  const uint32_t q = static_cast<uint32_t>((static_cast<uint64_t>(n) * v.m) >> v.s);
-  rest = n - q * v.d;
-  return q;
-}
-
 struct AttnArgs {
   Plan pl;
-  Divisor by_pairs, by_heads, by_L, by_grid_w, by_s_h, by_s_w;
+  Divisor by_pairs, by_heads;
+  WindowRule rule;
   const uint4* Q;       // [n_tok, H, d], read by the diagonal and mean terms; K and V by the diagonal term only
   const uint4* K;
   const uint4* V;
@@ -202,8 +185,6 @@ constexpr int kRegsLaunch = 96;   // 65536 / 640 threads, rounded down to the al
 constexpr int kRegsSoftmax = 112, kRegsOther = 32;
 static_assert(kRegsSoftmax * kSoftmaxWarps + kRegsOther * (kThreads / 32 - kSoftmaxWarps) <= kRegsLaunch * (kThreads / 32),
               "register budget after setmaxnreg exceeds the launch allocation");
-template <int N> __device__ __forceinline__ void reg_inc() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N)); }
-template <int N> __device__ __forceinline__ void reg_dec() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N)); }
 
 // A work item.
 struct WorkItem {
@@ -791,17 +772,6 @@ __device__ __forceinline__ float dot_bf16x8_f32(const uint4& x, const float4& a,
   return fmaf(__uint_as_float(x.w & 0xffff0000u), b.w, acc);
 }
 
-// The window rule: compact_slot(frame, slot) < 0
-__device__ __forceinline__ bool is_dropped(const AttnArgs& a, int row) {
-  uint32_t slot, c, rest_h, rest_w;
-  const uint32_t frame = divide(row, a.by_L, slot);
-  const uint32_t n_special = a.pl.n_special;
-  const uint32_t r = divide(slot >= n_special ? slot - n_special : 0u, a.by_grid_w, c);
-  divide(r, a.by_s_h, rest_h);
-  divide(c, a.by_s_w, rest_w);
-  return slot >= n_special && !(a.pl.keep_first && frame == 0) && (rest_h | rest_w) != 0;
-}
-
 // What the epilogue of a work item needs of its rows' running state (shared memory; a row's warp writes and reads it).
 struct RowResults {
   float neg_m[kQTiles * kTileQ];     // minus the reference maximum
@@ -862,7 +832,7 @@ __device__ __forceinline__ bool softmax_epilogue(const AttnArgs& a, Barriers* ba
       for (int hi = 0; hi < 2; ++hi) {
         const int row = tile.q0 + r0 + 8 * hi;
         if (row >= tile.first && row < tile.last) {
-          dropped[hi] = a.slot_of_token != nullptr ? a.slot_of_token[row] < 0 : is_dropped(a, row);
+          dropped[hi] = a.slot_of_token != nullptr ? a.slot_of_token[row] < 0 : compact_position(a.rule, pl, row) < 0;
         }
       }
 #pragma unroll
@@ -1248,10 +1218,7 @@ cudaError_t launch_attn(const Plan& pl, int sm_count, bool frame_mode, const voi
   a.pairs = static_cast<int32_t>((rows + a.item_rows - 1) / a.item_rows);
   a.by_pairs = make_divisor(a.pairs);
   a.by_heads = make_divisor(pl.H);
-  a.by_L = make_divisor(pl.L);
-  a.by_grid_w = make_divisor(pl.grid_w);
-  a.by_s_h = make_divisor(pl.s_h);
-  a.by_s_w = make_divisor(pl.s_w);
+  a.rule = make_window_rule(pl);
   a.n_work = static_cast<int32_t>(a.pairs * problems);
 
   // token-major [n_tok, H*d] maps for Q and, in frame attention, K and V; head-major [H, M, d] maps for Kc, Vc otherwise
