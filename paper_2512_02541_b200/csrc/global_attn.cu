@@ -111,7 +111,8 @@ struct AttnArgs {
   int32_t n_work;       // work items (pairs of query tiles x heads x problems) of the launch; a CTA takes the items
                         // blockIdx.x, blockIdx.x + gridDim.x, ...
   int32_t item_rows;    // query rows of a work item: 256 (two full tiles), or 128 or 64 spread over both tiles
-  int32_t pairs;        // work items of one problem and head
+  int32_t pairs;        // work items of one problem and head (kShortLast: the full ones)
+  int32_t n_full, ragged_rows;   // kShortLast: pairs x heads x problems; query rows of the items after them
   int32_t use_diag;     // diag on and |D| > 0
   int32_t use_mean;     // mean_fill on and |D| > 0
   float scale_log2;     // softmax scale * log2(e)
@@ -201,11 +202,22 @@ struct QueryTile {
 };
 
 // Items are numbered with the pair of query tiles fastest, then the head, then (frame
-// attention) the frame, so that the CTAs running side by side share one head's keys in L2.
+// attention) the frame, so that the CTAs running side by side share one head's keys in L2.  kShortLast (launches without the
+// extra columns, i.e. frame attention, and the dense layer, where it makes no difference): the ragged last items of the problems
+// come after all the full ones, so that every CTA meets some (with six items per frame and head and 148 CTAs every second CTA
+// never met a short one).  With the trimmed last key tile, frame attention of 10 frames 125.3 -> 122.0 us, of 100 frames
+// 1187 -> 1171 us; with tile 1 left out of items of one tile 118.8 and 1139 us (of the same run: 124.4 and 1177 before).  The
+// card is at its power limit there, so it is the products not made that count more than the balance.
+template <bool kShortLast>
 __device__ __forceinline__ WorkItem work_item(const AttnArgs& a, uint32_t item) {
   WorkItem w;
   uint32_t qp, head;
-  const uint32_t frame = divide(divide(item, a.by_pairs, qp), a.by_heads, head);
+  uint32_t rest = divide(item, a.by_pairs, qp);
+  if (kShortLast && item >= static_cast<uint32_t>(a.n_full)) {
+    rest = item - a.n_full;
+    qp = a.pairs;
+  }
+  const uint32_t frame = divide(rest, a.by_heads, head);
   w.head = static_cast<int>(head);
   w.key_row0 = static_cast<int>(frame) * a.pl.L;   // the subsampled layer has one problem
   w.row0 = w.key_row0 + static_cast<int>(qp) * a.item_rows;
@@ -217,8 +229,17 @@ __device__ __forceinline__ WorkItem work_item(const AttnArgs& a, uint32_t item) 
 // An item with rows for one tile only is cut in two halves by groups of 16 rows (one softmax warp), the second
 // half in the upper lanes of its tile: every scheduler then has two warps with work at most, and both tiles' products
 // overlap.  Warps without rows compute nothing.
+//
+// kShortLast: tile 0 takes all the rows and tile 1 sits the item out, products and all.  (The subsampled layer meets such an
+// item once per head, or is so small that nothing but latency counts; there the halves are as good and the code simpler.)
+template <bool kShortLast>
 __device__ __forceinline__ QueryTile query_tile(const WorkItem& w, int t) {
   QueryTile q;
+  if (kShortLast) {
+    q.q0 = q.first = w.row0 + t * kTileQ;
+    q.last = t == 0 && w.end - w.row0 > kTileQ ? static_cast<int64_t>(w.row0) + kTileQ : w.end;
+    return q;
+  }
   const bool two = w.end - w.row0 > kTileQ;
   const int groups = two ? 16 : static_cast<int>(w.end - w.row0 + 15) >> 4;
   const int cut = w.row0 + 16 * ((groups + 1) >> 1);   // first row of tile 1
@@ -246,7 +267,13 @@ __device__ __forceinline__ bool wait_bar_warp(uint64_t* bar, uint32_t parity, Ba
   return __all_sync(kFullMask, wait_bar(bar, parity, bars, a, where, iter, check_abort));
 }
 
+// kShortLast: tile 1 has rows in the item
+__device__ __forceinline__ bool tile_has_rows(const AttnArgs& a, uint32_t item) {
+  return a.item_rows > kTileQ && (item < static_cast<uint32_t>(a.n_full) || a.ragged_rows > kTileQ);
+}
+
 // ------------------------------------------------------------------ TMA producer (one warp)
+template <bool kShortLast>
 __device__ __forceinline__ void producer_role(const CUtensorMap* tm_q, const CUtensorMap* tm_k, const CUtensorMap* tm_v,
                                               const AttnArgs& a, Barriers* bars, const SmemLayout& sm) {
   const int n_kv = a.n_kv_tiles;
@@ -263,7 +290,7 @@ __device__ __forceinline__ void producer_role(const CUtensorMap* tm_q, const CUt
   int n_done = 0;              // work items completed by this role
   int q_issued = 0;            // work items whose Q copies have been issued
   for (uint32_t item = blockIdx.x; item < static_cast<uint32_t>(a.n_work) && ok; item += gridDim.x, ++n_done) {
-    const WorkItem wi = work_item(a, item);
+    const WorkItem wi = work_item<kShortLast>(a, item);
     const int head = wi.head;
     const int place = n_done & 1;
     // a wait has run out in another thread block: the launch is abandoned
@@ -280,7 +307,7 @@ __device__ __forceinline__ void producer_role(const CUtensorMap* tm_q, const CUt
       mbar_arrive_expect_tx(qb, kQTiles * kTileBytes);
 #pragma unroll
       for (int t = 0; t < kQTiles; ++t)
-        tma_load_2d(smem_u32(sm.q + (place * kQTiles + t) * kTileBytes), tm_q, head * kHeadDim, query_tile(wi, t).q0, qb);
+        tma_load_2d(smem_u32(sm.q + (place * kQTiles + t) * kTileBytes), tm_q, head * kHeadDim, query_tile<kShortLast>(wi, t).q0, qb);
     }
     __syncwarp();
     ++q_issued;
@@ -343,9 +370,9 @@ __device__ __forceinline__ void producer_role(const CUtensorMap* tm_q, const CUt
 // warps, so each instruction of it counts: the lower halves of the operand descriptors advance by additions of a constant, the
 // upper halves are constants, and of several waits the one that is satisfied last comes last.
 template <int t>
-__device__ __forceinline__ void issue_qk(Barriers* bars, uint32_t tmem, uint32_t desc_q, uint32_t desc_k, int stage, bool odd) {
+__device__ __forceinline__ void issue_qk(Barriers* bars, uint32_t tmem, uint32_t desc_q, uint32_t desc_k, int stage, bool odd,
+                                         uint32_t idesc) {
   if (elect_one()) {
-    constexpr uint32_t idesc = umma_idesc_bf16(kTileQ, kTileKV, false);
     const uint32_t d = tmem + t * kTmemTileStride + (odd ? kColSOdd : 0);
 #pragma unroll
     for (int k = 0; k < kHeadDim / 16; ++k) umma_ss_lo(d, desc_q + (k * 32 >> 4), desc_k + (k * 32 >> 4), idesc, k > 0);
@@ -357,8 +384,9 @@ __device__ __forceinline__ void issue_qk(Barriers* bars, uint32_t tmem, uint32_t
 
 // O_t += P_t V and, as columns 64..79 of the same product, the row sums of P: the descriptor's leading byte offset leads
 // from a slice of 16 keys of the V tile to the ones block, which serves as value columns 64..79 of every slice.
-template <int t>
-__device__ __forceinline__ void issue_pv(Barriers* bars, uint32_t tmem, uint32_t desc_v, int stage, bool odd, bool first) {
+template <int t, bool kTrim>
+__device__ __forceinline__ void issue_pv(Barriers* bars, uint32_t tmem, uint32_t desc_v, int stage, bool odd, bool first,
+                                         int slices) {
   if (elect_one()) {
     constexpr uint32_t idesc = umma_idesc_bf16(kTileQ, kPvCols, true);
     constexpr uint32_t kSlice = 16 * kHeadDim * 2;   // bytes of 16 keys: the start moves on, the offset to the ones shrinks
@@ -367,14 +395,16 @@ __device__ __forceinline__ void issue_pv(Barriers* bars, uint32_t tmem, uint32_t
     umma_ts_lo(tmem + t * kTmemTileStride + kColO, p, desc_v, idesc, !first);
 #pragma unroll
     for (int k = 1; k < kTileKV / 16; ++k)
-      umma_ts_lo(tmem + t * kTmemTileStride + kColO, p + k * 8, desc_v + k * kAdvance, idesc, true);
+      if (!kTrim || k < slices) umma_ts_lo(tmem + t * kTmemTileStride + kColO, p + k * 8, desc_v + k * kAdvance, idesc, true);
     umma_commit(smem_u32(&bars->o_done[t][odd]));
     umma_commit(smem_u32(&bars->v_empty[stage]));
   }
   __syncwarp();
 }
 
-template <int t>
+// kTrim: of a ragged last tile compute only as many columns and slices of 16 keys as hold keys.  Worth its instructions where steps
+// are few (frame attention of 1,374 tokens has 30 keys in the last of 13 tiles: 1.5 %); in the subsampled layer they cost 1 %.
+template <int t, bool kTrim>
 __device__ __forceinline__ void mma_issue_loop(const AttnArgs& a, Barriers* bars, const SmemLayout& sm, uint32_t tmem) {
   static_assert(kStages >= 2, "the K ring must hold the tile in use and the next one");
   const int n_kv = a.n_kv_tiles;
@@ -384,6 +414,9 @@ __device__ __forceinline__ void mma_issue_loop(const AttnArgs& a, Barriers* bars
   constexpr uint32_t kStage = kKeyTileBytes >> 4;         // a stage further on the start advances ...
   constexpr uint32_t kStageV = kStage - (kStage << 16);   // ... and the offset to the ones shrinks
   if (n_kv == 0) return;   // no retained keys: the epilogue's two extra columns are the whole layer
+  const int ragged_slices = a.last_tile_keys != 0 ? (a.last_tile_keys + 15) >> 4 : kTileKV / 16;
+  constexpr uint32_t kDescQk = umma_idesc_bf16(kTileQ, kTileKV, false);
+  const uint32_t ragged_desc_qk = umma_idesc_bf16(kTileQ, 16 * ragged_slices, false);
 
   // Running over all work items of the CTA: the ring positions of the next K and V tile, and g, the number of key
   // steps of this tile so far (the phase of the per-step barriers).
@@ -391,10 +424,30 @@ __device__ __forceinline__ void mma_issue_loop(const AttnArgs& a, Barriers* bars
   uint32_t k_parity = 0, v_parity = 0;   // parity of their "full" phase
   int g = 0;
   int n_done = 0;
-  for (uint32_t item = blockIdx.x; item < static_cast<uint32_t>(a.n_work); item += gridDim.x, ++n_done, g += n_kv) {
-    const bool more = item + gridDim.x < static_cast<uint32_t>(a.n_work);
-    // j = -1: Q K^T of the CTA's first step, which no P V precedes
-    for (int j = n_done == 0 ? -1 : 0; j < n_kv; ++j) {
+  int n_active = 0;          // work items this tile had rows in
+  bool first_issued = false; // Q K^T of the item's first step went out with the item before
+  for (uint32_t item = blockIdx.x; item < static_cast<uint32_t>(a.n_work); item += gridDim.x, ++n_done) {
+    if (kTrim && t > 0 && !tile_has_rows(a, item)) {
+      // the tile sits this item out: pass its tiles on in step
+      if (!wait_bar_warp(&bars->q_full[n_done & 1], (n_done >> 1) & 1, bars, a, 20, n_done)) return;
+      if (elect_one()) mbar_arrive(smem_u32(&bars->q_empty[n_done & 1]));
+      __syncwarp();
+      for (int j = 0; j < n_kv; ++j) {
+        if (!wait_bar_warp(&bars->k_full[k_stage], k_parity, bars, a, 24 + t, j)) return;
+        if (elect_one()) mbar_arrive(smem_u32(&bars->k_empty[k_stage]));
+        __syncwarp();
+        if (++k_stage == kStages) { k_stage = 0; k_parity ^= 1; }
+        if (!wait_bar_warp(&bars->v_full[v_stage], v_parity, bars, a, 28 + t, j)) return;
+        if (elect_one()) mbar_arrive(smem_u32(&bars->v_empty[v_stage]));
+        __syncwarp();
+        if (++v_stage == kStages) { v_stage = 0; v_parity ^= 1; }
+      }
+      continue;
+    }
+    const bool more = item + gridDim.x < static_cast<uint32_t>(a.n_work) &&
+                      (!kTrim || t == 0 || tile_has_rows(a, item + gridDim.x));
+    // j = -1: Q K^T of the first step, where it has not been issued with the item before
+    for (int j = first_issued ? 0 : -1; j < n_kv; ++j) {
       const bool last = j + 1 == n_kv;
       if (!last || more) {
         const int next = last ? 0 : j + 1;                  // step within its work item
@@ -402,9 +455,10 @@ __device__ __forceinline__ void mma_issue_loop(const AttnArgs& a, Barriers* bars
         const int place = next_item & 1;
         if (next == 0 && !wait_bar_warp(&bars->q_full[place], (next_item >> 1) & 1, bars, a, 20, n_done)) return;
         if (!wait_bar_warp(&bars->k_full[k_stage], k_parity, bars, a, 24 + t, g + j)) return;
-        if (j >= 0 && !wait_bar_warp(&bars->s_free[t], (g + j) & 1, bars, a, 22 + t, g + j)) return;
+        if (g + j >= 0 && !wait_bar_warp(&bars->s_free[t], (g + j) & 1, bars, a, 22 + t, g + j)) return;
         tc_fence_after();
-        issue_qk<t>(bars, tmem, q_desc + place * (kQTiles * kTileBytes >> 4), k_desc + k_stage * kStage, k_stage, ((g + j + 1) & 1) != 0);
+        issue_qk<t>(bars, tmem, q_desc + place * (kQTiles * kTileBytes >> 4), k_desc + k_stage * kStage, k_stage, ((g + j + 1) & 1) != 0,
+                    kTrim && next + 1 == n_kv ? ragged_desc_qk : kDescQk);
         if (++k_stage == kStages) { k_stage = 0; k_parity ^= 1; }
         if (next + 1 == n_kv) {   // every Q K^T of the work item has been issued: when they have completed, Q may be overwritten
           if (elect_one()) umma_commit(smem_u32(&bars->q_empty[place]));
@@ -414,21 +468,24 @@ __device__ __forceinline__ void mma_issue_loop(const AttnArgs& a, Barriers* bars
       if (j < 0) continue;
       if (!wait_bar_warp(&bars->v_full[v_stage], v_parity, bars, a, 28 + t, g + j)) return;
       // the first P V of a work item overwrites O_t: the previous item's epilogue must have read it out
-      if (j == 0 && n_done > 0 && !wait_bar_warp(&bars->o_free[t], (n_done - 1) & 1, bars, a, 29, n_done)) return;
+      if (j == 0 && n_active > 0 && !wait_bar_warp(&bars->o_free[t], (n_active - 1) & 1, bars, a, 29, n_done)) return;
       if (!wait_bar_warp(&bars->p_full[t][(g + j) & 1], ((g + j) >> 1) & 1, bars, a, 26 + t, g + j)) return;
       tc_fence_after();
-      issue_pv<t>(bars, tmem, v_desc + v_stage * kStageV, v_stage, ((g + j) & 1) != 0, j == 0);
+      issue_pv<t, kTrim>(bars, tmem, v_desc + v_stage * kStageV, v_stage, ((g + j) & 1) != 0, j == 0, last ? ragged_slices : kTileKV / 16);
       if (++v_stage == kStages) { v_stage = 0; v_parity ^= 1; }
     }
+    first_issued = more;
+    g += n_kv;
+    ++n_active;
   }
 }
 
 // The issue loop, then (on every path out of it, a wait that ran out included) a wait until the
 // tensor core has finished everything this warp issued: the CTA must not free its tensor memory
 // or leave its shared memory while a tcgen05.mma still reads or writes them.
-template <int t>
+template <int t, bool kTrim>
 __device__ __forceinline__ void mma_role(const AttnArgs& a, Barriers* bars, const SmemLayout& sm, uint32_t tmem) {
-  mma_issue_loop<t>(a, bars, sm, tmem);
+  mma_issue_loop<t, kTrim>(a, bars, sm, tmem);
   __syncwarp();
   if (elect_one()) umma_commit(smem_u32(&bars->mma_idle[t]));
   __syncwarp();
@@ -787,8 +844,8 @@ template <bool kLse, bool kExtra>
 __device__ __forceinline__ bool softmax_epilogue(const AttnArgs& a, Barriers* bars, const SoftmaxThread& me, const RowResults* res,
                                                  uint32_t item, int last) {
   const Plan& pl = a.pl;
-  const WorkItem wi = work_item(a, item);
-  const QueryTile tile = query_tile(wi, me.t);
+  const WorkItem wi = work_item<!kExtra>(a, item);
+  const QueryTile tile = query_tile<!kExtra>(wi, me.t);
   const int t = me.t, head = wi.head;
   const int i = me.lane & 3;                             // position in the quad
   const int r0 = 32 * me.q + 16 * me.h + (me.lane >> 2);   // the thread's two rows within the tile: r0, r0 + 8
@@ -952,11 +1009,12 @@ __device__ __forceinline__ void softmax_items(const AttnArgs& a, Barriers* bars,
   const bool ragged = a.last_tile_keys != 0;
   bool res_rows = false;   // the warp had rows in the item before
   int gj = 0;              // this tile's key steps so far, over all work items of the CTA: the phase of the per-step barriers
+  bool pending = false;    // the epilogue of the item before
 #pragma unroll 1
   for (uint32_t item = blockIdx.x;; item += gridDim.x) {
     const bool have = item < static_cast<uint32_t>(a.n_work);
-    bool pending = item != blockIdx.x;   // the epilogue of the item before
     if (!have && !pending) return;
+    const bool active = have && (kExtra || t == 0 || tile_has_rows(a, item));   // the tile has rows in this item
     RowState st;
 #pragma unroll
     for (int hi = 0; hi < 2; ++hi) {
@@ -966,8 +1024,8 @@ __device__ __forceinline__ void softmax_items(const AttnArgs& a, Barriers* bars,
     }
     bool rows = false;
     if (have) {
-      const WorkItem wi = work_item(a, item);
-      const QueryTile tile = query_tile(wi, t);
+      const WorkItem wi = work_item<!kExtra>(a, item);
+      const QueryTile tile = query_tile<!kExtra>(wi, t);
       const int row0 = tile.q0 + 32 * me.q + 16 * me.h;   // the warp's first row
       rows = row0 + 16 > tile.first && row0 < tile.last;
       if (kExtra && a.use_diag) {   // each thread asks for one line: K of row lane / 2, or V
@@ -976,7 +1034,7 @@ __device__ __forceinline__ void softmax_items(const AttnArgs& a, Barriers* bars,
           prefetch_l2(((me.lane & 1) ? a.V : a.K) + (static_cast<size_t>(row) * a.pl.H + wi.head) * (kHeadDim / 8));
       }
     }
-    int left = have ? n_kv : 0;
+    int left = active ? n_kv : 0;
 #pragma unroll 1
     do {
       const int most = pending ? 1 : kFlushSteps;
@@ -1015,6 +1073,8 @@ __device__ __forceinline__ void softmax_items(const AttnArgs& a, Barriers* bars,
       }
     } while (left > 0);
     if (!have) return;
+    pending = active;
+    if (!active) continue;
     __syncwarp();   // every lane has read the results of the item before
 #pragma unroll
     for (int hi = 0; hi < 2; ++hi) {
@@ -1114,9 +1174,9 @@ global_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
     softmax_role<kLse, kExtra>(a, &bars, &row_results, tmem, warp, tid & 31);
   } else {
     reg_dec<kRegsOther>();
-    if (warp == kTmaWarp) producer_role(&tm_q, &tm_k, &tm_v, a, &bars, sm);
-    else if (warp == kMmaWarp) mma_role<0>(a, &bars, sm, tmem);
-    else if (warp == kMmaWarp + 1) mma_role<1>(a, &bars, sm, tmem);
+    if (warp == kTmaWarp) producer_role<!kExtra>(&tm_q, &tm_k, &tm_v, a, &bars, sm);
+    else if (warp == kMmaWarp) mma_role<0, !kExtra>(a, &bars, sm, tmem);
+    else if (warp == kMmaWarp + 1) mma_role<1, !kExtra>(a, &bars, sm, tmem);
   }
 
   // a role that left on a wait that ran out may have tensor-memory loads or stores in flight
@@ -1215,11 +1275,15 @@ cudaError_t launch_attn(const Plan& pl, int sm_count, bool frame_mode, const voi
   const int64_t rows = frame_mode ? pl.L : pl.n_tok;
   const int64_t problems = static_cast<int64_t>(pl.H) * (frame_mode ? pl.n_frames : 1);
   a.item_rows = choose_item_rows(rows, problems, sm_count);
-  a.pairs = static_cast<int32_t>((rows + a.item_rows - 1) / a.item_rows);
-  a.by_pairs = make_divisor(a.pairs);
+  const bool short_last = !(a.use_diag || a.use_mean);
+  const int64_t ragged = rows % a.item_rows != 0 ? 1 : 0;
+  a.pairs = static_cast<int32_t>(rows / a.item_rows + (short_last ? 0 : ragged));
+  a.n_full = static_cast<int32_t>(a.pairs * problems);
+  a.ragged_rows = static_cast<int32_t>(rows % a.item_rows);
+  a.by_pairs = make_divisor(a.pairs > 0 ? a.pairs : 1);
   a.by_heads = make_divisor(pl.H);
   a.rule = make_window_rule(pl);
-  a.n_work = static_cast<int32_t>(a.pairs * problems);
+  a.n_work = static_cast<int32_t>(a.n_full + (short_last ? ragged * problems : 0));
 
   // token-major [n_tok, H*d] maps for Q and, in frame attention, K and V; head-major [H, M, d] maps for Kc, Vc otherwise
   CUtensorMap tm_q, tm_k, tm_v;

@@ -9,6 +9,7 @@ import paper_2512_02541_b200 as P
 from paper_2512_02541_b200 import binding as B
 from paper_2512_02541_b200 import inputs
 
+import test_gpu_frame_attn as frame_attn
 from test_gpu_parity import _check_attn, _host, _run_gpu
 
 pytestmark = pytest.mark.gpu
@@ -49,3 +50,13 @@ def test_layer_call_gives_the_bits_of_its_two_calls(sigma, mean_fill):
     with pytest.raises(B.AvggtError):   # everything is rejected before anything is enqueued
         B.avggt_layer(params, Q, K, V, layer.Kc, layer.Vc, layer.idx, layer.kmean, layer.vmean, O, None, layer.build_ws, 0,
                       layer.attn_ws, layer.attn_ws.numel(), None)
+
+
+# 12 frames x 16 heads, tokens per frame with one tile of rows only, with a full item and a last one of 1, 127, 128, 129 or 255
+# rows, and with key tails of 1, 16, 17 and 111 of a 112-key step: several items per thread block, tile 1 sitting some out
+@pytest.mark.parametrize("L", (100, 113, 257, 383, 384, 385, 511, 240, 223))
+def test_frame_items_with_a_short_last_one(L):
+    wl = inputs.Workload("frame_items", 12, 1, L - 5, 5, 16, 64, 4, 1, 2, "iid")
+    for lse in (False, True):
+        run = frame_attn._run(wl, seed=L, want_lse=lse)
+        frame_attn._check(*run)
