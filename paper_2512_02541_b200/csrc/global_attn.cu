@@ -1064,8 +1064,12 @@ __device__ __forceinline__ void softmax_items(const AttnArgs& a, Barriers* bars,
       if (pending) {
         if (res_rows) {
           if (!softmax_epilogue<kLse, kExtra>(a, bars, me, res, item - gridDim.x, stop - chunk - 1)) return;
-        } else if (me.lane == 0 && n_kv > 0) {
-          mbar_arrive(smem_u32(&bars->o_free[t]));
+        } else if (n_kv > 0) {
+          // Not before the item's last P V: a warp without rows could otherwise be an item ahead and arrive a second time in
+          // the phase in which another warp has not yet read O.
+          const int last = stop - chunk - 1;
+          if (!wait_bar(&bars->o_done[t][last & 1], (last >> 1) & 1, bars, a, 51, last)) return;
+          if (me.lane == 0) mbar_arrive(smem_u32(&bars->o_free[t]));
         }
         pending = false;
       } else if (left > 0 && rows && !flush_row_sums(me, gj - 1, bars, a)) {

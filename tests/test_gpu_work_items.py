@@ -60,3 +60,11 @@ def test_frame_items_with_a_short_last_one(L):
     for lse in (False, True):
         run = frame_attn._run(wl, seed=L, want_lse=lse)
         frame_attn._check(*run)
+
+
+def test_layer_items_of_two_steps():
+    """121 keys, 160 items on a GPU of fewer SMs: a warp without rows must not run an item ahead of the others."""
+    wl = inputs.Workload("two_steps", 1, 33, 33, 0, 32, 64, 9, 1, 2, "iid")
+    for seed in range(3):
+        _, ocfg, _, Q, K, V, O = _run_gpu(wl, seed=seed)
+        _check_attn(ocfg, Q, _host(K), _host(V), O)
