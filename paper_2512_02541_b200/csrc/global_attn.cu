@@ -110,7 +110,8 @@ struct AttnArgs {
   int32_t last_tile_keys;   // keys of a ragged last tile, else 0
   int32_t n_work;       // work items (pairs of query tiles x heads x problems) of the launch; a CTA takes the items
                         // blockIdx.x, blockIdx.x + gridDim.x, ...
-  int32_t item_rows;    // query rows of a work item: 256 (two full tiles), or 128 or 64 spread over both tiles
+  int32_t item_rows;    // query rows of a work item: 256 (two full tiles), or fewer, spread over both tiles
+  int32_t split_rows[2], split_lanes[2];   // rows of tile 0 and lanes left free in tile 1: of a work item, of a ragged one
   int32_t pairs;        // work items of one problem and head (kShortLast: the full ones)
   int32_t n_full, ragged_rows;   // kShortLast: pairs x heads x problems; query rows of the items after them
   int32_t use_diag;     // diag on and |D| > 0
@@ -193,6 +194,7 @@ struct WorkItem {
   int key_row0;   // frame attention: token index of the frame's first key
   int row0;       // first query row (token index)
   int64_t end;    // one past the item's last query row
+  int split;      // 0: item of item_rows rows, 1: ragged one
 };
 // One of its query tiles.
 struct QueryTile {
@@ -223,28 +225,21 @@ __device__ __forceinline__ WorkItem work_item(const AttnArgs& a, uint32_t item) 
   w.row0 = w.key_row0 + static_cast<int>(qp) * a.item_rows;
   const int64_t end = a.frame_mode ? static_cast<int64_t>(w.key_row0) + a.pl.L : a.pl.n_tok;
   w.end = end - w.row0 > a.item_rows ? static_cast<int64_t>(w.row0) + a.item_rows : end;
+  w.split = kShortLast ? (item >= static_cast<uint32_t>(a.n_full) ? 1 : 0) : (end - w.row0 < a.item_rows ? 1 : 0);
   return w;
 }
 
-// An item with rows for one tile only is cut in two halves by groups of 16 rows (one softmax warp), the second
-// half in the upper lanes of its tile: every scheduler then has two warps with work at most, and both tiles' products
-// overlap.  Warps without rows compute nothing.
+// An item of fewer than 256 rows is cut in two halves by groups of 16 rows (one softmax warp), the second half in the upper lanes
+// of its tile: the warps with work are spread over the four schedulers, and both tiles' products overlap.  Warps without rows
+// compute nothing.
 //
-// kShortLast: tile 0 takes all the rows and tile 1 sits the item out, products and all.  (The subsampled layer meets such an
-// item once per head, or is so small that nothing but latency counts; there the halves are as good and the code simpler.)
-template <bool kShortLast>
-__device__ __forceinline__ QueryTile query_tile(const WorkItem& w, int t) {
+// kShortLast: a last item of one tile is left to tile 0, and tile 1 sits it out, products and all.  (The subsampled layer meets
+// such an item once per head, or is so small that nothing but latency counts; there the halves are as good and the code simpler.)
+__device__ __forceinline__ QueryTile query_tile(const AttnArgs& a, const WorkItem& w, int t) {
   QueryTile q;
-  if (kShortLast) {
-    q.q0 = q.first = w.row0 + t * kTileQ;
-    q.last = t == 0 && w.end - w.row0 > kTileQ ? static_cast<int64_t>(w.row0) + kTileQ : w.end;
-    return q;
-  }
-  const bool two = w.end - w.row0 > kTileQ;
-  const int groups = two ? 16 : static_cast<int>(w.end - w.row0 + 15) >> 4;
-  const int cut = w.row0 + 16 * ((groups + 1) >> 1);   // first row of tile 1
+  const int cut = w.row0 + a.split_rows[w.split];   // first row of tile 1
   q.first = t == 0 ? w.row0 : cut;
-  q.q0 = t == 0 ? w.row0 : (two ? cut : cut - kTileQ / 2);
+  q.q0 = t == 0 ? w.row0 : cut - a.split_lanes[w.split];
   q.last = t == 0 && cut < w.end ? cut : w.end;
   return q;
 }
@@ -307,7 +302,7 @@ __device__ __forceinline__ void producer_role(const CUtensorMap* tm_q, const CUt
       mbar_arrive_expect_tx(qb, kQTiles * kTileBytes);
 #pragma unroll
       for (int t = 0; t < kQTiles; ++t)
-        tma_load_2d(smem_u32(sm.q + (place * kQTiles + t) * kTileBytes), tm_q, head * kHeadDim, query_tile<kShortLast>(wi, t).q0, qb);
+        tma_load_2d(smem_u32(sm.q + (place * kQTiles + t) * kTileBytes), tm_q, head * kHeadDim, query_tile(a, wi, t).q0, qb);
     }
     __syncwarp();
     ++q_issued;
@@ -845,7 +840,7 @@ __device__ __forceinline__ bool softmax_epilogue(const AttnArgs& a, Barriers* ba
                                                  uint32_t item, int last) {
   const Plan& pl = a.pl;
   const WorkItem wi = work_item<!kExtra>(a, item);
-  const QueryTile tile = query_tile<!kExtra>(wi, me.t);
+  const QueryTile tile = query_tile(a, wi, me.t);
   const int t = me.t, head = wi.head;
   const int i = me.lane & 3;                             // position in the quad
   const int r0 = 32 * me.q + 16 * me.h + (me.lane >> 2);   // the thread's two rows within the tile: r0, r0 + 8
@@ -1025,7 +1020,7 @@ __device__ __forceinline__ void softmax_items(const AttnArgs& a, Barriers* bars,
     bool rows = false;
     if (have) {
       const WorkItem wi = work_item<!kExtra>(a, item);
-      const QueryTile tile = query_tile<!kExtra>(wi, t);
+      const QueryTile tile = query_tile(a, wi, t);
       const int row0 = tile.q0 + 32 * me.q + 16 * me.h;   // the warp's first row
       rows = row0 + 16 > tile.first && row0 < tile.last;
       if (kExtra && a.use_diag) {   // each thread asks for one line: K of row lane / 2, or V
@@ -1240,11 +1235,29 @@ cudaError_t prepare_kernels() {
   return cudaSuccess;
 }
 
-// Query rows of a work item.  Half items leave half of a tile's products idle and cost 0.6 of a full one at best (a lone wave
-// of 13 key steps: 32.8 us in two rounds against 23.7 us in one), so they pay only where the chip has room for all of them at
-// once (1,044 queries x 532 keys x 16 heads, 80 items or 144: 18.3 against 16.2 us).
-int choose_item_rows(int64_t rows, int64_t problems, int sm_count) {
-  return (rows + kTileQ - 1) / kTileQ * problems <= sm_count ? kTileQ : kQTiles * kTileQ;
+// Query rows of a work item: 256, or, in a launch of one or two rounds of the chip, 160, 144 or 128 where that ends sooner
+// by this measure: an item of r <= 160 rows takes 0.68 + 0.32 r / 256 of a full one's time (measured at 128: 0.84; the key steps
+// are a chain; between 160 and 256 some scheduler has four warps with work again), and the ragged last items of a kShortLast launch fill up the last round of the others.  2,748 queries x 732 keys
+// x 16 heads, 176 items of 256 rows or 288 of 160: 28.5 against 25.6 us; frame attention of two frames of 1,374 tokens 35.8
+// against 31.9.  Longer launches keep 256: there the gain is small, and rows that do not exist cost power.
+int choose_item_rows(int64_t rows, int64_t problems, int sm_count, bool short_last) {
+  const auto rounds = [&](int64_t items) { return (items + sm_count - 1) / sm_count; };
+  const auto cost = [](int64_t r) { return 0.68 + 0.32 * static_cast<double>(r) / (kQTiles * kTileQ); };
+  const auto end = [&](int r) {
+    if (!short_last) return static_cast<double>(rounds((rows + r - 1) / r * problems)) * cost(r);
+    const int64_t full = rows / r * problems, last = rows % r != 0 ? problems : 0;
+    const int64_t idle = rounds(full) * sm_count - full;
+    return static_cast<double>(rounds(full)) * cost(r) + (last > idle ? static_cast<double>(rounds(last - idle)) * cost(rows % r) : 0.0);
+  };
+  int best = kQTiles * kTileQ;
+  if (rounds((rows + best - 1) / best * problems) > 2) return best;
+  double least = 0.97 * end(best);   // (not for next to nothing)
+  for (int r = 160; r >= kTileQ; r -= 16)
+    if (end(r) < least) {
+      least = end(r);
+      best = r;
+    }
+  return best;
 }
 
 // Tensor maps and launch shared by the two entry points.  frame_mode: see AttnArgs.
@@ -1278,9 +1291,15 @@ cudaError_t launch_attn(const Plan& pl, int sm_count, bool frame_mode, const voi
   a.poly_range = (kRescaleThreshold - kPolyLowest) * a.inv_scale_log2;
   const int64_t rows = frame_mode ? pl.L : pl.n_tok;
   const int64_t problems = static_cast<int64_t>(pl.H) * (frame_mode ? pl.n_frames : 1);
-  a.item_rows = choose_item_rows(rows, problems, sm_count);
   const bool short_last = !(a.use_diag || a.use_mean);
+  a.item_rows = choose_item_rows(rows, problems, sm_count, short_last);
   const int64_t ragged = rows % a.item_rows != 0 ? 1 : 0;
+  for (int i = 0; i < 2; ++i) {
+    const int n = static_cast<int>(i == 0 || !ragged ? a.item_rows : rows % a.item_rows);
+    const int groups = (n + 15) / 16, groups0 = short_last && n <= kTileQ ? groups : (groups + 1) / 2;
+    a.split_rows[i] = 16 * groups0;
+    a.split_lanes[i] = kTileQ - 16 * (groups - groups0);
+  }
   a.pairs = static_cast<int32_t>(rows / a.item_rows + (short_last ? 0 : ragged));
   a.n_full = static_cast<int32_t>(a.pairs * problems);
   a.ragged_rows = static_cast<int32_t>(rows % a.item_rows);

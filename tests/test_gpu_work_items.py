@@ -15,9 +15,10 @@ from test_gpu_parity import _check_attn, _host, _run_gpu
 pytestmark = pytest.mark.gpu
 
 
-# 32 heads: 7 or more half items per head do not fit the chip at once, so the items are full ones and some thread blocks have
-# two; the last item has 1, 16, 17, 128, 129 or 255 rows.  4 heads: half items.
-@pytest.mark.parametrize("heads,n_tok", [(32, 768 + r) for r in (1, 16, 17, 128, 129, 255)] + [(4, r) for r in (6, 64, 65, 129, 300)])
+# 32 heads: 769 to 1,023 queries make one round of 256-row items, 1,281 two rounds of 160- or 144-row ones, 2,305 three rounds (several
+# items per thread block); the last item has 1, 16, 17, 128, 129 or 255 rows of 256.  4 heads: 128-row items.
+@pytest.mark.parametrize("heads,n_tok", [(32, 768 + r) for r in (1, 16, 17, 128, 129, 255)] + [(32, 1280 + r) for r in (0, 1, 129, 160)]
+                         + [(32, 2304 + r) for r in (1, 129)] + [(4, r) for r in (6, 64, 65, 129, 300)])
 @pytest.mark.parametrize("sigma,lse", [(1, False), (2, True)])
 def test_rows_of_the_last_item(heads, n_tok, sigma, lse):
     wl = inputs.Workload("items", 1, 1, n_tok - 5, 5, heads, 64, sigma, 1, 2, "iid")
