@@ -115,8 +115,8 @@ int avggt_workspace_bytes(const avggt_params* p, size_t* build_ws_bytes, size_t*
  *   kmean, vmean  device, float [H, d]           written when mean_fill != 0 and |D| > 0
  *                                                (zero-filled when |D| == 0); may be NULL when
  *                                                mean_fill == 0
- *   ws      device scratch of at least build_ws_bytes; holds per-block partial sums and is
- *           fully rewritten by each call, so it needs no initialisation.  The reduction order is
+ *   ws      device scratch of at least build_ws_bytes; holds per-block partial sums (of a few
+ *           thousand tokens at most: nothing) and needs no initialisation.  The reduction order is
  *           fixed: results are identical from run to run.
  */
 int avggt_build_kv(const avggt_params* p, const void* K, const void* V,

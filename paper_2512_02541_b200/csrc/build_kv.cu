@@ -21,6 +21,10 @@ namespace {
 
 constexpr int kBuildThreads = 256;
 constexpr int kBuildWarps = kBuildThreads / 32;
+// Blocks of build_kv_kernel<PASSES> that an SM holds (by its registers), and as many as the grid has per SM: a second wave of
+// blocks would only double the partial sums (592 blocks instead of 296 on 148 SMs: 16.2 instead of 13.5 us at 8 frames,
+// 30.8 instead of 27.7 at 24; no difference at 333).
+constexpr int kBuildBlocks[9] = {0, 5, 3, 2, 2, 1, 1, 1, 1};
 
 __device__ __forceinline__ uint4 ld_stream(const uint4* p) {
   uint4 v;
@@ -125,6 +129,105 @@ build_kv_kernel(const Plan pl, const uint4* __restrict__ K, const uint4* __restr
     }
     __syncthreads();
   }
+}
+
+// The same for few tokens, in one launch: a cluster of thread blocks takes one head of K or of V, each block every
+// cluster-size-th group of 128 rows, and adds the blocks' sums up through distributed shared memory.  No partial sums in
+// global memory (for a few frames as many bytes as K and V themselves) and no second kernel.  A row's 128 bytes of the
+// head are read by 8 threads, 16 bytes each, four rows in flight per thread.
+constexpr int kSmallThreads = 1024;
+constexpr int kSmallRows = kSmallThreads / 8;   // rows a block reads at once
+
+// Up to so many tokens per block of a cluster.  Above, the bytes are the bound, which more blocks per SM and warps that read
+// whole rows serve better.  The two kernels' times in us, this one first (148 SMs): 16 heads, clusters of 4, limit 5,760:
+// 4.5 and 6.2 at 1,374 tokens, 7.9 and 10.4 at 4,122, 10.3 and 12.0 at 5,496, 16.2 and 14.1 at 8,244.  6 heads, clusters of 8,
+// limit 11,520: 4.2 and 4.9 at 1,374, 6.0 and 8.8 at 5,496, 9.1 and 11.3 at 10,992, 19.8 and 17.9 at 21,984.  24 heads, clusters
+// of 2, limit 2,880: 5.9 and 8.6 at 1,374.  Of 261 tokens and up to 8 heads it is 0.4 us slower (3.7 and 3.3) and saves
+// the host a launch.
+constexpr int64_t kSmallTokensPerBlock = 1440;
+
+struct SmallArgs {
+  Plan pl;
+  WindowRule rule;
+  const uint4* K;
+  const uint4* V;
+  uint4* Kc;
+  uint4* Vc;
+  int64_t kc_rows;
+  int32_t* idx;
+  const int32_t* slot_of_token;
+  float* kmean;        // null: no mean pair
+  float* vmean;
+  float scale;         // 1 / number of dropped rows, or 1 for the sums; 0: zero-fill
+  uint32_t* status;
+};
+
+__global__ void __launch_bounds__(kSmallThreads)
+build_kv_small_kernel(const SmallArgs a) {
+  __shared__ float red[kSmallThreads / 32][64];
+  __shared__ float part[64];   // this block's sums, read by the cluster's first block
+  const Plan& pl = a.pl;
+  const uint32_t rank = cluster_cta_rank(), n_ranks = cluster_size();
+  const int which_head = blockIdx.x / n_ranks;
+  const int which = which_head >= pl.H ? 1 : 0, head = which_head - which * pl.H;
+  const uint32_t c = threadIdx.x & 7u;
+  const uint4* src = (which == 0 ? a.K : a.V) + head * 8 + c;
+  uint4* dst = (which == 0 ? a.Kc : a.Vc) + static_cast<size_t>(head) * static_cast<size_t>(a.kc_rows) * 8u + c;
+  const uint32_t chunks_per_row = static_cast<uint32_t>(pl.H) * 8u, n_tok = static_cast<uint32_t>(pl.n_tok);
+  const bool add = a.kmean != nullptr && a.scale != 0.f;
+  float acc[8];
+#pragma unroll
+  for (int e = 0; e < 8; ++e) acc[e] = 0.f;
+
+  grid_dependency_wait();
+  if (blockIdx.x == 0 && a.status != nullptr && threadIdx.x < kAttnStatusBytes / 4) a.status[threadIdx.x] = 0u;
+  constexpr int kInFlight = 4;
+  for (uint32_t row0 = rank * kSmallRows + (threadIdx.x >> 3); row0 < n_tok; row0 += kInFlight * n_ranks * kSmallRows) {
+    uint4 v[kInFlight];
+    int32_t m[kInFlight];
+#pragma unroll
+    for (int i = 0; i < kInFlight; ++i) {
+      const uint32_t row = row0 + i * n_ranks * kSmallRows;
+      v[i] = make_uint4(0u, 0u, 0u, 0u);   // beyond the last row: adds nothing
+      m[i] = -1;
+      if (row < n_tok) {
+        m[i] = a.slot_of_token != nullptr ? a.slot_of_token[row] : compact_position(a.rule, pl, row);
+        if (m[i] >= 0 || add) v[i] = ld_stream(src + static_cast<size_t>(row) * chunks_per_row);
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < kInFlight; ++i) {
+      if (m[i] >= 0) {
+        dst[static_cast<size_t>(m[i]) * 8u] = v[i];
+        if (which_head == 0 && c == 0 && a.idx != nullptr) a.idx[m[i]] = static_cast<int32_t>(row0 + i * n_ranks * kSmallRows);
+      } else {
+        add_bf16x8(acc, v[i]);
+      }
+    }
+  }
+  grid_launch_dependents();
+  if (a.kmean == nullptr) return;   // the same for every block of the launch
+  // the warp's four rows, then the block's 32 warps, then the cluster's blocks, in a fixed order
+#pragma unroll
+  for (int e = 0; e < 8; ++e) {
+    acc[e] += __shfl_xor_sync(0xffffffffu, acc[e], 8);
+    acc[e] += __shfl_xor_sync(0xffffffffu, acc[e], 16);
+    if ((threadIdx.x & 31) < 8) red[threadIdx.x >> 5][8 * c + e] = acc[e];
+  }
+  __syncthreads();
+  if (threadIdx.x < 64) {
+    float s = 0.f;
+#pragma unroll
+    for (int w = 0; w < kSmallThreads / 32; ++w) s += red[w][threadIdx.x];
+    part[threadIdx.x] = s;
+  }
+  cluster_sync();
+  if (rank == 0 && threadIdx.x < 64) {
+    float s = 0.f;
+    for (uint32_t r = 0; r < n_ranks; ++r) s += ld_cluster_f32(cluster_addr(smem_u32(&part[threadIdx.x]), r));
+    (which == 0 ? a.kmean : a.vmean)[head * 64 + threadIdx.x] = s * a.scale;
+  }
+  cluster_sync();   // no block leaves while another may read its sums
 }
 
 // out[col] = (sum over blocks of partials[b][col]) / n_dropped, col in [0, 2*cols)
@@ -240,9 +343,21 @@ cudaError_t launch_assemble_shards(const void* gathered, int n_ranks, const int6
   return cudaSuccess;
 }
 
+// Blocks per cluster of the few-token kernel: as many as leave one block per SM, up to 8; clusters of 8 find a place on at most
+// three quarters of the SMs at once (8 heads, 16 clusters of 8: 7.6 us at 1,374 tokens, in two waves).
+int small_ranks(const Plan& pl, int sm_count) {
+  int ranks = 8;
+  while (ranks > 1 && 2 * pl.H * ranks > (ranks == 8 ? sm_count * 3 / 4 : sm_count)) ranks /= 2;
+  return ranks;
+}
+
+int build_passes(const Plan& pl) { return (pl.H * 8 + 31) / 32; }
+
+int build_kv_blocks_per_sm(const Plan& pl) { return kBuildBlocks[build_passes(pl)]; }
+
 int build_kv_grid(const Plan& pl, int sm_count) {
   const int64_t by_rows = (pl.n_tok + kBuildWarps - 1) / kBuildWarps;
-  int64_t g = static_cast<int64_t>(sm_count) * 4;
+  int64_t g = static_cast<int64_t>(sm_count) * build_kv_blocks_per_sm(pl);
   if (g > by_rows) g = by_rows;
   if (g < 1) g = 1;
   return static_cast<int>(g);
@@ -266,6 +381,24 @@ cudaError_t launch_build_kv(const Plan& pl, int sm_count, const void* K, const v
     if (e0 != cudaSuccess) return e0;
     idx = nullptr;
   }
+  const int ranks = small_ranks(pl, sm_count);
+  if (pl.n_tok <= ranks * kSmallTokensPerBlock) {
+    SmallArgs a;
+    a.pl = pl;
+    a.rule = make_window_rule(pl);
+    a.K = static_cast<const uint4*>(K);
+    a.V = static_cast<const uint4*>(V);
+    a.Kc = static_cast<uint4*>(Kc);
+    a.Vc = static_cast<uint4*>(Vc);
+    a.kc_rows = kc_rows;
+    a.idx = idx;
+    a.slot_of_token = slot_of_token;
+    a.kmean = pl.mean_fill != 0 ? kmean : nullptr;
+    a.vmean = vmean;
+    a.scale = pl.n_dropped <= 0 ? 0.f : sums_only ? 1.0f : 1.0f / static_cast<float>(pl.n_dropped);
+    a.status = static_cast<uint32_t*>(clear_status);
+    return launch_dependent_cluster(build_kv_small_kernel, 2 * pl.H * ranks, ranks, kSmallThreads, 0, st, a);
+  }
   const int grid = build_kv_grid(pl, sm_count);
   const int do_mean = (pl.mean_fill != 0 && pl.n_dropped > 0) ? 1 : 0;
   float* partials = static_cast<float*>(ws);
@@ -273,7 +406,7 @@ cudaError_t launch_build_kv(const Plan& pl, int sm_count, const void* K, const v
   const bool zero_mean = pl.mean_fill != 0 && !do_mean;
   float* zk = zero_mean ? kmean : nullptr;
   float* zv = zero_mean ? vmean : nullptr;
-  const int passes = (pl.H * 8 + 31) / 32;
+  const int passes = build_passes(pl);
   cudaError_t e;
   switch (passes) {
     case 1: e = launch_build<1>(pl, grid, K, V, Kc, Vc, kc_rows, idx, partials, do_mean, slot_of_token, status, zk, zv, st); break;

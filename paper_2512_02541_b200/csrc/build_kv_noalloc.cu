@@ -20,7 +20,7 @@ namespace {
 
 // Capacity: partial rows of 2 * H * d floats, one per thread block of the compaction kernel.
 constexpr int kStaticMaxCols2 = 2 * 16 * 64;   // H * d <= 1024
-constexpr int kStaticMaxBlocks = 296;          // four blocks per SM on up to 74 SMs' worth of grid (see the entry point)
+constexpr int kStaticMaxBlocks = 296;          // two blocks on each of 148 SMs at 16 heads (see the entry point)
 constexpr size_t kStaticScratchBytes = static_cast<size_t>(kStaticMaxBlocks) * kStaticMaxCols2 * sizeof(float);
 
 // In host code this name is only a handle for the runtime's symbol lookup, not a device
@@ -84,10 +84,11 @@ extern "C" int avggt_build_kv_noalloc(const avggt_params* p, const void* K, cons
   PerDevice* pd = nullptr;
   rc = setup_current_device(&pd);
   if (rc != AVGGT_OK) return rc;
-  // The compaction kernel runs four blocks per SM it is told about; telling it about fewer SMs
+  // The compaction kernel runs a fixed number of blocks per SM it is told about; telling it about fewer SMs
   // keeps its partial rows within the fixed array.
   int sm_eff = di.sm_count;
-  if (sm_eff > kStaticMaxBlocks / 4) sm_eff = kStaticMaxBlocks / 4;
+  const int most = kStaticMaxBlocks / build_kv_blocks_per_sm(pl);
+  if (sm_eff > most) sm_eff = most;
   if (build_kv_ws_bytes(pl, sm_eff) > kStaticScratchBytes) return AVGGT_ERR_STATIC_SCRATCH;
   return record_cuda(launch_build_kv(pl, sm_eff, K, V, Kc, Vc, idx, kmean, vmean, pd->scratch,
                                      static_cast<cudaStream_t>(cuda_stream)));

@@ -20,19 +20,29 @@ int record_message(const char* text);
 
 // Launch of a kernel that may be scheduled, up to its grid_dependency_wait, while the kernel before it in the stream ends:
 // the launch and the preparation of the layer's kernels (tensor memory, barriers) hide behind one another.
+// cluster: thread blocks per cluster.
 template <typename... P, typename... A>
-cudaError_t launch_dependent(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t st, const A&... args) {
-  cudaLaunchAttribute attr;
-  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr.val.programmaticStreamSerializationAllowed = 1;
+cudaError_t launch_dependent_cluster(void (*kernel)(P...), unsigned grid, unsigned cluster, unsigned block, size_t smem, cudaStream_t st,
+                                     const A&... args) {
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = cluster;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
   cfg.blockDim = dim3(block);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  cfg.attrs = &attr;
-  cfg.numAttrs = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = cluster > 1 ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+template <typename... P, typename... A>
+cudaError_t launch_dependent(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t st, const A&... args) {
+  return launch_dependent_cluster(kernel, grid, 1, block, smem, st, args...);
 }
 
 constexpr size_t kAttnStatusBytes = 256;   // status block at the start of the attention workspace
@@ -42,6 +52,7 @@ cudaError_t launch_clear_status(void* status, cudaStream_t st);
 
 // ---- K/V compaction (build_kv.cu)
 int build_kv_grid(const Plan& pl, int sm_count);
+int build_kv_blocks_per_sm(const Plan& pl);
 size_t build_kv_ws_bytes(const Plan& pl, int sm_count);
 // caller_idx / slot_of_token: both null for the window rule of Sec. 4.3; for a caller-chosen retained set,
 // the M retained token indices (device) and the [n_tok] map the call fills (device).

@@ -202,13 +202,18 @@ __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32
       : "memory");
 }
 
-// ---------------------------------------------------------------- CTA pairs (clusters of two)
+// ---------------------------------------------------------------- clusters, CTA pairs
 __device__ __forceinline__ uint32_t cluster_cta_rank() {
   uint32_t r;
   asm("mov.u32 %0, %cluster_ctarank;" : "=r"(r));
   return r;
 }
-// every thread of both CTAs; what was written before it (barrier initialisation included) is visible to the pair after it
+__device__ __forceinline__ uint32_t cluster_size() {
+  uint32_t n;
+  asm("mov.u32 %0, %cluster_nctaid.x;" : "=r"(n));
+  return n;
+}
+// every thread of the cluster; what was written before it (barrier initialisation included) is visible to all of them after it
 __device__ __forceinline__ void cluster_sync() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
@@ -217,6 +222,11 @@ __device__ __forceinline__ uint32_t cluster_addr(uint32_t saddr, uint32_t rank) 
   uint32_t a;
   asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(saddr), "r"(rank));
   return a;
+}
+__device__ __forceinline__ float ld_cluster_f32(uint32_t cluster_saddr) {
+  float v;
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(cluster_saddr) : "memory");
+  return v;
 }
 // Orders nothing but what the tcgen05 fences order (a releasing arrival waits until the thread's stores to global memory have
 // completed, some 2,000 clocks in the projection's epilogue).
