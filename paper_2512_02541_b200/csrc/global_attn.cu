@@ -92,7 +92,7 @@ constexpr uint32_t kPolyBlocks = AVGGT_POLY_BLOCKS;
 
 struct AttnArgs {
   Plan pl;
-  Divisor by_pairs, by_heads;
+  Divisor by_pairs, by_heads, by_window;
   WindowRule rule;
   const uint4* Q;       // [n_tok, H, d], read by the diagonal and mean terms; K and V by the diagonal term only
   const uint4* K;
@@ -113,7 +113,9 @@ struct AttnArgs {
   int32_t item_rows;    // query rows of a work item: 256 (two full tiles), or fewer, spread over both tiles
   int32_t split_rows[2], split_lanes[2];   // rows of tile 0 and lanes left free in tile 1: of a work item, of a ragged one
   int32_t pairs;        // work items of one problem and head (kShortLast: the full ones)
-  int32_t n_full, ragged_rows;   // kShortLast: pairs x heads x problems; query rows of the items after them
+  int32_t n_problems;   // kShortLast: problems x heads
+  int32_t window;       // kShortLast: so many of them make a window of the numbering (work_item)
+  int32_t ragged_rows;  // kShortLast: query rows of a problem's last item, 0 if it is a full one
   int32_t use_diag;     // diag on and |D| > 0
   int32_t use_mean;     // mean_fill on and |D| > 0
   float scale_log2;     // softmax scale * log2(e)
@@ -203,21 +205,44 @@ struct QueryTile {
   int64_t last;
 };
 
+// Where an item stands in the numbering of kShortLast.
+struct Place {
+  uint32_t problem0;   // first problem (x heads) of the item's window
+  uint32_t n;          // the item's number in the window
+  uint32_t n_full;     // full items of the window; the ragged ones follow
+};
+__device__ __forceinline__ Place place_of(const AttnArgs& a, uint32_t item) {
+  Place p;
+  p.problem0 = divide(item, a.by_window, p.n) * a.window;
+  const uint32_t left = a.n_problems - p.problem0;
+  p.n_full = (left < static_cast<uint32_t>(a.window) ? left : a.window) * a.pairs;
+  return p;
+}
+
 // Items are numbered with the pair of query tiles fastest, then the head, then (frame
 // attention) the frame, so that the CTAs running side by side share one head's keys in L2.  kShortLast (launches without the
-// extra columns, i.e. frame attention, and the dense layer, where it makes no difference): the ragged last items of the problems
-// come after all the full ones, so that every CTA meets some (with six items per frame and head and 148 CTAs every second CTA
-// never met a short one).  With the trimmed last key tile, frame attention of 10 frames 125.3 -> 122.0 us, of 100 frames
-// 1187 -> 1171 us; with tile 1 left out of items of one tile 118.8 and 1139 us (of the same run: 124.4 and 1177 before).  The
-// card is at its power limit there, so it is the products not made that count more than the balance.
+// extra columns, i.e. frame attention, and the dense layer, where it makes no difference): the ragged last items come after the
+// full ones of their window of the numbering (choose_window), so that every CTA meets some (with six items per frame and head and
+// 148 CTAs every second CTA never met a short one).  With the trimmed last key tile and one window, frame attention of 10 frames
+// 125.3 -> 122.0 us, of 100 frames 1187 -> 1171 us; with tile 1 left out of items of one tile 118.8 and 1139 us (of the same
+// run: 124.4 and 1177 before).  The card is at its power limit there, so it is the products not made that count more than
+// the balance.
 template <bool kShortLast>
 __device__ __forceinline__ WorkItem work_item(const AttnArgs& a, uint32_t item) {
   WorkItem w;
   uint32_t qp, head;
-  uint32_t rest = divide(item, a.by_pairs, qp);
-  if (kShortLast && item >= static_cast<uint32_t>(a.n_full)) {
-    rest = item - a.n_full;
-    qp = a.pairs;
+  uint32_t rest;
+  bool ragged = false;
+  if (kShortLast) {
+    const Place p = place_of(a, item);
+    rest = p.problem0 + divide(p.n, a.by_pairs, qp);
+    ragged = p.n >= p.n_full;
+    if (ragged) {
+      rest = p.problem0 + p.n - p.n_full;
+      qp = a.pairs;
+    }
+  } else {
+    rest = divide(item, a.by_pairs, qp);
   }
   const uint32_t frame = divide(rest, a.by_heads, head);
   w.head = static_cast<int>(head);
@@ -225,7 +250,7 @@ __device__ __forceinline__ WorkItem work_item(const AttnArgs& a, uint32_t item) 
   w.row0 = w.key_row0 + static_cast<int>(qp) * a.item_rows;
   const int64_t end = a.frame_mode ? static_cast<int64_t>(w.key_row0) + a.pl.L : a.pl.n_tok;
   w.end = end - w.row0 > a.item_rows ? static_cast<int64_t>(w.row0) + a.item_rows : end;
-  w.split = kShortLast ? (item >= static_cast<uint32_t>(a.n_full) ? 1 : 0) : (end - w.row0 < a.item_rows ? 1 : 0);
+  w.split = kShortLast ? (ragged ? 1 : 0) : (end - w.row0 < a.item_rows ? 1 : 0);
   return w;
 }
 
@@ -264,7 +289,10 @@ __device__ __forceinline__ bool wait_bar_warp(uint64_t* bar, uint32_t parity, Ba
 
 // kShortLast: tile 1 has rows in the item
 __device__ __forceinline__ bool tile_has_rows(const AttnArgs& a, uint32_t item) {
-  return a.item_rows > kTileQ && (item < static_cast<uint32_t>(a.n_full) || a.ragged_rows > kTileQ);
+  if (a.item_rows <= kTileQ) return false;
+  if (a.ragged_rows == 0 || a.ragged_rows > kTileQ) return true;
+  const Place p = place_of(a, item);
+  return p.n < p.n_full;
 }
 
 // ------------------------------------------------------------------ TMA producer (one warp)
@@ -1260,6 +1288,17 @@ int choose_item_rows(int64_t rows, int64_t problems, int sm_count, bool short_la
   return best;
 }
 
+// Frames x heads in a window of frame attention's items (work_item): all, or, where Q, K, V and O are more than L2 holds, as many
+// frames as move 32 MB, so that the ragged items find their frame's keys and values still there.  At 30 frames of 1,374 tokens
+// and 16 heads one window read 426 MB where Q, K and V are 253; 100 frames 1162 -> 1139 us (windows of 24, 48, 64 and 100 MB
+// 1144, 1143, 1147 and 1153; one frame 1146); 10 frames, which fit L2, are no faster.
+int32_t choose_window(const Plan& pl) {
+  const int64_t mb = int64_t(1) << 20, frame_bytes = 4 * static_cast<int64_t>(pl.L) * pl.H * pl.d * 2;
+  if (frame_bytes * pl.n_frames <= 128 * mb) return pl.n_frames * pl.H;
+  const int64_t frames = 32 * mb / frame_bytes;
+  return static_cast<int32_t>(frames > 1 ? frames : 1) * pl.H;
+}
+
 // Tensor maps and launch shared by the two entry points.  frame_mode: see AttnArgs.
 cudaError_t launch_attn(const Plan& pl, int sm_count, bool frame_mode, const void* Q, const void* K, const void* V, const void* Kc,
                         const void* Vc, const float* kmean, const float* vmean, void* O, float* lse, void* ws,
@@ -1301,12 +1340,16 @@ cudaError_t launch_attn(const Plan& pl, int sm_count, bool frame_mode, const voi
     a.split_lanes[i] = kTileQ - 16 * (groups - groups0);
   }
   a.pairs = static_cast<int32_t>(rows / a.item_rows + (short_last ? 0 : ragged));
-  a.n_full = static_cast<int32_t>(a.pairs * problems);
   a.ragged_rows = static_cast<int32_t>(rows % a.item_rows);
   a.by_pairs = make_divisor(a.pairs > 0 ? a.pairs : 1);
   a.by_heads = make_divisor(pl.H);
   a.rule = make_window_rule(pl);
-  a.n_work = static_cast<int32_t>(a.n_full + (short_last ? ragged * problems : 0));
+  a.n_problems = static_cast<int32_t>(problems);
+  a.window = a.n_problems;
+  if (short_last && frame_mode && ragged) a.window = choose_window(pl);
+  const int64_t items = a.pairs + (short_last ? ragged : 0);   // of one problem
+  a.by_window = make_divisor(static_cast<uint32_t>(a.window * items));
+  a.n_work = static_cast<int32_t>(problems * items);
 
   // token-major [n_tok, H*d] maps for Q and, in frame attention, K and V; head-major [H, M, d] maps for Kc, Vc otherwise
   CUtensorMap tm_q, tm_k, tm_v;

@@ -63,6 +63,14 @@ def test_frame_items_with_a_short_last_one(L):
         frame_attn._check(*run)
 
 
+# more bytes than L2 holds, so that the short last items follow the full ones of every two frames (of 16 heads) or of each
+# (of 32): 13 frames, the last of them on its own, and 6
+@pytest.mark.parametrize("n_frames,heads", ((13, 16), (6, 32)))
+def test_frame_items_in_windows(n_frames, heads):
+    wl = inputs.Workload("frame_windows", n_frames, 37, 37, 5, heads, 64, 4, 1, 2, "iid")
+    frame_attn._check(*frame_attn._run(wl, seed=heads))
+
+
 def test_layer_items_of_two_steps():
     """121 keys, 160 items on a GPU of fewer SMs: a warp without rows must not run an item ahead of the others."""
     wl = inputs.Workload("two_steps", 1, 33, 33, 0, 32, 64, 9, 1, 2, "iid")
