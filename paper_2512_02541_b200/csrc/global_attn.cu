@@ -120,7 +120,8 @@ struct AttnArgs {
   int32_t use_mean;     // mean_fill on and |D| > 0
   float scale_log2;     // softmax scale * log2(e)
   float inv_scale_log2;
-  float poly_range;     // raw score units from the polynomial's lowest score (kPolyLowest) to the threshold of a rescale
+  float poly_range;     // raw score units from kLookBelow to the threshold of a rescale
+  float poly_floor;     // the raw score of kPolyFloor
   float log2_count[2];  // log2 weight of the mean column for a retained and for a dropped query (0: unit weight; -inf: absent)
 };
 
@@ -533,7 +534,17 @@ __device__ __forceinline__ void exp2_poly_pair(uint64_t x2, float& p0, float& p1
   p0 = __uint_as_float(__float_as_uint(q0) + (__float_as_uint(t0) << 23));
   p1 = __uint_as_float(__float_as_uint(q1) + (__float_as_uint(t1) << 23));
 }
-constexpr float kPolyLowest = -125.0f;   // scores are raised to this many log2 units below the reference before the polynomial sees them
+// A step looks at its rows (softmax_step) when one of its scores lies more than so many log2 units below the reference, and gives
+// those more than kPolyLowest below a score that comes out of the polynomial as 2^-122.  Above it the polynomial is right, down
+// to -126.5.  The look is decided on raw scores, whose rounding shifts it by up to |m| 2^-20 log2 units at a reference m: less
+// than the one unit between the two for |m| < kLargeReference.  A row with a larger reference looks at every step.
+constexpr float kLookBelow = -125.0f, kPolyLowest = -126.0f;
+constexpr float kLargeReference = 1048576.0f;
+// That score, in log2 units: so far below any reference that it does not matter which, and beyond 2^48, where the polynomial finds
+// r = 0 and takes the exponent from the lowest bits of x: 390 of 512 is -122 (within 2, for the roundings of the raw score,
+// its product with the scale and the reference).  A score raised to the polynomial's range by its raw value, as one would, misses that
+// range for |m| > 2^23, where the raw scores are further apart.
+constexpr float kPolyFloor = -0x1.00030cp80f;
 
 // What a softmax thread knows about itself.  A softmax warp works on 16 query rows of its tile, all columns
 // of a key step: the tensor-memory lanes [32 q + 16 h, 32 q + 16 h + 16) of the tile.  Its tensor-memory
@@ -645,7 +656,7 @@ __device__ __forceinline__ void quad_transpose(uint32_t& w0, uint32_t& w1, uint3
 // Running state of the thread's two rows (the same in all four threads of a quad, except the partial sums).
 struct RowState {
   float neg_m[2];         // minus the reference maximum of the stored exponentials (log2 units); +inf before the first tile
-  float jump_above[2];    // raw score above which the reference has to move; -inf before the first tile
+  float look_above[2];    // raw score above which the reference may have to move; -inf before the first tile
   float l_exact[2];       // this thread's part of the sum of the unrounded 2^(scale_log2 * s - m): log-sum-exp output only
 };
 
@@ -693,8 +704,9 @@ __device__ __forceinline__ void exp_group(const uint32_t (&s)[4 * kBlocks], cons
 // far above its reference (lazy rescale: more than 2^8), so the first group of exponentials is computed against the old
 // references while the maxima are being taken, and the common case ends in one vote: no shuffles, no wait for the previous
 // P V (P has a place of its own in alternate steps).  The other case moves the references (a row decides by its own maximum,
-// so its bits do not depend on its neighbours), rescales O and the row sums, raises the scores that lie below the range of
-// the polynomial, and computes the first group again.
+// so its bits do not depend on its neighbours), rescales O and the row sums, replaces the scores that lie below the range of
+// the polynomial, and computes the first group again.  The vote compares raw scores with a limit that errs towards looking;
+// what to do is then decided in log2 units, where a large reference costs no more than its own rounding.
 // Measured with the tensor core in the loop but without memory traffic, for 2 tiles x 128 keys on one SM: 2270 clocks
 // with the maxima shuffled, the sums taken by the softmax warps and a wait for P V in every step, 1990 without those
 // waits and sums, 1860 with the vote instead of the shuffles, 1740 with the first group ahead of it, 1695 with the range check
@@ -745,21 +757,23 @@ __device__ __forceinline__ bool softmax_step(const SoftmaxThread& me, int gj, in
 #pragma unroll
     for (int b = 0; b < kBlocks; ++b)
       if ((kPoly >> b) & 1) mn[hi] = min3(mn[hi], __uint_as_float(s[4 * b + 2 * hi]), __uint_as_float(s[4 * b + 2 * hi + 1]));
-    look = look || mx[hi] > st.jump_above[hi] || (kPoly != 0 && mn[hi] < st.jump_above[hi] - a.poly_range);
+    look = look || mx[hi] > st.look_above[hi] || (kPoly != 0 && mn[hi] < st.look_above[hi] - a.poly_range);
   }
   if (__any_sync(0xffffffffu, look)) {
     float alpha[2];
     bool jump_any = false;
 #pragma unroll
     for (int hi = 0; hi < 2; ++hi) {
-      const float row_max = quad_max(mx[hi]);
+      const float m = quad_max(mx[hi]) * a.scale_log2;
       alpha[hi] = 1.0f;
-      if (row_max > st.jump_above[hi]) {
-        const float m = row_max * a.scale_log2;
+      if (m > kRescaleThreshold - st.neg_m[hi]) {
         jump_any = jump_any || st.neg_m[hi] != INFINITY;   // nothing to rescale on the first tile
         alpha[hi] = ex2_approx(-m - st.neg_m[hi]);
         st.neg_m[hi] = -m;
-        st.jump_above[hi] = (m + kRescaleThreshold) * a.inv_scale_log2;
+        // less what the roundings on the way to this limit and to the next m can amount to
+        st.look_above[hi] = fabsf(m) < kLargeReference
+                                ? (m + kRescaleThreshold - (fabsf(m) + kRescaleThreshold) * 0x1p-21f) * a.inv_scale_log2
+                                : -INFINITY;
         if (kLse) st.l_exact[hi] *= alpha[hi];
       }
     }
@@ -788,7 +802,8 @@ __device__ __forceinline__ bool softmax_step(const SoftmaxThread& me, int gj, in
     if (kPoly != 0) {
 #pragma unroll
       for (int c = 0; c < 4 * kBlocks; ++c)
-        if ((kPoly >> (c >> 2)) & 1) s[c] = __float_as_uint(fmaxf(__uint_as_float(s[c]), st.jump_above[(c >> 1) & 1] - a.poly_range));
+        if (((kPoly >> (c >> 2)) & 1) && fmaf(__uint_as_float(s[c]), a.scale_log2, st.neg_m[(c >> 1) & 1]) < kPolyLowest)
+          s[c] = __float_as_uint(a.poly_floor);
     }
     if (kAhead) exp_group<0, kMasked, kLse, kPoly>(s, st, scale2, sum_exact2, pk, n_blocks);
   }
@@ -1042,7 +1057,7 @@ __device__ __forceinline__ void softmax_items(const AttnArgs& a, Barriers* bars,
 #pragma unroll
     for (int hi = 0; hi < 2; ++hi) {
       st.neg_m[hi] = INFINITY;
-      st.jump_above[hi] = -INFINITY;
+      st.look_above[hi] = -INFINITY;
       st.l_exact[hi] = 0.f;
     }
     bool rows = false;
@@ -1327,7 +1342,8 @@ cudaError_t launch_attn(const Plan& pl, int sm_count, bool frame_mode, const voi
   a.use_mean = (!frame_mode && pl.mean_fill != 0 && pl.n_dropped > 0) ? 1 : 0;
   a.scale_log2 = pl.scale * kLog2e;
   a.inv_scale_log2 = 1.0f / a.scale_log2;
-  a.poly_range = (kRescaleThreshold - kPolyLowest) * a.inv_scale_log2;
+  a.poly_range = (kRescaleThreshold - kLookBelow) * a.inv_scale_log2;
+  a.poly_floor = kPolyFloor / a.scale_log2;
   const int64_t rows = frame_mode ? pl.L : pl.n_tok;
   const int64_t problems = static_cast<int64_t>(pl.H) * (frame_mode ? pl.n_frames : 1);
   const bool short_last = !(a.use_diag || a.use_mean);
