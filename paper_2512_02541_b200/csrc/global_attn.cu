@@ -77,6 +77,7 @@ constexpr float kRescaleThreshold = 8.0f;   // log2 units
 // seven products of a step (measured 1.8e-3 after 4,086 steps, as large as a bf16 rounding step).  Every so many steps the
 // row sums are therefore moved to the next column, to which P V adds exact zeros; what is left of the error is 2.7e-5.
 constexpr int kFlushSteps = 64;
+static_assert(kFlushSteps > 1, "an item's first step, under which the item before is finished, ends without a flush");
 
 // Blocks of 8 key columns (bit b: columns [8 b, 8 b + 8) of a step) whose exponentials come from a polynomial on the
 // FMA pipe instead of the special-function unit, which at 16 results per clock per SM would otherwise set the pace.
@@ -1075,7 +1076,8 @@ __device__ __forceinline__ void softmax_items(const AttnArgs& a, Barriers* bars,
     int left = active ? n_kv : 0;
 #pragma unroll 1
     do {
-      const int most = pending ? 1 : kFlushSteps;
+      // up to the next multiple of kFlushSteps of the item's own steps, so that a row's sums do not depend on the item's place
+      const int most = pending ? 1 : kFlushSteps - (n_kv - left) % kFlushSteps;
       const int chunk = left < most ? left : most;
       left -= chunk;
       const int stop = gj + chunk;

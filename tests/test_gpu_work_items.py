@@ -7,7 +7,7 @@ import torch
 
 import paper_2512_02541_b200 as P
 from paper_2512_02541_b200 import binding as B
-from paper_2512_02541_b200 import inputs
+from paper_2512_02541_b200 import inputs, sharded
 
 import test_gpu_frame_attn as frame_attn
 from test_gpu_parity import _check_attn, _host, _run_gpu
@@ -77,3 +77,28 @@ def test_layer_items_of_two_steps():
     for seed in range(3):
         _, ocfg, _, Q, K, V, O = _run_gpu(wl, seed=seed)
         _check_attn(ocfg, Q, _host(K), _host(V), O)
+
+
+# 8,244 and 8,784 keys, 74 and 79 steps: past the step after which the row sums move on; several items per thread block, which the
+# groups of the host-buffer path and the shards number differently (an item is the first of its block in one and not in the other)
+@pytest.mark.parametrize("n_frames,sigma,diag,mean_fill", [(6, 1, 0, 0), (24, 4, 1, 2)])
+def test_bits_do_not_depend_on_the_place_of_an_item(n_frames, sigma, diag, mean_fill):
+    wl = inputs.Workload("places", n_frames, 37, 37, 5, 16, 64, sigma, diag, mean_fill, "proj")
+    params, _, layer, Q, K, V, O = _run_gpu(wl, seed=2)
+    hQ, hK, hV = (t.cpu().pin_memory() for t in (Q, K, V))
+    hO = torch.empty_like(hQ).pin_memory()
+    for n_chunks in (1, 3, 6):
+        hO.fill_(float("nan"))
+        layer.forward_host(hQ, hK, hV, hO, n_chunks=n_chunks)
+        layer.check_status()
+        assert torch.equal(hO, O.cpu()), n_chunks
+    L = wl.tokens_per_frame
+    for world in (2, 5):
+        for f0, f1 in (sharded.shard_frames(n_frames, world, r) for r in range(world)):
+            part = P.make_params(f1 - f0, 37, 37, 5, 16, 64, sigma, diag=diag, mean_fill=mean_fill)
+            sl = slice(f0 * L, f1 * L)
+            out = torch.full_like(Q[sl], float("nan"))
+            P.avggt_global_attn_shard(part, layer.M, layer.n_dropped, Q[sl], K[sl], V[sl], layer.Kc, layer.Vc, layer.kmean,
+                                      layer.vmean, out, None, layer.attn_ws, layer.attn_ws.numel())
+            layer.check_status()
+            assert torch.equal(out, O[sl]), (world, f0)
