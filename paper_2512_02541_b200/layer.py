@@ -1,25 +1,33 @@
 """Buffer management around the two library calls (PyTorch is used for device memory and streams only)."""
 
 import threading
+import weakref
 
 import torch
 
 from . import binding as B
 
 
-_upload_streams = {}   # device index -> stream
-_upload_lock = threading.Lock()
+class _Uploads:
+    """The stream on which the host-buffer calls made on one stream copy their inputs, whichever layers they are for.  Their
+    copies are then served in the order of the calls; with a stream per layer the copy engine shared itself out between the
+    inputs of this call and those of calls several places behind it (three layers in rotation, 100 frames: 28.0 ms a call instead of
+    24).  Calls on one stream follow one another there in any case.  Those of another stream have copies of their own,
+    which wait for nothing of this one's."""
 
+    def __init__(self, index):
+        self.stream = torch.cuda.Stream(index)
 
-def _upload_stream(index):
-    """The one stream per device on which the host-buffer calls of all layers copy their inputs.  The copies are then served in
-    the order of the calls; with a stream per layer the copy engine shared itself out between the inputs of this call and
-    those of calls several places behind it (three layers in rotation, 100 frames: 28.0 ms a call instead of 24).  A copy only ever
-    waits for work enqueued before it, so calls from several threads cannot wait for one another in a circle."""
-    with _upload_lock:
-        if index not in _upload_streams:
-            _upload_streams[index] = torch.cuda.Stream(index)
-        return _upload_streams[index]
+    _of_caller = weakref.WeakValueDictionary()   # (device index, caller's stream) -> _Uploads; kept by the layers that use it
+    _lock = threading.Lock()
+
+    @classmethod
+    def of(cls, index, caller):
+        with cls._lock:
+            uploads = cls._of_caller.get((index, caller.cuda_stream))
+            if uploads is None:
+                uploads = cls._of_caller[index, caller.cuda_stream] = cls(index)
+            return uploads
 
 
 def host_groups(n_frames, n_chunks):
@@ -127,9 +135,10 @@ class SubsampledGlobalAttention:
             shape = (self.n_tok, p.n_heads, p.head_dim)
             new = lambda: torch.empty(shape, dtype=torch.bfloat16, device=dev)
             self._host_path = dict(
-                Q=new(), O=new(), K=[new(), new()], V=[new(), new()], h2d=_upload_stream(self._index), d2h=torch.cuda.Stream(dev),
+                Q=new(), O=new(), K=[new(), new()], V=[new(), new()], uploads=None, d2h=torch.cuda.Stream(dev),
                 turn=torch.cuda.Stream(dev),
                 calls=0,
+                uploaded=None,           # the previous call's inputs have arrived
                 kv_free=[[], []],        # per K/V buffer: the call that used it last has finished with it
                 bounds=None,             # frame groups of the previous call
                 q_free=[], o_free=[],    # per group of the previous call: its attention has read Q / its output copy has left O
@@ -138,7 +147,11 @@ class SubsampledGlobalAttention:
         hp = self._host_path
         which = hp["calls"] & 1
         hp["calls"] += 1
-        dQ, dK, dV, dO, h2d, d2h = hp["Q"], hp["K"][which], hp["V"][which], hp["O"], hp["h2d"], hp["d2h"]
+        dQ, dK, dV, dO, d2h = hp["Q"], hp["K"][which], hp["V"][which], hp["O"], hp["d2h"]
+        hp["uploads"] = _Uploads.of(self._index, cur)
+        h2d = hp["uploads"].stream
+        if hp["uploaded"] is not None:
+            h2d.wait_event(hp["uploaded"])     # on another stream, perhaps
         L = p.tokens_per_frame
         n_chunks = max(1, min(n_chunks, p.n_frames))
         bounds = host_groups(p.n_frames, n_chunks)
@@ -165,6 +178,7 @@ class SubsampledGlobalAttention:
                     ev = torch.cuda.Event()
                     ev.record(h2d)
                     q_ready.append(ev)
+            hp["uploaded"] = q_ready[-1]
             cur.wait_event(kv_ready)
             self.build_kv(dK, dV)
             built = torch.cuda.Event()
