@@ -879,6 +879,8 @@ struct RowResults {
 //
 // The queries' own Q, K and V rows are read straight from global memory (at the item's start the warp asked for them to be
 // brought to L2), 16 bytes per thread and half row, and asked for before the first use.
+// By the read-only path: the kernel before this one does not write them, and those before that had ended when this one began (the
+// compaction and clear_status_kernel let it begin after their own wait).
 template <bool kLse, bool kExtra>
 __device__ __forceinline__ bool softmax_epilogue(const AttnArgs& a, Barriers* bars, const SoftmaxThread& me, const RowResults* res,
                                                  uint32_t item, int last) {

@@ -405,7 +405,7 @@ project_kv_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
 
 // kmean[col] = (sum over the CTAs that own col's block, and their four epilogue warps, in a fixed order) / n_dropped
 __global__ void __launch_bounds__(256)
-project_mean_kernel(const float* __restrict__ partials, int grid, int n_col_tiles, int cols_total, float inv_count,
+project_mean_kernel(const float* partials, int grid, int n_col_tiles, int cols_total, float inv_count,
                     float* __restrict__ kmean, float* __restrict__ vmean) {
   grid_launch_dependents();
   grid_dependency_wait();

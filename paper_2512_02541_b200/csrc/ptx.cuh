@@ -32,7 +32,9 @@ __device__ __forceinline__ bool elect_one() {
 
 // Programmatic dependent launch: wait until every kernel before this one in the stream has completed and its writes are
 // visible (returns at once in a kernel launched the ordinary way); let the next kernel of the stream start its own
-// preparation as soon as every block has said so or ended.
+// preparation as soon as every block has said so or ended.  What a kernel before it writes must not be read by the read-only path
+// (ld.global.nc, __ldg, const __restrict__): the read comes after the wait, but the data changed in the reader's lifetime.  A
+// kernel that lets the next one start before its own wait does so for the kernels before itself as well.
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
