@@ -1076,10 +1076,10 @@ __device__ __forceinline__ void softmax_items(const AttnArgs& a, Barriers* bars,
       }
     }
     int left = active ? n_kv : 0;
+    // steps up to the next multiple of kFlushSteps of the item's own, so that a row's sums do not depend on the item's place
+    int most = pending ? 1 : kFlushSteps;
 #pragma unroll 1
     do {
-      // up to the next multiple of kFlushSteps of the item's own steps, so that a row's sums do not depend on the item's place
-      const int most = pending ? 1 : kFlushSteps - (n_kv - left) % kFlushSteps;
       const int chunk = left < most ? left : most;
       left -= chunk;
       const int stop = gj + chunk;
@@ -1114,8 +1114,10 @@ __device__ __forceinline__ void softmax_items(const AttnArgs& a, Barriers* bars,
           if (me.lane == 0) mbar_arrive(smem_u32(&bars->o_free[t]));
         }
         pending = false;
-      } else if (left > 0 && rows && !flush_row_sums(me, gj - 1, bars, a)) {
-        return;
+        most = kFlushSteps - 1;
+      } else {
+        if (left > 0 && rows && !flush_row_sums(me, gj - 1, bars, a)) return;
+        most = kFlushSteps;
       }
     } while (left > 0);
     if (!have) return;
