@@ -19,6 +19,7 @@
 //   warp 1      MMA issuer (even CTA): tcgen05.mma, M 256 x N 256 x K 16, fp32 accumulators in tensor memory;
 //               two accumulators of 256 columns, so the next tile's products run under this
 //               tile's epilogue
+//   warp 2      hands a read accumulator back to the even CTA
 //   warps 4-11  epilogue, one token row and half of the tile's columns per thread: accumulator -> registers, bias, bf16; a head's
 //               64 values of the warp's 32 rows are staged in shared memory (128-byte swizzle),
 //               from where one TMA store writes them to the full K / V array and the retained
@@ -56,7 +57,7 @@ constexpr uint32_t kBytesB = kTileCol / 2 * kBlockK * 2;   // 16 KiB: a CTA's ha
 constexpr uint32_t kStageBytes = 32 * 128;   // epilogue staging: 32 rows x one head (64 bf16), one per epilogue warp
 constexpr int kEpiWarps = 8;        // warps 4..11: warp % 4 is the lane quarter of tensor memory, (warp - 4) / 4 the half of
                                     // the tile's 256 columns (two heads each)
-constexpr int kFirstEpiWarp = 4;    // warps 2 and 3 idle: they complete the first warpgroup, so that registers can be moved
+constexpr int kFirstEpiWarp = 4;    // warp 3 is idle: it completes the first warpgroup, so that registers can be moved
 constexpr int kProjThreads = 32 * (kFirstEpiWarp + kEpiWarps);
 // Registers per thread after the roles have split (an epilogue thread keeps 128 column sums).  The sum over all warps must not
 // exceed what the launch allocated, or setmaxnreg.inc waits for ever: prepare_kernel refuses a build that allocates less.
@@ -90,7 +91,8 @@ struct __align__(8) ProjBarriers {
   uint64_t full[kProjStages];    // even CTA's: both CTAs' copies of the stage have landed
   uint64_t empty[kProjStages];   // either CTA's own: the products have read the stage
   uint64_t acc_full[2];          // either CTA's own: the tile's products have completed
-  uint64_t acc_empty[2];         // even CTA's: the epilogue warps of both CTAs have read the accumulator
+  uint64_t acc_read[2];          // either CTA's own: its epilogue warps have read the accumulator
+  uint64_t acc_empty[2];         // even CTA's: those of both CTAs have (one arrival from each, see warp 2)
   uint64_t mma_idle;             // MMA issuer -> itself: every product it issued has completed
   uint32_t tmem_base;
   uint32_t abort_flag;
@@ -175,7 +177,8 @@ project_kv_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(smem_u32(&bars.acc_full[b]), 1);
-      mbar_init(smem_u32(&bars.acc_empty[b]), 2 * kEpiWarps);
+      mbar_init(smem_u32(&bars.acc_read[b]), kEpiWarps);
+      mbar_init(smem_u32(&bars.acc_empty[b]), 2);
     }
     mbar_init(smem_u32(&bars.mma_idle), 1);
     bars.abort_flag = 0;
@@ -275,6 +278,20 @@ project_kv_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
         __syncwarp();
         (void)proj_wait_warp(&bars.mma_idle, 0, &bars, a, 22, it, false);
       }
+    } else if (warp == 2) {
+      // ------------------------------------------------------------ hands the accumulators back to the even CTA
+      // An arrival on the other CTA's barrier that releases what came before it waits until the thread's stores to global memory have
+      // completed (some 2,000 clocks in the epilogue).  So the epilogue warps arrive on their own CTA's barrier, and this warp, which
+      // stores nothing, passes the arrival on.
+      int it = 0;
+      for (int tt = tok0; tt < a.n_tok_tiles; tt += a.tok_stride, ++it) {
+        const int buf = it & 1;
+        if (!proj_wait_warp(&bars.acc_read[buf], (it >> 1) & 1, &bars, a, 31, it)) break;
+        tc_fence_after();
+        tc_fence_before();
+        if (elect_one()) mbar_arrive_cluster(cluster_addr(smem_u32(&bars.acc_empty[buf]), 0));
+        __syncwarp();
+      }
     }
   } else {
     reg_inc<kRegsEpi>();
@@ -326,7 +343,7 @@ project_kv_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
           tmem_wait_ld();
           if (hh == 1 && half == 1) {   // this warp is done with the accumulator
             tc_fence_before();
-            if (elect_one()) mbar_arrive_cluster(cluster_addr(smem_u32(&bars.acc_empty[buf]), 0));
+            if (elect_one()) mbar_arrive(smem_u32(&bars.acc_read[buf]));
           }
           uint64_t v[16];
 #pragma unroll
@@ -377,7 +394,7 @@ project_kv_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
       }
       if (2 * col_half * 64 + 64 + col_tile * kTileCol >= cols_total) {   // a second head (or both) beyond the last: not reached above
         tc_fence_before();
-        if (elect_one()) mbar_arrive_cluster(cluster_addr(smem_u32(&bars.acc_empty[buf]), 0));
+        if (elect_one()) mbar_arrive(smem_u32(&bars.acc_read[buf]));
       }
     }
     if (lane == 0) bulk_wait<0>();   // the staging tiles stay put until the last store has read them

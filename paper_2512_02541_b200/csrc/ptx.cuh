@@ -230,10 +230,9 @@ __device__ __forceinline__ float ld_cluster_f32(uint32_t cluster_saddr) {
   asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(cluster_saddr) : "memory");
   return v;
 }
-// Orders nothing but what the tcgen05 fences order (a releasing arrival waits until the thread's stores to global memory have
-// completed, some 2,000 clocks in the projection's epilogue).
+// arrival on a barrier of any CTA of the cluster
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_bar) {
-  asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_bar) : "memory");
+  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_bar) : "memory");
 }
 // mbar_try_wait that also acquires what the other CTA released
 __device__ __forceinline__ bool mbar_try_wait_cluster(uint32_t bar, uint32_t parity) {

@@ -97,6 +97,14 @@ def test_vggt_shape_twenty_frames():
     _check(wl, 1024, seed=5)
 
 
+# 27,480 tokens: each pair of thread blocks uses both accumulators three times and more, with few channels, so that the products wait
+# for the epilogue to hand one back; 1, 5 and 6 heads leave epilogue warps without a second head, or without any
+@pytest.mark.parametrize("heads", (1, 5, 6, 16))
+def test_accumulators_handed_back(heads):
+    wl = inputs.WORKLOADS["vggt_n100_s4"].with_(n_frames=20, n_heads=heads, name="handed_back")
+    _check(wl, 64, seed=20 + heads)
+
+
 def test_results_are_deterministic_and_feed_the_attention():
     wl = inputs.Workload("proj_det", 4, 12, 12, 5, 8, 64, 4, 1, 2, "iid")
     params = P.make_params(wl.n_frames, wl.grid_h, wl.grid_w, wl.n_special, wl.n_heads, wl.head_dim, wl.sigma)
