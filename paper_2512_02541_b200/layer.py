@@ -113,7 +113,7 @@ class SubsampledGlobalAttention:
                       self.build_ws.numel(), self.attn_ws, self.attn_ws.numel(), self._stream())
         return out
 
-    def forward_host(self, hQ, hK, hV, hO, n_chunks=8):
+    def forward_host(self, hQ, hK, hV, hO, n_chunks=8, inputs_ready=None):
         """The layer on host buffers (pinned memory), with the copies hidden behind the kernels.
 
         K and V go to the device first (the compaction and the mean need all of them); Q then arrives in
@@ -122,9 +122,14 @@ class SubsampledGlobalAttention:
         every group's output leaves on a second copy stream.  The groups' kernels take turns on the current stream and a
         stream of the layer's own, so that the thread blocks of a group move in as those of the group before run out
         (eight launches in a row on one stream left a tenth of the chip's time unused: 100 frames 28.0 -> 27.2 ms a call,
-        33.3 -> 30.7 ms for a call on its own).  Everything is ordered with events and the call
-        returns without waiting for the device: the current stream waits for the last output copy.  The device
-        copies of K and V alternate between two buffers, so that the K and V of a call made right after this one
+        33.3 -> 30.7 ms for a call on its own).  The call returns without waiting for the device: what it does is ordered
+        with events, and the current stream waits for the last output copy.
+
+        The inputs must be in the host buffers when the call is made: their copies do not wait for the current stream, which
+        is what lets them travel under the call before.  Where something on the device still writes them (an asynchronous copy to the
+        host), pass the event recorded behind it as ``inputs_ready``.  ``hO`` is written after what is on the current stream.
+
+        The device copies of K and V alternate between two buffers, so that the K and V of a call made right after this one
         travel while this one's attention runs; Q and O have one buffer, guarded group by group.  The device
         staging buffers are allocated on first use.
         """
@@ -163,6 +168,8 @@ class SubsampledGlobalAttention:
             h2d.wait_stream(d2h)
         with torch.cuda.device(dev):
             with torch.cuda.stream(h2d):
+                if inputs_ready is not None:
+                    h2d.wait_event(inputs_ready)
                 for ev in hp["kv_free"][which]:
                     h2d.wait_event(ev)
                 dK.copy_(hK, non_blocking=True)

@@ -60,3 +60,21 @@ def test_a_layer_called_on_one_stream_and_then_on_another():
         a.wait_stream(b)
     layer.check_status()
     assert torch.equal(o1, w1) and torch.equal(o2, w2)
+
+
+def test_inputs_that_a_copy_still_writes():
+    """Pinned inputs filled by an asynchronous copy on the calling stream, in a second call (a first one waits for the stream)."""
+    (h1, o1, w1), (h2, _, w2) = _case(5), _case(6)
+    device = [t.cuda() for t in h2]
+    layer = P.SubsampledGlobalAttention(_cfgs(WL)[0])
+    layer.forward_host(*h1, o1)
+    torch.cuda.synchronize()
+    assert torch.equal(o1, w1)
+    torch.cuda._sleep(int(1e8))       # so that the copies below are far from done when the call is made
+    for host, dev in zip(h1, device):
+        host.copy_(dev, non_blocking=True)
+    written = torch.cuda.Event()
+    written.record()
+    layer.forward_host(*h1, o1, inputs_ready=written)
+    layer.check_status()
+    assert torch.equal(o1, w2)
