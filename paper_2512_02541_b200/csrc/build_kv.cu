@@ -21,8 +21,8 @@ namespace {
 
 constexpr int kBuildThreads = 256;
 constexpr int kBuildWarps = kBuildThreads / 32;
-// Blocks of build_kv_kernel<PASSES> that an SM holds (by its registers), and as many as the grid has per SM: a second wave of
-// blocks would only double the partial sums (592 blocks instead of 296 on 148 SMs: 16.2 instead of 13.5 us at 8 frames,
+// Blocks of build_kv_kernel<PASSES> that an SM holds (by its registers; the launch bounds see to it that they fit), and as many as
+// the grid has per SM: a second wave of blocks would only double the partial sums (592 blocks instead of 296 on 148 SMs: 16.2 instead of 13.5 us at 8 frames,
 // 30.8 instead of 27.7 at 24; no difference at 333).
 constexpr int kBuildBlocks[9] = {0, 5, 3, 2, 2, 1, 1, 1, 1};
 
@@ -52,7 +52,7 @@ __device__ __forceinline__ void add_bf16x8(float (&acc)[8], const uint4& v) {
 // kc_rows: rows per head of the compact arrays (M, or more when the caller's arrays are a slot of a
 // larger exchange buffer).
 template <int PASSES>
-__global__ void __launch_bounds__(kBuildThreads)
+__global__ void __launch_bounds__(kBuildThreads, kBuildBlocks[PASSES])
 build_kv_kernel(const Plan pl, const uint4* K, const uint4* V, uint4* __restrict__ Kc,
                 uint4* __restrict__ Vc, const int64_t kc_rows, int32_t* __restrict__ idx, float* __restrict__ partials,
                 const int do_mean, const int32_t* slot_of_token, uint32_t* __restrict__ status,
