@@ -28,3 +28,24 @@ def test_compaction(heads, n_frames, mean_fill, keep_first):
     layer.build_kv(K, V)
     torch.cuda.synchronize()
     _check_build(ocfg, layer, K, V)
+
+
+# both kernels with nothing to average: the mean pair is zero-filled, as the first part of the layer writes it and as a shard's sums
+@pytest.mark.parametrize("n_frames", (3, 30))
+def test_nothing_dropped(n_frames):
+    wl = inputs.Workload("whole", n_frames, 15, 27, 5, 16, 64, 1, 1, 2, "iid")
+    params, ocfg = _cfgs(wl)
+    _, K, V = inputs.make_qkv(wl, seed=1, device="cuda")
+    layer = P.SubsampledGlobalAttention(params)
+    for t in (layer.kmean, layer.vmean):
+        t.fill_(float("nan"))
+    layer.build_kv(K, V)
+    slot_rows = layer.M + 3
+    slot = torch.full((2, wl.n_heads, slot_rows, 64), float("nan"), dtype=torch.bfloat16, device="cuda")
+    sums = torch.full((2, wl.n_heads, 64), float("nan"), device="cuda")
+    P.avggt_build_kv_shard(params, K, V, slot, slot_rows, None, sums, layer.build_ws, layer.build_ws.numel())
+    torch.cuda.synchronize()
+    _check_build(ocfg, layer, K, V)
+    assert not layer.kmean.any() and not layer.vmean.any() and not sums.any()
+    assert torch.equal(slot[0, :, :layer.M], layer.Kc) and torch.equal(slot[1, :, :layer.M], layer.Vc)
+    assert torch.isnan(slot[:, :, layer.M:].float()).all()

@@ -14,8 +14,9 @@ from test_gpu_parity import _cfgs, _check_attn, _host
 pytestmark = pytest.mark.gpu
 
 
-# Q and K scaled by sqrt(magnitude): references of 4e4 log2 units at 1e4 to 4e8 at 1e8, either side of the size (2^20) from which a
-# row looks at every step, and with one ordinary row in sixteen among them
+# Q and K scaled by sqrt(magnitude): scores with a standard deviation of 4e4 log2 units at 1e4 to 4e8 at 1e8, so that the references lie
+# on either side of the size (2^20) from which a row looks at every step; one ordinary row in sixteen among them.  (Sizes at
+# which no row's two largest scores lie within their rounding of each other.)
 @pytest.mark.parametrize("magnitude", (1e4, 1e5, 3e6, 1e7, 1e8))
 @pytest.mark.parametrize("sigma,diag,mean_fill", [(4, 1, 2), (1, 0, 0)])
 @pytest.mark.parametrize("want_lse", (False, True))

@@ -80,7 +80,7 @@ def _check(wl, C, seed, with_bias=True, want_full=True):
 @pytest.mark.parametrize("C", (64, 192, 1024))
 @pytest.mark.parametrize("sigma", (1, 4, 9))
 def test_small_shapes(C, sigma):
-    wl = inputs.Workload("proj", 3, 9, 11, 5, 4, 64, sigma, 1, 2, "iid")          # 312 tokens: tiles 128, 128, 56
+    wl = inputs.Workload("proj", 3, 9, 11, 5, 4, 64, sigma, 1, 2, "iid")          # 312 tokens: tiles of 256 and 56
     _check(wl, C, seed=10 + sigma)
 
 

@@ -78,6 +78,29 @@ def test_shards_reproduce_the_whole_sequence(world, keep_first):
     assert err.max() <= 2e-2 and err.mean() <= 2e-3, (err.max(), err.mean())
 
 
+@pytest.mark.parametrize("keep_first", (False, True))
+def test_shards_of_many_tokens(keep_first):
+    """6 and 5 frames of 1,374 tokens, 16 heads: more than the one-launch compaction takes, so that the sums go through the second
+    kernel, and a slot of the exchange buffer with more rows than the second rank fills.  Compact arrays and means in full,
+    the output on a sample of rows."""
+    wl = inputs.Workload("big_shards", 11, 37, 37, 5, 16, 64, 4, 1, 2, "proj", keep_first_frame=int(keep_first))
+    Q, K, V, O, Kc, Vc, kmean, vmean = _shard_run(wl, 2, keep_first, seed=9)
+    ocfg = orc.SGAConfig(wl.n_frames, wl.grid_h, wl.grid_w, wl.n_special, wl.n_heads, wl.head_dim, wl.sigma,
+                         keep_first_frame=keep_first)
+    Qh, Kh, Vh = (t.float().cpu().numpy() for t in (Q, K, V))
+    Kc_w, Vc_w, _, kmean_w, vmean_w = orc.build_kv(ocfg, Kh, Vh)
+    np.testing.assert_array_equal(Kc.float().cpu().numpy().transpose(1, 0, 2), Kc_w)
+    np.testing.assert_array_equal(Vc.float().cpu().numpy().transpose(1, 0, 2), Vc_w)
+    for got_m, want_m, src in ((kmean, kmean_w, Kh), (vmean, vmean_w, Vh)):
+        assert np.abs(got_m.cpu().numpy().astype(np.float64) - want_m).max() <= 1e-5 * float(np.abs(src).mean())
+    rows = inputs.sample_rows(wl, 300).numpy()
+    want = orc.global_attn_blocked(ocfg, Qh, Kh, Vh, rows)
+    got = O[torch.as_tensor(rows, device=O.device)].float().cpu().numpy().astype(np.float64)
+    assert torch.isfinite(O.float()).all()
+    err = np.abs(got - want)
+    assert err.max() <= 2e-2 and err.mean() <= 2e-3, (err.max(), err.mean())
+
+
 def test_class_with_a_one_rank_group():
     """FrameShardedAttention end to end with a process group of one rank (NCCL on this GPU)."""
     with socket.socket() as s:

@@ -3,7 +3,7 @@
 Every device-side wait of the kernel is bounded: when one runs out, the thread block records
 (code, block, site, iteration) in the workspace's status block, raises a block-wide abort flag,
 lets its roles leave in order (copies in flight land, issued tensor-core work completes, tensor
-memory is freed) and the blocks that start later leave at once; `avggt_check_status` then returns
+memory is freed) and the other blocks begin no further work item; `avggt_check_status` then returns
 AVGGT_ERR_DEVICE_TIMEOUT.  A second build of the same sources (`libavggt_waittest.so`: a 0.5 ms
 limit, and the first thread block's producer leaves out one K tile, i.e. a flag that nothing
 sets) makes such a wait run out.  The product library does not contain that switch.
@@ -41,8 +41,8 @@ def _forward(L, params, Q, K, V, layer, O):
 
 
 def test_a_wait_that_runs_out_is_reported_and_the_context_stays_usable():
-    # 100 frames of 261 tokens, 16 heads: 1632 thread blocks of 104 key tiles each, about eleven waves of ~0.15 ms,
-    # so that the first block's wait (0.5 ms) runs out while most blocks have not started yet
+    # 100 frames of 261 tokens, 16 heads: 1632 work items of 119 key steps each, eleven or twelve of about 0.12 ms for each of
+    # 148 thread blocks, so that the first block's wait (0.5 ms) runs out while the others have most of theirs before them
     wl = inputs.Workload("wait_limit", 100, 16, 16, 5, 16, 64, 2, 1, 2, "iid")
     params = P.make_params(wl.n_frames, wl.grid_h, wl.grid_w, wl.n_special, wl.n_heads, wl.head_dim, wl.sigma,
                            diag=wl.diag, mean_fill=wl.mean_fill)
@@ -59,7 +59,7 @@ def test_a_wait_that_runs_out_is_reported_and_the_context_stays_usable():
     # on a ring stage that is never released (sites 10, 11), an MMA issuer on the tile itself (24, 25) or a
     # softmax warp on the scores of step 1 (40, 41); all within the first cycle of the four-stage ring
     assert site in (10, 11, 24, 25, 40, 41) and iteration <= 5
-    # the blocks of the last head start after the time-out and leave at once: their rows were never written
+    # the items of the last head were not begun: the blocks had seen the time-out by then
     assert torch.isnan(O[:, wl.n_heads - 1].float()).any()
 
     # the same workspace and buffers through the product library right afterwards: correct output

@@ -2,6 +2,7 @@
 item whose rows are spread over both tiles, several items per thread block, key counts around the 112-key step; and the
 one-call layer against its two calls."""
 
+import numpy as np
 import pytest
 import torch
 
@@ -10,13 +11,15 @@ from paper_2512_02541_b200 import binding as B
 from paper_2512_02541_b200 import inputs, sharded
 
 import test_gpu_frame_attn as frame_attn
+import test_gpu_indexed as indexed
 from test_gpu_parity import _check_attn, _host, _run_gpu
 
 pytestmark = pytest.mark.gpu
 
 
 # 32 heads: 769 to 1,023 queries make one round of 256-row items, 1,281 two rounds of 160- or 144-row ones, 2,305 three rounds (several
-# items per thread block); the last item has 1, 16, 17, 128, 129 or 255 rows of 256.  4 heads: 128-row items.
+# items per thread block); the last item has 1, 16, 17, 128, 129 or 255 rows of 256.  4 heads: items of 128 rows, or of 256 with
+# nothing dropped and up to 129 queries.
 @pytest.mark.parametrize("heads,n_tok", [(32, 768 + r) for r in (1, 16, 17, 128, 129, 255)] + [(32, 1280 + r) for r in (0, 1, 129, 160)]
                          + [(32, 2304 + r) for r in (1, 129)] + [(4, r) for r in (6, 64, 65, 129, 300)])
 @pytest.mark.parametrize("sigma,lse", [(1, False), (2, True)])
@@ -72,11 +75,21 @@ def test_frame_items_in_windows(n_frames, heads):
 
 
 def test_layer_items_of_two_steps():
-    """121 keys, 160 items on a GPU of fewer SMs: a warp without rows must not run an item ahead of the others."""
+    """121 keys, 288 items of 128 rows."""
     wl = inputs.Workload("two_steps", 1, 33, 33, 0, 32, 64, 9, 1, 2, "iid")
     for seed in range(3):
         _, ocfg, _, Q, K, V, O = _run_gpu(wl, seed=seed)
         _check_attn(ocfg, Q, _host(K), _host(V), O)
+
+
+# 32 heads x 2,400 queries: 320 items of 256 rows, three rounds of the chip, the last of a head with 96 rows; 113 to 224 keys.  A warp
+# without rows must not run an item ahead of the others.
+@pytest.mark.parametrize("n_keys", (113, 121, 224))
+def test_items_of_two_steps_in_three_rounds(n_keys):
+    wl = inputs.Workload("two_steps_256", 1, 40, 60, 0, 32, 64, 4, 1, 2, "iid")
+    for seed in range(3):
+        idx = np.sort(np.random.default_rng(seed).permutation(wl.n_tokens)[:n_keys]).astype(np.int32)
+        indexed._check(wl, idx, seed)
 
 
 # 8,244 and 8,784 keys, 74 and 79 steps: past the step after which the row sums move on; several items per thread block, which the
