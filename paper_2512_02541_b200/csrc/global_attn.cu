@@ -14,7 +14,9 @@
 //               maximum is two shuffles away and every row lives in one warp.  Four softmax warps per scheduler keep the exponential unit
 //               busy while others wait on tensor memory or barriers.
 //   warp  16    TMA producer: Q tiles once per work item (two places), then the compacted
-//               K/V of the head through a ring of shared-memory stages (128-byte swizzle)
+//               K/V of the head through a ring of shared-memory stages (128-byte swizzle), then, for the
+//               epilogue, the query rows' own K and V and the head's mean pair; it also writes the record of the item
+//               (ItemInfo)
 //   warps 17-18 MMA issuers, one per query tile: S_t = Q_t Kc_j^T and
 //               O_t += P_t Vc_j with tcgen05.mma, bf16 operands, fp32
 //               accumulators in tensor memory
@@ -51,10 +53,10 @@ constexpr uint32_t kTileBytes = kTileQ * kHeadDim * 2;      // 16 KiB: one tile 
 constexpr uint32_t kKeyTileBytes = kTileKV * kHeadDim * 2;  // 14 KiB: one tile of keys or values, one ring stage
 static_assert(kKeyTileBytes % 1024 == 0, "swizzle atoms");
 constexpr uint32_t kOnesBytes = 2 * 1024;                   // the block of value columns 64..79 (ones_block)
-// K ring and V ring depth.  2, 3, 4 and 5 stages measure the same: layer of 100 frames 22.44, 22.48, 22.47 and 22.47 ms, frame
-// attention of 100 frames 1099, 1102, 1105 and 1107 us (an earlier form, with an item per CTA, gained 6 % there from the fourth).
+// K ring and V ring depth.  2, 3, 4 and 5 stages measured the same (layer of 100 frames 22.44, 22.48, 22.47 and 22.47 ms, frame
+// attention of 100 frames 1099, 1102, 1105 and 1107 us); three leave room for the query rows' own K and V.
 #ifndef AVGGT_STAGES
-#define AVGGT_STAGES 4
+#define AVGGT_STAGES 3
 #endif
 constexpr int kStages = AVGGT_STAGES;
 constexpr int kThreads = 640;
@@ -97,9 +99,6 @@ struct AttnArgs {
   Plan pl;
   Divisor by_pairs, by_heads, by_window;
   WindowRule rule;
-  const uint4* Q;       // [n_tok, H, d], read by the diagonal and mean terms; K and V by the diagonal term only
-  const uint4* K;
-  const uint4* V;
   const float* kmean;   // [H, d] or null
   const float* vmean;
   __nv_bfloat16* O;     // [n_tok, H, d]
@@ -128,9 +127,15 @@ struct AttnArgs {
   float log2_count[2];  // log2 weight of the mean column for a retained and for a dropped query (0: unit weight; -inf: absent)
 };
 
+// Records of work items (ItemInfo): so many that one is never overwritten while a warp may still read it.  When the producer writes
+// the record of item n, every Q K^T of item n - 2 has completed, so that every softmax warp has read scores of item n - 3 and, with
+// one step per item, may still be before the epilogue of item n - 4.
+constexpr int kInfos = 8;
+
 struct __align__(8) Barriers {
   uint64_t q_full[2];          // producer -> MMA: the work item's Q tiles are in shared memory (items take the two places in turn)
-  uint64_t q_empty[2];         // MMA issuers -> producer: every Q K^T of the work item has completed, Q may be overwritten
+  uint64_t q_empty[2];         // MMA issuers -> producer: every Q K^T of the work item has completed; with extra columns, softmax ->
+                               // producer as well: the epilogue has read Q.  Q may be overwritten
   uint64_t o_free[kQTiles];    // softmax -> MMA: O_t of the finished work item has been read out
   uint64_t k_full[kStages], k_empty[kStages];
   uint64_t v_full[kStages], v_empty[kStages];
@@ -140,6 +145,9 @@ struct __align__(8) Barriers {
                                // have finished a step before another warp of its tile has finished the step before
   uint64_t o_done[kQTiles][2]; // MMA -> softmax: P_t(j) V_j has completed; even and odd steps apart, since the softmax learns of
                                // P V of step j-2 from the scores of step j only, and of later ones here
+  uint64_t info_full[kInfos];  // producer -> softmax: the item's record is in shared memory
+  uint64_t own_full;           // producer -> softmax: the item's own rows of K and V and the mean pair are in shared memory
+  uint64_t own_empty;          // softmax -> producer: its epilogue has read them
   uint64_t mma_idle[kQTiles];  // MMA issuer t -> itself: every tcgen05.mma it issued has completed
   uint32_t tmem_base;
   uint32_t abort_flag;
@@ -273,10 +281,21 @@ __device__ __forceinline__ QueryTile query_tile(const AttnArgs& a, const WorkIte
   return q;
 }
 
+// What the softmax warps need to know of a work item: found once, by the producer (sixteen warps that each found it for themselves,
+// at the start and again in the epilogue, spent some 150 instructions a time on it).
+struct ItemInfo {
+  int head;
+  int active[kQTiles];   // the tile takes part in the item
+  int q0[kQTiles], first[kQTiles], last[kQTiles];   // QueryTile
+};
+
 struct SmemLayout {
   uint8_t* q;   // 2 places of kQTiles tiles
   uint8_t* k;   // kStages tiles
   uint8_t* v;   // kStages tiles
+  uint8_t* own_v;   // kQTiles tiles: V of the query rows; the epilogue turns O around here, each warp in its own rows
+  uint8_t* own_k;   // kQTiles tiles: K of the query rows (with extra columns only, as what follows)
+  float* means;     // the head's mean Key and mean Value
   uint8_t* ones;   // 16 rows of 64 values: 1 in column 0, else 0 (ones_block)
 };
 
@@ -302,13 +321,18 @@ __device__ __forceinline__ bool tile_has_rows(const AttnArgs& a, uint32_t item) 
 // ------------------------------------------------------------------ TMA producer (one warp)
 template <bool kShortLast>
 __device__ __forceinline__ void producer_role(const CUtensorMap* tm_q, const CUtensorMap* tm_k, const CUtensorMap* tm_v,
-                                              const AttnArgs& a, Barriers* bars, const SmemLayout& sm) {
-  const int n_kv = a.n_kv_tiles;
-  if (n_kv == 0) return;   // no retained keys: nothing goes through shared memory
+                                              const CUtensorMap* tm_own_k, const CUtensorMap* tm_own_v, const AttnArgs& a, Barriers* bars,
+                                              ItemInfo* infos, const SmemLayout& sm) {
+  constexpr bool kExtra = !kShortLast;
+  const int n_kv = a.n_kv_tiles;   // 0 where there are no retained keys
   if (elect_one()) {
     prefetch_tensormap(tm_q);
     prefetch_tensormap(tm_k);
     prefetch_tensormap(tm_v);
+    if (kExtra) {
+      prefetch_tensormap(tm_own_k);
+      prefetch_tensormap(tm_own_v);
+    }
   }
   int k_issued = 0, v_issued = 0;   // K / V copies issued so far, over all work items
   int stage = 0;
@@ -316,10 +340,26 @@ __device__ __forceinline__ void producer_role(const CUtensorMap* tm_q, const CUt
   bool ok = true;
   int n_done = 0;              // work items completed by this role
   int q_issued = 0;            // work items whose Q copies have been issued
+  int own_issued = 0;          // ... whose own rows' copies have been issued
   for (uint32_t item = blockIdx.x; item < static_cast<uint32_t>(a.n_work) && ok; item += gridDim.x, ++n_done) {
     const WorkItem wi = work_item<kShortLast>(a, item);
     const int head = wi.head;
     const int place = n_done & 1;
+    const QueryTile tile[kQTiles] = {query_tile(a, wi, 0), query_tile(a, wi, 1)};
+    if (elect_one()) {
+      ItemInfo& info = infos[n_done % kInfos];
+      info.head = head;
+      info.active[0] = 1;
+      info.active[1] = kExtra || tile_has_rows(a, item) ? 1 : 0;
+#pragma unroll
+      for (int t = 0; t < kQTiles; ++t) {
+        info.q0[t] = tile[t].q0;
+        info.first[t] = tile[t].first;
+        info.last[t] = static_cast<int>(tile[t].last);
+      }
+      mbar_arrive(smem_u32(&bars->info_full[n_done % kInfos]));
+    }
+    __syncwarp();
     // a wait has run out in another thread block: the launch is abandoned
     if (n_done > 0 && __any_sync(kFullMask, *reinterpret_cast<volatile uint32_t*>(a.status) != 0u)) {
       *reinterpret_cast<volatile uint32_t*>(&bars->abort_flag) = 1u;
@@ -334,7 +374,7 @@ __device__ __forceinline__ void producer_role(const CUtensorMap* tm_q, const CUt
       mbar_arrive_expect_tx(qb, kQTiles * kTileBytes);
 #pragma unroll
       for (int t = 0; t < kQTiles; ++t)
-        tma_load_2d(smem_u32(sm.q + (place * kQTiles + t) * kTileBytes), tm_q, head * kHeadDim, query_tile(a, wi, t).q0, qb);
+        tma_load_2d(smem_u32(sm.q + (place * kQTiles + t) * kTileBytes), tm_q, head * kHeadDim, tile[t].q0, qb);
     }
     __syncwarp();
     ++q_issued;
@@ -368,14 +408,39 @@ __device__ __forceinline__ void producer_role(const CUtensorMap* tm_q, const CUt
       ++v_issued;
       if (++stage == kStages) { stage = 0; empty_parity ^= 1; }
     }
+    // The query rows' own K and V and the mean pair, which the epilogue of the item before has to have read: it comes after this
+    // item's first step, whose keys and values are on their way.
+    if (kExtra && ok) {
+      ok = wait_bar_warp(&bars->own_empty, (n_done & 1) ^ 1, bars, a, 15, n_done);
+      if (!ok) break;
+      if (elect_one()) {
+        const uint32_t ob = smem_u32(&bars->own_full);
+        constexpr uint32_t kMeanBytes = kHeadDim * sizeof(float);
+        mbar_arrive_expect_tx(ob, (a.use_diag ? 2 * kQTiles * kTileBytes : 0) + (a.use_mean ? 2 * kMeanBytes : 0));
+        if (a.use_diag) {
+#pragma unroll
+          for (int t = 0; t < kQTiles; ++t) {
+            tma_load_2d(smem_u32(sm.own_k + t * kTileBytes), tm_own_k, head * kHeadDim, tile[t].q0, ob);
+            tma_load_2d(smem_u32(sm.own_v + t * kTileBytes), tm_own_v, head * kHeadDim, tile[t].q0, ob);
+          }
+        }
+        if (a.use_mean) {
+          bulk_load(smem_u32(sm.means), a.kmean + head * kHeadDim, kMeanBytes, ob);
+          bulk_load(smem_u32(sm.means + kHeadDim), a.vmean + head * kHeadDim, kMeanBytes, ob);
+        }
+      }
+      __syncwarp();
+      ++own_issued;
+    }
   }
   if (!ok) {
     // let the copies still in flight land before the CTA gives up its shared memory: the Q tiles of the last two work
-    // items begun, and the last kStages issued into either ring (earlier ones completed before their stage was reused)
+    // items begun, the last own rows, and the last kStages issued into either ring (earlier ones completed before their stage was reused)
     for (int back = 1; back <= 2; ++back) {
       const int jq = q_issued - back;
       if (jq >= 0) (void)wait_bar_warp(&bars->q_full[jq & 1], (jq >> 1) & 1, bars, a, 12, jq, false);
     }
+    if (own_issued > 0) (void)wait_bar_warp(&bars->own_full, (own_issued - 1) & 1, bars, a, 16, own_issued, false);
     for (int back = 1; back <= kStages; ++back) {
       const int jk = k_issued - back, jv = v_issued - back;
       if (jk >= 0) (void)wait_bar_warp(&bars->k_full[jk % kStages], (jk / kStages) & 1, bars, a, 12, jk, false);
@@ -641,21 +706,6 @@ __device__ __forceinline__ float quad_sum(float v) {
   return v + __shfl_xor_sync(0xffffffffu, v, 2);
 }
 
-// 4 x 4 transpose over a quad: thread i gives word b and ends with the four words that the threads 0..3 held in
-// their place i (two exchanges, with the neighbour at distance 1 and then 2; every lane of the warp takes part)
-__device__ __forceinline__ void quad_transpose(uint32_t& w0, uint32_t& w1, uint32_t& w2, uint32_t& w3, int i) {
-  const bool odd = (i & 1) != 0, upper = (i & 2) != 0;
-  uint32_t got;
-  got = __shfl_xor_sync(0xffffffffu, odd ? w0 : w1, 1);
-  if (odd) w0 = got; else w1 = got;
-  got = __shfl_xor_sync(0xffffffffu, odd ? w2 : w3, 1);
-  if (odd) w2 = got; else w3 = got;
-  got = __shfl_xor_sync(0xffffffffu, upper ? w0 : w2, 2);
-  if (upper) w0 = got; else w2 = got;
-  got = __shfl_xor_sync(0xffffffffu, upper ? w1 : w3, 2);
-  if (upper) w1 = got; else w3 = got;
-}
-
 // Running state of the thread's two rows (the same in all four threads of a quad, except the partial sums).
 struct RowState {
   float neg_m[2];         // minus the reference maximum of the stored exponentials (log2 units); +inf before the first tile
@@ -852,124 +902,126 @@ __device__ __forceinline__ bool flush_row_sums(const SoftmaxThread& me, int last
   return true;
 }
 
-// acc + the sum over the 8 products of two 16-byte pieces of bf16, or of one with 8 floats
-__device__ __forceinline__ float dot_bf16x8(const uint4& x, const uint4& y, float acc) {
-  acc = fma_bf16x2_to_f32(x.x, y.x, acc);
-  acc = fma_bf16x2_to_f32(x.y, y.y, acc);
-  acc = fma_bf16x2_to_f32(x.z, y.z, acc);
-  return fma_bf16x2_to_f32(x.w, y.w, acc);
-}
-__device__ __forceinline__ float dot_bf16x8_f32(const uint4& x, const float4& a, const float4& b, float acc) {
-  acc = fmaf(__uint_as_float(x.x << 16), a.x, acc);
-  acc = fmaf(__uint_as_float(x.x & 0xffff0000u), a.y, acc);
-  acc = fmaf(__uint_as_float(x.y << 16), a.z, acc);
-  acc = fmaf(__uint_as_float(x.y & 0xffff0000u), a.w, acc);
-  acc = fmaf(__uint_as_float(x.z << 16), b.x, acc);
-  acc = fmaf(__uint_as_float(x.z & 0xffff0000u), b.y, acc);
-  acc = fmaf(__uint_as_float(x.w << 16), b.z, acc);
-  return fmaf(__uint_as_float(x.w & 0xffff0000u), b.w, acc);
-}
-
 // What the epilogue of a work item needs of its rows' running state (shared memory; a row's warp writes and reads it).
 struct RowResults {
   float neg_m[kQTiles * kTileQ];     // minus the reference maximum
   float l_exact[kQTiles * kTileQ];   // sum of the unrounded exponentials: log-sum-exp output only
 };
 
-// Epilogue of a work item: diagonal and mean-fill terms, normalisation, store of this thread's 16 output dimensions of two
-// rows.  last: the tile's latest key step, the item's last.
+// 16 rows x 16 dimensions of a 128-byte-swizzled tile of 64 values a row (`row`: shared-memory address of the row that this lane
+// points at, 16 h + lane % 16 of the tile's quarter; `chunk`: which 16 bytes of it, 2 k + lane / 16), in the layout of O: register 0:
+// block 2 k of 8 dimensions of the thread's first row, 1: of its second row, 2 and 3: block 2 k + 1.
+__device__ __forceinline__ uint32_t row_chunk(uint32_t row, int lane, int k) {
+  return row + (((2 * k + (lane >> 4)) ^ (lane & 7)) << 4);
+}
+__device__ __forceinline__ void ld_rows16(uint32_t addr, uint32_t (&r)[4]) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ void st_rows16(uint32_t addr, uint32_t r0, uint32_t r1, uint32_t r2, uint32_t r3) {
+  asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(r0), "r"(r1), "r"(r2), "r"(r3) : "memory");
+}
+__device__ __forceinline__ uint64_t unpack_bf16x2(uint32_t w) {
+  return pack_f32x2(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u));
+}
+
+// Epilogue of a work item: diagonal and mean-fill terms, normalisation, store of the warp's 16 rows.  n: the item's number in this
+// CTA, last: the tile's latest key step, the item's last.
 //
-// The queries' own Q, K and V rows are read straight from global memory (at the item's start the warp asked for them to be
-// brought to L2), 16 bytes per thread and half row, and asked for before the first use.
-// By the read-only path: the kernel before this one does not write them, and those before that had ended when this one began (the
-// compaction and clear_status_kernel let it begin after their own wait).
+// The queries' own Q, K and V rows and the mean pair are in shared memory (the producer brings them while the item runs).  A thread
+// has two rows, and of each block of 8 dimensions the pair 2 i, 2 i + 1, as in O: ldmatrix gives rows of a tile in that layout, and
+// stmatrix turns the result into rows, which are stored 128 contiguous bytes at a time.
+//
+// An item boundary is bound by instructions: all four warps of a scheduler are in it at once.  Before, with the own rows and the mean
+// pair read from global memory 16 bytes per thread, V and the result turned around by shuffles within the quad, and the item found
+// anew by every warp, a boundary cost the layer 1,215 instructions a warp, as many as 4.6 key steps, and the last epilogue of a launch
+// 4,900 clocks.  Layer of 10 frames 269 -> 261 us, 31 frames 1154 -> 1126 us, 4 frames of 16 x 16 17.2 -> 16.8 us, frame
+// attention of 100 frames 1090 -> 1062 us, of 10 frames 116 -> 114.5 us.
 template <bool kLse, bool kExtra>
 __device__ __forceinline__ bool softmax_epilogue(const AttnArgs& a, Barriers* bars, const SoftmaxThread& me, const RowResults* res,
-                                                 uint32_t item, int last) {
+                                                 const ItemInfo* infos, const SmemLayout& sm, int n, int last) {
   const Plan& pl = a.pl;
-  const WorkItem wi = work_item<!kExtra>(a, item);
-  const QueryTile tile = query_tile(a, wi, me.t);
-  const int t = me.t, head = wi.head;
+  const ItemInfo& info = infos[n % kInfos];
+  const int t = me.t, head = info.head, first = info.first[t], end = info.last[t];
   const int i = me.lane & 3;                             // position in the quad
-  const int r0 = 32 * me.q + 16 * me.h + (me.lane >> 2);   // the thread's two rows within the tile: r0, r0 + 8
+  const int lane0 = 32 * me.q + 16 * me.h;               // the warp's first row within the tile
+  const int row0 = info.q0[t] + lane0;                   // ... and in the sequence; the thread's rows: + lane / 4, + lane / 4 + 8
+  const uint32_t at = static_cast<uint32_t>(t) * kTileBytes + static_cast<uint32_t>(lane0 + (me.lane & 15)) * (kHeadDim * 2);
 
-  // base-2 logits of the two extra columns: each thread of the quad takes 16 dimensions (8 i .. and 32 + 8 i ..), then the quad
-  // adds up (every thread runs the shuffles; rows without the term carry zeros)
+  // base-2 logits of the two extra columns (every thread runs the shuffles; rows without the term carry what is not used)
   float l_d[2] = {-INFINITY, -INFINITY}, l_m[2] = {-INFINITY, -INFINITY};
-  uint32_t vw[2][8];   // the row's own V: chunks i and 4 + i of 16 bytes, then the words 4 b + i
   if (kExtra) {
-    uint4 q[2][2], k[2][2];
-    float4 km[4];
     bool dropped[2] = {false, false};
+    if (a.use_diag) {   // lanes 0..15: a row each
+      const int row = row0 + (me.lane & 15);
+      bool mine = row >= first && row < end;
+      if (mine) mine = a.slot_of_token != nullptr ? a.slot_of_token[row] < 0 : compact_position(a.rule, pl, row) < 0;
+      const uint32_t rows = __ballot_sync(kFullMask, mine) >> (me.lane >> 2);
+      dropped[0] = (rows & 1) != 0;
+      dropped[1] = (rows & 0x100) != 0;
+    }
+    const uint32_t q_row = smem_u32(sm.q) + (n & 1) * (kQTiles * kTileBytes) + at, k_row = smem_u32(sm.own_k) + at;
+    if (!wait_bar(&bars->q_full[n & 1], (n >> 1) & 1, bars, a, 52, n)) return false;
+    if (!wait_bar(&bars->own_full, n & 1, bars, a, 53, n)) return false;
+    float d[2] = {0.f, 0.f};
+    uint64_t m[2] = {pack_f32x2(0.f, 0.f), pack_f32x2(0.f, 0.f)};
+#pragma unroll
+    for (int k = 0; k < kHeadDim / 16; ++k) {
+      uint32_t q[4], own[4];
+      ld_rows16(row_chunk(q_row, me.lane, k), q);
+      if (a.use_diag) {
+        ld_rows16(row_chunk(k_row, me.lane, k), own);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) d[c & 1] = fma_bf16x2_to_f32(q[c], own[c], d[c & 1]);
+      }
+      if (a.use_mean) {
+#pragma unroll
+        for (int b = 0; b < 2; ++b) {
+          const uint64_t mean = *reinterpret_cast<const uint64_t*>(sm.means + 16 * k + 8 * b + 2 * i);
+          m[0] = fma_f32x2(unpack_bf16x2(q[2 * b]), mean, m[0]);
+          m[1] = fma_f32x2(unpack_bf16x2(q[2 * b + 1]), mean, m[1]);
+        }
+      }
+    }
 #pragma unroll
     for (int hi = 0; hi < 2; ++hi) {
-      const int row = tile.q0 + r0 + 8 * hi;   // query token
-      uint4 v0 = make_uint4(0u, 0u, 0u, 0u), v1 = v0;
-      q[hi][0] = q[hi][1] = k[hi][0] = k[hi][1] = v0;
-      if (row >= tile.first && row < tile.last) {
-        const size_t at = (static_cast<size_t>(row) * pl.H + head) * (kHeadDim / 8) + i;
-        q[hi][0] = __ldg(a.Q + at);
-        q[hi][1] = __ldg(a.Q + at + 4);
-        if (a.use_diag) {
-          k[hi][0] = __ldg(a.K + at);
-          k[hi][1] = __ldg(a.K + at + 4);
-          v0 = __ldg(a.V + at);
-          v1 = __ldg(a.V + at + 4);
-        }
+      if (a.use_diag) {
+        const float dot = quad_sum(d[hi]);
+        if (dropped[hi]) l_d[hi] = dot * a.scale_log2;
       }
-      vw[hi][0] = v0.x; vw[hi][1] = v0.y; vw[hi][2] = v0.z; vw[hi][3] = v0.w;
-      vw[hi][4] = v1.x; vw[hi][5] = v1.y; vw[hi][6] = v1.z; vw[hi][7] = v1.w;
-    }
-    if (a.use_mean) {   // (past L1: written by the kernel before this one, which may have ended after this one began)
-      const float4* src = reinterpret_cast<const float4*>(a.kmean + head * kHeadDim + 8 * i);
-      km[0] = __ldcg(src);
-      km[1] = __ldcg(src + 1);
-      km[2] = __ldcg(src + 8);
-      km[3] = __ldcg(src + 9);
-    }
-    if (a.use_diag) {
-#pragma unroll
-      for (int hi = 0; hi < 2; ++hi) {
-        const int row = tile.q0 + r0 + 8 * hi;
-        if (row >= tile.first && row < tile.last) {
-          dropped[hi] = a.slot_of_token != nullptr ? a.slot_of_token[row] < 0 : compact_position(a.rule, pl, row) < 0;
-        }
-      }
-#pragma unroll
-      for (int hi = 0; hi < 2; ++hi) {
-        const float acc = quad_sum(dot_bf16x8(q[hi][1], k[hi][1], dot_bf16x8(q[hi][0], k[hi][0], 0.f)));
-        if (dropped[hi]) l_d[hi] = acc * a.scale_log2;
+      if (a.use_mean) {
+        float m0, m1;
+        unpack_f32x2(m[hi], m0, m1);
+        l_m[hi] = fmaf(quad_sum(m0 + m1), a.scale_log2, a.log2_count[dropped[hi] ? 1 : 0]);
       }
     }
-    if (a.use_mean) {
-#pragma unroll
-      for (int hi = 0; hi < 2; ++hi) {
-        const float acc = quad_sum(dot_bf16x8_f32(q[hi][1], km[2], km[3], dot_bf16x8_f32(q[hi][0], km[0], km[1], 0.f)));
-        l_m[hi] = fmaf(acc, a.scale_log2, a.log2_count[dropped[hi] ? 1 : 0]);
-      }
-    }
-    if (a.use_diag) {
-#pragma unroll
-      for (int hi = 0; hi < 2; ++hi) {
-        quad_transpose(vw[hi][0], vw[hi][1], vw[hi][2], vw[hi][3], i);
-        quad_transpose(vw[hi][4], vw[hi][5], vw[hi][6], vw[hi][7], i);
-      }
-    }
+    __syncwarp();
+    if (elect_one()) mbar_arrive(smem_u32(&bars->q_empty[n & 1]));
   }
 
   uint32_t l[4] = {0u, 0u, 0u, 0u};   // thread 0 of a quad: the row sums, in two parts, in registers 0 + 1 (row 0) and 2 + 3 (row 1)
+  uint32_t o[2][16];   // register 4 b + 2 hi + e of a half: row hi, output dimension 32 half + 8 b + 2 i + e; zero with no retained keys
+#pragma unroll
+  for (int half = 0; half < 2; ++half)
+#pragma unroll
+    for (int c = 0; c < 16; ++c) o[half][c] = 0u;
   if (a.n_kv_tiles > 0) {
     if (!wait_bar(&bars->o_done[t][last & 1], (last >> 1) & 1, bars, a, 50 + t, last)) return false;
     tc_fence_after();
     tmem_ld_rows16_c8(me.base + kColL, l);
+    tmem_ld_rows16_c32(me.base + kColO, o[0]);
+    tmem_ld_rows16_c32(me.base + kColO + 32, o[1]);
     tmem_wait_ld();
+    // O_t has been read: the next work item's first P V may overwrite it
+    tc_fence_before();
+    if (elect_one()) mbar_arrive(smem_u32(&bars->o_free[t]));
   }
-  float w_s[2], w_d[2], w_m[2];   // weights of the accumulator, of the row's own V and of the mean Value
+  uint64_t w_s[2], w_d[2], w_m[2];   // weights of the accumulator, of the row's own V and of the mean Value
 #pragma unroll
   for (int hi = 0; hi < 2; ++hi) {
-    const int r = r0 + 8 * hi;
+    const int r = lane0 + (me.lane >> 2) + 8 * hi;
     // the row's sums: of the rounded probabilities (the normaliser), of the unrounded ones (log-sum-exp)
-    const float l_run = __shfl_sync(0xffffffffu, __uint_as_float(l[2 * hi]) + __uint_as_float(l[2 * hi + 1]), me.lane & ~3);
+    const float l_run = __shfl_sync(kFullMask, __uint_as_float(l[2 * hi]) + __uint_as_float(l[2 * hi + 1]), me.lane & ~3);
     float p_d = 0.f, p_m = 0.f, a_s = 1.0f, m_fin = 0.f;
     if (kExtra || kLse) {
       const float m = -res->neg_m[t * kTileQ + r];
@@ -983,62 +1035,47 @@ __device__ __forceinline__ bool softmax_epilogue(const AttnArgs& a, Barriers* ba
     }
     const float z = fmaf(l_run, a_s, p_d + p_m);
     const float inv_z = __fdividef(1.0f, z);   // z is at least one exponential of a row maximum, far from the ends of the range
-    w_s[hi] = a_s * inv_z;
-    w_d[hi] = p_d * inv_z;
-    w_m[hi] = p_m * inv_z;
+    w_s[hi] = pack_f32x2(a_s * inv_z, a_s * inv_z);
+    w_d[hi] = pack_f32x2(p_d * inv_z, p_d * inv_z);
+    w_m[hi] = pack_f32x2(p_m * inv_z, p_m * inv_z);
     if (kLse && i == 0) {
-      const int row = tile.q0 + r;
+      const int row = info.q0[t] + r;
       const float z_exact = fmaf(res->l_exact[t * kTileQ + r], a_s, p_d + p_m);
-      if (row >= tile.first && row < tile.last)
+      if (row >= first && row < end)
         a.lse[static_cast<size_t>(row) * pl.H + head] = (m_fin + log2f(z_exact)) * 0.6931471805599453f;
     }
   }
+  const uint32_t v_row = smem_u32(sm.own_v) + at;
 #pragma unroll
-  for (int half = 0; half < 2; ++half) {   // 32 output dimensions at a time: with more the registers run over
-    float2 vm[4];     // the mean Value at the thread's output dimensions 8 b + 2 i, 8 b + 2 i + 1
-    if (kExtra && a.use_mean) {
-      const float2* src = reinterpret_cast<const float2*>(a.vmean + head * kHeadDim + 32 * half) + i;
+  for (int k = 0; k < kHeadDim / 16; ++k) {
+    uint32_t own[4], w[4];
+    if (kExtra && a.use_diag) ld_rows16(row_chunk(v_row, me.lane, k), own);
 #pragma unroll
-      for (int b = 0; b < 4; ++b) vm[b] = __ldcg(src + 4 * b);
+    for (int c = 0; c < 4; ++c) {
+      const int hi = c & 1, reg = 4 * (2 * (k & 1) + (c >> 1)) + 2 * hi;
+      uint64_t v = mul_f32x2(pack_f32x2(__uint_as_float(o[k >> 1][reg]), __uint_as_float(o[k >> 1][reg + 1])), w_s[hi]);
+      if (kExtra && a.use_diag) v = fma_f32x2(w_d[hi], unpack_bf16x2(own[c]), v);
+      if (kExtra && a.use_mean)
+        v = fma_f32x2(w_m[hi], *reinterpret_cast<const uint64_t*>(sm.means + kHeadDim + 16 * k + 8 * (c >> 1) + 2 * i), v);
+      w[c] = pack_bf16x2(v);
     }
-    uint32_t o[16];   // register 4 b + 2 hi + e: row hi, output dimension 8 b + 2 i + e; zero with no retained keys at all
+    __syncwarp();   // every lane has its part of V
+    st_rows16(row_chunk(v_row, me.lane, k), w[0], w[1], w[2], w[3]);
+  }
+  __syncwarp();
+  // four rows at a time, eight lanes x 16 bytes per row
 #pragma unroll
-    for (int c = 0; c < 16; ++c) o[c] = 0u;
-    if (a.n_kv_tiles > 0) {
-      tmem_ld_rows16_c32(me.base + kColO + 32 * half, o);
-      tmem_wait_ld();
-      if (half == 1) {   // O_t has been read: the next work item's first P V may overwrite it
-        tc_fence_before();
-        if (elect_one()) mbar_arrive(smem_u32(&bars->o_free[t]));
-      }
-    }
-#pragma unroll
-    for (int hi = 0; hi < 2; ++hi) {
-      const int row = tile.q0 + r0 + 8 * hi;
-      uint32_t w[4];   // the thread's words of the output row: word 4 b + i (dimensions 8 b + 2 i, 8 b + 2 i + 1)
-#pragma unroll
-      for (int b = 0; b < 4; ++b) {
-        uint64_t v = mul_f32x2(pack_f32x2(__uint_as_float(o[4 * b + 2 * hi]), __uint_as_float(o[4 * b + 2 * hi + 1])),
-                               pack_f32x2(w_s[hi], w_s[hi]));
-        if (kExtra && a.use_diag) {
-          const uint32_t own = vw[hi][4 * half + b];
-          v = fma_f32x2(pack_f32x2(w_d[hi], w_d[hi]), pack_f32x2(__uint_as_float(own << 16), __uint_as_float(own & 0xffff0000u)), v);
-        }
-        if (kExtra && a.use_mean) v = fma_f32x2(pack_f32x2(w_m[hi], w_m[hi]), pack_f32x2(vm[b].x, vm[b].y), v);
-        float v0, v1;
-        unpack_f32x2(v, v0, v1);
-        w[b] = pack_bf16x2(v0, v1);
-      }
-      // Transposed within the quad, a thread holds 16 contiguous bytes of the row: 4 stores of 16 bytes
-      // per thread instead of 16 of 4 bytes (whose 8 rows x 16 bytes per warp instruction kept the store path of the
-      // SM busy for thousands of clocks per work item).
-      quad_transpose(w[0], w[1], w[2], w[3], i);
-      if (row >= tile.first && row < tile.last) {
-        uint4* dst = reinterpret_cast<uint4*>(a.O + (static_cast<size_t>(row) * pl.H + head) * kHeadDim);
-        dst[4 * half + i] = make_uint4(w[0], w[1], w[2], w[3]);
-      }
+  for (int k = 0; k < 4; ++k) {
+    const int r = 4 * k + (me.lane >> 3), row = row0 + r;
+    if (row >= first && row < end) {
+      const uint8_t* src = sm.own_v + t * kTileBytes + (lane0 + r) * (kHeadDim * 2) + (((me.lane ^ r) & 7) << 4);
+      uint4* dst = reinterpret_cast<uint4*>(a.O + (static_cast<size_t>(row) * pl.H + head) * kHeadDim) + (me.lane & 7);
+      *dst = *reinterpret_cast<const uint4*>(src);
     }
   }
+  if (kExtra) fence_proxy_async_smem();   // the next copy of own rows comes after these accesses
+  __syncwarp();
+  if (kExtra && elect_one()) mbar_arrive(smem_u32(&bars->own_empty));
   return true;
 }
 
@@ -1046,18 +1083,19 @@ __device__ __forceinline__ bool softmax_epilogue(const AttnArgs& a, Barriers* ba
 // P V has completed, the next item's P V waits for O to be read out (o_free) but its scores do not, and the tensor core and the
 // copies are a step ahead.
 template <bool kLse, bool kExtra>
-__device__ __forceinline__ void softmax_items(const AttnArgs& a, Barriers* bars, const SoftmaxThread& me, RowResults* res) {
+__device__ __forceinline__ void softmax_items(const AttnArgs& a, Barriers* bars, const SoftmaxThread& me, RowResults* res, const ItemInfo* infos,
+                                              const SmemLayout& sm) {
   const int n_kv = a.n_kv_tiles;
   const int t = me.t;
   const bool ragged = a.last_tile_keys != 0;
   bool res_rows = false;   // the warp had rows in the item before
   int gj = 0;              // this tile's key steps so far, over all work items of the CTA: the phase of the per-step barriers
   bool pending = false;    // the epilogue of the item before
+  int n = 0;               // items so far
 #pragma unroll 1
-  for (uint32_t item = blockIdx.x;; item += gridDim.x) {
+  for (uint32_t item = blockIdx.x;; item += gridDim.x, ++n) {
     const bool have = item < static_cast<uint32_t>(a.n_work);
     if (!have && !pending) return;
-    const bool active = have && (kExtra || t == 0 || tile_has_rows(a, item));   // the tile has rows in this item
     RowState st;
 #pragma unroll
     for (int hi = 0; hi < 2; ++hi) {
@@ -1065,17 +1103,13 @@ __device__ __forceinline__ void softmax_items(const AttnArgs& a, Barriers* bars,
       st.look_above[hi] = -INFINITY;
       st.l_exact[hi] = 0.f;
     }
-    bool rows = false;
+    bool active = false, rows = false;   // the tile takes part in this item, the warp has rows in it
     if (have) {
-      const WorkItem wi = work_item<!kExtra>(a, item);
-      const QueryTile tile = query_tile(a, wi, t);
-      const int row0 = tile.q0 + 32 * me.q + 16 * me.h;   // the warp's first row
-      rows = row0 + 16 > tile.first && row0 < tile.last;
-      if (kExtra && a.use_diag) {   // each thread asks for one line: K of row lane / 2, or V
-        const int row = row0 + (me.lane >> 1);
-        if (row >= tile.first && row < tile.last)
-          prefetch_l2(((me.lane & 1) ? a.V : a.K) + (static_cast<size_t>(row) * a.pl.H + wi.head) * (kHeadDim / 8));
-      }
+      if (!wait_bar(&bars->info_full[n % kInfos], (n / kInfos) & 1, bars, a, 54, n)) return;
+      const ItemInfo& info = infos[n % kInfos];
+      active = info.active[t] != 0;
+      const int row0 = info.q0[t] + 32 * me.q + 16 * me.h;   // the warp's first row
+      rows = row0 + 16 > info.first[t] && row0 < info.last[t];
     }
     int left = active ? n_kv : 0;
     // steps up to the next multiple of kFlushSteps of the item's own, so that a row's sums do not depend on the item's place
@@ -1107,13 +1141,22 @@ __device__ __forceinline__ void softmax_items(const AttnArgs& a, Barriers* bars,
       }
       if (pending) {
         if (res_rows) {
-          if (!softmax_epilogue<kLse, kExtra>(a, bars, me, res, item - gridDim.x, stop - chunk - 1)) return;
-        } else if (n_kv > 0) {
-          // Not before the item's last P V: a warp without rows could otherwise be an item ahead and arrive a second time in
-          // the phase in which another warp has not yet read O.
-          const int last = stop - chunk - 1;
-          if (!wait_bar(&bars->o_done[t][last & 1], (last >> 1) & 1, bars, a, 51, last)) return;
-          if (me.lane == 0) mbar_arrive(smem_u32(&bars->o_free[t]));
+          if (!softmax_epilogue<kLse, kExtra>(a, bars, me, res, infos, sm, n - 1, stop - chunk - 1)) return;
+        } else {
+          if (n_kv > 0) {
+            // Not before the item's last P V: a warp without rows could otherwise be an item ahead and arrive a second time in
+            // the phase in which another warp has not yet read O.
+            const int last = stop - chunk - 1;
+            if (!wait_bar(&bars->o_done[t][last & 1], (last >> 1) & 1, bars, a, 51, last)) return;
+            if (me.lane == 0) mbar_arrive(smem_u32(&bars->o_free[t]));
+          }
+          if (kExtra) {   // (nor before the item's own rows have come, for the same reason)
+            if (!wait_bar(&bars->own_full, (n - 1) & 1, bars, a, 53, n)) return;
+            if (me.lane == 0) {
+              mbar_arrive(smem_u32(&bars->q_empty[(n - 1) & 1]));
+              mbar_arrive(smem_u32(&bars->own_empty));
+            }
+          }
         }
         pending = false;
         most = kFlushSteps - 1;
@@ -1141,14 +1184,15 @@ __device__ __forceinline__ void softmax_items(const AttnArgs& a, Barriers* bars,
 }
 
 template <bool kLse, bool kExtra>
-__device__ __forceinline__ void softmax_role(const AttnArgs& a, Barriers* bars, RowResults* res, uint32_t tmem, int warp, int lane) {
+__device__ __forceinline__ void softmax_role(const AttnArgs& a, Barriers* bars, RowResults* res, const ItemInfo* infos, const SmemLayout& sm,
+                                             uint32_t tmem, int warp, int lane) {
   SoftmaxThread me;
   me.t = warp >> 3;
   me.h = (warp >> 2) & 1;
   me.q = warp & 3;
   me.lane = lane;
   me.base = tmem + me.t * kTmemTileStride + (static_cast<uint32_t>(32 * me.q + 16 * me.h) << 16);   // TMEM lane = row
-  softmax_items<kLse, kExtra>(a, bars, me, res);
+  softmax_items<kLse, kExtra>(a, bars, me, res, infos, sm);
 }
 
 // Value columns 64..79 of a slice of 16 keys, in the 128-byte-swizzled layout of the V tiles: column 64 all ones, the others
@@ -1168,7 +1212,8 @@ __device__ __forceinline__ void ones_block(uint8_t* ones, int tid) {
 template <bool kLse, bool kExtra>
 __global__ void __launch_bounds__(kThreads, 1)
 global_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
-                   const __grid_constant__ CUtensorMap tm_v, const AttnArgs a) {
+                   const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_own_k,
+                   const __grid_constant__ CUtensorMap tm_own_v, const AttnArgs a) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   SmemLayout sm;
@@ -1176,16 +1221,23 @@ global_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
   sm.k = smem + 2 * kQTiles * kTileBytes;
   sm.v = sm.k + kStages * kKeyTileBytes;
   sm.ones = sm.v + kStages * kKeyTileBytes;
+  sm.own_v = sm.ones + kOnesBytes;
+  sm.own_k = sm.own_v + kQTiles * kTileBytes;
+  sm.means = reinterpret_cast<float*>(sm.own_k + kQTiles * kTileBytes);
   __shared__ RowResults row_results;
   __shared__ Barriers bars;
+  __shared__ ItemInfo infos[kInfos];
 
   const int tid = threadIdx.x;
   const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // warp-uniform by construction
   if (tid == 0) {
     for (int e = 0; e < 2; ++e) {
       mbar_init(smem_u32(&bars.q_full[e]), 1);
-      mbar_init(smem_u32(&bars.q_empty[e]), kQTiles);
+      mbar_init(smem_u32(&bars.q_empty[e]), (a.n_kv_tiles > 0 ? kQTiles : 0) + (kExtra ? kSoftmaxWarps : 0));
     }
+    for (int e = 0; e < kInfos; ++e) mbar_init(smem_u32(&bars.info_full[e]), 1);
+    mbar_init(smem_u32(&bars.own_full), 1);
+    mbar_init(smem_u32(&bars.own_empty), kSoftmaxWarps);
     for (int s = 0; s < kStages; ++s) {
       mbar_init(smem_u32(&bars.k_full[s]), 1);
       mbar_init(smem_u32(&bars.k_empty[s]), kQTiles);
@@ -1221,10 +1273,10 @@ global_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
   if (abandoned) {
   } else if (warp < kSoftmaxWarps) {
     reg_inc<kRegsSoftmax>();
-    softmax_role<kLse, kExtra>(a, &bars, &row_results, tmem, warp, tid & 31);
+    softmax_role<kLse, kExtra>(a, &bars, &row_results, infos, sm, tmem, warp, tid & 31);
   } else {
     reg_dec<kRegsOther>();
-    if (warp == kTmaWarp) producer_role<!kExtra>(&tm_q, &tm_k, &tm_v, a, &bars, sm);
+    if (warp == kTmaWarp) producer_role<!kExtra>(&tm_q, &tm_k, &tm_v, &tm_own_k, &tm_own_v, a, &bars, infos, sm);
     else if (warp == kMmaWarp) mma_role<0, !kExtra>(a, &bars, sm, tmem);
     else if (warp == kMmaWarp + 1) mma_role<1, !kExtra>(a, &bars, sm, tmem);
   }
@@ -1244,7 +1296,11 @@ __global__ void clear_status_kernel(uint32_t* status) {
   if (threadIdx.x < kAttnStatusBytes / 4) status[threadIdx.x] = 0u;
 }
 
-constexpr size_t kAttnSmemBytes = static_cast<size_t>(kTileBytes) * (2 * kQTiles) + static_cast<size_t>(kKeyTileBytes) * (2 * kStages) + kOnesBytes + 1024;
+// kExtra: with the query rows' own K and the mean pair
+constexpr size_t attn_smem_bytes(bool extra) {
+  return static_cast<size_t>(kTileBytes) * (2 * kQTiles) + static_cast<size_t>(kKeyTileBytes) * (2 * kStages) + kOnesBytes +
+         kQTiles * kTileBytes + (extra ? kQTiles * kTileBytes + 2 * kHeadDim * sizeof(float) : 0) + 1024;
+}
 
 }  // namespace
 
@@ -1260,7 +1316,7 @@ namespace {
 // registers the role split hands out.  setmaxnreg.inc waits, without a time limit, for registers that other
 // warps release; if the compiler gave the kernel fewer than kRegsLaunch registers per thread the pool could
 // never cover the softmax warps' share and the kernel would hang, so such a build refuses to launch.
-typedef void (*AttnKernel)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const AttnArgs);
+typedef void (*AttnKernel)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const CUtensorMap, const CUtensorMap, const AttnArgs);
 constexpr AttnKernel kAttnKernels[4] = {global_attn_kernel<false, false>, global_attn_kernel<false, true>,
                                         global_attn_kernel<true, false>, global_attn_kernel<true, true>};
 
@@ -1273,13 +1329,14 @@ cudaError_t prepare_kernels() {
   if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
   std::lock_guard<std::mutex> lock(mu);
   if (ready[dev]) return cudaSuccess;
-  for (AttnKernel k : kAttnKernels) {
+  for (int which = 0; which < 4; ++which) {
+    const AttnKernel k = kAttnKernels[which];
     cudaFuncAttributes fa;
     e = cudaFuncGetAttributes(&fa, k);
     if (e != cudaSuccess) return e;
     if (fa.numRegs * (kThreads / 32) < kRegsSoftmax * kSoftmaxWarps + kRegsOther * (kThreads / 32 - kSoftmaxWarps))
       return cudaErrorLaunchOutOfResources;
-    e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kAttnSmemBytes));
+    e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(attn_smem_bytes((which & 1) != 0)));
     if (e != cudaSuccess) return e;
   }
   ready[dev] = true;
@@ -1330,9 +1387,6 @@ cudaError_t launch_attn(const Plan& pl, int sm_count, bool frame_mode, const voi
   AttnArgs a;
   a.pl = pl;
   a.slot_of_token = slot_of_token;
-  a.Q = static_cast<const uint4*>(Q);
-  a.K = static_cast<const uint4*>(K);
-  a.V = static_cast<const uint4*>(V);
   a.kmean = kmean;
   a.vmean = vmean;
   a.O = static_cast<__nv_bfloat16*>(O);
@@ -1376,7 +1430,7 @@ cudaError_t launch_attn(const Plan& pl, int sm_count, bool frame_mode, const voi
   a.n_work = static_cast<int32_t>(problems * items);
 
   // token-major [n_tok, H*d] maps for Q and, in frame attention, K and V; head-major [H, M, d] maps for Kc, Vc otherwise
-  CUtensorMap tm_q, tm_k, tm_v;
+  CUtensorMap tm_q, tm_k, tm_v, tm_own_k, tm_own_v;
   const uint64_t tok_dims[2] = {static_cast<uint64_t>(pl.H) * pl.d, static_cast<uint64_t>(pl.n_tok)};
   const uint64_t tok_str[1] = {static_cast<uint64_t>(pl.H) * pl.d * 2};
   const uint32_t q_box[2] = {kHeadDim, kTileQ};
@@ -1394,6 +1448,12 @@ cudaError_t launch_attn(const Plan& pl, int sm_count, bool frame_mode, const voi
   } else {
     tm_k = tm_v = tm_q;   // not read
   }
+  if (a.use_diag) {   // the query rows' own K and V
+    good = good && make_tmap_bf16(&tm_own_k, K, 2, tok_dims, tok_str, q_box);
+    good = good && make_tmap_bf16(&tm_own_v, V, 2, tok_dims, tok_str, q_box);
+  } else {
+    tm_own_k = tm_own_v = tm_q;   // not read
+  }
   if (!good) { *tmap_failed = true; return cudaSuccess; }
 
   cudaError_t e = prepare_kernels();
@@ -1404,7 +1464,7 @@ cudaError_t launch_attn(const Plan& pl, int sm_count, bool frame_mode, const voi
   }
   const unsigned grid = static_cast<unsigned>(a.n_work < sm_count ? a.n_work : sm_count);
   const int which = (lse != nullptr ? 2 : 0) + (a.use_diag || a.use_mean ? 1 : 0);
-  return launch_dependent(kAttnKernels[which], grid, kThreads, kAttnSmemBytes, st, tm_q, tm_k, tm_v, a);
+  return launch_dependent(kAttnKernels[which], grid, kThreads, attn_smem_bytes((which & 1) != 0), st, tm_q, tm_k, tm_v, tm_own_k, tm_own_v, a);
 }
 
 }  // namespace
