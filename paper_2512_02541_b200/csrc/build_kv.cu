@@ -2,35 +2,29 @@
 // one pass over K and V that copies the retained rows into the head-major
 // compact arrays and sums the dropped patch rows for the mean Key/Value pair.
 //
-// Memory-bound: every row of K and V is read once with 16-byte loads (a warp
-// covers 512 contiguous bytes per load instruction), retained rows are written
-// once as full 128-byte lines.  Sums are kept in registers per lane (a lane owns
-// fixed columns), reduced across the warps of a block in shared memory in a
-// fixed order, written as one partial row per block, and reduced across blocks
-// by a second small kernel with a fixed shuffle tree: no floating-point
+// Memory-bound: every row of K and V is read once, retained rows are written once as full 128-byte lines.  Many tokens with a mean:
+// build_kv_stream_kernel, contiguous tiles through shared memory; without one (only retained rows are read): build_kv_gather_kernel,
+// tiles of compact rows; few tokens: build_kv_small_kernel, a cluster of thread blocks per head.  Sums are kept in
+// registers per lane (a lane owns fixed columns), reduced within a block in a fixed order, written as one partial row per block, and
+// reduced across blocks by a second small kernel with a fixed shuffle tree: no floating-point
 // atomics, so the result does not change from run to run.
+#include <mutex>
+
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
 #include "internal.h"
 #include "ptx.cuh"
+#include "tmap.h"
 
 namespace avggt {
 
 namespace {
 
-constexpr int kBuildThreads = 256;
-constexpr int kBuildWarps = kBuildThreads / 32;
-// Blocks of build_kv_kernel<PASSES> that an SM holds (by its registers; the launch bounds see to it that they fit), and as many as
-// the grid has per SM: a second wave of blocks would only double the partial sums (592 blocks instead of 296 on 148 SMs: 16.2 instead of 13.5 us at 8 frames,
-// 30.8 instead of 27.7 at 24; no difference at 333).
-constexpr int kBuildBlocks[9] = {0, 5, 3, 2, 2, 1, 1, 1, 1};
-
 // The kernels here begin while the kernel before them in the stream, and one before that which has already let it begin, may still
 // be writing what they read after their wait: K and V (the projection), the map from tokens to compact positions, a caller's
 // list of retained tokens.  They therefore read none of it by the read-only path, which is for data that does not change in a
 // kernel's lifetime, or through a pointer the compiler may take for one to such data: K and V by this load, the rest by __ldcg.
-// (The compaction of 333 frames takes the same time with either load, 396 us.)
 __device__ __forceinline__ uint4 ld_stream(const uint4* p) {
   uint4 v;
   asm volatile("ld.global.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];"
@@ -48,92 +42,391 @@ __device__ __forceinline__ void add_bf16x8(float (&acc)[8], const uint4& v) {
   }
 }
 
-// PASSES = ceil(H * 8 / 32): 16-byte chunks of one row handled per lane.
-// kc_rows: rows per head of the compact arrays (M, or more when the caller's arrays are a slot of a
-// larger exchange buffer).
-template <int PASSES>
-__global__ void __launch_bounds__(kBuildThreads, kBuildBlocks[PASSES])
-build_kv_kernel(const Plan pl, const uint4* K, const uint4* V, uint4* __restrict__ Kc,
-                uint4* __restrict__ Vc, const int64_t kc_rows, int32_t* __restrict__ idx, float* __restrict__ partials,
-                const int do_mean, const int32_t* slot_of_token, uint32_t* __restrict__ status,
-                float* __restrict__ zero_kmean, float* __restrict__ zero_vmean) {
-  extern __shared__ float red[];   // [kBuildWarps][PASSES * 256]
-  const int lane = threadIdx.x & 31;
-  const int warp = threadIdx.x >> 5;
-  const uint32_t chunks_per_row = static_cast<uint32_t>(pl.H) * 8u;   // 16-byte chunks (d = 64 bf16 = 8 chunks per head)
-  const uint32_t n_tok = static_cast<uint32_t>(pl.n_tok);
-  const uint32_t warps_total = gridDim.x * kBuildWarps;
+// Many tokens, with a mean: two thread blocks per SM walk over tiles of consecutive tokens, whose rows of K and V
+// (contiguous: two bulk copies) go through a ring of shared-memory stages.  One warp issues the copies and, as a tile arrives, one
+// TMA store per retained row and array, which takes the row's heads to their places in the head-major array; the other eight
+// warps only add: a thread owns 16 bytes of a row (eight columns) and takes every row of the tile that is dropped.
+//
+// What bounds it is HBM.  457,542 tokens of 16 heads, a quarter retained (2.37 GB): 396 -> 356 us (6.0 -> 6.7 TB/s) against a warp per
+// row with 16 bytes per lane in flight, whose loads stop while it adds and stores; 13,740 tokens 13.9 -> 11.4 us, 137,400
+// tokens, a ninth retained, 107.0 -> 102.5.  Stages of 16 + 16 KB, three in each of two blocks per SM: six in one block 377 us (14.0 at 13,740 tokens),
+// four 356 (14.3), three of 32 + 32 KB 353 (14.2); of 8 + 8 KB 536 and more in one block (the copying warp's chain of waits per tile),
+// 362 in two; two of 16 + 16 KB in two blocks 395, in three 355.
+constexpr int kStreamSums = 256;                    // adding threads
+constexpr int kStreamThreads = kStreamSums + 32;    // and the warp that copies
+constexpr int kStreamBlocks = 2;                    // per SM
+constexpr int kStreamStages = 3;
+constexpr uint32_t kStreamBytes = 16 * 1024;        // of K, and of V, in a stage (at most)
+constexpr int kStreamRows = 32;                     // rows of a tile (at most): the copying warp has a lane for each
+constexpr int kStreamFlush = 8;                     // tiles after which a thread's sums move on: short chains round less
+constexpr size_t kStreamSmemBytes = 2 * kStreamStages * kStreamBytes + 128;
 
+struct StreamArgs {
+  Plan pl;
+  WindowRule rule;
+  const uint8_t* K;
+  const uint8_t* V;
+  int32_t rows;        // of a tile
+  int32_t* idx;
+  const int32_t* slot_of_token;
+  float* partials;     // [gridDim.x][2 * H * d]
+  uint32_t* status;
+};
+
+struct __align__(8) StreamBarriers {
+  uint64_t full[kStreamStages], empty[kStreamStages];
+};
+
+// A wait for a copy or for the other warps; false after the time limit.
+__device__ __forceinline__ bool stream_wait(uint64_t* bar, uint32_t parity) {
+  const uint32_t b = smem_u32(bar);
+  if (mbar_try_wait(b, parity)) return true;
+  const uint64_t t0 = globaltimer_ns();
+  while (!mbar_try_wait(b, parity))
+    if (globaltimer_ns() - t0 > AVGGT_WAIT_LIMIT_NS) return false;
+  return true;
+}
+
+// A wait that ran out: in the status block, where the call has one (the attention that follows then does nothing).
+__device__ __forceinline__ void stream_report(uint32_t* status, int lane) {
+  if (status == nullptr || lane != 0 || atomicCAS(status, 0u, 1u) != 0u) return;
+  status[1] = blockIdx.x;
+  status[2] = 90;
+  status[3] = 0;
+}
+
+// PASSES: chunks of 16 bytes per adding thread (2 * H * 8 of them in a row of K and V).
+template <int PASSES>
+__global__ void __launch_bounds__(kStreamThreads, kStreamBlocks)
+build_kv_stream_kernel(const __grid_constant__ CUtensorMap tm_kc, const __grid_constant__ CUtensorMap tm_vc, const StreamArgs a) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* stages = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~uintptr_t(127));
+  __shared__ StreamBarriers bars;
+  __shared__ uint32_t kept_mask[kStreamStages];
+  __shared__ float red[PASSES == 1 ? kStreamSums * 8 : 1];
+  const Plan& pl = a.pl;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
+  const uint32_t row_bytes = static_cast<uint32_t>(pl.H) * 128u, n_tok = static_cast<uint32_t>(pl.n_tok);
+  const uint32_t rows = a.rows, n_tiles = (n_tok + rows - 1) / rows;
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < kStreamStages; ++s) {
+      mbar_init(smem_u32(&bars.full[s]), 2);
+      mbar_init(smem_u32(&bars.empty[s]), kStreamSums / 32);
+    }
+    fence_mbar_init();
+  }
+  grid_dependency_wait();
+  if (blockIdx.x == 0 && a.status != nullptr && threadIdx.x < kAttnStatusBytes / 4) a.status[threadIdx.x] = 0u;
+  __syncthreads();
+
+  if (warp == kStreamSums / 32) {
+    if (lane == 0 && pl.M > 0) {
+      prefetch_tensormap(&tm_kc);
+      prefetch_tensormap(&tm_vc);
+    }
+    // compact position of the row of tile t that this lane stands for, -1 if it is dropped, -2 if it does not exist
+    const auto position = [&](uint32_t t) {
+      const uint32_t row = t * rows + lane;
+      if (t >= n_tiles || lane >= static_cast<int>(rows) || row >= n_tok) return -2;
+      return a.slot_of_token != nullptr ? __ldcg(a.slot_of_token + row) : compact_position(a.rule, pl, row);
+    };
+    const auto load = [&](uint32_t t, int stage) {
+      if (lane == 0) {
+        const uint32_t row0 = t * rows, n = n_tok - row0 < rows ? n_tok - row0 : rows;
+        const uint32_t fb = smem_u32(&bars.full[stage]), dst = smem_u32(stages + 2 * stage * kStreamBytes);
+        mbar_arrive_expect_tx(fb, 2 * n * row_bytes);
+        bulk_load(dst, a.K + static_cast<size_t>(row0) * row_bytes, n * row_bytes, fb);
+        bulk_load(dst + kStreamBytes, a.V + static_cast<size_t>(row0) * row_bytes, n * row_bytes, fb);
+      }
+    };
+    const auto tell = [&](int stage, int m) {   // the adding warps which rows of the tile are retained; m: the lane's position
+      const uint32_t mask = __ballot_sync(0xffffffffu, m >= 0);
+      if (lane == 0) {
+        kept_mask[stage] = mask;
+        mbar_arrive(smem_u32(&bars.full[stage]));
+      }
+      __syncwarp();
+    };
+    int pos[kStreamStages];   // of the lane's row, by stage
+#pragma unroll
+    for (int s = 0; s < kStreamStages; ++s) {
+      if (blockIdx.x + s * gridDim.x < n_tiles) load(blockIdx.x + s * gridDim.x, s);
+    }
+#pragma unroll
+    for (int s = 0; s < kStreamStages; ++s) {   // under the copies
+      pos[s] = position(blockIdx.x + s * gridDim.x);
+      if (blockIdx.x + s * gridDim.x < n_tiles) tell(s, pos[s]);
+    }
+    bool ok = true;
+    int round = 0;
+    for (uint32_t t0 = blockIdx.x; t0 < n_tiles && ok; t0 += kStreamStages * gridDim.x, ++round) {
+#pragma unroll
+      for (int s = 0; s < kStreamStages; ++s) {
+        const uint32_t t = t0 + s * gridDim.x;
+        if (t >= n_tiles || !ok) break;
+        const uint32_t refill = t + (kStreamStages - 1) * gridDim.x;   // the tile for the stage before this one
+        const int before = s == 0 ? kStreamStages - 1 : s - 1;
+        const bool more = refill < n_tiles && (round > 0 || s > 0);
+        const int next = more ? position(refill) : -2;
+        ok = __all_sync(0xffffffffu, stream_wait(&bars.full[s], round & 1));
+        if (!ok) break;
+        const int m = pos[s];
+        uint32_t mask = __ballot_sync(0xffffffffu, m >= 0);
+        if (m >= 0 && a.idx != nullptr) a.idx[m] = static_cast<int32_t>(t * rows + lane);
+        const uint32_t src = smem_u32(stages + 2 * s * kStreamBytes);
+        while (mask != 0) {
+          const int r = __ffs(mask) - 1;
+          mask &= mask - 1;
+          const int at = __shfl_sync(0xffffffffu, m, r);
+          if (lane == 0) {
+            tma_store_3d(&tm_kc, src + r * row_bytes, 0, 0, at);
+            tma_store_3d(&tm_vc, src + kStreamBytes + r * row_bytes, 0, 0, at);
+          }
+        }
+        if (lane == 0) {
+          bulk_commit();
+          if (more) bulk_wait_read<1>();   // the stores of the tile before this one have read their stage
+        }
+        __syncwarp();
+        if (more) {
+          ok = __all_sync(0xffffffffu, stream_wait(&bars.empty[before], (s == 0 ? round - 1 : round) & 1));
+          if (!ok) break;
+          load(refill, before);
+          tell(before, next);
+          pos[before] = next;
+        }
+      }
+    }
+    if (!ok) {   // a wait ran out: whatever is still on its way arrives before the block gives up its shared memory
+      stream_report(a.status, lane);
+      for (int s = 0; s < kStreamStages; ++s) (void)stream_wait(&bars.full[s], 0), (void)stream_wait(&bars.full[s], 1);
+    }
+    if (lane == 0) bulk_wait_read<0>();   // the stores complete before the kernel does
+    __syncwarp();
+  } else {
+    const int chunks = pl.H * 16, groups = PASSES == 1 ? kStreamSums / chunks : 1;
+    const int group = PASSES == 1 ? static_cast<int>(threadIdx.x) / chunks : 0;
+    const int c0 = PASSES == 1 ? static_cast<int>(threadIdx.x) - group * chunks : static_cast<int>(threadIdx.x);
+    const int half = pl.H * 8;
+    uint64_t run[PASSES][4], sum[PASSES][4];
+    uint32_t at[PASSES];
+#pragma unroll
+    for (int p = 0; p < PASSES; ++p) {
+      const int c = c0 + p * kStreamSums;
+      at[p] = c < half ? c * 16 : kStreamBytes + (c - half) * 16;
+#pragma unroll
+      for (int e = 0; e < 4; ++e) run[p][e] = sum[p][e] = pack_f32x2(0.f, 0.f);
+    }
+    bool ok = true;
+    int stage = 0, since = 0;
+    uint32_t parity = 0;
+    for (uint32_t t = blockIdx.x; t < n_tiles; t += gridDim.x) {
+      ok = __all_sync(0xffffffffu, stream_wait(&bars.full[stage], parity));
+      if (!ok) break;
+      const uint8_t* src = stages + 2 * stage * kStreamBytes;
+      const uint32_t n = n_tok - t * rows < rows ? n_tok - t * rows : rows;
+      const uint32_t kept = kept_mask[stage];
+      if (group < groups) {
+        for (uint32_t r = group; r < n; r += groups) {
+          if ((kept >> r) & 1u) continue;
+#pragma unroll
+          for (int p = 0; p < PASSES; ++p) {
+            if (PASSES > 1 && c0 + p * kStreamSums >= chunks) break;
+            const uint4 v = *reinterpret_cast<const uint4*>(src + at[p] + r * row_bytes);
+            run[p][0] = add_f32x2(run[p][0], unpack_bf16x2(v.x));
+            run[p][1] = add_f32x2(run[p][1], unpack_bf16x2(v.y));
+            run[p][2] = add_f32x2(run[p][2], unpack_bf16x2(v.z));
+            run[p][3] = add_f32x2(run[p][3], unpack_bf16x2(v.w));
+          }
+        }
+      }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(smem_u32(&bars.empty[stage]));
+      if (++stage == kStreamStages) { stage = 0; parity ^= 1; }
+      if (++since == kStreamFlush) {
+        since = 0;
+#pragma unroll
+        for (int p = 0; p < PASSES; ++p)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) { sum[p][e] = add_f32x2(sum[p][e], run[p][e]); run[p][e] = pack_f32x2(0.f, 0.f); }
+      }
+    }
+    float* out = a.partials + static_cast<size_t>(blockIdx.x) * (static_cast<size_t>(chunks) * 8);
+#pragma unroll
+    for (int p = 0; p < PASSES; ++p) {
+      const int c = c0 + p * kStreamSums;
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        float lo, hi;
+        unpack_f32x2(add_f32x2(sum[p][e], run[p][e]), lo, hi);
+        if (!ok) lo = hi = __int_as_float(0x7fffffff);   // a copy that never came shows in the means
+        if (PASSES > 1 || groups == 1) {
+          if (group < groups && c < chunks) *reinterpret_cast<float2*>(out + c * 8 + 2 * e) = make_float2(lo, hi);
+        } else if (group < groups) {
+          red[(group * chunks + c) * 8 + 2 * e] = lo;
+          red[(group * chunks + c) * 8 + 2 * e + 1] = hi;
+        }
+      }
+    }
+  }
+  grid_launch_dependents();
+  __syncthreads();
+  const int cols = pl.H * 128, groups = kStreamSums / (pl.H * 16);
+  if (PASSES == 1 && groups > 1) {   // the groups' sums, in order
+    for (int col = threadIdx.x; col < cols; col += kStreamThreads) {
+      float s = 0.f;
+      for (int g = 0; g < groups; ++g) s += red[g * cols + col];
+      a.partials[static_cast<size_t>(blockIdx.x) * cols + col] = s;
+    }
+  }
+}
+
+// Many tokens, nothing to average: only the retained rows are read.  A block is one warp, which walks over tiles of consecutive compact
+// rows: a bulk copy per row and array (one per array where the tile's tokens are consecutive) into a stage, and a TMA store of the
+// whole tile per array to the head-major places.  HBM is the bound.  Against a warp per token with 16-byte loads: 457,542 tokens of
+// 16 heads, a quarter retained (1.0 GB) 233 -> 171 us (5.8 TB/s), 137,400 tokens all retained 203 -> 185 us (6.1 TB/s), 82,440 tokens, a
+// ninth retained, 21 -> 10 us, 137,400 tokens of 6 heads, a quarter retained, 38 -> 17 us.
+struct GatherArgs {
+  Plan pl;
+  Divisor by_Lc, by_kept_w;
+  const uint8_t* K;
+  const uint8_t* V;
+  int32_t rows;        // of a tile
+  int32_t* idx;
+  const int32_t* caller_idx;   // caller-chosen retained set: token of every compact row; else null
+  uint32_t* status;
+  float* zero_kmean;   // mean pair of a problem that drops nothing, or null
+  float* zero_vmean;
+};
+
+// Token of compact row m by the window rule.
+__device__ __forceinline__ int32_t token_of_compact(const GatherArgs& a, uint32_t m) {
+  const Plan& pl = a.pl;
+  uint32_t f = 0, c = m;
+  if (!pl.keep_first) {
+    f = divide(m, a.by_Lc, c);
+  } else if (m >= static_cast<uint32_t>(pl.L)) {
+    f = 1 + divide(m - static_cast<uint32_t>(pl.L), a.by_Lc, c);
+  } else {
+    return static_cast<int32_t>(m);
+  }
+  const uint32_t n_special = static_cast<uint32_t>(pl.n_special);
+  uint32_t u = c;
+  if (c >= n_special) {
+    uint32_t col;
+    const uint32_t r = divide(c - n_special, a.by_kept_w, col);
+    u = n_special + r * pl.s_h * pl.grid_w + col * pl.s_w;
+  }
+  return static_cast<int32_t>(f * pl.L + u);
+}
+
+__global__ void __launch_bounds__(32)
+build_kv_gather_kernel(const __grid_constant__ CUtensorMap tm_kc, const __grid_constant__ CUtensorMap tm_vc,
+                       const __grid_constant__ CUtensorMap tm_kc_row, const __grid_constant__ CUtensorMap tm_vc_row, const GatherArgs a) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* stages = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~uintptr_t(127));
+  __shared__ __align__(8) uint64_t full[kStreamStages];
+  const Plan& pl = a.pl;
+  const int lane = threadIdx.x;
+  const uint32_t row_bytes = static_cast<uint32_t>(pl.H) * 128u, rows = a.rows, M = static_cast<uint32_t>(pl.M);
+  const uint32_t n_tiles = (M + rows - 1) / rows;
+  if (lane == 0) {
+    for (int s = 0; s < kStreamStages; ++s) mbar_init(smem_u32(&full[s]), 1);
+    fence_mbar_init();
+    if (M > 0) {
+      prefetch_tensormap(&tm_kc);
+      prefetch_tensormap(&tm_vc);
+    }
+  }
+  __syncwarp();
   grid_dependency_wait();
   if (blockIdx.x == 0) {
     // what would otherwise be launches of their own: the status block of the attention that follows, and the mean pair of
     // a problem that drops nothing
-    if (status != nullptr && threadIdx.x < kAttnStatusBytes / 4) status[threadIdx.x] = 0u;
-    if (zero_kmean != nullptr)
-      for (int i = threadIdx.x; i < pl.H * pl.d; i += kBuildThreads) { zero_kmean[i] = 0.f; zero_vmean[i] = 0.f; }
+    if (a.status != nullptr)
+      for (int i = lane; i < static_cast<int>(kAttnStatusBytes / 4); i += 32) a.status[i] = 0u;
+    if (a.zero_kmean != nullptr)
+      for (int i = lane; i < pl.H * pl.d; i += 32) { a.zero_kmean[i] = 0.f; a.zero_vmean[i] = 0.f; }
   }
-
-  float acc_k[PASSES][8], acc_v[PASSES][8];
-#pragma unroll
-  for (int p = 0; p < PASSES; ++p)
-#pragma unroll
-    for (int e = 0; e < 8; ++e) { acc_k[p][e] = 0.f; acc_v[p][e] = 0.f; }
-
-  for (uint32_t row = blockIdx.x * kBuildWarps + warp; row < n_tok; row += warps_total) {
-    const int32_t f = static_cast<int32_t>(row / static_cast<uint32_t>(pl.L));
-    const int32_t u = static_cast<int32_t>(row - static_cast<uint32_t>(f) * static_cast<uint32_t>(pl.L));
-    // compact position within the frame's block by the window rule, or, for a caller-chosen retained set,
-    // the global compact position from the caller's map
-    const int32_t cs = slot_of_token != nullptr ? __ldcg(slot_of_token + row) : compact_slot(pl, f, u);
-    if (cs < 0 && !do_mean) continue;
-    const uint4* krow = K + static_cast<size_t>(row) * chunks_per_row;
-    const uint4* vrow = V + static_cast<size_t>(row) * chunks_per_row;
-    uint4 kv[PASSES], vv[PASSES];
-#pragma unroll
-    for (int p = 0; p < PASSES; ++p) {
-      const uint32_t c = p * 32 + lane;
-      if (c < chunks_per_row) { kv[p] = ld_stream(krow + c); vv[p] = ld_stream(vrow + c); }
-      else { kv[p] = make_uint4(0, 0, 0, 0); vv[p] = make_uint4(0, 0, 0, 0); }
-    }
-    if (cs >= 0) {
-      const int64_t m = slot_of_token != nullptr ? cs : compact_frame_base(pl, f) + cs;
-      if (lane == 0 && idx != nullptr) idx[m] = static_cast<int32_t>(row);
-#pragma unroll
-      for (int p = 0; p < PASSES; ++p) {
-        const uint32_t c = p * 32 + lane;
-        if (c < chunks_per_row) {
-          const size_t dst = (static_cast<size_t>(c >> 3) * static_cast<size_t>(kc_rows) + static_cast<size_t>(m)) * 8u + (c & 7u);
-          Kc[dst] = kv[p];
-          Vc[dst] = vv[p];
-        }
+  // token of the lane's row of tile t; -1 if there is none
+  const auto token = [&](uint32_t t) {
+    const uint32_t m = t * rows + lane;
+    if (t >= n_tiles || lane >= static_cast<int>(rows) || m >= M) return -1;
+    const int32_t tok = a.caller_idx != nullptr ? __ldcg(a.caller_idx + m) : token_of_compact(a, m);
+    return tok < pl.n_tok ? tok : -1;   // (entries of a caller's list that are no token are passed over)
+  };
+  const auto load = [&](int stage, int tok) {
+    const uint32_t have = __ballot_sync(0xffffffffu, tok >= 0);
+    const int tok0 = __shfl_sync(0xffffffffu, tok, 0);
+    const uint32_t fb = smem_u32(&full[stage]), dst = smem_u32(stages + 2 * stage * kStreamBytes);
+    const uint32_t bytes = __popc(have) * row_bytes;
+    if (lane == 0) mbar_arrive_expect_tx(fb, 2 * bytes);
+    __syncwarp();
+    // consecutive tokens, from the first row on
+    if ((have & (have + 1)) == 0 && __all_sync(0xffffffffu, tok < 0 || tok == tok0 + lane)) {
+      if (lane == 0 && have != 0) {
+        bulk_load(dst, a.K + static_cast<size_t>(tok0) * row_bytes, bytes, fb);
+        bulk_load(dst + kStreamBytes, a.V + static_cast<size_t>(tok0) * row_bytes, bytes, fb);
       }
-    } else {
+    } else if (tok >= 0) {
+      bulk_load(dst + lane * row_bytes, a.K + static_cast<size_t>(tok) * row_bytes, row_bytes, fb);
+      bulk_load(dst + kStreamBytes + lane * row_bytes, a.V + static_cast<size_t>(tok) * row_bytes, row_bytes, fb);
+    }
+    __syncwarp();
+  };
+  int toks[kStreamStages];   // of the lane's row, by stage
 #pragma unroll
-      for (int p = 0; p < PASSES; ++p) { add_bf16x8(acc_k[p], kv[p]); add_bf16x8(acc_v[p], vv[p]); }
+  for (int s = 0; s < kStreamStages; ++s) {
+    const uint32_t t = blockIdx.x + s * gridDim.x;
+    toks[s] = token(t);
+    if (t < n_tiles) load(s, toks[s]);
+  }
+  bool ok = true;
+  int round = 0;
+  for (uint32_t t0 = blockIdx.x; t0 < n_tiles && ok; t0 += kStreamStages * gridDim.x, ++round) {
+#pragma unroll
+    for (int s = 0; s < kStreamStages; ++s) {
+      const uint32_t t = t0 + s * gridDim.x;
+      if (t >= n_tiles) break;
+      const uint32_t refill = t + (kStreamStages - 1) * gridDim.x;   // the tile for the stage before this one
+      const int before = s == 0 ? kStreamStages - 1 : s - 1;
+      const bool more = refill < n_tiles && (round > 0 || s > 0);
+      const int next = more ? token(refill) : -1;
+      ok = __all_sync(0xffffffffu, stream_wait(&full[s], round & 1));
+      if (!ok) break;
+      const int tok = toks[s];
+      const uint32_t m0 = t * rows;
+      if (tok >= 0 && a.idx != nullptr) a.idx[m0 + lane] = tok;
+      const uint32_t src = smem_u32(stages + 2 * s * kStreamBytes);
+      uint32_t have = __ballot_sync(0xffffffffu, tok >= 0);
+      if (lane == 0) {
+        if (__popc(have) == static_cast<int>(rows)) {
+          tma_store_3d(&tm_kc, src, 0, 0, m0);
+          tma_store_3d(&tm_vc, src + kStreamBytes, 0, 0, m0);
+        } else {   // the last tile (what follows the retained rows is not this call's), or one with rows passed over
+          for (; have != 0; have &= have - 1) {
+            const int r = __ffs(have) - 1;
+            tma_store_3d(&tm_kc_row, src + r * row_bytes, 0, 0, m0 + r);
+            tma_store_3d(&tm_vc_row, src + kStreamBytes + r * row_bytes, 0, 0, m0 + r);
+          }
+        }
+        bulk_commit();
+        if (more) bulk_wait_read<1>();   // the stores of the tile before this one have read their stage
+      }
+      __syncwarp();
+      if (more) {
+        load(before, next);
+        toks[before] = next;
+      }
     }
   }
-
-  // the next kernel may take its place on the chip while the blocks reduce and end (earlier it would only be in the way)
+  if (!ok) {   // a wait ran out: whatever is still on its way arrives before the block gives up its shared memory
+    stream_report(a.status, lane);
+    for (int s = 0; s < kStreamStages; ++s) (void)stream_wait(&full[s], 0), (void)stream_wait(&full[s], 1);
+  }
+  if (lane == 0) bulk_wait_read<0>();   // the stores complete before the kernel does
+  __syncwarp();
   grid_launch_dependents();
-  if (!do_mean) return;
-  // block reduction, K then V, fixed order over warps
-  const int cols = pl.H * pl.d;   // = chunks_per_row * 8
-#pragma unroll
-  for (int which = 0; which < 2; ++which) {
-    float* mine = red + warp * (PASSES * 256);
-#pragma unroll
-    for (int p = 0; p < PASSES; ++p)
-#pragma unroll
-      for (int e = 0; e < 8; ++e) mine[(p * 32 + lane) * 8 + e] = which == 0 ? acc_k[p][e] : acc_v[p][e];
-    __syncthreads();
-    for (int col = threadIdx.x; col < cols; col += kBuildThreads) {
-      float s = 0.f;
-#pragma unroll
-      for (int w = 0; w < kBuildWarps; ++w) s += red[w * (PASSES * 256) + col];
-      partials[static_cast<size_t>(blockIdx.x) * (2 * cols) + which * cols + col] = s;
-    }
-    __syncthreads();
-  }
 }
 
 // The same for few tokens, in one launch: a cluster of thread blocks takes one head of K or of V, each block every
@@ -143,13 +436,11 @@ build_kv_kernel(const Plan pl, const uint4* K, const uint4* V, uint4* __restrict
 constexpr int kSmallThreads = 1024;
 constexpr int kSmallRows = kSmallThreads / 8;   // rows a block reads at once
 
-// Up to so many tokens per block of a cluster.  Above, the bytes are the bound, which more blocks per SM and warps that read
-// whole rows serve better.  The two kernels' times in us, this one first (148 SMs): 16 heads, clusters of 4, limit 5,760:
-// 4.5 and 6.2 at 1,374 tokens, 7.9 and 10.4 at 4,122, 10.3 and 12.0 at 5,496, 16.2 and 14.1 at 8,244.  6 heads, clusters of 8,
-// limit 11,520: 4.2 and 4.9 at 1,374, 6.0 and 8.8 at 5,496, 9.1 and 11.3 at 10,992, 19.8 and 17.9 at 21,984.  24 heads, clusters
-// of 2, limit 2,880: 5.9 and 8.6 at 1,374.  Of 261 tokens and up to 8 heads it is 0.4 us slower (3.7 and 3.3) and saves
-// the host a launch.
-constexpr int64_t kSmallTokensPerBlock = 1440;
+// Up to so many tokens per block of a cluster.  Above, the bytes are the bound.  Times in us, this kernel first, then
+// build_kv_stream_kernel with its reduction (148 SMs): 16 heads, clusters of 4, limit 4,400: 4.5 and 5.4 at 1,374 tokens, 7.0 and 7.0 at
+// 4,122, 8.1 and 7.5 at 5,496, 15.3 and 9.8 at 10,992.  6 heads, clusters of 8, limit 8,800: 4.2 and 5.1 at 1,374, 6.0 and 6.0 at 5,496,
+// 7.1 and 7.5 at 8,244, 8.2 and 7.7 at 10,992.  24 heads, clusters of 2, limit 2,200: 5.8 and 6.0 at 1,374, 8.1 and 7.0 at 2,748.
+constexpr int64_t kSmallTokensPerBlock = 1100;
 
 struct SmallArgs {
   Plan pl;
@@ -246,8 +537,17 @@ mean_finalize_kernel(const float* partials, int n_blocks, int cols2, float inv_c
   const int c = threadIdx.x & 31, g = threadIdx.x >> 5;
   const int col = blockIdx.x * 32 + c;
   float s = 0.f;
-  if (col < cols2)
-    for (int b = g; b < n_blocks; b += 32) s += __ldcg(partials + static_cast<size_t>(b) * cols2 + col);
+  if (col < cols2) {
+    constexpr int kAhead = 10;   // 296 blocks in one go: the loads wait for one another otherwise
+    for (int b0 = g; b0 < n_blocks; b0 += 32 * kAhead) {
+      float part[kAhead];
+#pragma unroll
+      for (int i = 0; i < kAhead; ++i)
+        part[i] = b0 + 32 * i < n_blocks ? __ldcg(partials + static_cast<size_t>(b0 + 32 * i) * cols2 + col) : 0.f;
+#pragma unroll
+      for (int i = 0; i < kAhead; ++i) s += part[i];
+    }
+  }
   tile[c][g] = s;
   __syncthreads();
   // warp g now owns column blockIdx.x*32 + g; lane c holds the partial of group c
@@ -280,18 +580,80 @@ __global__ void scatter_slots_kernel(const int32_t* idx, int64_t M, int32_t* __r
   }
 }
 
-template <int PASSES>
-cudaError_t launch_build(const Plan& pl, int grid, const void* K, const void* V, void* Kc, void* Vc, int64_t kc_rows,
-                         int32_t* idx, float* partials, int do_mean, const int32_t* slot_of_token, uint32_t* status,
-                         float* zero_kmean, float* zero_vmean, cudaStream_t st) {
-  const size_t smem = do_mean ? static_cast<size_t>(kBuildWarps) * PASSES * 256 * sizeof(float) : 0;
-  if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(build_kv_kernel<PASSES>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+int stream_rows(const Plan& pl) {
+  const int rows = static_cast<int>(kStreamBytes) / (pl.H * 128);
+  return rows < kStreamRows ? rows : kStreamRows;
+}
+
+// Once per device: the dynamic shared-memory limit.
+cudaError_t prepare_stream_kernels() {
+  static std::mutex mu;
+  static bool ready[64] = {};
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+  std::lock_guard<std::mutex> lock(mu);
+  if (ready[dev]) return cudaSuccess;
+  for (const void* kernel : {reinterpret_cast<const void*>(build_kv_stream_kernel<1>), reinterpret_cast<const void*>(build_kv_stream_kernel<2>),
+                             reinterpret_cast<const void*>(build_kv_gather_kernel)}) {
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kStreamSmemBytes));
     if (e != cudaSuccess) return e;
   }
-  return launch_dependent(build_kv_kernel<PASSES>, grid, kBuildThreads, smem, st, pl, static_cast<const uint4*>(K),
-                          static_cast<const uint4*>(V), static_cast<uint4*>(Kc), static_cast<uint4*>(Vc), kc_rows, idx, partials,
-                          do_mean, slot_of_token, status, zero_kmean, zero_vmean);
+  ready[dev] = true;
+  return cudaSuccess;
+}
+
+// The compact arrays as [kc_rows, H, d]: a box is all heads of `rows` rows.
+bool make_compact_tmap(CUtensorMap* tm, const Plan& pl, void* base, int64_t kc_rows, int rows) {
+  const uint64_t dims[3] = {static_cast<uint64_t>(pl.d), static_cast<uint64_t>(pl.H), static_cast<uint64_t>(kc_rows)};
+  const uint64_t strides[2] = {static_cast<uint64_t>(kc_rows) * pl.d * 2, static_cast<uint64_t>(pl.d) * 2};
+  const uint32_t box[3] = {static_cast<uint32_t>(pl.d), static_cast<uint32_t>(pl.H), static_cast<uint32_t>(rows)};
+  return make_tmap_bf16(tm, base, 3, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_NONE);
+}
+
+cudaError_t launch_stream(const Plan& pl, int grid, const void* K, const void* V, void* Kc, void* Vc, int64_t kc_rows, int32_t* idx,
+                          float* partials, const int32_t* slot_of_token, uint32_t* status, cudaStream_t st) {
+  StreamArgs a;
+  a.pl = pl;
+  a.rule = make_window_rule(pl);
+  a.K = static_cast<const uint8_t*>(K);
+  a.V = static_cast<const uint8_t*>(V);
+  a.rows = stream_rows(pl);
+  a.idx = idx;
+  a.slot_of_token = slot_of_token;
+  a.partials = partials;
+  a.status = status;
+  CUtensorMap tm_kc = {}, tm_vc = {};
+  if (kc_rows > 0 && !(make_compact_tmap(&tm_kc, pl, Kc, kc_rows, 1) && make_compact_tmap(&tm_vc, pl, Vc, kc_rows, 1)))
+    return cudaErrorInvalidValue;
+  const cudaError_t e = prepare_stream_kernels();
+  if (e != cudaSuccess) return e;
+  return launch_dependent(pl.H <= 16 ? build_kv_stream_kernel<1> : build_kv_stream_kernel<2>, grid, kStreamThreads, kStreamSmemBytes, st,
+                          tm_kc, tm_vc, a);
+}
+
+cudaError_t launch_gather(const Plan& pl, int grid, const void* K, const void* V, void* Kc, void* Vc, int64_t kc_rows, int32_t* idx,
+                          const int32_t* caller_idx, uint32_t* status, float* zero_kmean, float* zero_vmean, cudaStream_t st) {
+  GatherArgs a;
+  a.pl = pl;
+  a.by_Lc = make_divisor(pl.Lc > 0 ? pl.Lc : 1);
+  a.by_kept_w = make_divisor(pl.kept_w);
+  a.K = static_cast<const uint8_t*>(K);
+  a.V = static_cast<const uint8_t*>(V);
+  a.rows = stream_rows(pl);
+  a.idx = idx;
+  a.caller_idx = caller_idx;
+  a.status = status;
+  a.zero_kmean = zero_kmean;
+  a.zero_vmean = zero_vmean;
+  CUtensorMap tm_kc = {}, tm_vc = {}, tm_kc_row = {}, tm_vc_row = {};
+  if (kc_rows > 0 && !(make_compact_tmap(&tm_kc, pl, Kc, kc_rows, a.rows) && make_compact_tmap(&tm_vc, pl, Vc, kc_rows, a.rows) &&
+                       make_compact_tmap(&tm_kc_row, pl, Kc, kc_rows, 1) && make_compact_tmap(&tm_vc_row, pl, Vc, kc_rows, 1)))
+    return cudaErrorInvalidValue;
+  const cudaError_t e = prepare_stream_kernels();
+  if (e != cudaSuccess) return e;
+  return launch_dependent(build_kv_gather_kernel, grid, 32, kStreamSmemBytes, st, tm_kc, tm_vc, tm_kc_row, tm_vc_row, a);
 }
 
 // Exchange buffer [n_ranks][2][H][slot_rows][d] (every rank's compact K then V, padded to slot_rows rows per
@@ -355,16 +717,14 @@ int small_ranks(const Plan& pl, int sm_count) {
   return ranks;
 }
 
-int build_passes(const Plan& pl) { return (pl.H * 8 + 31) / 32; }
+int build_kv_blocks_per_sm() { return kStreamBlocks; }
 
-int build_kv_blocks_per_sm(const Plan& pl) { return kBuildBlocks[build_passes(pl)]; }
-
+// Blocks of build_kv_stream_kernel; build_kv_gather_kernel has as many.
 int build_kv_grid(const Plan& pl, int sm_count) {
-  const int64_t by_rows = (pl.n_tok + kBuildWarps - 1) / kBuildWarps;
-  int64_t g = static_cast<int64_t>(sm_count) * build_kv_blocks_per_sm(pl);
-  if (g > by_rows) g = by_rows;
-  if (g < 1) g = 1;
-  return static_cast<int>(g);
+  const int rows = stream_rows(pl);
+  const int64_t tiles = (pl.n_tok + rows - 1) / rows;
+  const int64_t most = static_cast<int64_t>(sm_count) * build_kv_blocks_per_sm();
+  return static_cast<int>(tiles < most ? tiles : most);
 }
 
 size_t build_kv_ws_bytes(const Plan& pl, int sm_count) {
@@ -410,19 +770,8 @@ cudaError_t launch_build_kv(const Plan& pl, int sm_count, const void* K, const v
   const bool zero_mean = pl.mean_fill != 0 && !do_mean;
   float* zk = zero_mean ? kmean : nullptr;
   float* zv = zero_mean ? vmean : nullptr;
-  const int passes = build_passes(pl);
-  cudaError_t e;
-  switch (passes) {
-    case 1: e = launch_build<1>(pl, grid, K, V, Kc, Vc, kc_rows, idx, partials, do_mean, slot_of_token, status, zk, zv, st); break;
-    case 2: e = launch_build<2>(pl, grid, K, V, Kc, Vc, kc_rows, idx, partials, do_mean, slot_of_token, status, zk, zv, st); break;
-    case 3: e = launch_build<3>(pl, grid, K, V, Kc, Vc, kc_rows, idx, partials, do_mean, slot_of_token, status, zk, zv, st); break;
-    case 4: e = launch_build<4>(pl, grid, K, V, Kc, Vc, kc_rows, idx, partials, do_mean, slot_of_token, status, zk, zv, st); break;
-    case 5: e = launch_build<5>(pl, grid, K, V, Kc, Vc, kc_rows, idx, partials, do_mean, slot_of_token, status, zk, zv, st); break;
-    case 6: e = launch_build<6>(pl, grid, K, V, Kc, Vc, kc_rows, idx, partials, do_mean, slot_of_token, status, zk, zv, st); break;
-    case 7: e = launch_build<7>(pl, grid, K, V, Kc, Vc, kc_rows, idx, partials, do_mean, slot_of_token, status, zk, zv, st); break;
-    case 8: e = launch_build<8>(pl, grid, K, V, Kc, Vc, kc_rows, idx, partials, do_mean, slot_of_token, status, zk, zv, st); break;
-    default: return cudaErrorInvalidValue;
-  }
+  const cudaError_t e = do_mean ? launch_stream(pl, grid, K, V, Kc, Vc, kc_rows, idx, partials, slot_of_token, status, st)
+                                : launch_gather(pl, grid, K, V, Kc, Vc, kc_rows, idx, caller_idx, status, zk, zv, st);
   if (e != cudaSuccess || !do_mean) return e;
   const int cols2 = 2 * pl.H * pl.d;
   const float inv_count = sums_only ? 1.0f : 1.0f / static_cast<float>(pl.n_dropped);

@@ -87,7 +87,7 @@ extern "C" int avggt_build_kv_noalloc(const avggt_params* p, const void* K, cons
   // The compaction kernel runs a fixed number of blocks per SM it is told about; telling it about fewer SMs
   // keeps its partial rows within the fixed array.
   int sm_eff = di.sm_count;
-  const int most = kStaticMaxBlocks / build_kv_blocks_per_sm(pl);
+  const int most = kStaticMaxBlocks / build_kv_blocks_per_sm();
   if (sm_eff > most) sm_eff = most;
   if (build_kv_ws_bytes(pl, sm_eff) > kStaticScratchBytes) return AVGGT_ERR_STATIC_SCRATCH;
   return record_cuda(launch_build_kv(pl, sm_eff, K, V, Kc, Vc, idx, kmean, vmean, pd->scratch,

@@ -921,9 +921,6 @@ __device__ __forceinline__ void ld_rows16(uint32_t addr, uint32_t (&r)[4]) {
 __device__ __forceinline__ void st_rows16(uint32_t addr, uint32_t r0, uint32_t r1, uint32_t r2, uint32_t r3) {
   asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(r0), "r"(r1), "r"(r2), "r"(r3) : "memory");
 }
-__device__ __forceinline__ uint64_t unpack_bf16x2(uint32_t w) {
-  return pack_f32x2(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u));
-}
 
 // Epilogue of a work item: diagonal and mean-fill terms, normalisation, store of the warp's 16 rows.  n: the item's number in this
 // CTA, last: the tile's latest key step, the item's last.

@@ -52,7 +52,7 @@ cudaError_t launch_clear_status(void* status, cudaStream_t st);
 
 // ---- K/V compaction (build_kv.cu)
 int build_kv_grid(const Plan& pl, int sm_count);
-int build_kv_blocks_per_sm(const Plan& pl);
+int build_kv_blocks_per_sm();
 size_t build_kv_ws_bytes(const Plan& pl, int sm_count);
 // caller_idx / slot_of_token: both null for the window rule of Sec. 4.3; for a caller-chosen retained set,
 // the M retained token indices (device) and the [n_tok] map the call fills (device).

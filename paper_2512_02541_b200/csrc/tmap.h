@@ -25,9 +25,10 @@ inline EncodeTiledFn encode_tiled_fn() {
 
 // bf16 tensor of up to 3 dimensions, innermost first.  dims[i] elements,
 // strides_bytes[i] = byte stride of dimension i+1 (i < rank-1), box[i] elements.
-// 128-byte swizzle, zero fill outside the tensor.  Returns false on failure.
+// Zero fill outside the tensor.  Returns false on failure.
 inline bool make_tmap_bf16(CUtensorMap* out, const void* base, int rank, const uint64_t* dims,
-                           const uint64_t* strides_bytes, const uint32_t* box) {
+                           const uint64_t* strides_bytes, const uint32_t* box,
+                           CUtensorMapSwizzle swizzle = CU_TENSOR_MAP_SWIZZLE_128B) {
   EncodeTiledFn fn = encode_tiled_fn();
   if (!fn) return false;
   cuuint64_t gdim[3];
@@ -37,7 +38,7 @@ inline bool make_tmap_bf16(CUtensorMap* out, const void* base, int rank, const u
   for (int i = 0; i < rank; ++i) { gdim[i] = dims[i]; bx[i] = box[i]; }
   for (int i = 0; i + 1 < rank; ++i) gstr[i] = strides_bytes[i];
   CUresult r = fn(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, static_cast<cuuint32_t>(rank), const_cast<void*>(base), gdim,
-                  gstr, bx, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                  gstr, bx, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle,
                   CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS;
 }

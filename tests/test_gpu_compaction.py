@@ -1,5 +1,5 @@
-"""The two compaction kernels (few tokens: a cluster of thread blocks per head; many: a warp per row) over the head counts that
-select their variants, against the oracle: bit copies, indices, and the mean pair."""
+"""The compaction kernels (few tokens: a cluster of thread blocks per head; many, with a mean: tiles of tokens; without: tiles of compact
+rows) over the head counts that select their variants, against the oracle: bit copies, indices, and the mean pair."""
 
 import pytest
 import torch
@@ -12,8 +12,9 @@ from test_gpu_parity import _cfgs, _check_build
 pytestmark = pytest.mark.gpu
 
 
-# 1 to 8 chunks of 16 bytes per lane and row in the many-token kernel; clusters of 8, 4, 2 blocks in the other, whose
-# limit lies at 11,520 tokens for up to 6 heads, 5,760 up to 18, 2,880 above; 12,300 and 1,230 tokens, not a multiple of any group
+# 16 to 1 groups of adding threads and one or two chunks per thread in the many-token kernel, tiles of 4 to 32 rows; clusters of 8, 4, 2
+# blocks in the few-token kernel, whose limit lies at 8,800 tokens for up to 6 heads, 4,400 up to 18, 2,200 above; 12,300 and 1,230 tokens,
+# not a multiple of any group
 @pytest.mark.parametrize("heads", (1, 3, 6, 7, 8, 12, 16, 19, 24, 28, 32))
 @pytest.mark.parametrize("n_frames", (3, 30))
 @pytest.mark.parametrize("mean_fill,keep_first", [(2, 1), (0, 0)])
@@ -49,3 +50,41 @@ def test_nothing_dropped(n_frames):
     assert not layer.kmean.any() and not layer.vmean.any() and not sums.any()
     assert torch.equal(slot[0, :, :layer.M], layer.Kc) and torch.equal(slot[1, :, :layer.M], layer.Vc)
     assert torch.isnan(slot[:, :, layer.M:].float()).all()
+
+
+# Tiles of 8 tokens (16 heads) or 4 (32), 296 blocks, three tiles in flight in each: token counts around a tile, around the tiles of all
+# blocks together, and around the ring; with a mean and, over the compact rows, without
+@pytest.mark.parametrize("heads,n_tok", [(16, t) for t in (4401, 4409, 4736 * 8 - 1, 7104, 7105, 7111)] + [(32, 2201), (32, 3 * 1184 + 5)])
+@pytest.mark.parametrize("sigma,mean_fill", [(4, 2), (4, 0), (1, 2)])
+def test_tokens_around_a_tile(heads, n_tok, sigma, mean_fill):
+    wl = inputs.Workload("tiles", 1, 3, (n_tok - 2) // 3, 2 + (n_tok - 2) % 3, heads, 64, sigma, 1, mean_fill, "iid")
+    assert wl.n_tokens == n_tok
+    params, ocfg = _cfgs(wl)
+    _, K, V = inputs.make_qkv(wl, seed=n_tok, device="cuda")
+    layer = P.SubsampledGlobalAttention(params)
+    for t in (layer.Kc, layer.Vc, layer.kmean, layer.vmean):
+        t.fill_(float("nan"))
+    layer.idx.fill_(-1)
+    layer.build_kv(K, V)
+    torch.cuda.synchronize()
+    _check_build(ocfg, layer, K, V)
+
+
+def test_a_list_with_entries_that_are_no_token():
+    """Their compact rows are left as they were; without a mean the list itself says what is read."""
+    wl = inputs.Workload("listed", 4, 37, 37, 5, 16, 64, 4, 1, 0, "iid")
+    params, _ = _cfgs(wl)
+    _, K, V = inputs.make_qkv(wl, seed=1, device="cuda")
+    for n_kept in (5, 64, 701):
+        idx = torch.sort(torch.randperm(wl.n_tokens, device="cuda")[:n_kept]).values.to(torch.int32)
+        idx[-1] = wl.n_tokens + 3
+        idx[0] = -1
+        Kc, Vc = (torch.full((wl.n_heads, n_kept, 64), 7.0, dtype=torch.bfloat16, device="cuda") for _ in range(2))
+        slots = torch.empty((wl.n_tokens,), dtype=torch.int32, device="cuda")
+        ws = torch.empty((P.avggt_workspace_bytes(params)[0],), dtype=torch.uint8, device="cuda")
+        P.avggt_build_kv_indexed(params, idx, n_kept, K, V, Kc, Vc, slots, None, None, ws, ws.numel())
+        torch.cuda.synchronize()
+        kept = idx[1:-1].long()
+        for full, compact in ((K, Kc), (V, Vc)):
+            assert torch.equal(compact[:, 1:-1], full[kept].transpose(0, 1))
+            assert (compact[:, 0] == 7).all() and (compact[:, -1] == 7).all()
