@@ -20,7 +20,7 @@
 //   warps 17-18 MMA issuers, one per query tile: S_t = Q_t Kc_j^T and
 //               O_t += P_t Vc_j with tcgen05.mma, bf16 operands, fp32
 //               accumulators in tensor memory
-//   warp  19    idle (it completes the fifth warpgroup so that registers can
+//   warp  19    allocates tensor memory (and completes the fifth warpgroup so that registers can
 //               be moved to the softmax warpgroups)
 // Tensor memory per tile (256 columns): two places for S and P that alternate (see kColSOdd), O (64) and the row
 // sums of P (16).  A softmax thread pulls its 56 scores of S into registers and the warp frees its rows at once,
@@ -31,6 +31,7 @@
 // diagonal and the mean-fill column into the same normalisation:
 //   O = (a_S O_S + p_d v_i + p_m vmean) / (a_S l_S + p_d + p_m).
 #include <cmath>
+#include <cstddef>
 #include <mutex>
 
 #include <cuda_bf16.h>
@@ -63,6 +64,7 @@ constexpr int kThreads = 640;
 constexpr int kSoftmaxWarps = 16;
 constexpr int kTmaWarp = 16;
 constexpr int kMmaWarp = 17;
+constexpr int kTmemWarp = 19;
 constexpr uint32_t kTmemCols = 512;
 // Tensor memory of a query tile (256 columns): scores and probabilities of the even steps of the tile, S at 0 and P at 0
 // (over the scores it was computed from); of the odd steps, S at 64 and P at 112; O at 176, the row sums of P at 240.
@@ -132,26 +134,47 @@ struct AttnArgs {
 // one step per item, may still be before the epilogue of item n - 4.
 constexpr int kInfos = 8;
 
+// Ordered by the arrivals that a phase counts, so that as many threads can initialise them at once (init_barriers).
 struct __align__(8) Barriers {
+  // one arrival
   uint64_t q_full[2];          // producer -> MMA: the work item's Q tiles are in shared memory (items take the two places in turn)
-  uint64_t q_empty[2];         // MMA issuers -> producer: every Q K^T of the work item has completed; with extra columns, softmax ->
-                               // producer as well: the epilogue has read Q.  Q may be overwritten
-  uint64_t o_free[kQTiles];    // softmax -> MMA: O_t of the finished work item has been read out
-  uint64_t k_full[kStages], k_empty[kStages];
-  uint64_t v_full[kStages], v_empty[kStages];
+  uint64_t k_full[kStages], v_full[kStages];
   uint64_t s_full[kQTiles];    // MMA -> softmax: S_t(j) is in tensor memory
-  uint64_t s_free[kQTiles];    // softmax -> MMA: S_t(j) has been read into registers
-  uint64_t p_full[kQTiles][2]; // softmax -> MMA: P_t(j) stored (and O_t rescaled); even and odd steps apart, since a warp may
-                               // have finished a step before another warp of its tile has finished the step before
   uint64_t o_done[kQTiles][2]; // MMA -> softmax: P_t(j) V_j has completed; even and odd steps apart, since the softmax learns of
                                // P V of step j-2 from the scores of step j only, and of later ones here
   uint64_t info_full[kInfos];  // producer -> softmax: the item's record is in shared memory
   uint64_t own_full;           // producer -> softmax: the item's own rows of K and V and the mean pair are in shared memory
-  uint64_t own_empty;          // softmax -> producer: its epilogue has read them
   uint64_t mma_idle[kQTiles];  // MMA issuer t -> itself: every tcgen05.mma it issued has completed
+  // one of each tile's issuer
+  uint64_t k_empty[kStages], v_empty[kStages];
+  // one of each of a tile's softmax warps
+  uint64_t o_free[kQTiles];    // softmax -> MMA: O_t of the finished work item has been read out
+  uint64_t s_free[kQTiles];    // softmax -> MMA: S_t(j) has been read into registers
+  uint64_t p_full[kQTiles][2]; // softmax -> MMA: P_t(j) stored (and O_t rescaled); even and odd steps apart, since a warp may
+                               // have finished a step before another warp of its tile has finished the step before
+  // one of each softmax warp
+  uint64_t own_empty;          // softmax -> producer: its epilogue has read the own rows
+  // of the issuers, where there are keys, and with extra columns of the softmax warps
+  uint64_t q_empty[2];         // MMA issuers -> producer: every Q K^T of the work item has completed; with extra columns, softmax ->
+                               // producer as well: the epilogue has read Q.  Q may be overwritten
   uint32_t tmem_base;
   uint32_t abort_flag;
 };
+// A thread each: one thread alone takes 400 clocks for them.
+template <bool kExtra>
+__device__ __forceinline__ void init_barriers(Barriers* bars, const AttnArgs& a, int tid) {
+  constexpr int kSize = sizeof(uint64_t);
+  constexpr int kTwo = offsetof(Barriers, k_empty) / kSize, kTile = offsetof(Barriers, o_free) / kSize,
+                kAll = offsetof(Barriers, own_empty) / kSize, kQ = offsetof(Barriers, q_empty) / kSize;
+  static_assert(kAll + 1 == kQ && kQ + 2 == offsetof(Barriers, tmem_base) / kSize, "order of the barriers");
+  if (tid < kQ + 2) {
+    const uint32_t count = tid < kTwo ? 1 : tid < kTile ? kQTiles : tid < kAll ? kSoftmaxWarps / kQTiles : tid < kQ ? kSoftmaxWarps
+                           : (a.n_kv_tiles > 0 ? kQTiles : 0) + (kExtra ? kSoftmaxWarps : 0);
+    mbar_init(smem_u32(bars) + tid * kSize, count);
+    fence_mbar_init();
+  }
+  if (tid == 0) bars->abort_flag = 0;
+}
 
 __device__ __forceinline__ void report_timeout(const AttnArgs& a, Barriers* bars, uint32_t where, uint32_t iter) {
   if (atomicCAS(a.status, 0u, 1u) == 0u) {
@@ -322,18 +345,9 @@ __device__ __forceinline__ bool tile_has_rows(const AttnArgs& a, uint32_t item) 
 template <bool kShortLast>
 __device__ __forceinline__ void producer_role(const CUtensorMap* tm_q, const CUtensorMap* tm_k, const CUtensorMap* tm_v,
                                               const CUtensorMap* tm_own_k, const CUtensorMap* tm_own_v, const AttnArgs& a, Barriers* bars,
-                                              ItemInfo* infos, const SmemLayout& sm) {
+                                              ItemInfo* infos, const SmemLayout& sm, WorkItem wi, QueryTile tile0, QueryTile tile1) {
   constexpr bool kExtra = !kShortLast;
   const int n_kv = a.n_kv_tiles;   // 0 where there are no retained keys
-  if (elect_one()) {
-    prefetch_tensormap(tm_q);
-    prefetch_tensormap(tm_k);
-    prefetch_tensormap(tm_v);
-    if (kExtra) {
-      prefetch_tensormap(tm_own_k);
-      prefetch_tensormap(tm_own_v);
-    }
-  }
   int k_issued = 0, v_issued = 0;   // K / V copies issued so far, over all work items
   int stage = 0;
   uint32_t empty_parity = 1;   // a fresh barrier passes the wait on the "previous" phase at once
@@ -342,10 +356,34 @@ __device__ __forceinline__ void producer_role(const CUtensorMap* tm_q, const CUt
   int q_issued = 0;            // work items whose Q copies have been issued
   int own_issued = 0;          // ... whose own rows' copies have been issued
   for (uint32_t item = blockIdx.x; item < static_cast<uint32_t>(a.n_work) && ok; item += gridDim.x, ++n_done) {
-    const WorkItem wi = work_item<kShortLast>(a, item);
+    const uint32_t failed = *reinterpret_cast<volatile uint32_t*>(a.status);
+    if (n_done > 0) {
+      wi = work_item<kShortLast>(a, item);
+      tile0 = query_tile(a, wi, 0);
+      tile1 = query_tile(a, wi, 1);
+    }
     const int head = wi.head;
     const int place = n_done & 1;
-    const QueryTile tile[kQTiles] = {query_tile(a, wi, 0), query_tile(a, wi, 1)};
+    const QueryTile tile[kQTiles] = {tile0, tile1};
+    // the Q tiles of the work item before the last one are no longer read by any Q K^T
+    ok = wait_bar_warp(&bars->q_empty[place], ((n_done >> 1) & 1) ^ 1, bars, a, 14, n_done);
+    if (!ok) break;
+    if (elect_one()) {
+      const uint32_t qb = smem_u32(&bars->q_full[place]);
+      mbar_arrive_expect_tx(qb, kQTiles * kTileBytes);
+#pragma unroll
+      for (int t = 0; t < kQTiles; ++t)
+        tma_load_2d(smem_u32(sm.q + (place * kQTiles + t) * kTileBytes), tm_q, head * kHeadDim, tile[t].q0, qb);
+    }
+    __syncwarp();
+    ++q_issued;
+    // A wait has run out in another thread block (or had before this one began): the launch is abandoned.  Looked at here because
+    // the word takes some 700 clocks to come, which a launch of a single item would wait for.
+    if (__any_sync(kFullMask, failed != 0u)) {
+      *reinterpret_cast<volatile uint32_t*>(&bars->abort_flag) = 1u;
+      ok = false;
+      break;
+    }
     if (elect_one()) {
       ItemInfo& info = infos[n_done % kInfos];
       info.head = head;
@@ -360,24 +398,6 @@ __device__ __forceinline__ void producer_role(const CUtensorMap* tm_q, const CUt
       mbar_arrive(smem_u32(&bars->info_full[n_done % kInfos]));
     }
     __syncwarp();
-    // a wait has run out in another thread block: the launch is abandoned
-    if (n_done > 0 && __any_sync(kFullMask, *reinterpret_cast<volatile uint32_t*>(a.status) != 0u)) {
-      *reinterpret_cast<volatile uint32_t*>(&bars->abort_flag) = 1u;
-      ok = false;
-      break;
-    }
-    // the Q tiles of the work item before the last one are no longer read by any Q K^T
-    ok = wait_bar_warp(&bars->q_empty[place], ((n_done >> 1) & 1) ^ 1, bars, a, 14, n_done);
-    if (!ok) break;
-    if (elect_one()) {
-      const uint32_t qb = smem_u32(&bars->q_full[place]);
-      mbar_arrive_expect_tx(qb, kQTiles * kTileBytes);
-#pragma unroll
-      for (int t = 0; t < kQTiles; ++t)
-        tma_load_2d(smem_u32(sm.q + (place * kQTiles + t) * kTileBytes), tm_q, head * kHeadDim, tile[t].q0, qb);
-    }
-    __syncwarp();
-    ++q_issued;
     for (int it = 0; it < n_kv; ++it) {
       ok = wait_bar_warp(&bars->k_empty[stage], empty_parity, bars, a, 10, it);
       if (!ok) break;
@@ -1227,53 +1247,46 @@ global_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
 
   const int tid = threadIdx.x;
   const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // warp-uniform by construction
-  if (tid == 0) {
-    for (int e = 0; e < 2; ++e) {
-      mbar_init(smem_u32(&bars.q_full[e]), 1);
-      mbar_init(smem_u32(&bars.q_empty[e]), (a.n_kv_tiles > 0 ? kQTiles : 0) + (kExtra ? kSoftmaxWarps : 0));
-    }
-    for (int e = 0; e < kInfos; ++e) mbar_init(smem_u32(&bars.info_full[e]), 1);
-    mbar_init(smem_u32(&bars.own_full), 1);
-    mbar_init(smem_u32(&bars.own_empty), kSoftmaxWarps);
-    for (int s = 0; s < kStages; ++s) {
-      mbar_init(smem_u32(&bars.k_full[s]), 1);
-      mbar_init(smem_u32(&bars.k_empty[s]), kQTiles);
-      mbar_init(smem_u32(&bars.v_full[s]), 1);
-      mbar_init(smem_u32(&bars.v_empty[s]), kQTiles);
-    }
-    for (int t = 0; t < kQTiles; ++t) {
-      mbar_init(smem_u32(&bars.s_full[t]), 1);
-      mbar_init(smem_u32(&bars.s_free[t]), kSoftmaxWarps / kQTiles);
-      for (int e = 0; e < 2; ++e) {
-        mbar_init(smem_u32(&bars.p_full[t][e]), kSoftmaxWarps / kQTiles);
-        mbar_init(smem_u32(&bars.o_done[t][e]), 1);
-      }
-      mbar_init(smem_u32(&bars.mma_idle[t]), 1);
-      mbar_init(smem_u32(&bars.o_free[t]), kSoftmaxWarps / kQTiles);
-    }
-    bars.abort_flag = 0;
-    fence_mbar_init();
-  }
-  if (warp == kTmaWarp) {
+  init_barriers<kExtra>(&bars, a, tid);
+  if (warp == kTmemWarp) {
     tmem_alloc(smem_u32(&bars.tmem_base), kTmemCols);
     tmem_relinquish();
   }
-  ones_block(sm.ones, tid);
+  // The first item is found while other warps prepare the rest (found after them, behind a read of the status word and with one thread
+  // initialising the barriers, the first key step came 2,000 clocks later: 4 frames of 16 x 16 16.8 -> 15.8 us, one frame of 37 x 37
+  // 16.6 -> 15.6 us).
+  WorkItem wi = {};
+  QueryTile tile0 = {}, tile1 = {};
+  if (warp == kTmaWarp) {
+    wi = work_item<!kExtra>(a, blockIdx.x);
+    tile0 = query_tile(a, wi, 0);
+    tile1 = query_tile(a, wi, 1);
+    if (elect_one()) {
+      prefetch_tensormap(&tm_q);
+      prefetch_tensormap(&tm_k);
+      prefetch_tensormap(&tm_v);
+      if (kExtra) {
+        prefetch_tensormap(&tm_own_k);
+        prefetch_tensormap(&tm_own_v);
+      }
+    }
+    __syncwarp();
+  } else if (warp < kSoftmaxWarps) {
+    ones_block(sm.ones, tid);
+  }
   // everything above may run while the kernel before this one ends
   grid_dependency_wait();
   tc_fence_before();
-  // a launch in which a wait has already run out is abandoned: the remaining CTAs leave at once
-  const bool abandoned = __syncthreads_or(*reinterpret_cast<volatile uint32_t*>(a.status) != 0u) != 0;
+  __syncthreads();
   tc_fence_after();
   const uint32_t tmem = bars.tmem_base;
 
-  if (abandoned) {
-  } else if (warp < kSoftmaxWarps) {
+  if (warp < kSoftmaxWarps) {
     reg_inc<kRegsSoftmax>();
     softmax_role<kLse, kExtra>(a, &bars, &row_results, infos, sm, tmem, warp, tid & 31);
   } else {
     reg_dec<kRegsOther>();
-    if (warp == kTmaWarp) producer_role<!kExtra>(&tm_q, &tm_k, &tm_v, &tm_own_k, &tm_own_v, a, &bars, infos, sm);
+    if (warp == kTmaWarp) producer_role<!kExtra>(&tm_q, &tm_k, &tm_v, &tm_own_k, &tm_own_v, a, &bars, infos, sm, wi, tile0, tile1);
     else if (warp == kMmaWarp) mma_role<0, !kExtra>(a, &bars, sm, tmem);
     else if (warp == kMmaWarp + 1) mma_role<1, !kExtra>(a, &bars, sm, tmem);
   }
@@ -1283,7 +1296,7 @@ global_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
   tmem_wait_st();
   tc_fence_before();
   __syncthreads();
-  if (warp == kTmaWarp) tmem_dealloc(tmem, kTmemCols);
+  if (warp == kTmemWarp) tmem_dealloc(tmem, kTmemCols);
 }
 
 // The status block of a launch that no compaction precedes.
