@@ -34,6 +34,7 @@
 // fetched from HBM once and from L2 by the others.  Per-CTA partial sums go to the workspace and
 // a small second kernel adds them in a fixed order: no floating-point atomics, results identical
 // from run to run.
+#include <cstddef>
 #include <mutex>
 
 #include <cuda_bf16.h>
@@ -170,20 +171,15 @@ project_kv_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
   const int tok0 = pair / (2 * a.n_col_tiles);                    // first token tile
   const int n_kb = a.C / kBlockK;
 
-  if (threadIdx.x == 0) {
-    for (int s = 0; s < kProjStages; ++s) {
-      mbar_init(smem_u32(&bars.full[s]), 1);
-      mbar_init(smem_u32(&bars.empty[s]), 1);
-    }
-    for (int b = 0; b < 2; ++b) {
-      mbar_init(smem_u32(&bars.acc_full[b]), 1);
-      mbar_init(smem_u32(&bars.acc_read[b]), kEpiWarps);
-      mbar_init(smem_u32(&bars.acc_empty[b]), 2);
-    }
-    mbar_init(smem_u32(&bars.mma_idle), 1);
-    bars.abort_flag = 0;
+  // a thread for each barrier (one alone takes hundreds of clocks for them)
+  constexpr int kBarriers = static_cast<int>(offsetof(ProjBarriers, tmem_base) / sizeof(uint64_t));
+  constexpr int kAccRead = static_cast<int>(offsetof(ProjBarriers, acc_read) / sizeof(uint64_t));
+  if (threadIdx.x < kBarriers) {
+    const int which_bar = static_cast<int>(threadIdx.x) - kAccRead;
+    mbar_init(smem_u32(&bars) + threadIdx.x * sizeof(uint64_t), which_bar == 0 || which_bar == 1 ? kEpiWarps : which_bar == 2 || which_bar == 3 ? 2 : 1);
     fence_mbar_init();
   }
+  if (threadIdx.x == 0) bars.abort_flag = 0;
   if (warp == 0) {
     tmem_alloc_pair(smem_u32(&bars.tmem_base), kProjTmemCols);
     tmem_relinquish_pair();
@@ -199,13 +195,12 @@ project_kv_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
     for (int i = threadIdx.x; i < a.pl.H * a.pl.d; i += 256) { a.kmean[i] = 0.f; a.vmean[i] = 0.f; }
   }
   tc_fence_before();
-  const bool abandoned = __syncthreads_or(*reinterpret_cast<volatile uint32_t*>(a.status) != 0u) != 0;
+  __syncthreads();
   cluster_sync();   // the other CTA's barriers are initialised
   tc_fence_after();
   const uint32_t tmem = bars.tmem_base;
 
-  if (abandoned) {
-  } else if (warp < kFirstEpiWarp) {
+  if (warp < kFirstEpiWarp) {
     reg_dec<kRegsIssue>();
     if (warp == 0) {
       // ------------------------------------------------------------ TMA producer
@@ -397,7 +392,7 @@ project_kv_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
         if (elect_one()) mbar_arrive(smem_u32(&bars.acc_read[buf]));
       }
     }
-    if (lane == 0) bulk_wait<0>();   // the staging tiles stay put until the last store has read them
+    if (lane == 0) bulk_wait_read<0>();   // the staging tiles stay put until the last store has read them
     __syncwarp();
     if (ok && a.do_mean) {
       float* dst = a.partials + (static_cast<size_t>(blockIdx.x) * 4 + quarter) * kTileCol + 128 * col_half;
