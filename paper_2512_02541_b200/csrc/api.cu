@@ -136,7 +136,7 @@ static int check_build(const Plan& pl, const void* K, const void* V, const void*
     return AVGGT_ERR_ALIGNMENT;
   const int rc = device_info(di);
   if (rc != AVGGT_OK) return rc;
-  return ws_bytes < build_kv_ws_bytes(pl, di->sm_count) ? AVGGT_ERR_WORKSPACE_TOO_SMALL : AVGGT_OK;
+  return ws_bytes < build_kv_min_ws_bytes(pl, di->sm_count) ? AVGGT_ERR_WORKSPACE_TOO_SMALL : AVGGT_OK;
 }
 
 int avggt_build_kv(const avggt_params* p, const void* K, const void* V, void* Kc, void* Vc, int32_t* idx,
@@ -147,7 +147,8 @@ int avggt_build_kv(const avggt_params* p, const void* K, const void* V, void* Kc
   DeviceInfo di;
   rc = check_build(pl, K, V, Kc, Vc, idx, kmean, vmean, ws, ws_bytes, &di);
   if (rc != AVGGT_OK) return rc;
-  return record_cuda(launch_build_kv(pl, di.sm_count, K, V, Kc, Vc, idx, kmean, vmean, ws, static_cast<cudaStream_t>(cuda_stream)));
+  return record_cuda(launch_build_kv(pl, di.sm_count, K, V, Kc, Vc, idx, kmean, vmean, ws, ws_bytes,
+                                     static_cast<cudaStream_t>(cuda_stream)));
 }
 
 // One attention call: which buffers, on which stream.
@@ -220,7 +221,8 @@ int avggt_layer(const avggt_params* p, const void* Q, const void* K, const void*
   AttnCall c{Q, K, V, Kc, Vc, kmean, vmean, O, lse, attn_ws, attn_ws_bytes, cuda_stream, nullptr, false};
   rc = check_attn(pl, c, &di);
   if (rc != AVGGT_OK) return rc;
-  rc = record_cuda(launch_build_kv(pl, di.sm_count, K, V, Kc, Vc, idx, kmean, vmean, build_ws, static_cast<cudaStream_t>(cuda_stream),
+  rc = record_cuda(launch_build_kv(pl, di.sm_count, K, V, Kc, Vc, idx, kmean, vmean, build_ws, build_ws_bytes,
+                                   static_cast<cudaStream_t>(cuda_stream),
                                    nullptr, nullptr, 0, false, attn_ws));
   if (rc != AVGGT_OK) return rc;
   c.status_cleared = true;
@@ -256,8 +258,8 @@ int avggt_build_kv_indexed(const avggt_params* p, const int32_t* idx, int64_t n_
   DeviceInfo di;
   rc = device_info(&di);
   if (rc != AVGGT_OK) return rc;
-  if (ws_bytes < build_kv_ws_bytes(pl, di.sm_count)) return AVGGT_ERR_WORKSPACE_TOO_SMALL;
-  return record_cuda(launch_build_kv(pl, di.sm_count, K, V, Kc, Vc, nullptr, kmean, vmean, ws,
+  if (ws_bytes < build_kv_min_ws_bytes(pl, di.sm_count)) return AVGGT_ERR_WORKSPACE_TOO_SMALL;
+  return record_cuda(launch_build_kv(pl, di.sm_count, K, V, Kc, Vc, nullptr, kmean, vmean, ws, ws_bytes,
                                      static_cast<cudaStream_t>(cuda_stream), idx, slot_of_token));
 }
 
@@ -335,11 +337,11 @@ int avggt_build_kv_shard(const avggt_params* p, const void* K, const void* V, vo
   DeviceInfo di;
   rc = device_info(&di);
   if (rc != AVGGT_OK) return rc;
-  if (ws_bytes < build_kv_ws_bytes(pl, di.sm_count)) return AVGGT_ERR_WORKSPACE_TOO_SMALL;
+  if (ws_bytes < build_kv_min_ws_bytes(pl, di.sm_count)) return AVGGT_ERR_WORKSPACE_TOO_SMALL;
   const size_t part = static_cast<size_t>(pl.H) * static_cast<size_t>(slot_rows) * pl.d;   // elements of the K part of a slot
   void* Vc = static_cast<char*>(slot) + part * 2;
   float* vsum = sums ? sums + static_cast<size_t>(pl.H) * pl.d : nullptr;
-  return record_cuda(launch_build_kv(pl, di.sm_count, K, V, slot, Vc, idx, sums, vsum, ws,
+  return record_cuda(launch_build_kv(pl, di.sm_count, K, V, slot, Vc, idx, sums, vsum, ws, ws_bytes,
                                      static_cast<cudaStream_t>(cuda_stream), nullptr, nullptr, slot_rows, true));
 }
 

@@ -732,12 +732,19 @@ int build_kv_grid(const Plan& pl, int sm_count) {
   return static_cast<int>(tiles < most ? tiles : most);
 }
 
+size_t build_kv_min_ws_bytes(const Plan& pl, int sm_count) {
+  const int grid = build_kv_grid(pl, sm_count);
+  const int64_t groups = (pl.n_tok + 7) / 8;
+  const int64_t least = pl.H <= 16 ? grid : groups < sm_count ? groups : sm_count;
+  return static_cast<size_t>(least < grid ? least : grid) * 2 * pl.H * pl.d * sizeof(float);
+}
+
 size_t build_kv_ws_bytes(const Plan& pl, int sm_count) {
   return static_cast<size_t>(build_kv_grid(pl, sm_count)) * 2 * pl.H * pl.d * sizeof(float);
 }
 
 cudaError_t launch_build_kv(const Plan& pl, int sm_count, const void* K, const void* V, void* Kc, void* Vc,
-                            int32_t* idx, float* kmean, float* vmean, void* ws, cudaStream_t st,
+                            int32_t* idx, float* kmean, float* vmean, void* ws, size_t ws_bytes, cudaStream_t st,
                             const int32_t* caller_idx, int32_t* slot_of_token, int64_t kc_rows, bool sums_only,
                             void* clear_status) {
   if (kc_rows <= 0) kc_rows = pl.M;
@@ -768,8 +775,10 @@ cudaError_t launch_build_kv(const Plan& pl, int sm_count, const void* K, const v
     a.status = static_cast<uint32_t*>(clear_status);
     return launch_dependent_cluster(build_kv_small_kernel, 2 * pl.H * ranks, ranks, kSmallThreads, 0, st, a);
   }
-  const int grid = build_kv_grid(pl, sm_count);
   const int do_mean = (pl.mean_fill != 0 && pl.n_dropped > 0) ? 1 : 0;
+  int grid = build_kv_grid(pl, sm_count);
+  const size_t room = ws_bytes / (2 * static_cast<size_t>(pl.H) * pl.d * sizeof(float));   // partial rows
+  if (do_mean && room < static_cast<size_t>(grid)) grid = static_cast<int>(room);
   float* partials = static_cast<float*>(ws);
   uint32_t* status = static_cast<uint32_t*>(clear_status);
   const bool zero_mean = pl.mean_fill != 0 && !do_mean;

@@ -54,13 +54,15 @@ cudaError_t launch_clear_status(void* status, cudaStream_t st);
 int build_kv_grid(const Plan& pl, int sm_count);
 int build_kv_blocks_per_sm();
 size_t build_kv_ws_bytes(const Plan& pl, int sm_count);
+// What a call gets by with, on fewer blocks (above 16 heads a block per SM).
+size_t build_kv_min_ws_bytes(const Plan& pl, int sm_count);
 // caller_idx / slot_of_token: both null for the window rule of Sec. 4.3; for a caller-chosen retained set,
 // the M retained token indices (device) and the [n_tok] map the call fills (device).
 // kc_rows: rows per head of Kc / Vc (0 = M; larger when they are one rank's slot of an exchange buffer).
 // sums_only: kmean / vmean receive the un-normalised sums over the dropped rows instead of the means.
 // clear_status: the status block (kAttnStatusBytes) of the attention launch that follows in the stream, or null.
 cudaError_t launch_build_kv(const Plan& pl, int sm_count, const void* K, const void* V, void* Kc, void* Vc,
-                            int32_t* idx, float* kmean, float* vmean, void* ws, cudaStream_t st,
+                            int32_t* idx, float* kmean, float* vmean, void* ws, size_t ws_bytes, cudaStream_t st,
                             const int32_t* caller_idx = nullptr, int32_t* slot_of_token = nullptr,
                             int64_t kc_rows = 0, bool sums_only = false, void* clear_status = nullptr);
 

@@ -88,3 +88,19 @@ def test_a_list_with_entries_that_are_no_token():
         for full, compact in ((K, Kc), (V, Vc)):
             assert torch.equal(compact[:, 1:-1], full[kept].transpose(0, 1))
             assert (compact[:, 0] == 7).all() and (compact[:, -1] == 7).all()
+
+
+def test_a_workspace_for_a_block_per_sm():
+    """Above 16 heads a call gets by with half of what avggt_workspace_bytes asks for, on half as many blocks."""
+    wl = inputs.Workload("half", 6, 37, 37, 5, 20, 64, 4, 1, 2, "iid")
+    params, ocfg = _cfgs(wl)
+    _, K, V = inputs.make_qkv(wl, seed=2, device="cuda")
+    layer = P.SubsampledGlobalAttention(params)
+    half = torch.cuda.get_device_properties(0).multi_processor_count * 2 * 20 * 64 * 4
+    assert half < layer.build_ws_bytes
+    ws = torch.empty((half,), dtype=torch.uint8, device="cuda")
+    P.avggt_build_kv(params, K, V, layer.Kc, layer.Vc, layer.idx, layer.kmean, layer.vmean, ws, half)
+    torch.cuda.synchronize()
+    _check_build(ocfg, layer, K, V)
+    with pytest.raises(P.AvggtError):
+        P.avggt_build_kv(params, K, V, layer.Kc, layer.Vc, layer.idx, layer.kmean, layer.vmean, ws, half - 1)
