@@ -42,11 +42,11 @@ from paper_2512_02541_b200 import inputs  # noqa: E402
 # profiles/; None where no capture covers the workload.  Both kernels are captured on the 30-frame copy of the
 # headline layer (profiles/*_vggt_n30_s9.md); their traffic is proportional to the frame count, so the 800-frame
 # figures are those captures x 800/30.
-_ATTN_N30_S9 = 0.275387648e9 + 0.068802048e9
-_BUILD_N30_S9 = 0.168858624e9 + 0.006855424e9
+_ATTN_N30_S9 = 275201024.0 + 66723840.0
+_BUILD_N30_S9 = 168868096.0 + 13229056.0
 NCU_TRAFFIC = {
-    "vggt_n30_s9": {"global_attn_kernel": _ATTN_N30_S9, "build_kv_kernel": _BUILD_N30_S9},
-    "vggt_n800_s9": {"global_attn_kernel": _ATTN_N30_S9 * 800 / 30, "build_kv_kernel": _BUILD_N30_S9 * 800 / 30},
+    "vggt_n30_s9": {"global_attn_kernel": _ATTN_N30_S9, "build_kv_stream_kernel": _BUILD_N30_S9},
+    "vggt_n800_s9": {"global_attn_kernel": _ATTN_N30_S9 * 800 / 30, "build_kv_stream_kernel": _BUILD_N30_S9 * 800 / 30},
 }
 
 METRIC = "subsampled_global_attn_queries_per_sec"
@@ -524,10 +524,10 @@ def run_ours(args, wl):
             "frame_attn_tflops": (4.0 * n_q_local * wl.tokens_per_frame * H * d / (frame_ms * 1e-3) / 1e12) if frame_ms else None,
             "project_build_kv": proj,
             "roofline": roof,
-            "roofline_build_kv": {"bound": "hbm", "kernel": "build_kv_kernel", "achieved": build_gbs,
+            "roofline_build_kv": {"bound": "hbm", "kernel": "build_kv_stream_kernel", "achieved": build_gbs,
                                   "peak": peaks["hbm_gbs"], "unit": "GB/s", "frac": build_gbs / peaks["hbm_gbs"],
                                   "frac_of_nominal_8000": build_gbs / NOMINAL_HBM_GBS,
-                                  "traffic": NCU_TRAFFIC.get(wl.name, {}).get("build_kv_kernel") if not shard_mode else None,
+                                  "traffic": NCU_TRAFFIC.get(wl.name, {}).get("build_kv_stream_kernel") if not shard_mode else None,
                                   "bytes_per_launch": bbytes,
                                   "peak_source": f"{peaks['source']} copy bandwidth"},
             "e2e": {"value": units_all * e2e_steps / (e2e_ms * 1e-3), "unit": UNIT,
