@@ -171,7 +171,7 @@ int avggt_build_kv_noalloc(const avggt_params* p, const void* K, const void* V,
  *   lse           device, float [N*L, H] or NULL: natural-log normaliser ln(Z) + max-shift
  *   ws            device scratch of at least attn_ws_bytes.  It starts with a 256-byte status
  *                 block that the call clears on the stream and whose first 16 bytes
- *                 avggt_check_status reads.  The kernel looks at the block when it starts (a
+ *                 avggt_check_status reads.  The kernel looks at the block with each work item (a
  *                 launch in which a wait has run out is abandoned by its remaining thread
  *                 blocks), so one workspace serves one attention launch at a time: launches that
  *                 may be in flight together need a workspace each.
