@@ -24,7 +24,7 @@
 //               be moved to the softmax warpgroups)
 // Tensor memory per tile (256 columns): two places for S and P that alternate (see kColSOdd), O (64) and the row
 // sums of P (16).  A softmax thread pulls its 56 scores of S into registers and the warp frees its rows at once,
-// so the next Q K^T runs under the exponentials; P V of step j runs under the softmax of step j+1.  Three
+// so the next Q K^T runs under the exponentials; P V of step j runs under the softmax of step j+1.  Two
 // blocks of 8 key columns in fourteen take their exponentials from a polynomial on
 // the FMA pipe.  The accumulator is rescaled lazily: only when the running
 // maximum grew by more than 2^8 since the last rescale.  The epilogue folds the
@@ -88,15 +88,13 @@ static_assert(kFlushSteps > 1, "an item's first step, under which the item befor
 // Blocks of 8 key columns (bit b: columns [8 b, 8 b + 8) of a step) whose exponentials come from a polynomial on the
 // FMA pipe instead of the special-function unit, which at 16 results per clock per SM would otherwise set the pace.
 // The polynomial costs more instructions and more energy, and the long launches run at the card's power limit, so the
-// choice that takes the fewest clocks gains least.  Where the blocks lie counts as much as their number: one in each group of four
-// blocks but the first (which is computed ahead of the vote, and again where a row moves its reference) spreads the instructions.
-// Dense layer of 40 frames, layer of 31 and 10, frame attention of 100 (ms, us, us, us; clocks of the dense launch): 6 and 13:
-// 12.90, 1110, 256.5, 1049 (20.3 M); one block 13.4, 1143, -, 1065 (21.4 M); 4, 9 and 12: 12.78, 1092, 252,
-// 1047 (19.4 M); 4, 9 and 13, or 4, 8 and 12: 1 % more clocks; 3, 8 and 13 12.95, 1139, -, 1086; 4, 9, 11 and 13: 13.05, 1108, -, 1068 (19.2 M).
-// Error of the outputs against 64 bits with 6 and 13, and with 4, 9 and 12 (relative 2-norm, 768 rows): independent normal inputs
-// 1.91729e-3 and 1.91726e-3, 10 frames 1.66249e-3 both, dense 1.67474e-3 and 1.67476e-3.
+// choice that takes the fewest clocks gains least.  Two blocks and no more: the polynomial's error (7.5e-5) vanishes in the rounding of
+// the probabilities to bf16, but not in the sum of the unrounded ones behind the log-sum-exp (7.2e-5 where one key of such a block
+// takes the whole softmax), and every further block adds to it.  A third block (4, 9 and 12 instead of 6 and 13) is not worth that:
+// 10 frames of 1,374 tokens, a quarter retained, 269.8 us against 271.8; 100 frames 22.20 ms against 22.54, dense 81.1 against 82.9; frame
+// attention of 10 frames 118.1 us against 119.7.
 #ifndef AVGGT_POLY_BLOCKS
-#define AVGGT_POLY_BLOCKS 0x1210
+#define AVGGT_POLY_BLOCKS 0x2040
 #endif
 constexpr uint32_t kPolyBlocks = AVGGT_POLY_BLOCKS;
 
