@@ -130,9 +130,9 @@ struct AttnArgs {
   float log2_count[2];  // log2 weight of the mean column for a retained and for a dropped query (0: unit weight; -inf: absent)
 };
 
-// Records of work items (ItemInfo): so many that one is never overwritten while a warp may still read it.  When the producer writes
-// the record of item n, every Q K^T of item n - 2 has completed, so that every softmax warp has read scores of item n - 3 and, with
-// one step per item, may still be before the epilogue of item n - 4.
+// Records of work items (ItemInfo).  The producer writes record n when every softmax warp is done with that of item n - kInfos
+// (info_empty): no other barrier says so, since the softmax warps of a tile that sits items out arrive on none for them.  With so many
+// the producer does not wait: it is at most four items ahead of the epilogues of a tile at work.
 constexpr int kInfos = 8;
 
 // Ordered by the arrivals that a phase counts, so that as many threads can initialise them at once (init_barriers).
@@ -154,6 +154,7 @@ struct __align__(8) Barriers {
   uint64_t p_full[kQTiles][2]; // softmax -> MMA: P_t(j) stored (and O_t rescaled); even and odd steps apart, since a warp may
                                // have finished a step before another warp of its tile has finished the step before
   // one of each softmax warp
+  uint64_t info_empty[kInfos]; // softmax -> producer: the warp has read the item's record for the last time
   uint64_t own_empty;          // softmax -> producer: its epilogue has read the own rows
   // of the issuers, where there are keys, and with extra columns of the softmax warps
   uint64_t q_empty[2];         // MMA issuers -> producer: every Q K^T of the work item has completed; with extra columns, softmax ->
@@ -166,8 +167,8 @@ template <bool kExtra>
 __device__ __forceinline__ void init_barriers(Barriers* bars, const AttnArgs& a, int tid) {
   constexpr int kSize = sizeof(uint64_t);
   constexpr int kTwo = offsetof(Barriers, k_empty) / kSize, kTile = offsetof(Barriers, o_free) / kSize,
-                kAll = offsetof(Barriers, own_empty) / kSize, kQ = offsetof(Barriers, q_empty) / kSize;
-  static_assert(kAll + 1 == kQ && kQ + 2 == offsetof(Barriers, tmem_base) / kSize, "order of the barriers");
+                kAll = offsetof(Barriers, info_empty) / kSize, kQ = offsetof(Barriers, q_empty) / kSize;
+  static_assert(kAll + kInfos + 1 == kQ && kQ + 2 == offsetof(Barriers, tmem_base) / kSize, "order of the barriers");
   if (tid < kQ + 2) {
     const uint32_t count = tid < kTwo ? 1 : tid < kTile ? kQTiles : tid < kAll ? kSoftmaxWarps / kQTiles : tid < kQ ? kSoftmaxWarps
                            : (a.n_kv_tiles > 0 ? kQTiles : 0) + (kExtra ? kSoftmaxWarps : 0);
@@ -385,6 +386,8 @@ __device__ __forceinline__ void producer_role(const CUtensorMap* tm_q, const CUt
       ok = false;
       break;
     }
+    ok = wait_bar_warp(&bars->info_empty[n_done % kInfos], ((n_done / kInfos) & 1) ^ 1, bars, a, 17, n_done);
+    if (!ok) break;
     if (elect_one()) {
       ItemInfo& info = infos[n_done % kInfos];
       info.head = head;
@@ -1176,6 +1179,8 @@ __device__ __forceinline__ void softmax_items(const AttnArgs& a, Barriers* bars,
             }
           }
         }
+        __syncwarp();   // every lane has read the record
+        if (elect_one()) mbar_arrive(smem_u32(&bars->info_empty[(n - 1) % kInfos]));
         pending = false;
         most = kFlushSteps - 1;
       } else {
@@ -1185,8 +1190,11 @@ __device__ __forceinline__ void softmax_items(const AttnArgs& a, Barriers* bars,
     } while (left > 0);
     if (!have) return;
     pending = active;
-    if (!active) continue;
-    __syncwarp();   // every lane has read the results of the item before
+    __syncwarp();   // every lane has read the results of the item before, and of the record what it needs before the epilogue
+    if (!active) {
+      if (elect_one()) mbar_arrive(smem_u32(&bars->info_empty[n % kInfos]));
+      continue;
+    }
 #pragma unroll
     for (int hi = 0; hi < 2; ++hi) {
       const int at = t * kTileQ + 32 * me.q + 16 * me.h + (me.lane >> 2) + 8 * hi;

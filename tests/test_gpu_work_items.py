@@ -66,6 +66,15 @@ def test_frame_items_with_a_short_last_one(L):
         frame_attn._check(*run)
 
 
+# 54 items per thread block, all of one tile, so that tile 1 never takes part; 6 or 7 in a row behind as many full ones
+@pytest.mark.parametrize("L,n_frames", ((100, 500), (261, 62)))
+def test_items_that_a_tile_sits_out_in_a_row(L, n_frames):
+    wl = inputs.Workload("sit_out", n_frames, 1, L - 5, 5, 16, 64, 4, 1, 2, "iid")
+    for lse in (False, True):
+        run = frame_attn._run(wl, seed=L, want_lse=lse)
+        frame_attn._check(*run, rows=np.arange(0, wl.n_tokens, 23))
+
+
 # more bytes than L2 holds, so that the short last items follow the full ones of every two frames (of 16 heads) or of each
 # (of 32): 13 frames, the last of them on its own, and 6
 @pytest.mark.parametrize("n_frames,heads", ((13, 16), (6, 32)))
