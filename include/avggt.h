@@ -118,6 +118,8 @@ int avggt_workspace_bytes(const avggt_params* p, size_t* build_ws_bytes, size_t*
  *   ws      device scratch of at least build_ws_bytes; holds per-block partial sums (of a few
  *           thousand tokens at most: nothing) and needs no initialisation.  The reduction order is
  *           fixed: results are identical from run to run.
+ * The kernel waits for its own copies, for 0.2 s at most.  Compact rows that were not copied because such a wait ran out are NaN, and so
+ * is the mean pair that lacks a row; avggt_layer reports it in the status block as well.
  */
 int avggt_build_kv(const avggt_params* p, const void* K, const void* V,
                    void* Kc, void* Vc, int32_t* idx, float* kmean, float* vmean,

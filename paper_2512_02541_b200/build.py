@@ -8,11 +8,12 @@ import sys
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libavggt.so")
-# A second library for one GPU test: the same sources with a 0.5 ms limit on device-side waits and one K tile
-# left out by the first thread block of the attention kernel, so that the time-out path can be exercised
-# without hanging or faulting anything.  The product library never contains that switch.
+# A second library for the GPU tests of the time-out paths: the same sources with a 0.5 ms limit on device-side waits, one K tile
+# left out by the first thread block of the attention kernel and, in calls of fewer than 20,000 tokens, the copies of one tile by the
+# first thread block of the compaction kernels, so that those paths can be exercised without hanging or faulting anything.  The product
+# library never contains those switches.
 WAIT_TEST_LIB = os.path.join(HERE, "libavggt_waittest.so")
-WAIT_TEST_DEFINES = ["-DAVGGT_TEST_SKIP_K_LOAD=1", "-DAVGGT_WAIT_LIMIT_NS=500000ull"]
+WAIT_TEST_DEFINES = ["-DAVGGT_TEST_SKIP_K_LOAD=1", "-DAVGGT_TEST_SKIP_TILE_LOAD_BELOW=20000", "-DAVGGT_WAIT_LIMIT_NS=500000ull"]
 SOURCES = ["api.cu", "build_kv.cu", "build_kv_noalloc.cu", "global_attn.cu", "project_kv.cu"]
 HEADERS = ["internal.h", "plan.h", "ptx.cuh", "tmap.h", os.path.join("..", "..", "include", "avggt.h")]
 

@@ -66,6 +66,9 @@ struct StreamArgs {
   WindowRule rule;
   const uint8_t* K;
   const uint8_t* V;
+  uint4* Kc;           // for rows that a wait which ran out kept from being copied (as kc_rows)
+  uint4* Vc;
+  int64_t kc_rows;
   int32_t rows;        // of a tile
   int32_t* idx;
   const int32_t* slot_of_token;
@@ -94,6 +97,25 @@ __device__ __forceinline__ void stream_report(uint32_t* status, int lane) {
   status[2] = 90;
   status[3] = 0;
 }
+
+// Row m of the compact arrays, all heads, by a warp that could not copy it because a wait ran out: NaN, so that a call without a status
+// block does not pass for a good one.
+__device__ __forceinline__ void mark_row(uint4* Kc, uint4* Vc, int64_t kc_rows, int H, int m, int lane) {
+  const uint4 nan = make_uint4(0x7fff7fffu, 0x7fff7fffu, 0x7fff7fffu, 0x7fff7fffu);
+  for (int c = lane; c < H * 8; c += 32) {
+    const size_t at = (static_cast<size_t>(c >> 3) * static_cast<size_t>(kc_rows) + static_cast<size_t>(m)) * 8u + (c & 7);
+    Kc[at] = nan;
+    Vc[at] = nan;
+  }
+}
+
+// Build for the wait-limit test only (never part of libavggt.so): in calls of fewer tokens than this the first thread block leaves out the
+// copies of its second tile.
+#ifdef AVGGT_TEST_SKIP_TILE_LOAD_BELOW
+#define AVGGT_SKIP_TILE(n_tok, stage) (blockIdx.x == 0 && (stage) == 1 && (n_tok) < AVGGT_TEST_SKIP_TILE_LOAD_BELOW)
+#else
+#define AVGGT_SKIP_TILE(n_tok, stage) false
+#endif
 
 // PASSES: chunks of 16 bytes per adding thread (2 * H * 8 of them in a row of K and V).
 template <int PASSES>
@@ -131,7 +153,7 @@ build_kv_stream_kernel(const __grid_constant__ CUtensorMap tm_kc, const __grid_c
       return a.slot_of_token != nullptr ? __ldcg(a.slot_of_token + row) : compact_position(a.rule, pl, row);
     };
     const auto load = [&](uint32_t t, int stage) {
-      if (lane == 0) {
+      if (lane == 0 && !AVGGT_SKIP_TILE(n_tok, stage)) {
         const uint32_t row0 = t * rows, n = n_tok - row0 < rows ? n_tok - row0 : rows;
         const uint32_t fb = smem_u32(&bars.full[stage]), dst = smem_u32(stages + 2 * stage * kStreamBytes);
         mbar_arrive_expect_tx(fb, 2 * n * row_bytes);
@@ -158,6 +180,7 @@ build_kv_stream_kernel(const __grid_constant__ CUtensorMap tm_kc, const __grid_c
       if (blockIdx.x + s * gridDim.x < n_tiles) tell(s, pos[s]);
     }
     bool ok = true;
+    uint32_t left = n_tiles;   // first tile whose rows are not stored, where a wait ran out
     int round = 0;
     for (uint32_t t0 = blockIdx.x; t0 < n_tiles && ok; t0 += kStreamStages * gridDim.x, ++round) {
 #pragma unroll
@@ -169,7 +192,10 @@ build_kv_stream_kernel(const __grid_constant__ CUtensorMap tm_kc, const __grid_c
         const bool more = refill < n_tiles && (round > 0 || s > 0);
         const int next = more ? position(refill) : -2;
         ok = __all_sync(0xffffffffu, stream_wait(&bars.full[s], round & 1));
-        if (!ok) break;
+        if (!ok) {
+          left = t;
+          break;
+        }
         const int m = pos[s];
         uint32_t mask = __ballot_sync(0xffffffffu, m >= 0);
         if (m >= 0 && a.idx != nullptr) a.idx[m] = static_cast<int32_t>(t * rows + lane);
@@ -190,7 +216,10 @@ build_kv_stream_kernel(const __grid_constant__ CUtensorMap tm_kc, const __grid_c
         __syncwarp();
         if (more) {
           ok = __all_sync(0xffffffffu, stream_wait(&bars.empty[before], (s == 0 ? round - 1 : round) & 1));
-          if (!ok) break;
+          if (!ok) {
+            left = t + gridDim.x;
+            break;
+          }
           load(refill, before);
           tell(before, next);
           pos[before] = next;
@@ -200,6 +229,11 @@ build_kv_stream_kernel(const __grid_constant__ CUtensorMap tm_kc, const __grid_c
     if (!ok) {   // a wait ran out: whatever is still on its way arrives before the block gives up its shared memory
       stream_report(a.status, lane);
       for (int s = 0; s < kStreamStages; ++s) (void)stream_wait(&bars.full[s], 0), (void)stream_wait(&bars.full[s], 1);
+      for (uint32_t t = left; t < n_tiles; t += gridDim.x) {
+        const int m = position(t);
+        for (uint32_t mask = __ballot_sync(0xffffffffu, m >= 0); mask != 0; mask &= mask - 1)
+          mark_row(a.Kc, a.Vc, a.kc_rows, pl.H, __shfl_sync(0xffffffffu, m, __ffs(mask) - 1), lane);
+      }
     }
     if (lane == 0) bulk_wait_read<0>();   // the stores complete before the kernel does
     __syncwarp();
@@ -291,6 +325,9 @@ struct GatherArgs {
   Divisor by_Lc, by_kept_w;
   const uint8_t* K;
   const uint8_t* V;
+  uint4* Kc;           // as in StreamArgs
+  uint4* Vc;
+  int64_t kc_rows;
   int32_t rows;        // of a tile
   int32_t* idx;
   const int32_t* caller_idx;   // caller-chosen retained set: token of every compact row; else null
@@ -356,6 +393,7 @@ build_kv_gather_kernel(const __grid_constant__ CUtensorMap tm_kc, const __grid_c
     return tok < pl.n_tok ? tok : -1;   // (entries of a caller's list that are no token are passed over)
   };
   const auto load = [&](int stage, int tok) {
+    if (AVGGT_SKIP_TILE(pl.n_tok, stage)) return;
     const uint32_t have = __ballot_sync(0xffffffffu, tok >= 0);
     const int tok0 = __shfl_sync(0xffffffffu, tok, 0);
     const uint32_t fb = smem_u32(&full[stage]), dst = smem_u32(stages + 2 * stage * kStreamBytes);
@@ -382,6 +420,7 @@ build_kv_gather_kernel(const __grid_constant__ CUtensorMap tm_kc, const __grid_c
     if (t < n_tiles) load(s, toks[s]);
   }
   bool ok = true;
+  uint32_t left = n_tiles;   // first tile whose rows are not stored, where a wait ran out
   int round = 0;
   for (uint32_t t0 = blockIdx.x; t0 < n_tiles && ok; t0 += kStreamStages * gridDim.x, ++round) {
 #pragma unroll
@@ -393,7 +432,10 @@ build_kv_gather_kernel(const __grid_constant__ CUtensorMap tm_kc, const __grid_c
       const bool more = refill < n_tiles && (round > 0 || s > 0);
       const int next = more ? token(refill) : -1;
       ok = __all_sync(0xffffffffu, stream_wait(&full[s], round & 1));
-      if (!ok) break;
+      if (!ok) {
+        left = t;
+        break;
+      }
       const int tok = toks[s];
       const uint32_t m0 = t * rows;
       if (tok >= 0 && a.idx != nullptr) a.idx[m0 + lane] = tok;
@@ -423,6 +465,10 @@ build_kv_gather_kernel(const __grid_constant__ CUtensorMap tm_kc, const __grid_c
   if (!ok) {   // a wait ran out: whatever is still on its way arrives before the block gives up its shared memory
     stream_report(a.status, lane);
     for (int s = 0; s < kStreamStages; ++s) (void)stream_wait(&full[s], 0), (void)stream_wait(&full[s], 1);
+    for (uint32_t t = left; t < n_tiles; t += gridDim.x) {
+      for (uint32_t have = __ballot_sync(0xffffffffu, token(t) >= 0); have != 0; have &= have - 1)
+        mark_row(a.Kc, a.Vc, a.kc_rows, pl.H, static_cast<int>(t * rows) + __ffs(have) - 1, lane);
+    }
   }
   if (lane == 0) bulk_wait_read<0>();   // the stores complete before the kernel does
   __syncwarp();
@@ -624,6 +670,9 @@ cudaError_t launch_stream(const Plan& pl, int grid, const void* K, const void* V
   a.rule = make_window_rule(pl);
   a.K = static_cast<const uint8_t*>(K);
   a.V = static_cast<const uint8_t*>(V);
+  a.Kc = static_cast<uint4*>(Kc);
+  a.Vc = static_cast<uint4*>(Vc);
+  a.kc_rows = kc_rows;
   a.rows = stream_rows(pl);
   a.idx = idx;
   a.slot_of_token = slot_of_token;
@@ -646,6 +695,9 @@ cudaError_t launch_gather(const Plan& pl, int grid, const void* K, const void* V
   a.by_kept_w = make_divisor(pl.kept_w);
   a.K = static_cast<const uint8_t*>(K);
   a.V = static_cast<const uint8_t*>(V);
+  a.Kc = static_cast<uint4*>(Kc);
+  a.Vc = static_cast<uint4*>(Vc);
+  a.kc_rows = kc_rows;
   a.rows = stream_rows(pl);
   a.idx = idx;
   a.caller_idx = caller_idx;

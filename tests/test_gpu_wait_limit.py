@@ -75,3 +75,54 @@ def test_a_wait_that_runs_out_is_reported_and_the_context_stays_usable():
     want = orc.global_attn_blocked(ocfg, Qh, Kh, Vh, rows)
     err = np.abs(O[torch.as_tensor(rows, device="cuda")].float().cpu().numpy().astype(np.float64) - want)
     assert err.max() <= 2e-2 and err.mean() <= 2e-3
+
+
+def _small(mean_fill):
+    # 13,740 tokens of 16 heads, a quarter retained: 1,718 tiles of 8 tokens, or 458 of 8 compact rows, over 296 thread blocks
+    wl = inputs.Workload("wait_limit_small", 10, 37, 37, 5, 16, 64, 4, 1, mean_fill, "iid")
+    params = P.make_params(wl.n_frames, wl.grid_h, wl.grid_w, wl.n_special, wl.n_heads, wl.head_dim, wl.sigma,
+                           diag=wl.diag, mean_fill=wl.mean_fill)
+    return params, P.SubsampledGlobalAttention(params), inputs.make_qkv(wl, seed=1, device="cuda")
+
+
+@pytest.mark.parametrize("mean_fill", (2, 0))   # tiles of tokens, tiles of compact rows
+def test_a_compaction_that_lost_a_tile_shows(mean_fill):
+    params, layer, (Q, K, V) = _small(mean_fill)
+    vp = ctypes.c_void_p
+    st = vp(torch.cuda.current_stream().cuda_stream)
+    broken = binding.load_library(build.build_wait_test())
+    buffers = (layer.Kc, layer.Vc, layer.idx, layer.kmean, layer.vmean)
+    for t in buffers[:2]:
+        t.zero_()
+    args = [vp(t.data_ptr()) for t in (K, V) + buffers]
+    assert broken.avggt_build_kv(ctypes.byref(params), *args, vp(layer.build_ws.data_ptr()), layer.build_ws.numel(), st) == 0
+    torch.cuda.synchronize()
+    got = [t.clone() for t in buffers]
+
+    layer.build_kv(K, V)   # the product library, the same buffers
+    layer.check_status()
+    lost = torch.isnan(got[0].float()).any(dim=2).any(dim=0)
+    assert 0 < int(lost.sum()) < layer.M // 4   # what the first thread block had before it
+    for bad, good in zip(got[:2], buffers[:2]):
+        assert torch.isfinite(good.float()).all()
+        assert torch.isnan(bad[:, lost].float()).all() and torch.equal(bad[:, ~lost], good[:, ~lost])
+    if mean_fill:
+        assert torch.isnan(got[3]).all() and torch.isnan(got[4]).all() and torch.isfinite(layer.kmean).all()
+
+
+@pytest.mark.parametrize("mean_fill", (2, 0))
+def test_the_layer_reports_a_compaction_that_lost_a_tile(mean_fill):
+    params, layer, (Q, K, V) = _small(mean_fill)
+    vp = ctypes.c_void_p
+    st = vp(torch.cuda.current_stream().cuda_stream)
+    broken = binding.load_library(build.build_wait_test())
+    O = torch.empty_like(Q)
+    args = [vp(t.data_ptr()) for t in (Q, K, V, layer.Kc, layer.Vc, layer.idx, layer.kmean, layer.vmean, O)]
+    assert broken.avggt_layer(ctypes.byref(params), *args, None, vp(layer.build_ws.data_ptr()), layer.build_ws.numel(),
+                              vp(layer.attn_ws.data_ptr()), layer.attn_ws.numel(), st) == 0
+    torch.cuda.synchronize()
+    detail = (ctypes.c_uint32 * 4)()
+    assert broken.avggt_check_status(vp(layer.attn_ws.data_ptr()), detail) == binding.AVGGT_ERR_DEVICE_TIMEOUT
+    assert tuple(detail)[:3] == (1, 0, 90)
+    layer.forward(Q, K, V)
+    layer.check_status()
