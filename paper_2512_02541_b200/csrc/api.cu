@@ -147,8 +147,10 @@ int avggt_build_kv(const avggt_params* p, const void* K, const void* V, void* Kc
   DeviceInfo di;
   rc = check_build(pl, K, V, Kc, Vc, idx, kmean, vmean, ws, ws_bytes, &di);
   if (rc != AVGGT_OK) return rc;
-  return record_cuda(launch_build_kv(pl, di.sm_count, K, V, Kc, Vc, idx, kmean, vmean, ws, ws_bytes,
-                                     static_cast<cudaStream_t>(cuda_stream)));
+  bool tmap_failed = false;
+  const cudaError_t e = launch_build_kv(pl, di.sm_count, K, V, Kc, Vc, idx, kmean, vmean, ws, ws_bytes,
+                                        static_cast<cudaStream_t>(cuda_stream), &tmap_failed);
+  return record_launch(e, tmap_failed);
 }
 
 // One attention call: which buffers, on which stream.
@@ -190,8 +192,7 @@ static int enqueue_attn(const Plan& pl, const DeviceInfo& di, const AttnCall& c)
       ? launch_frame_attn(pl, di.sm_count, c.Q, c.K, c.V, c.O, c.lse, c.ws, st, &tmap_failed)
       : launch_global_attn(pl, di.sm_count, c.Q, c.K, c.V, c.Kc, c.Vc, c.kmean, c.vmean, c.O, c.lse, c.ws, st,
                            &tmap_failed, c.slot_of_token, c.status_cleared);
-  if (tmap_failed) return record_message("cuTensorMapEncodeTiled failed");
-  return record_cuda(e);
+  return record_launch(e, tmap_failed);
 }
 
 static int run_attn(const Plan& pl, const AttnCall& c) {
@@ -221,9 +222,10 @@ int avggt_layer(const avggt_params* p, const void* Q, const void* K, const void*
   AttnCall c{Q, K, V, Kc, Vc, kmean, vmean, O, lse, attn_ws, attn_ws_bytes, cuda_stream, nullptr, false};
   rc = check_attn(pl, c, &di);
   if (rc != AVGGT_OK) return rc;
-  rc = record_cuda(launch_build_kv(pl, di.sm_count, K, V, Kc, Vc, idx, kmean, vmean, build_ws, build_ws_bytes,
-                                   static_cast<cudaStream_t>(cuda_stream),
-                                   nullptr, nullptr, 0, false, attn_ws));
+  bool tmap_failed = false;
+  const cudaError_t e = launch_build_kv(pl, di.sm_count, K, V, Kc, Vc, idx, kmean, vmean, build_ws, build_ws_bytes,
+                                        static_cast<cudaStream_t>(cuda_stream), &tmap_failed, nullptr, nullptr, 0, false, attn_ws);
+  rc = record_launch(e, tmap_failed);
   if (rc != AVGGT_OK) return rc;
   c.status_cleared = true;
   return enqueue_attn(pl, di, c);
@@ -259,8 +261,10 @@ int avggt_build_kv_indexed(const avggt_params* p, const int32_t* idx, int64_t n_
   rc = device_info(&di);
   if (rc != AVGGT_OK) return rc;
   if (ws_bytes < build_kv_min_ws_bytes(pl, di.sm_count)) return AVGGT_ERR_WORKSPACE_TOO_SMALL;
-  return record_cuda(launch_build_kv(pl, di.sm_count, K, V, Kc, Vc, nullptr, kmean, vmean, ws, ws_bytes,
-                                     static_cast<cudaStream_t>(cuda_stream), idx, slot_of_token));
+  bool tmap_failed = false;
+  const cudaError_t e = launch_build_kv(pl, di.sm_count, K, V, Kc, Vc, nullptr, kmean, vmean, ws, ws_bytes,
+                                        static_cast<cudaStream_t>(cuda_stream), &tmap_failed, idx, slot_of_token);
+  return record_launch(e, tmap_failed);
 }
 
 int avggt_global_attn_indexed(const avggt_params* p, int64_t n_kept, const int32_t* slot_of_token, const void* Q,
@@ -319,8 +323,7 @@ int avggt_project_build_kv(const avggt_params* p, int32_t model_dim, const void*
   bool tmap_failed = false;
   const cudaError_t e = launch_project_kv(pl, di.sm_count, model_dim, X, Wk, Wv, bias_k, bias_v, K, V, Kc, Vc, idx, kmean,
                                           vmean, ws, static_cast<cudaStream_t>(cuda_stream), &tmap_failed);
-  if (tmap_failed) return record_message("cuTensorMapEncodeTiled failed");
-  return record_cuda(e);
+  return record_launch(e, tmap_failed);
 }
 
 int avggt_build_kv_shard(const avggt_params* p, const void* K, const void* V, void* slot, int64_t slot_rows,
@@ -341,8 +344,10 @@ int avggt_build_kv_shard(const avggt_params* p, const void* K, const void* V, vo
   const size_t part = static_cast<size_t>(pl.H) * static_cast<size_t>(slot_rows) * pl.d;   // elements of the K part of a slot
   void* Vc = static_cast<char*>(slot) + part * 2;
   float* vsum = sums ? sums + static_cast<size_t>(pl.H) * pl.d : nullptr;
-  return record_cuda(launch_build_kv(pl, di.sm_count, K, V, slot, Vc, idx, sums, vsum, ws, ws_bytes,
-                                     static_cast<cudaStream_t>(cuda_stream), nullptr, nullptr, slot_rows, true));
+  bool tmap_failed = false;
+  const cudaError_t e = launch_build_kv(pl, di.sm_count, K, V, slot, Vc, idx, sums, vsum, ws, ws_bytes,
+                                        static_cast<cudaStream_t>(cuda_stream), &tmap_failed, nullptr, nullptr, slot_rows, true);
+  return record_launch(e, tmap_failed);
 }
 
 int avggt_shard_assemble(const avggt_params* p, const void* gathered, int32_t n_ranks, const int64_t* kept,

@@ -657,6 +657,7 @@ cudaError_t prepare_stream_kernels() {
 
 // The compact arrays as [kc_rows, H, d]: a box is all heads of `rows` rows.
 bool make_compact_tmap(CUtensorMap* tm, const Plan& pl, void* base, int64_t kc_rows, int rows) {
+  if (kc_rows >= (int64_t(1) << 40) / (pl.d * 2)) return false;   // the strides a tensor map can have
   const uint64_t dims[3] = {static_cast<uint64_t>(pl.d), static_cast<uint64_t>(pl.H), static_cast<uint64_t>(kc_rows)};
   const uint64_t strides[2] = {static_cast<uint64_t>(kc_rows) * pl.d * 2, static_cast<uint64_t>(pl.d) * 2};
   const uint32_t box[3] = {static_cast<uint32_t>(pl.d), static_cast<uint32_t>(pl.H), static_cast<uint32_t>(rows)};
@@ -664,7 +665,7 @@ bool make_compact_tmap(CUtensorMap* tm, const Plan& pl, void* base, int64_t kc_r
 }
 
 cudaError_t launch_stream(const Plan& pl, int grid, const void* K, const void* V, void* Kc, void* Vc, int64_t kc_rows, int32_t* idx,
-                          float* partials, const int32_t* slot_of_token, uint32_t* status, cudaStream_t st) {
+                          float* partials, const int32_t* slot_of_token, uint32_t* status, cudaStream_t st, bool* tmap_failed) {
   StreamArgs a;
   a.pl = pl;
   a.rule = make_window_rule(pl);
@@ -679,8 +680,10 @@ cudaError_t launch_stream(const Plan& pl, int grid, const void* K, const void* V
   a.partials = partials;
   a.status = status;
   CUtensorMap tm_kc = {}, tm_vc = {};
-  if (kc_rows > 0 && !(make_compact_tmap(&tm_kc, pl, Kc, kc_rows, 1) && make_compact_tmap(&tm_vc, pl, Vc, kc_rows, 1)))
-    return cudaErrorInvalidValue;
+  if (kc_rows > 0 && !(make_compact_tmap(&tm_kc, pl, Kc, kc_rows, 1) && make_compact_tmap(&tm_vc, pl, Vc, kc_rows, 1))) {
+    *tmap_failed = true;
+    return cudaSuccess;
+  }
   const cudaError_t e = prepare_stream_kernels();
   if (e != cudaSuccess) return e;
   return launch_dependent(pl.H <= 16 ? build_kv_stream_kernel<1> : build_kv_stream_kernel<2>, grid, kStreamThreads, kStreamSmemBytes, st,
@@ -688,7 +691,8 @@ cudaError_t launch_stream(const Plan& pl, int grid, const void* K, const void* V
 }
 
 cudaError_t launch_gather(const Plan& pl, int grid, const void* K, const void* V, void* Kc, void* Vc, int64_t kc_rows, int32_t* idx,
-                          const int32_t* caller_idx, uint32_t* status, float* zero_kmean, float* zero_vmean, cudaStream_t st) {
+                          const int32_t* caller_idx, uint32_t* status, float* zero_kmean, float* zero_vmean, cudaStream_t st,
+                          bool* tmap_failed) {
   GatherArgs a;
   a.pl = pl;
   a.by_Lc = make_divisor(pl.Lc > 0 ? pl.Lc : 1);
@@ -706,8 +710,10 @@ cudaError_t launch_gather(const Plan& pl, int grid, const void* K, const void* V
   a.zero_vmean = zero_vmean;
   CUtensorMap tm_kc = {}, tm_vc = {}, tm_kc_row = {}, tm_vc_row = {};
   if (kc_rows > 0 && !(make_compact_tmap(&tm_kc, pl, Kc, kc_rows, a.rows) && make_compact_tmap(&tm_vc, pl, Vc, kc_rows, a.rows) &&
-                       make_compact_tmap(&tm_kc_row, pl, Kc, kc_rows, 1) && make_compact_tmap(&tm_vc_row, pl, Vc, kc_rows, 1)))
-    return cudaErrorInvalidValue;
+                       make_compact_tmap(&tm_kc_row, pl, Kc, kc_rows, 1) && make_compact_tmap(&tm_vc_row, pl, Vc, kc_rows, 1))) {
+    *tmap_failed = true;
+    return cudaSuccess;
+  }
   const cudaError_t e = prepare_stream_kernels();
   if (e != cudaSuccess) return e;
   return launch_dependent(build_kv_gather_kernel, grid, 32, kStreamSmemBytes, st, tm_kc, tm_vc, tm_kc_row, tm_vc_row, a);
@@ -797,8 +803,9 @@ size_t build_kv_ws_bytes(const Plan& pl, int sm_count) {
 
 cudaError_t launch_build_kv(const Plan& pl, int sm_count, const void* K, const void* V, void* Kc, void* Vc,
                             int32_t* idx, float* kmean, float* vmean, void* ws, size_t ws_bytes, cudaStream_t st,
-                            const int32_t* caller_idx, int32_t* slot_of_token, int64_t kc_rows, bool sums_only,
+                            bool* tmap_failed, const int32_t* caller_idx, int32_t* slot_of_token, int64_t kc_rows, bool sums_only,
                             void* clear_status) {
+  *tmap_failed = false;
   if (kc_rows <= 0) kc_rows = pl.M;
   if (slot_of_token != nullptr) {
     // caller-chosen retained set: build the token -> compact position map first
@@ -836,9 +843,9 @@ cudaError_t launch_build_kv(const Plan& pl, int sm_count, const void* K, const v
   const bool zero_mean = pl.mean_fill != 0 && !do_mean;
   float* zk = zero_mean ? kmean : nullptr;
   float* zv = zero_mean ? vmean : nullptr;
-  const cudaError_t e = do_mean ? launch_stream(pl, grid, K, V, Kc, Vc, kc_rows, idx, partials, slot_of_token, status, st)
-                                : launch_gather(pl, grid, K, V, Kc, Vc, kc_rows, idx, caller_idx, status, zk, zv, st);
-  if (e != cudaSuccess || !do_mean) return e;
+  const cudaError_t e = do_mean ? launch_stream(pl, grid, K, V, Kc, Vc, kc_rows, idx, partials, slot_of_token, status, st, tmap_failed)
+                                : launch_gather(pl, grid, K, V, Kc, Vc, kc_rows, idx, caller_idx, status, zk, zv, st, tmap_failed);
+  if (e != cudaSuccess || *tmap_failed || !do_mean) return e;
   const int cols2 = 2 * pl.H * pl.d;
   const float inv_count = sums_only ? 1.0f : 1.0f / static_cast<float>(pl.n_dropped);
   return launch_dependent(mean_finalize_kernel, (cols2 + 31) / 32, 1024, 0, st, partials, grid, cols2, inv_count, kmean, vmean);

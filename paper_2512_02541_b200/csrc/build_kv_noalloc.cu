@@ -90,6 +90,8 @@ extern "C" int avggt_build_kv_noalloc(const avggt_params* p, const void* K, cons
   const int most = kStaticMaxBlocks / build_kv_blocks_per_sm();
   if (sm_eff > most) sm_eff = most;
   if (build_kv_ws_bytes(pl, sm_eff) > kStaticScratchBytes) return AVGGT_ERR_STATIC_SCRATCH;
-  return record_cuda(launch_build_kv(pl, sm_eff, K, V, Kc, Vc, idx, kmean, vmean, pd->scratch, kStaticScratchBytes,
-                                     static_cast<cudaStream_t>(cuda_stream)));
+  bool tmap_failed = false;
+  const cudaError_t e = launch_build_kv(pl, sm_eff, K, V, Kc, Vc, idx, kmean, vmean, pd->scratch, kStaticScratchBytes,
+                                        static_cast<cudaStream_t>(cuda_stream), &tmap_failed);
+  return record_launch(e, tmap_failed);
 }

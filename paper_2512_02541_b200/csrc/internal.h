@@ -17,6 +17,10 @@ int device_info(DeviceInfo* out);
 int record_cuda(cudaError_t e);
 // Keep `text` for avggt_last_cuda_error; returns AVGGT_ERR_CUDA.
 int record_message(const char* text);
+// The outcome of a launcher that encodes tensor maps.
+inline int record_launch(cudaError_t e, bool tmap_failed) {
+  return tmap_failed ? record_message("cuTensorMapEncodeTiled failed") : record_cuda(e);
+}
 
 // Launch of a kernel that may be scheduled, up to its grid_dependency_wait, while the kernel before it in the stream ends:
 // the launch and the preparation of the layer's kernels (tensor memory, barriers) hide behind one another.
@@ -61,8 +65,9 @@ size_t build_kv_min_ws_bytes(const Plan& pl, int sm_count);
 // kc_rows: rows per head of Kc / Vc (0 = M; larger when they are one rank's slot of an exchange buffer).
 // sums_only: kmean / vmean receive the un-normalised sums over the dropped rows instead of the means.
 // clear_status: the status block (kAttnStatusBytes) of the attention launch that follows in the stream, or null.
+// Returns cudaSuccess, or an error; *tmap_failed is set when a tensor map could not be encoded.
 cudaError_t launch_build_kv(const Plan& pl, int sm_count, const void* K, const void* V, void* Kc, void* Vc,
-                            int32_t* idx, float* kmean, float* vmean, void* ws, size_t ws_bytes, cudaStream_t st,
+                            int32_t* idx, float* kmean, float* vmean, void* ws, size_t ws_bytes, cudaStream_t st, bool* tmap_failed,
                             const int32_t* caller_idx = nullptr, int32_t* slot_of_token = nullptr,
                             int64_t kc_rows = 0, bool sums_only = false, void* clear_status = nullptr);
 

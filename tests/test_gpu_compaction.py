@@ -104,3 +104,17 @@ def test_a_workspace_for_a_block_per_sm():
     _check_build(ocfg, layer, K, V)
     with pytest.raises(P.AvggtError):
         P.avggt_build_kv(params, K, V, layer.Kc, layer.Vc, layer.idx, layer.kmean, layer.vmean, ws, half - 1)
+
+
+def test_a_tensor_map_that_cannot_be_encoded_is_named():
+    """Tensor maps have strides below 2^40 bytes; a slot of more rows than that is refused before anything is launched."""
+    wl = inputs.Workload("stride", 6, 37, 37, 5, 16, 64, 4, 1, 2, "iid")
+    params, _ = _cfgs(wl)
+    _, K, V = inputs.make_qkv(wl, seed=3, device="cuda")
+    layer = P.SubsampledGlobalAttention(params)
+    sums = torch.zeros((2, wl.n_heads, 64), device="cuda")
+    for p in (params, P.make_params(6, 37, 37, 5, 16, 64, 4, diag=0, mean_fill=0)):
+        with pytest.raises(P.AvggtError, match="cuTensorMapEncodeTiled"):
+            P.avggt_build_kv_shard(p, K, V, layer.Kc, 1 << 34, None, sums, layer.build_ws, layer.build_ws.numel())
+    torch.cuda.synchronize()
+    assert not sums.any()
