@@ -331,6 +331,7 @@ struct GatherArgs {
   int32_t rows;        // of a tile
   int32_t* idx;
   const int32_t* caller_idx;   // caller-chosen retained set: token of every compact row; else null
+  const int32_t* slot_of_token;   // and compact row of every token: of a token listed twice only this row is written
   uint32_t* status;
   float* zero_kmean;   // mean pair of a problem that drops nothing, or null
   float* zero_vmean;
@@ -389,8 +390,10 @@ build_kv_gather_kernel(const __grid_constant__ CUtensorMap tm_kc, const __grid_c
   const auto token = [&](uint32_t t) {
     const uint32_t m = t * rows + lane;
     if (t >= n_tiles || lane >= static_cast<int>(rows) || m >= M) return -1;
-    const int32_t tok = a.caller_idx != nullptr ? __ldcg(a.caller_idx + m) : token_of_compact(a, m);
-    return tok < pl.n_tok ? tok : -1;   // (entries of a caller's list that are no token are passed over)
+    if (a.caller_idx == nullptr) return token_of_compact(a, m);
+    const int32_t tok = __ldcg(a.caller_idx + m);
+    // (entries of a caller's list that are no token are passed over)
+    return tok >= 0 && tok < pl.n_tok && __ldcg(a.slot_of_token + tok) == static_cast<int32_t>(m) ? tok : -1;
   };
   const auto load = [&](int stage, int tok) {
     if (AVGGT_SKIP_TILE(pl.n_tok, stage)) return;
@@ -691,7 +694,7 @@ cudaError_t launch_stream(const Plan& pl, int grid, const void* K, const void* V
 }
 
 cudaError_t launch_gather(const Plan& pl, int grid, const void* K, const void* V, void* Kc, void* Vc, int64_t kc_rows, int32_t* idx,
-                          const int32_t* caller_idx, uint32_t* status, float* zero_kmean, float* zero_vmean, cudaStream_t st,
+                          const int32_t* caller_idx, const int32_t* slot_of_token, uint32_t* status, float* zero_kmean, float* zero_vmean, cudaStream_t st,
                           bool* tmap_failed) {
   GatherArgs a;
   a.pl = pl;
@@ -705,6 +708,7 @@ cudaError_t launch_gather(const Plan& pl, int grid, const void* K, const void* V
   a.rows = stream_rows(pl);
   a.idx = idx;
   a.caller_idx = caller_idx;
+  a.slot_of_token = slot_of_token;
   a.status = status;
   a.zero_kmean = zero_kmean;
   a.zero_vmean = zero_vmean;
@@ -844,7 +848,7 @@ cudaError_t launch_build_kv(const Plan& pl, int sm_count, const void* K, const v
   float* zk = zero_mean ? kmean : nullptr;
   float* zv = zero_mean ? vmean : nullptr;
   const cudaError_t e = do_mean ? launch_stream(pl, grid, K, V, Kc, Vc, kc_rows, idx, partials, slot_of_token, status, st, tmap_failed)
-                                : launch_gather(pl, grid, K, V, Kc, Vc, kc_rows, idx, caller_idx, status, zk, zv, st, tmap_failed);
+                                : launch_gather(pl, grid, K, V, Kc, Vc, kc_rows, idx, caller_idx, slot_of_token, status, zk, zv, st, tmap_failed);
   if (e != cudaSuccess || *tmap_failed || !do_mean) return e;
   const int cols2 = 2 * pl.H * pl.d;
   const float inv_count = sums_only ? 1.0f : 1.0f / static_cast<float>(pl.n_dropped);

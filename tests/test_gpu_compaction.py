@@ -90,6 +90,31 @@ def test_a_list_with_entries_that_are_no_token():
             assert (compact[:, 0] == 7).all() and (compact[:, -1] == 7).all()
 
 
+# on either side of the few-token limit of 16 heads (4,400 tokens), with a mean and without
+@pytest.mark.parametrize("n_frames", (3, 4))
+@pytest.mark.parametrize("mean_fill", (0, 2))
+def test_a_list_with_a_repeated_entry(n_frames, mean_fill):
+    """One of its two compact rows, the one that the map names, is written."""
+    wl = inputs.Workload("repeated", n_frames, 37, 37, 5, 16, 64, 4, 1, mean_fill, "iid")
+    params, _ = _cfgs(wl)
+    _, K, V = inputs.make_qkv(wl, seed=1, device="cuda")
+    n_kept = 300
+    idx = torch.sort(torch.randperm(wl.n_tokens, device="cuda")[:n_kept]).values.to(torch.int32)
+    for m in (1, 9, 100, n_kept - 1):   # within a tile of eight, across two, at the end
+        idx[m] = idx[m - 1]
+    Kc, Vc = (torch.full((wl.n_heads, n_kept, 64), 7.0, dtype=torch.bfloat16, device="cuda") for _ in range(2))
+    slots = torch.empty((wl.n_tokens,), dtype=torch.int32, device="cuda")
+    kmean, vmean = (torch.zeros((wl.n_heads, 64), device="cuda") for _ in range(2))
+    ws = torch.empty((P.avggt_workspace_bytes(params)[0],), dtype=torch.uint8, device="cuda")
+    P.avggt_build_kv_indexed(params, idx, n_kept, K, V, Kc, Vc, slots, kmean, vmean, ws, ws.numel())
+    torch.cuda.synchronize()
+    named = slots[idx.long()] == torch.arange(n_kept, dtype=torch.int32, device="cuda")
+    assert int((~named).sum()) == 4
+    for full, compact in ((K, Kc), (V, Vc)):
+        assert torch.equal(compact[:, named], full[idx.long()[named]].transpose(0, 1))
+        assert (compact[:, ~named] == 7).all()
+
+
 def test_a_workspace_for_a_block_per_sm():
     """Above 16 heads a call gets by with half of what avggt_workspace_bytes asks for, on half as many blocks."""
     wl = inputs.Workload("half", 6, 37, 37, 5, 20, 64, 4, 1, 2, "iid")
