@@ -325,7 +325,7 @@ struct GatherArgs {
   Divisor by_Lc, by_kept_w;
   const uint8_t* K;
   const uint8_t* V;
-  uint4* Kc;           // as in StreamArgs
+  uint4* Kc;           // where a tile is not stored whole (and as in StreamArgs)
   uint4* Vc;
   int64_t kc_rows;
   int32_t rows;        // of a tile
@@ -359,8 +359,7 @@ __device__ __forceinline__ int32_t token_of_compact(const GatherArgs& a, uint32_
 }
 
 __global__ void __launch_bounds__(32)
-build_kv_gather_kernel(const __grid_constant__ CUtensorMap tm_kc, const __grid_constant__ CUtensorMap tm_vc,
-                       const __grid_constant__ CUtensorMap tm_kc_row, const __grid_constant__ CUtensorMap tm_vc_row, const GatherArgs a) {
+build_kv_gather_kernel(const __grid_constant__ CUtensorMap tm_kc, const __grid_constant__ CUtensorMap tm_vc, const GatherArgs a) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* stages = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~uintptr_t(127));
   __shared__ __align__(8) uint64_t full[kStreamStages];
@@ -442,19 +441,24 @@ build_kv_gather_kernel(const __grid_constant__ CUtensorMap tm_kc, const __grid_c
       const int tok = toks[s];
       const uint32_t m0 = t * rows;
       if (tok >= 0 && a.idx != nullptr) a.idx[m0 + lane] = tok;
-      const uint32_t src = smem_u32(stages + 2 * s * kStreamBytes);
-      uint32_t have = __ballot_sync(0xffffffffu, tok >= 0);
-      if (lane == 0) {
-        if (__popc(have) == static_cast<int>(rows)) {
-          tma_store_3d(&tm_kc, src, 0, 0, m0);
-          tma_store_3d(&tm_vc, src + kStreamBytes, 0, 0, m0);
-        } else {   // the last tile (what follows the retained rows is not this call's), or one with rows passed over
-          for (; have != 0; have &= have - 1) {
-            const int r = __ffs(have) - 1;
-            tma_store_3d(&tm_kc_row, src + r * row_bytes, 0, 0, m0 + r);
-            tma_store_3d(&tm_vc_row, src + kStreamBytes + r * row_bytes, 0, 0, m0 + r);
+      const uint8_t* src = stages + 2 * s * kStreamBytes;
+      const uint32_t have = __ballot_sync(0xffffffffu, tok >= 0), exist = M - m0 < rows ? M - m0 : rows;
+      if (__popc(have) == static_cast<int>(exist)) {
+        if (lane == 0) {   // (rows of the box beyond the last compact row are not written: the tensor map ends there)
+          tma_store_3d(&tm_kc, smem_u32(src), 0, 0, m0);
+          tma_store_3d(&tm_vc, smem_u32(src) + kStreamBytes, 0, 0, m0);
+        }
+      } else {   // with rows passed over
+        for (uint32_t left_rows = have; left_rows != 0; left_rows &= left_rows - 1) {
+          const int r = __ffs(left_rows) - 1;
+          for (int c = lane; c < pl.H * 8; c += 32) {
+            const size_t at = (static_cast<size_t>(c >> 3) * static_cast<size_t>(a.kc_rows) + m0 + r) * 8u + (c & 7);
+            a.Kc[at] = *reinterpret_cast<const uint4*>(src + r * row_bytes + c * 16);
+            a.Vc[at] = *reinterpret_cast<const uint4*>(src + kStreamBytes + r * row_bytes + c * 16);
           }
         }
+      }
+      if (lane == 0) {
         bulk_commit();
         if (more) bulk_wait_read<1>();   // the stores of the tile before this one have read their stage
       }
@@ -658,10 +662,10 @@ cudaError_t prepare_stream_kernels() {
   return cudaSuccess;
 }
 
-// The compact arrays as [kc_rows, H, d]: a box is all heads of `rows` rows.
+// The compact arrays as [M, H, d], a head every kc_rows rows: a box is all heads of `rows` rows.
 bool make_compact_tmap(CUtensorMap* tm, const Plan& pl, void* base, int64_t kc_rows, int rows) {
   if (kc_rows >= (int64_t(1) << 40) / (pl.d * 2)) return false;   // the strides a tensor map can have
-  const uint64_t dims[3] = {static_cast<uint64_t>(pl.d), static_cast<uint64_t>(pl.H), static_cast<uint64_t>(kc_rows)};
+  const uint64_t dims[3] = {static_cast<uint64_t>(pl.d), static_cast<uint64_t>(pl.H), static_cast<uint64_t>(pl.M)};
   const uint64_t strides[2] = {static_cast<uint64_t>(kc_rows) * pl.d * 2, static_cast<uint64_t>(pl.d) * 2};
   const uint32_t box[3] = {static_cast<uint32_t>(pl.d), static_cast<uint32_t>(pl.H), static_cast<uint32_t>(rows)};
   return make_tmap_bf16(tm, base, 3, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_NONE);
@@ -683,7 +687,7 @@ cudaError_t launch_stream(const Plan& pl, int grid, const void* K, const void* V
   a.partials = partials;
   a.status = status;
   CUtensorMap tm_kc = {}, tm_vc = {};
-  if (kc_rows > 0 && !(make_compact_tmap(&tm_kc, pl, Kc, kc_rows, 1) && make_compact_tmap(&tm_vc, pl, Vc, kc_rows, 1))) {
+  if (pl.M > 0 && !(make_compact_tmap(&tm_kc, pl, Kc, kc_rows, 1) && make_compact_tmap(&tm_vc, pl, Vc, kc_rows, 1))) {
     *tmap_failed = true;
     return cudaSuccess;
   }
@@ -712,15 +716,14 @@ cudaError_t launch_gather(const Plan& pl, int grid, const void* K, const void* V
   a.status = status;
   a.zero_kmean = zero_kmean;
   a.zero_vmean = zero_vmean;
-  CUtensorMap tm_kc = {}, tm_vc = {}, tm_kc_row = {}, tm_vc_row = {};
-  if (kc_rows > 0 && !(make_compact_tmap(&tm_kc, pl, Kc, kc_rows, a.rows) && make_compact_tmap(&tm_vc, pl, Vc, kc_rows, a.rows) &&
-                       make_compact_tmap(&tm_kc_row, pl, Kc, kc_rows, 1) && make_compact_tmap(&tm_vc_row, pl, Vc, kc_rows, 1))) {
+  CUtensorMap tm_kc = {}, tm_vc = {};
+  if (pl.M > 0 && !(make_compact_tmap(&tm_kc, pl, Kc, kc_rows, a.rows) && make_compact_tmap(&tm_vc, pl, Vc, kc_rows, a.rows))) {
     *tmap_failed = true;
     return cudaSuccess;
   }
   const cudaError_t e = prepare_stream_kernels();
   if (e != cudaSuccess) return e;
-  return launch_dependent(build_kv_gather_kernel, grid, 32, kStreamSmemBytes, st, tm_kc, tm_vc, tm_kc_row, tm_vc_row, a);
+  return launch_dependent(build_kv_gather_kernel, grid, 32, kStreamSmemBytes, st, tm_kc, tm_vc, a);
 }
 
 // Exchange buffer [n_ranks][2][H][slot_rows][d] (every rank's compact K then V, padded to slot_rows rows per
