@@ -52,12 +52,17 @@ __device__ __forceinline__ void add_bf16x8(float (&acc)[8], const uint4& v) {
 // tokens, a ninth retained, 107.0 -> 102.5.  Stages of 16 + 16 KB, three in each of two blocks per SM: six in one block 377 us (14.0 at 13,740 tokens),
 // four 356 (14.3), three of 32 + 32 KB 353 (14.2); of 8 + 8 KB 536 and more in one block (the copying warp's chain of waits per tile),
 // 362 in two; two of 16 + 16 KB in two blocks 395, in three 355.
+//
+// Where a block has a few tiles only, what follows the last copy counts: an adding thread reads four rows before it adds the first of them.
+// Row by row, a ninth retained, the kernel was slower than a warp per row: 8,244 tokens of 12 heads 11.8 us against 11.1, now 10.2;
+// 5,496 of 20 heads 12.2 against 11.9, now 11.1; 8,244 of 32 heads 18.9 against 18.6, now 18.5; 137,400 of 16 heads 102.5, now 100.2.
 constexpr int kStreamSums = 256;                    // adding threads
 constexpr int kStreamThreads = kStreamSums + 32;    // and the warp that copies
 constexpr int kStreamBlocks = 2;                    // per SM
 constexpr int kStreamStages = 3;
 constexpr uint32_t kStreamBytes = 16 * 1024;        // of K, and of V, in a stage (at most)
 constexpr int kStreamRows = 32;                     // rows of a tile (at most): the copying warp has a lane for each
+constexpr int kStreamTogether = 4;                  // rows that an adding thread reads before it adds the first
 constexpr int kStreamFlush = 8;                     // tiles after which a thread's sums move on: short chains round less
 constexpr size_t kStreamSmemBytes = 2 * kStreamStages * kStreamBytes + 128;
 
@@ -261,17 +266,27 @@ build_kv_stream_kernel(const __grid_constant__ CUtensorMap tm_kc, const __grid_c
       const uint32_t n = n_tok - t * rows < rows ? n_tok - t * rows : rows;
       const uint32_t kept = kept_mask[stage];
       if (group < groups) {
-        for (uint32_t r = group; r < n; r += groups) {
-          if ((kept >> r) & 1u) continue;
+        for (uint32_t r0 = group; r0 < n; r0 += kStreamTogether * groups) {
+          uint4 v[kStreamTogether][PASSES];   // zeros, which add nothing, for a row that is retained or does not exist
 #pragma unroll
-          for (int p = 0; p < PASSES; ++p) {
-            if (PASSES > 1 && c0 + p * kStreamSums >= chunks) break;
-            const uint4 v = *reinterpret_cast<const uint4*>(src + at[p] + r * row_bytes);
-            run[p][0] = add_f32x2(run[p][0], unpack_bf16x2(v.x));
-            run[p][1] = add_f32x2(run[p][1], unpack_bf16x2(v.y));
-            run[p][2] = add_f32x2(run[p][2], unpack_bf16x2(v.z));
-            run[p][3] = add_f32x2(run[p][3], unpack_bf16x2(v.w));
+          for (int i = 0; i < kStreamTogether; ++i) {
+            const uint32_t r = r0 + i * groups;
+            const bool add = r < n && ((kept >> r) & 1u) == 0;
+#pragma unroll
+            for (int p = 0; p < PASSES; ++p) {
+              v[i][p] = make_uint4(0u, 0u, 0u, 0u);
+              if (add && (PASSES == 1 || c0 + p * kStreamSums < chunks)) v[i][p] = *reinterpret_cast<const uint4*>(src + at[p] + r * row_bytes);
+            }
           }
+#pragma unroll
+          for (int i = 0; i < kStreamTogether; ++i)
+#pragma unroll
+            for (int p = 0; p < PASSES; ++p) {
+              run[p][0] = add_f32x2(run[p][0], unpack_bf16x2(v[i][p].x));
+              run[p][1] = add_f32x2(run[p][1], unpack_bf16x2(v[i][p].y));
+              run[p][2] = add_f32x2(run[p][2], unpack_bf16x2(v[i][p].z));
+              run[p][3] = add_f32x2(run[p][3], unpack_bf16x2(v[i][p].w));
+            }
         }
       }
       __syncwarp();
