@@ -335,6 +335,13 @@ build_kv_stream_kernel(const __grid_constant__ CUtensorMap tm_kc, const __grid_c
 // whole tile per array to the head-major places.  HBM is the bound.  Against a warp per token with 16-byte loads: 457,542 tokens of
 // 16 heads, a quarter retained (1.0 GB) 233 -> 171 us (5.8 TB/s), 137,400 tokens all retained 203 -> 185 us (6.1 TB/s), 82,440 tokens, a
 // ninth retained, 21 -> 10 us, 137,400 tokens of 6 heads, a quarter retained, 38 -> 17 us.
+//
+// Above 16 heads a block per SM has the three stages, 20 + 20 KB each: with two blocks of 16 + 16 KB a tile is few rows, and where all rows are
+// retained the kernel was slower than a warp per token.  A warp per token, two blocks, one of 32 + 32, of 24 + 24 and of 20 + 20 KB, us: 137,400
+// tokens of 24 heads 296, 311, 300, 289, 274; of 28 346, 354, 352, 332, 320; 54,960 of 32 160, 165, 161, 160, 157; 137,400 of 20 heads, a quarter
+// retained, 109, 70, 68, 67, 65.
+constexpr uint32_t kGatherBytesManyHeads = 20 * 1024;
+constexpr size_t gather_smem_bytes(uint32_t stage_bytes) { return 2 * kStreamStages * stage_bytes + 128; }
 struct GatherArgs {
   Plan pl;
   Divisor by_Lc, by_kept_w;
@@ -343,6 +350,7 @@ struct GatherArgs {
   uint4* Kc;           // where a tile is not stored whole (and as in StreamArgs)
   uint4* Vc;
   int64_t kc_rows;
+  uint32_t stage_bytes;   // of K, and of V, in a stage
   int32_t rows;        // of a tile
   int32_t* idx;
   const int32_t* caller_idx;   // caller-chosen retained set: token of every compact row; else null
@@ -413,7 +421,7 @@ build_kv_gather_kernel(const __grid_constant__ CUtensorMap tm_kc, const __grid_c
     if (AVGGT_SKIP_TILE(pl.n_tok, stage)) return;
     const uint32_t have = __ballot_sync(0xffffffffu, tok >= 0);
     const int tok0 = __shfl_sync(0xffffffffu, tok, 0);
-    const uint32_t fb = smem_u32(&full[stage]), dst = smem_u32(stages + 2 * stage * kStreamBytes);
+    const uint32_t fb = smem_u32(&full[stage]), dst = smem_u32(stages + 2 * stage * a.stage_bytes);
     const uint32_t bytes = __popc(have) * row_bytes;
     if (lane == 0) mbar_arrive_expect_tx(fb, 2 * bytes);
     __syncwarp();
@@ -421,11 +429,11 @@ build_kv_gather_kernel(const __grid_constant__ CUtensorMap tm_kc, const __grid_c
     if ((have & (have + 1)) == 0 && __all_sync(0xffffffffu, tok < 0 || tok == tok0 + lane)) {
       if (lane == 0 && have != 0) {
         bulk_load(dst, a.K + static_cast<size_t>(tok0) * row_bytes, bytes, fb);
-        bulk_load(dst + kStreamBytes, a.V + static_cast<size_t>(tok0) * row_bytes, bytes, fb);
+        bulk_load(dst + a.stage_bytes, a.V + static_cast<size_t>(tok0) * row_bytes, bytes, fb);
       }
     } else if (tok >= 0) {
       bulk_load(dst + lane * row_bytes, a.K + static_cast<size_t>(tok) * row_bytes, row_bytes, fb);
-      bulk_load(dst + kStreamBytes + lane * row_bytes, a.V + static_cast<size_t>(tok) * row_bytes, row_bytes, fb);
+      bulk_load(dst + a.stage_bytes + lane * row_bytes, a.V + static_cast<size_t>(tok) * row_bytes, row_bytes, fb);
     }
     __syncwarp();
   };
@@ -456,12 +464,12 @@ build_kv_gather_kernel(const __grid_constant__ CUtensorMap tm_kc, const __grid_c
       const int tok = toks[s];
       const uint32_t m0 = t * rows;
       if (tok >= 0 && a.idx != nullptr) a.idx[m0 + lane] = tok;
-      const uint8_t* src = stages + 2 * s * kStreamBytes;
+      const uint8_t* src = stages + 2 * s * a.stage_bytes;
       const uint32_t have = __ballot_sync(0xffffffffu, tok >= 0), exist = M - m0 < rows ? M - m0 : rows;
       if (__popc(have) == static_cast<int>(exist)) {
         if (lane == 0) {   // (rows of the box beyond the last compact row are not written: the tensor map ends there)
           tma_store_3d(&tm_kc, smem_u32(src), 0, 0, m0);
-          tma_store_3d(&tm_vc, smem_u32(src) + kStreamBytes, 0, 0, m0);
+          tma_store_3d(&tm_vc, smem_u32(src) + a.stage_bytes, 0, 0, m0);
         }
       } else {   // with rows passed over
         for (uint32_t left_rows = have; left_rows != 0; left_rows &= left_rows - 1) {
@@ -469,7 +477,7 @@ build_kv_gather_kernel(const __grid_constant__ CUtensorMap tm_kc, const __grid_c
           for (int c = lane; c < pl.H * 8; c += 32) {
             const size_t at = (static_cast<size_t>(c >> 3) * static_cast<size_t>(a.kc_rows) + m0 + r) * 8u + (c & 7);
             a.Kc[at] = *reinterpret_cast<const uint4*>(src + r * row_bytes + c * 16);
-            a.Vc[at] = *reinterpret_cast<const uint4*>(src + kStreamBytes + r * row_bytes + c * 16);
+            a.Vc[at] = *reinterpret_cast<const uint4*>(src + a.stage_bytes + r * row_bytes + c * 16);
           }
         }
       }
@@ -653,8 +661,8 @@ __global__ void scatter_slots_kernel(const int32_t* idx, int64_t M, int32_t* __r
   }
 }
 
-int stream_rows(const Plan& pl) {
-  const int rows = static_cast<int>(kStreamBytes) / (pl.H * 128);
+int stream_rows(const Plan& pl, uint32_t stage_bytes = kStreamBytes) {
+  const int rows = static_cast<int>(stage_bytes) / (pl.H * 128);
   return rows < kStreamRows ? rows : kStreamRows;
 }
 
@@ -668,11 +676,13 @@ cudaError_t prepare_stream_kernels() {
   if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
   std::lock_guard<std::mutex> lock(mu);
   if (ready[dev]) return cudaSuccess;
-  for (const void* kernel : {reinterpret_cast<const void*>(build_kv_stream_kernel<1>), reinterpret_cast<const void*>(build_kv_stream_kernel<2>),
-                             reinterpret_cast<const void*>(build_kv_gather_kernel)}) {
+  for (const void* kernel : {reinterpret_cast<const void*>(build_kv_stream_kernel<1>), reinterpret_cast<const void*>(build_kv_stream_kernel<2>)}) {
     e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kStreamSmemBytes));
     if (e != cudaSuccess) return e;
   }
+  e = cudaFuncSetAttribute(build_kv_gather_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           static_cast<int>(gather_smem_bytes(kGatherBytesManyHeads)));
+  if (e != cudaSuccess) return e;
   ready[dev] = true;
   return cudaSuccess;
 }
@@ -712,7 +722,7 @@ cudaError_t launch_stream(const Plan& pl, int grid, const void* K, const void* V
                           tm_kc, tm_vc, a);
 }
 
-cudaError_t launch_gather(const Plan& pl, int grid, const void* K, const void* V, void* Kc, void* Vc, int64_t kc_rows, int32_t* idx,
+cudaError_t launch_gather(const Plan& pl, int sm_count, const void* K, const void* V, void* Kc, void* Vc, int64_t kc_rows, int32_t* idx,
                           const int32_t* caller_idx, const int32_t* slot_of_token, uint32_t* status, float* zero_kmean, float* zero_vmean, cudaStream_t st,
                           bool* tmap_failed) {
   GatherArgs a;
@@ -724,7 +734,8 @@ cudaError_t launch_gather(const Plan& pl, int grid, const void* K, const void* V
   a.Kc = static_cast<uint4*>(Kc);
   a.Vc = static_cast<uint4*>(Vc);
   a.kc_rows = kc_rows;
-  a.rows = stream_rows(pl);
+  a.stage_bytes = pl.H > 16 ? kGatherBytesManyHeads : kStreamBytes;
+  a.rows = stream_rows(pl, a.stage_bytes);
   a.idx = idx;
   a.caller_idx = caller_idx;
   a.slot_of_token = slot_of_token;
@@ -738,7 +749,9 @@ cudaError_t launch_gather(const Plan& pl, int grid, const void* K, const void* V
   }
   const cudaError_t e = prepare_stream_kernels();
   if (e != cudaSuccess) return e;
-  return launch_dependent(build_kv_gather_kernel, grid, 32, kStreamSmemBytes, st, tm_kc, tm_vc, a);
+  const int64_t tiles = (pl.M + a.rows - 1) / a.rows, most = static_cast<int64_t>(sm_count) * (pl.H > 16 ? 1 : kStreamBlocks);
+  const int grid = static_cast<int>(tiles < 1 ? 1 : tiles < most ? tiles : most);
+  return launch_dependent(build_kv_gather_kernel, grid, 32, gather_smem_bytes(a.stage_bytes), st, tm_kc, tm_vc, a);
 }
 
 // Exchange buffer [n_ranks][2][H][slot_rows][d] (every rank's compact K then V, padded to slot_rows rows per
@@ -804,7 +817,7 @@ int small_ranks(const Plan& pl, int sm_count) {
 
 int build_kv_blocks_per_sm() { return kStreamBlocks; }
 
-// Blocks of build_kv_stream_kernel; build_kv_gather_kernel has as many.
+// Blocks of build_kv_stream_kernel.
 int build_kv_grid(const Plan& pl, int sm_count) {
   const int rows = stream_rows(pl);
   const int64_t tiles = (pl.n_tok + rows - 1) / rows;
@@ -866,7 +879,7 @@ cudaError_t launch_build_kv(const Plan& pl, int sm_count, const void* K, const v
   float* zk = zero_mean ? kmean : nullptr;
   float* zv = zero_mean ? vmean : nullptr;
   const cudaError_t e = do_mean ? launch_stream(pl, grid, K, V, Kc, Vc, kc_rows, idx, partials, slot_of_token, status, st, tmap_failed)
-                                : launch_gather(pl, grid, K, V, Kc, Vc, kc_rows, idx, caller_idx, slot_of_token, status, zk, zv, st, tmap_failed);
+                                : launch_gather(pl, sm_count, K, V, Kc, Vc, kc_rows, idx, caller_idx, slot_of_token, status, zk, zv, st, tmap_failed);
   if (e != cudaSuccess || *tmap_failed || !do_mean) return e;
   const int cols2 = 2 * pl.H * pl.d;
   const float inv_count = sums_only ? 1.0f : 1.0f / static_cast<float>(pl.n_dropped);

@@ -53,8 +53,9 @@ def test_nothing_dropped(n_frames):
 
 
 # Tiles of 8 tokens (16 heads) or 4 (32), 296 blocks, three tiles in flight in each: token counts around a tile, around the tiles of all
-# blocks together, and around the ring; with a mean and, over the compact rows, without
-@pytest.mark.parametrize("heads,n_tok", [(16, t) for t in (4401, 4409, 4736 * 8 - 1, 7104, 7105, 7111)] + [(32, 2201), (32, 3 * 1184 + 5)])
+# blocks together, and around the ring; with a mean and, over the compact rows (tiles of 6 of 24 heads, of 5 of 32, 148 blocks), without
+@pytest.mark.parametrize("heads,n_tok", [(16, t) for t in (4401, 4409, 4736 * 8 - 1, 7104, 7105, 7111)] + [(32, 2201), (32, 3 * 1184 + 5)]
+                         + [(24, t) for t in (2663, 2664, 2665)] + [(32, 2221)])
 @pytest.mark.parametrize("sigma,mean_fill", [(4, 2), (4, 0), (1, 2)])
 def test_tokens_around_a_tile(heads, n_tok, sigma, mean_fill):
     wl = inputs.Workload("tiles", 1, 3, (n_tok - 2) // 3, 2 + (n_tok - 2) % 3, heads, 64, sigma, 1, mean_fill, "iid")
