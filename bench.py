@@ -217,6 +217,16 @@ def fractions(tflops, peaks):
             "frac_of_measured_sustained": tflops / peaks["bf16_tflops_sustained"]}
 
 
+def compaction_kernels(n_tok, n_dropped, H, mean_fill):
+    """The kernels that the compaction of so many tokens launches on 148 SMs, its own first."""
+    blocks = 8 if H <= 6 else 4 if H <= 18 else 2          # per cluster of the few-token kernel, 1,100 tokens each
+    if n_tok <= 1100 * blocks:
+        return ["build_kv_small_kernel"]
+    if mean_fill and n_dropped > 0:
+        return ["build_kv_stream_kernel", "mean_finalize_kernel"]
+    return ["build_kv_gather_kernel"]
+
+
 def build_bytes(n_q, M, H, d, mean_fill):
     """Algorithmic bytes of one compaction launch: every K/V row read once when the mean is taken (else only the
     retained rows), every retained row written once."""
@@ -493,6 +503,7 @@ def run_ours(args, wl):
         peak_tf = peaks["bf16_tflops_sustained"] if long_run else peaks["bf16_tflops"]
         M_local = layer.kept[rank] if shard_mode else M
         bbytes = build_bytes(n_q_local, M_local, H, d, wl.mean_fill)
+        build_kernels = compaction_kernels(n_q_local, n_q_local - M_local, H, wl.mean_fill)
         build_gbs = bbytes / (build_avg * 1e-3) / 1e9
         if shard_mode:
             par, scaling = f"{world} ranks, {wl.n_frames} frames split {[b - a for a, b in layer.ranges]}", "strong"
@@ -524,15 +535,15 @@ def run_ours(args, wl):
             "frame_attn_tflops": (4.0 * n_q_local * wl.tokens_per_frame * H * d / (frame_ms * 1e-3) / 1e12) if frame_ms else None,
             "project_build_kv": proj,
             "roofline": roof,
-            "roofline_build_kv": {"bound": "hbm", "kernel": "build_kv_stream_kernel", "achieved": build_gbs,
+            "roofline_build_kv": {"bound": "hbm", "kernel": build_kernels[0], "achieved": build_gbs,
                                   "peak": peaks["hbm_gbs"], "unit": "GB/s", "frac": build_gbs / peaks["hbm_gbs"],
                                   "frac_of_nominal_8000": build_gbs / NOMINAL_HBM_GBS,
-                                  "traffic": NCU_TRAFFIC.get(wl.name, {}).get("build_kv_stream_kernel") if not shard_mode else None,
+                                  "traffic": NCU_TRAFFIC.get(wl.name, {}).get(build_kernels[0]) if not shard_mode else None,
                                   "bytes_per_launch": bbytes,
                                   "peak_source": f"{peaks['source']} copy bandwidth"},
             "e2e": {"value": units_all * e2e_steps / (e2e_ms * 1e-3), "unit": UNIT,
                     "h2d_bytes_per_step": in_bytes, "d2h_bytes_per_step": out_bytes, "steps": e2e_steps},
-            "gpu_launches": (5 if shard_mode else 3) * args.steps,
+            "gpu_launches": (len(build_kernels) + (4 if shard_mode else 2)) * args.steps,
             "clocks": clocks,
         }
         if cpu_tensors is not None:
