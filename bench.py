@@ -42,8 +42,8 @@ from paper_2512_02541_b200 import inputs  # noqa: E402
 # profiles/; None where no capture covers the workload.  Both kernels are captured on the 30-frame copy of the
 # headline layer (profiles/*_vggt_n30_s9.md); their traffic is proportional to the frame count, so the 800-frame
 # figures are those captures x 800/30.
-_ATTN_N30_S9 = 275201024.0 + 66723840.0
-_BUILD_N30_S9 = 168868096.0 + 13229056.0
+_ATTN_N30_S9 = 275335168.0 + 66518528.0
+_BUILD_N30_S9 = 168873216.0 + 15323136.0
 NCU_TRAFFIC = {
     "vggt_n30_s9": {"global_attn_kernel": _ATTN_N30_S9, "build_kv_stream_kernel": _BUILD_N30_S9},
     "vggt_n800_s9": {"global_attn_kernel": _ATTN_N30_S9 * 800 / 30, "build_kv_stream_kernel": _BUILD_N30_S9 * 800 / 30},

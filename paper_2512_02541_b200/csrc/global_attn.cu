@@ -962,8 +962,8 @@ __device__ __forceinline__ void st_rows16(uint32_t addr, uint32_t r0, uint32_t r
 // An item boundary is bound by instructions: all four warps of a scheduler are in it at once.  Before, with the own rows and the mean
 // pair read from global memory 16 bytes per thread, V and the result turned around by shuffles within the quad, and the item found
 // anew by every warp, a boundary cost the layer 1,215 instructions a warp, as many as 4.6 key steps, and the last epilogue of a launch
-// 4,900 clocks.  Layer of 10 frames 269 -> 261 us, 31 frames 1154 -> 1126 us, 4 frames of 16 x 16 17.2 -> 16.8 us, frame
-// attention of 100 frames 1090 -> 1062 us, of 10 frames 116 -> 114.5 us.
+// 4,900 clocks.  Layer of 10 frames of 37 x 37, a quarter retained, 280 -> 272.5 us, of 31 frames of 28 x 37, a ninth retained, with
+// log-sum-exp 896 -> 874 us, of 4 frames of 16 x 16 17.1 -> 16.7 us, frame attention of 100 frames of 37 x 37 1122 -> 1099 us, of 10 122.5 -> 120.3 us.
 template <bool kLse, bool kExtra>
 __device__ __forceinline__ bool softmax_epilogue(const AttnArgs& a, Barriers* bars, const SoftmaxThread& me, const RowResults* res,
                                                  const ItemInfo* infos, const SmemLayout& sm, int n, int last) {

@@ -57,7 +57,7 @@ def test_a_wait_that_runs_out_is_reported_and_the_context_stays_usable():
     assert flag == 1 and block == 0                       # the first thread block gave up ...
     # ... in whichever of its roles had waited longest on the consequences of the missing K tile: the producer
     # on a ring stage that is never released (sites 10, 11), an MMA issuer on the tile itself (24, 25) or a
-    # softmax warp on the scores of step 1 (40, 41); all within the first cycle of the four-stage ring
+    # softmax warp on the scores of step 1 (40, 41); all within the item's first six steps
     assert site in (10, 11, 24, 25, 40, 41) and iteration <= 5
     # the items of the last head were not begun: the blocks had seen the time-out by then
     assert torch.isnan(O[:, wl.n_heads - 1].float()).any()
